@@ -65,6 +65,14 @@ def _channels(rng, lo, hi, step=8):
 
 
 def draw(rng):
+    have = [{k: v for k, v in c.items() if k != "name"} for c in listed()]
+    while True:
+        c = _draw(rng)
+        if c not in have:
+            return c
+
+
+def _draw(rng):
     kind = rng.choice(["layer", "layer", "layer", "resnet", "convnext", "train", "train", "masks"])
     if kind == "resnet":
         return dict(kind=kind, batch=_log_int(rng, 1, 250))
@@ -157,8 +165,9 @@ def prepare(case, seed):
     s["x"] = _randn(g, case["n"], case["h"], case["w"], case["cin"])
     s["bias"] = _randn(g, case["cout"], std=0.1, dtype=torch.float32)
     w = _randn(g, case["cout"], case["k"], case["k"], k_in, std=1.0 / math.sqrt(case["k"] ** 2 * k_in))
+    s["w"] = w
     if kind == "train":
-        s["w"], n_groups = w, w.numel() // 4
+        n_groups = w.numel() // 4
         s["logits"], s["noise"] = _randn(g, n_groups, 6, dtype=torch.float32), _gumbel(g, n_groups, 6)
         s["dy"] = _randn(g, case["n"], ho, wo, case["cout"])
         s["m"], s["v"] = torch.zeros_like(s["logits"]), torch.zeros_like(s["logits"])
@@ -284,3 +293,137 @@ def tolerance(case):
     if case["kind"] == "convnext":
         return dict(rel=3.5e-2, max=0.15)
     return dict(rel=7e-3, max=2e-2)
+
+
+# ----------------------------------------------------------------------------- the same in 64 bits, plain torch
+_PAIRS = ((0, 1), (0, 2), (0, 3), (1, 2), (1, 3), (2, 3))   # the positions the six patterns keep
+
+
+def _keep_two(w):
+    """w with the two largest magnitudes of each group of four kept (of equal ones the earlier), fp64."""
+    v = w.double().reshape(-1, 4)
+    a = v.abs()
+    earlier = torch.ones(4, 4, dtype=torch.bool, device=v.device).tril(-1)                   # [i, j]: j before i
+    beaten = (a[:, None, :] > a[:, :, None]) | ((a[:, None, :] == a[:, :, None]) & earlier)
+    return torch.where(beaten.sum(2) < 2, v, torch.zeros_like(v)).reshape(w.shape)
+
+
+def _patches(t, kh, kw, stride, ho, wo):
+    return t[:, kh:kh + stride * (ho - 1) + 1:stride, kw:kw + stride * (wo - 1) + 1:stride]
+
+
+def _conv(x, w, bias, stride=1, pad=0, act="none", res=None):
+    """One matrix product per filter tap; x [N, H, W, C] and w [C_out, KH, KW, C]."""
+    w = w.double()
+    kh, kw = w.shape[1:3]
+    xp = torch.nn.functional.pad(x, (0, 0, pad, pad, pad, pad)).double()
+    ho, wo = (xp.shape[1] - kh) // stride + 1, (xp.shape[2] - kw) // stride + 1
+    y = bias.double().expand(x.shape[0], ho, wo, w.shape[0]).clone()
+    for i in range(kh):
+        for j in range(kw):
+            y += _patches(xp, i, j, stride, ho, wo) @ w[:, i, j].T
+    if res is not None:
+        y += res.double()
+    return y.relu_() if act == "relu" else torch.nn.functional.gelu(y) if act == "gelu" else y
+
+
+def _exact_layer(case, s, w):
+    x, groups = s["x"], case["groups"]
+    if case["dtype"] == "e4m3":
+        x = x.float().clamp(-448, 448).to(torch.float8_e4m3fn).float()
+        w = (w.float() * W_SCALE).clamp(-448, 448).to(torch.float8_e4m3fn).float()
+    w = _keep_two(w)
+    if case["dtype"] == "e4m3":
+        w = w / W_SCALE
+    y = [_conv(x_g, w_g, b_g, case["stride"], case["pad"], case["act"], s.get("residual")) for x_g, w_g, b_g in
+         zip(x.chunk(groups, 3), w.chunk(groups, 0), s["bias"].chunk(groups))]
+    return torch.cat(y, 3)
+
+
+def _exact_train(case, s):
+    k, st, pad = case["k"], case["stride"], case["pad"]
+    ho, wo = _extent(case)
+    d = torch.zeros(4, 6, dtype=torch.float64, device=DEV)
+    for i, kept in enumerate(_PAIRS):
+        d[list(kept), i] = 1.0
+    w, dy = s["w"].double(), s["dy"].double()
+    z = torch.softmax((s["logits"].double() + s["noise"].double()) / TAU, 1)
+    # (the effective weights are a bf16 tensor between two calls)
+    w_eff = ((z @ d.T) * w.reshape(-1, 4)).reshape(w.shape).to(torch.bfloat16).double()
+    xp = torch.nn.functional.pad(s["x"], (0, 0, pad, pad, pad, pad)).double()
+    dw, dxp = torch.zeros_like(w), torch.zeros_like(xp)
+    for i in range(k):
+        for j in range(k):
+            dw[:, i, j] = dy.reshape(-1, case["cout"]).T @ _patches(xp, i, j, st, ho, wo).reshape(-1, case["cin"])
+            _patches(dxp, i, j, st, ho, wo).add_(dy @ w_eff[:, i, j])
+    g_z = (dw.reshape(-1, 4) * w.reshape(-1, 4)) @ d
+    g = z * (g_z - (z * g_z).sum(1, keepdim=True)) / TAU
+    m, v = 0.1 * g, 0.001 * g * g                                 # the first step, from zero moments
+    theta = s["logits"].double()
+    theta = theta - 1e-3 * (m / 0.1 / ((v / 0.001).sqrt() + 1e-8) + 1e-4 * theta)
+    return dict(y=_conv(s["x"], w_eff, s["bias"], st, pad), dw=dw, dx=dxp[:, pad:pad + case["h"], pad:pad + case["w"]],
+                g_logits=g, logits=theta, m=m, v=v)
+
+
+def _exact_resnet(s):
+    net, outs = s["net"], []
+    last = {}                                                     # the step that reads an output last
+    for i, st in enumerate(net.steps):
+        last[st.src] = last[st.res] = i
+    for i, st in enumerate(net.steps):
+        x = s["x"] if st.src < 0 else outs[st.src]
+        if st.kind == "maxpool":
+            y = torch.nn.functional.max_pool2d(x.permute(0, 3, 1, 2), 3, 2, 1).permute(0, 2, 3, 1)
+        else:
+            sp = st.spec
+            inp = synth.make_weights(sp)
+            w = inp.w.to(DEV)
+            w = _keep_two(w) if st.kind == "conv" else w[..., :x.shape[3]]
+            y = _conv(x, w, inp.bias.to(DEV), sp.stride, sp.pad, "relu" if sp.relu else "none",
+                      outs[st.res] if st.res >= 0 else None)
+        outs.append(y)
+        for k in range(i):
+            if k not in s["taps"] and last.get(k, 0) <= i:
+                outs[k] = None
+    return [outs[i] for i in s["taps"]] + [outs[-1]]
+
+
+def _exact_convnext(s):
+    net, outs = s["net"], []
+    for i, (st, p) in enumerate(zip(net.steps, net.params)):
+        x = s["x"] if st.src < 0 else outs[st.src]
+        if st.kind == "s2d":
+            y = x                                                 # the dense stem below reads the image itself
+        elif st.kind == "dense":
+            y = _conv(x, p["w_host"].to(DEV), p["bias"], 4)
+        elif st.kind == "layernorm":
+            y = torch.nn.functional.layer_norm(x.double(), x.shape[3:], p["gamma"].double(), p["beta"].double(), convnext.LN_EPS)
+        elif st.kind == "depthwise":
+            xp = torch.nn.functional.pad(x, (0, 0, 3, 3, 3, 3))
+            y = p["bias"].double().expand(x.shape).clone()
+            for a in range(7):
+                for b in range(7):
+                    y += _patches(xp, a, b, 1, *x.shape[1:3]) * p["w"][a, b].double()
+        else:
+            y = _conv(x, _keep_two(p["w_host"].to(DEV)), p["bias"], st.desc.stride_h, 0, "gelu" if st.gelu else "none",
+                      outs[st.res] if st.res >= 0 else None)
+        outs.append(y)
+        for k in range(max(0, i - 3)):                            # a block's input is read at most four steps later
+            if k not in s["taps"]:
+                outs[k] = None
+    return [outs[i] for i in s["taps"]] + [outs[-1]]
+
+
+def exact(case, seed):
+    """What `run` returns for these inputs, in 64 bits and by plain torch operations.  A network is one chain in
+    64 bits, without the rounding of the tensors in between."""
+    if case["kind"] == "masks":
+        return None                                               # bytes
+    s = prepare(case, seed)
+    if case["kind"] == "resnet":
+        return _exact_resnet(s)
+    if case["kind"] == "convnext":
+        return _exact_convnext(s)
+    if case["kind"] == "train":
+        return _exact_train(case, s)
+    return _exact_layer(case, s, s["w"])
