@@ -1,0 +1,529 @@
+// Depthwise 7 x 7 convolution (unit stride, no dilation, C % 32 == 0) on the warp-level tensor-core
+// instruction mma.m16n8k16 (bf16 operands, fp32 accumulation).
+//
+// One channel's filter row is a band matrix: eight neighbouring outputs of a row are the product of the
+// sixteen image pixels under them (fourteen count) and a 16 x 8 matrix holding the seven taps on its
+// diagonals.  With sixteen such windows as the rows of A, one instruction does one filter row of 128 outputs
+// of one channel (7 of its 16 columns of K are taps: 2.3 multiply-adds issued per useful one), and seven of
+// them, one per filter row, reuse the same A fragment for the seven output rows the image row contributes
+// to.  tcgen05.mma has no use here: every channel is a matrix product of its own, with N = 8.
+//
+// What bounds it and why: on fp32 FMA pipes the 1.9 G multiply-adds of a 128 x 56 x 56 x 96 tensor take at
+// least 52 us, twice what moving the tensor takes (23 us); as band matrices they are 2.3 M instructions, 16 us
+// at the 8.4 cycles per scheduler that one takes.  What is left is bringing channels that are neighbours in
+// memory into one fragment per channel, which goes through shared memory.
+//
+// A block of 24 warps (one per SM, persistent) works on 32 channels and 16 windows (numbered over images and
+// blocks of eight columns, so any map width fills them) and walks down the image rows:
+//   4 warps bring pieces of 8 pixels x 32 channels in by TMA (zero outside the image, 8 rows ahead: at one row
+//     ahead the kernel was bound by the latency of its loads) and write each row transposed, channel by
+//     channel, to shared memory, where a window is two 16-byte rows of ldmatrix that neighbouring windows share;
+//   16 warps of two channels each keep the band matrices (28 registers) and the accumulators of the seven
+//     output rows in flight (56) and write each finished row to shared memory;
+//   4 warps store finished rows, 64 bytes per pixel.
+// The roles meet at mbarriers only.  Measured on that tensor under ncu: 61 us (the fp32 kernel with 4 x 8
+// outputs per thread before it: 122-127 us; one set of helper warps 65 us; no roles and one row of loads ahead
+// 72 us).  By events around one launch: 131 -> 64 us, 128 x 28 x 28 x 192 74 -> 47, 14 x 14 x 384 44 -> 33,
+// 7 x 7 x 768 33 -> 27 us.  The shared-memory pipe is 59 % busy, the tensor pipe 31 %.
+//
+// Zero entries of the band matrix meet pixels outside an output's window.  An infinity or NaN among those
+// would turn the output into a NaN, so a block that meets a non-finite accumulator looks at its outputs again at
+// the end and computes every NaN among them from the pixels of its own window alone (recompute_output).
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "layout.cuh"
+#include "sm100_ptx.cuh"
+#include "ssconv.h"
+
+namespace ssconv {
+
+constexpr int kDw7K = 7;
+constexpr int kDw7MainWarps = 16;                   // two channels each
+constexpr int kDw7HelperWarps = 4;                  // bring image rows in; as many more carry finished rows out
+constexpr int kDw7Threads = 32 * (kDw7MainWarps + 2 * kDw7HelperWarps);
+// Registers per thread: 80 at launch (the launch bound's limit), then 96 for the multiplying warps and 48 for the
+// helpers, together what the launch allotted.
+constexpr int kDw7LaunchRegs = 80, kDw7MainRegs = 96, kDw7HelperRegs = 48;
+static_assert(kDw7MainWarps * kDw7MainRegs + 2 * kDw7HelperWarps * kDw7HelperRegs <=
+                  (kDw7MainWarps + 2 * kDw7HelperWarps) * kDw7LaunchRegs,
+              "a register split above the launch's total never ends");
+constexpr uint32_t kDw7Spins = 1u << 20;            // polls of a barrier before a warp gives up on it
+constexpr int kDw7Channels = 32;                    // per block
+constexpr int kDw7Windows = 16;                     // per block: the rows of the MMA
+constexpr int kDw7Slots = 2 * kDw7Windows;          // most 8-pixel pieces of a row they touch
+constexpr int kDw7ChannelWords = kDw7Slots * 4;     // a channel's staged row, in 32-bit words
+// eight words between channels 8 apart: the four lanes that hold a pixel's channels write to different banks
+constexpr int kDw7StageWords = kDw7Channels * kDw7ChannelWords + 3 * 8;
+constexpr int kDw7OutWords = kDw7Windows * 8 * 17 + 4;
+constexpr int kDw7StageBufs = 3, kDw7OutBufs = 2;
+constexpr int kDw7StageBytes = 4 * kDw7StageWords, kDw7OutBytes = 4 * kDw7OutWords;
+// image rows as TMA brings them in: kDw7RawRows rows of every 8-pixel piece per copy, 64 bytes per pixel
+// (64-byte swizzle), kDw7RawBufs copies of each piece in flight
+constexpr int kDw7RawRows = 2, kDw7RawBufs = 4;
+constexpr int kDw7RawSlotBytes = kDw7RawRows * 8 * 64;
+constexpr int kDw7RawBytes = kDw7Slots * kDw7RawSlotBytes;
+// (alignment,) raw rows, staged and finished rows, barriers (full and empty per buffer; raw: one per helper warp
+// and buffer), table, bias, flags
+constexpr int kDw7SmemBytes = 1024 + kDw7RawBufs * kDw7RawBytes + kDw7StageBufs * kDw7StageBytes + kDw7OutBufs * kDw7OutBytes +
+                              8 * (2 * (kDw7StageBufs + kDw7OutBufs) + kDw7HelperWarps * kDw7RawBufs) +
+                              4 * (kDw7Windows * 8 + kDw7Channels + 2);
+
+// A finished row in shared memory: pixel col of window w at this word, 16 words of channel pairs.  17 words per
+// pixel and one more per four windows: a warp's fragment (8 windows x 4 columns) writes to 32 banks, and two
+// windows two apart are read from 32.
+__device__ __forceinline__ int dw7_out_word(int w, int col) { return w * (8 * 17) + (w >> 2) + col * 17; }
+
+struct Dw7Params {
+  const uint32_t* x;
+  const uint32_t* w;
+  const float* bias;
+  uint32_t* y;
+  int N, H, W, C, Ho, Wo, pad;
+  long long y_row;          // bytes per output row
+  int nblk;                 // windows per output row
+  int groups;               // groups of 16 windows (of N nblk)
+  int work_quot, work_rem;  // output rows per thread block (of groups * C / 32 * Ho): quotient and remainder
+  uint32_t flags;
+};
+
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void lds128(uint32_t addr, uint32_t (&v)[4]) {
+  asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(addr)
+               : "memory");
+}
+template <bool FIRST>  // FIRST: d = a b instead of d += a b
+__device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  if (FIRST)
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+  else
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// One output of channel pair c2 from its own window's pixels only.
+template <bool RELU>
+__device__ __forceinline__ uint32_t recompute_output(const Dw7Params& p, int n, int ho, int wo, int c2) {
+  const int C2 = p.C >> 1;
+  float lo = 0.0f, hi = 0.0f;
+  if (p.flags & SSCONV_FLAG_BIAS) {
+    lo = p.bias[2 * c2];
+    hi = p.bias[2 * c2 + 1];
+  }
+  for (int kh = 0; kh < kDw7K; ++kh) {
+    const int h = ho - p.pad + kh;
+    if (h < 0 || h >= p.H) continue;
+    for (int kw = 0; kw < kDw7K; ++kw) {
+      const int col = wo - p.pad + kw;
+      const uint32_t v = (col >= 0 && col < p.W) ? p.x[(((long long)n * p.H + h) * p.W + col) * C2 + c2] : 0u;
+      const uint32_t tap = p.w[(kh * kDw7K + kw) * C2 + c2];
+      lo = fmaf(bf16_lo(v), bf16_lo(tap), lo);
+      hi = fmaf(bf16_hi(v), bf16_hi(tap), hi);
+    }
+  }
+  return RELU ? pack_bf16x2<false>(fmaxf(lo, 0.0f), fmaxf(hi, 0.0f)) : pack_bf16x2<false>(lo, hi);
+}
+
+// Consecutive output rows of one group of windows and 32 channels, from row `pos` of the block's range on.
+struct Dw7Segment {
+  int z, win0, n_first, b_first, h0, S, rows, row0, row1;
+  __device__ __forceinline__ Dw7Segment(const Dw7Params& p, int& pos, int end) {
+    const int unit = pos / p.Ho;
+    h0 = pos - unit * p.Ho;
+    S = min(p.Ho - h0, end - pos);
+    pos += S;
+    z = unit / p.groups;
+    win0 = (unit - z * p.groups) * kDw7Windows;
+    n_first = win0 / p.nblk;
+    b_first = win0 - n_first * p.nblk;
+    rows = S + kDw7K - 1;
+    // rows [row0, row1) of the segment's are inside the image
+    row0 = max(0, p.pad - h0);
+    row1 = min(rows, p.H + p.pad - h0);
+  }
+};
+
+template <bool RELU>
+__global__ void __launch_bounds__(kDw7Threads, 1)
+depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ Dw7Params p) {
+  extern __shared__ uint8_t dw_smem_raw[];
+  uint8_t* const raw = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dw_smem_raw) + 1023) & ~uintptr_t(1023));
+  uint32_t* const stage_words = reinterpret_cast<uint32_t*>(raw + kDw7RawBufs * kDw7RawBytes);
+  uint32_t* const out_words = stage_words + kDw7StageBufs * kDw7StageWords;
+  uint64_t* const bars = reinterpret_cast<uint64_t*>(out_words + kDw7OutBufs * kDw7OutWords);
+  uint64_t* const raw_bars = bars + 2 * (kDw7StageBufs + kDw7OutBufs);
+  uint32_t* const out_at = reinterpret_cast<uint32_t*>(raw_bars + kDw7HelperWarps * kDw7RawBufs);  // [column][window]
+  float* const bias_s = reinterpret_cast<float*>(out_at + kDw7Windows * 8);
+  volatile int* const again = reinterpret_cast<int*>(bias_s + kDw7Channels);  // set: look for NaNs
+  volatile int* const failed = again + 1;                                     // set: a wait ran out, compute everything again
+  const uint32_t stage0 = smem_u32(stage_words), out0 = smem_u32(out_words);
+  // barriers: image row staged, image row read, finished row written, finished row stored
+  const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kDw7StageBufs;
+  const uint32_t ofull0 = empty0 + 8 * kDw7StageBufs, oempty0 = ofull0 + 8 * kDw7OutBufs;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);       // (uniform over the warp, and known to be)
+  if (tid == 0) {
+    *again = *failed = 0;
+    for (int b = 0; b < kDw7StageBufs; ++b) {
+      mbar_init(bars + b, kDw7HelperWarps);
+      mbar_init(bars + kDw7StageBufs + b, kDw7MainWarps);
+    }
+    for (int b = 0; b < kDw7OutBufs; ++b) {
+      mbar_init(bars + 2 * kDw7StageBufs + b, kDw7MainWarps);
+      mbar_init(bars + 2 * kDw7StageBufs + kDw7OutBufs + b, kDw7HelperWarps);
+    }
+    for (int b = 0; b < kDw7HelperWarps * kDw7RawBufs; ++b) mbar_init(raw_bars + b, 1);
+    mbar_fence_init();
+    prefetch_tensormap(&tm_x);
+  }
+  const int blk = (int)blockIdx.x;
+  int pos = blk * p.work_quot + min(blk, p.work_rem);
+  const int end = pos + p.work_quot + (blk < p.work_rem ? 1 : 0);
+  grid_launch_dependents();
+  grid_dependency_wait();
+  __syncthreads();
+
+  // Every role walks the block's segments; three block barriers per segment: tables written, outputs stored, done.
+  // Buffers in use and the parity of their barriers are carried on over segments.
+  uint32_t sbuf = 0, sphase = 0, obuf = 0, ophase = 0;
+  bool ok = true;
+  if (warp < kDw7MainWarps) {
+    // ------------------------------------------------------------------ multiplications and epilogue
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kDw7MainRegs));
+    const int g = lane >> 2, t = lane & 3;                      // fragment row and column group
+    while (pos < end) {
+      const Dw7Segment sg(p, pos, end);
+      if (tid < kDw7Windows * 8) {  // where outputs go, in units of 64 bytes (a block's channels of a pixel); ~0: outside
+        const int win = sg.win0 + (tid & 15), n = win / p.nblk, wo = 8 * (win - n * p.nblk) + (tid >> 4);
+        out_at[tid] = (n < p.N && wo < p.Wo)
+                          ? (uint32_t)((((long long)n * p.Ho + sg.h0) * p.Wo + wo) * (p.C / kDw7Channels) + sg.z)
+                          : ~0u;
+      }
+      if (tid < kDw7Channels) bias_s[tid] = (p.flags & SSCONV_FLAG_BIAS) ? __ldg(p.bias + sg.z * kDw7Channels + tid) : 0.0f;
+      // the two channels' band matrices: B[k][n] = tap k - n of the filter row, n = g
+      uint32_t band[2][kDw7K][2];
+      {
+        const int C2 = p.C >> 1;
+        const uint32_t* w = p.w + sg.z * (kDw7Channels / 2) + warp;
+#pragma unroll
+        for (int kh = 0; kh < kDw7K; ++kh) {
+          uint32_t v[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int kw = 2 * t + (e & 1) + 8 * (e >> 1) - g;
+            v[e] = (kw >= 0 && kw < kDw7K) ? __ldg(w + (kh * kDw7K + kw) * C2) : 0u;
+          }
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            band[0][kh][half] = __byte_perm(v[2 * half], v[2 * half + 1], 0x5410);
+            band[1][kh][half] = __byte_perm(v[2 * half], v[2 * half + 1], 0x7632);
+          }
+        }
+      }
+      // ldmatrix address: matrices 0, 1 = windows 0-7, 8-15 on their first 8 pixels, 2, 3 on the next 8
+      const int lw = lane & 15;
+      const int lslot = lw + (sg.win0 + lw) / p.nblk - sg.n_first + (lane >> 4);
+      const uint32_t a_addr = stage0 + 4u * ((2 * warp) * kDw7ChannelWords + (warp >> 2) * 8 + 4 * lslot);
+      const uint32_t out_dst = out0 + 4u * (dw7_out_word(g, 2 * t) + warp);
+      const uint32_t bias_at = smem_u32(bias_s) + 8u * warp;
+      __syncthreads();
+      float acc[2][kDw7K][4];
+#pragma unroll
+      for (int o = 0; o < kDw7K; ++o)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[0][o][e] = acc[1][o][e] = 0.0f;
+      const int rows = sg.rows, row0 = sg.row0, row1 = sg.row1;
+      for (int r0 = 0; r0 < rows && ok; r0 += kDw7K) {
+#pragma unroll
+        for (int ph = 0; ph < kDw7K; ++ph) {  // (unrolled: the accumulator of output row o is o mod 7)
+          const int r = r0 + ph;
+          if (r >= rows || !ok) break;
+          // Image row r under filter row kh is output row r - kh.  (Rows before the segment's first are dropped
+          // below, rows past its last never leave the accumulators.)
+          if (r >= row0 && r < row1) {
+            ok = mbar_spin_a(full0 + 8u * sbuf, sphase, kDw7Spins);
+            uint32_t a[2][4];
+            ldmatrix_x4(a_addr + sbuf * kDw7StageBytes, a[0]);
+            ldmatrix_x4(a_addr + sbuf * kDw7StageBytes + 4u * kDw7ChannelWords, a[1]);
+            if (lane == 0) mbar_arrive_a(empty0 + 8u * sbuf);
+#pragma unroll
+            for (int ch = 0; ch < 2; ++ch) {
+              // (the row's oldest output first: the epilogue below waits for it)
+#pragma unroll
+              for (int kh = kDw7K - 1; kh > 0; --kh)
+                mma_bf16_16816<false>(acc[ch][(ph - kh + kDw7K) % kDw7K], a[ch], band[ch][kh][0], band[ch][kh][1]);
+              mma_bf16_16816<true>(acc[ch][ph], a[ch], band[ch][0][0], band[ch][0][1]);
+            }
+            if (++sbuf == kDw7StageBufs) {
+              sbuf = 0;
+              sphase ^= 1u;
+            }
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[0][ph][e] = acc[1][ph][e] = 0.0f;
+          }
+          if (r >= kDw7K - 1) {  // the output row this image row completes
+            float(&d0)[4] = acc[0][(ph + 1) % kDw7K];
+            float(&d1)[4] = acc[1][(ph + 1) % kDw7K];
+            const float bias0 = __uint_as_float(lds32(bias_at)), bias1 = __uint_as_float(lds32(bias_at + 4u));
+            ok = mbar_spin_a(oempty0 + 8u * obuf, ophase ^ 1u, kDw7Spins) && ok;
+            const uint32_t o = out_dst + obuf * kDw7OutBytes;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              d0[e] += bias0;
+              d1[e] += bias1;
+              sts32(o + 4u * ((e >> 1) * (8 * 8 * 17 + 2) + (e & 1) * 17), pack_bf16x2<RELU>(d0[e], d1[e]));
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive_a(ofull0 + 8u * obuf);
+            if (++obuf == kDw7OutBufs) {
+              obuf = 0;
+              ophase ^= 1u;
+            }
+            // a NaN among the eight makes their sum one (a sum that is infinite only costs the second look)
+            const float sum = ((d0[0] + d0[1]) + (d0[2] + d0[3])) + ((d1[0] + d1[1]) + (d1[2] + d1[3]));
+            if (!(fabsf(sum) <= 3.0e38f)) *again = 1;
+          }
+        }
+      }
+      if (!ok) *failed = 1;
+      __syncthreads();  // (also: this block's stores are visible to all its threads)
+      if (*again != 0 || *failed != 0) {
+        for (int i = tid; i < sg.S * kDw7Windows * 8 * (kDw7Channels / 2); i += 32 * kDw7MainWarps) {
+          const int word = i & 15, at_col = (i >> 4) & 7, w = (i >> 7) & 15, o = i >> 11;
+          const uint32_t at = out_at[at_col * 16 + w];
+          if (at == ~0u) continue;
+          uint32_t* const dst = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(p.y + word) + 64ull * at + o * p.y_row);
+          const uint32_t v = *dst;
+          if (*failed == 0 && (v & 0x7FFFu) <= 0x7F80u && (v & 0x7FFF0000u) <= 0x7F800000u) continue;  // neither is a NaN
+          const int win = sg.win0 + w, n = win / p.nblk;
+          *dst = recompute_output<RELU>(p, n, sg.h0 + o, 8 * (win - n * p.nblk) + at_col, sg.z * (kDw7Channels / 2) + word);
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kDw7MainWarps) : "memory");
+        if (tid == 0) *again = 0;
+      }
+      __syncthreads();  // (the next segment writes the table)
+    }
+  } else if (warp < kDw7MainWarps + kDw7HelperWarps) {
+    // ------------------------------------------------------------------ image rows in
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kDw7HelperRegs));
+    const int ht = tid - 32 * kDw7MainWarps, hw = warp - kDw7MainWarps;
+    uint32_t rbuf = 0, rphase = 0;
+    while (pos < end) {
+      const Dw7Segment sg(p, pos, end);
+      // A warp brings in pieces 2 hw, 2 hw + 1, 2 hw + 8, ... of the rows by itself: lane l < 8 copies piece
+      // 2 hw + l % 2 + 8 (l / 2), zero outside the image, kDw7RawRows rows at a time.
+      const int slots = kDw7Windows + 1 + (sg.win0 + kDw7Windows - 1) / p.nblk - sg.n_first;  // (pieces in use)
+      const int my_slot = 2 * hw + (lane & 1) + 8 * (lane >> 1);
+      const bool my_copy = lane < 8 && my_slot < slots;
+      const uint32_t copies = __popc(__ballot_sync(0xffffffffu, my_copy));  // (at least two: slots >= 17)
+      const int my_piece = my_slot + sg.b_first;                // an image has nblk + 1 pieces per row
+      const int my_n = sg.n_first + my_piece / (p.nblk + 1), my_col = 8 * (my_piece % (p.nblk + 1)) - p.pad;
+      const uint32_t raw0 = smem_u32(raw), raw_bar0 = smem_u32(raw_bars) + 8u * kDw7RawBufs * hw;
+      int row_next = sg.row0;                                   // first row of the next copy
+      uint32_t cbuf = rbuf;
+      auto copy_rows = [&]() {  // (all lanes; the buffer's last rows have been read)
+        if (row_next >= sg.row1) return;
+        const uint32_t bar = raw_bar0 + 8u * cbuf;
+        if (lane == 0) mbar_expect_tx_a(bar, copies * kDw7RawSlotBytes);
+        __syncwarp();
+        if (my_copy)
+          tma_load_4d_a(raw0 + cbuf * kDw7RawBytes + my_slot * kDw7RawSlotBytes, &tm_x, bar, sg.z * kDw7Channels, my_col,
+                        sg.h0 - p.pad + row_next, my_n);
+        row_next += kDw7RawRows;
+        cbuf = (cbuf + 1 == kDw7RawBufs) ? 0u : cbuf + 1;
+      };
+      for (int k = 0; k < kDw7RawBufs; ++k) copy_rows();
+      // staging: pixels 2 q, 2 q + 1 of pieces s0 + 8 k, channels [8 cc, 8 cc + 8).  Lanes of odd q read the
+      // second pixel first (eight lanes then read 128 bytes on different banks).
+      const int cc = ht & 3, q = (ht >> 2) & 3, s0 = ht >> 4;
+      const uint32_t raw_src = raw0 + s0 * kDw7RawSlotBytes + (2 * q) * 64 + 16 * (cc ^ q);
+      const uint32_t first = (q & 1) ? 64u : 0u;
+      const uint32_t sel_lo = (q & 1) ? 0x1054u : 0x5410u, sel_hi = (q & 1) ? 0x3276u : 0x7632u;
+      const uint32_t st_dst = stage0 + 4u * (8 * cc * kDw7ChannelWords + 8 * cc + 4 * s0 + q);
+      __syncthreads();
+      for (int r = sg.row0; r < sg.row1 && ok; ++r) {
+        const int sub = (r - sg.row0) % kDw7RawRows;
+        if (sub == 0) ok = mbar_spin_a(raw_bar0 + 8u * rbuf, rphase, kDw7Spins);
+        ok = mbar_spin_a(empty0 + 8u * sbuf, sphase ^ 1u, kDw7Spins) && ok;
+        const uint32_t src = raw_src + rbuf * kDw7RawBytes + sub * 512u;
+#pragma unroll
+        for (int k2 = 0; k2 < 4; k2 += 2) {
+          if (8 * k2 >= slots) break;
+          uint32_t a[2][4], b[2][4];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            lds128(src + 8u * (k2 + k) * kDw7RawSlotBytes + first, a[k]);
+            lds128(src + 8u * (k2 + k) * kDw7RawSlotBytes + (64u - first), b[k]);
+          }
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            if (8 * (k2 + k) >= slots) break;
+            const uint32_t d = st_dst + sbuf * kDw7StageBytes + 4u * 32 * (k2 + k);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              sts32(d + 4u * (2 * i) * kDw7ChannelWords, __byte_perm(a[k][i], b[k][i], sel_lo));
+              sts32(d + 4u * (2 * i + 1) * kDw7ChannelWords, __byte_perm(a[k][i], b[k][i], sel_hi));
+            }
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive_a(full0 + 8u * sbuf);
+        if (++sbuf == kDw7StageBufs) {
+          sbuf = 0;
+          sphase ^= 1u;
+        }
+        if (sub == kDw7RawRows - 1 || r + 1 == sg.row1) {  // the copy is used up
+          copy_rows();
+          if (++rbuf == kDw7RawBufs) {
+            rbuf = 0;
+            rphase ^= 1u;
+          }
+        }
+      }
+      if (!ok) *failed = 1;
+      __syncthreads();
+      __syncthreads();
+    }
+  } else {
+    // ------------------------------------------------------------------ finished rows out
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kDw7HelperRegs));
+    const int hw = warp - kDw7MainWarps - kDw7HelperWarps;
+    // a warp stores the words of columns hw, hw + 4 of windows w2, w2 + 4, ... and w2 + 1, w2 + 5, ...
+    const int w2 = 2 * (lane >> 4);
+    const uint32_t out_src = out0 + 4u * (dw7_out_word(w2, hw) + (lane & 15));
+    const uint32_t out_tab = smem_u32(out_at) + 4u * (hw * 16 + w2);
+    while (pos < end) {
+      const Dw7Segment sg(p, pos, end);
+      char* y_row = reinterpret_cast<char*>(p.y + (lane & 15));
+      __syncthreads();
+      for (int o = 0; o < sg.S && ok; ++o) {
+        ok = mbar_spin_a(ofull0 + 8u * obuf, ophase, kDw7Spins);
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          uint32_t to[8], w[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {  // windows w2 + 4 (k / 2) + k % 2
+            to[k] = lds32(out_tab + 4u * (64 * c + 4 * (k >> 1) + (k & 1)));
+            w[k] = lds32(out_src + obuf * kDw7OutBytes + 4u * (4 * c * 17 + (k >> 1) * (4 * 8 * 17 + 1) + (k & 1) * 8 * 17));
+          }
+          if (c == 1) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive_a(oempty0 + 8u * obuf);
+          }
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (to[k] != ~0u) *reinterpret_cast<uint32_t*>(y_row + 64ull * to[k]) = w[k];
+        }
+        y_row += p.y_row;
+        if (++obuf == kDw7OutBufs) {
+          obuf = 0;
+          ophase ^= 1u;
+        }
+      }
+      if (!ok) *failed = 1;
+      __syncthreads();
+      __syncthreads();
+    }
+  }
+}
+
+// False: not a layer for this kernel (the caller goes on to the general ones).
+bool depthwise7_applies(int N, int H, int W, int C, int Ho, int Wo, int KH, int KW, int stride, int dil) {
+  return KH == kDw7K && KW == kDw7K && stride == 1 && dil == 1 && C % kDw7Channels == 0 &&
+         (long long)N * Ho * Wo * (C / kDw7Channels) < 0xFFFFFFFFll && (long long)H * W * C < (1ll << 38) &&
+         (long long)N * ((Wo + 7) / 8) * (C / kDw7Channels) * Ho < 0x7FFFFFF0ll / 2;
+}
+
+typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                             const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+cudaError_t launch_depthwise7(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho,
+                              int Wo, int pad, uint32_t flags, cudaStream_t st) {
+  Dw7Params p;
+  p.x = static_cast<const uint32_t*>(x);
+  p.w = static_cast<const uint32_t*>(w);
+  p.bias = bias;
+  p.y = static_cast<uint32_t*>(y);
+  p.N = N;
+  p.H = H;
+  p.W = W;
+  p.C = C;
+  p.Ho = Ho;
+  p.Wo = Wo;
+  p.pad = pad;
+  p.y_row = 2ll * Wo * C;
+  p.nblk = (Wo + 7) / 8;
+  p.groups = (N * p.nblk + kDw7Windows - 1) / kDw7Windows;
+  p.flags = flags;
+  const bool relu = (flags & SSCONV_FLAG_RELU) != 0;
+  const auto kernel = relu ? depthwise7_mma_kernel<true> : depthwise7_mma_kernel<false>;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  static int sm_count[64][2] = {{0}};  // (set once per device and form, after the kernel has been made ready there)
+  int sms = (dev >= 0 && dev < 64) ? sm_count[dev][relu] : 0;
+  if (sms == 0) {
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, kernel);
+    if (e == cudaSuccess && fa.numRegs != kDw7LaunchRegs) return cudaErrorInvalidConfiguration;  // (the register split counts on it)
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDw7SmemBytes);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) sm_count[dev][relu] = sms;
+  }
+  // output rows are dealt out evenly: a block walks a contiguous range of (32 channels, group of windows, row)
+  const long long work = (long long)p.groups * (C / kDw7Channels) * Ho;
+  const int blocks = (int)(work < sms ? work : sms);
+  p.work_quot = (int)(work / blocks);
+  p.work_rem = (int)(work % blocks);
+  CUtensorMap tm_x;
+  {
+    static EncodeFn encode = nullptr;  // (every thread finds the same function)
+    if (encode == nullptr) {
+      void* f = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q);
+      if (e != cudaSuccess) return e;
+      if (q != cudaDriverEntryPointSuccess || f == nullptr) return cudaErrorNotSupported;
+      encode = reinterpret_cast<EncodeFn>(f);
+    }
+    const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)N};
+    const cuuint64_t strides[3] = {2ull * C, 2ull * C * W, 2ull * C * W * H};
+    const cuuint32_t box[4] = {kDw7Channels, 8, kDw7RawRows, 1}, estr[4] = {1, 1, 1, 1};
+    if (encode(&tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return cudaErrorInvalidValue;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(kDw7Threads);
+  cfg.dynamicSmemBytes = kDw7SmemBytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, kernel, tm_x, p);
+}
+
+}  // namespace ssconv

@@ -1,0 +1,73 @@
+"""The 7 x 7 depthwise kernel on tensor cores at the sizes where its tiling can go wrong, against the fp64 oracle:
+groups of sixteen windows that end inside an image, span several or are mostly empty, map widths around multiples
+of eight, paddings up to the filter's width, one output row, more blocks' ranges than rows; and infinities and
+NaNs, which may only reach the outputs whose own window holds them."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import blocks
+from oracle.conv import ConvShape
+from paper_2411_00288_b200 import api, synth
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+CASES = [  # N, H, W, C, pad, relu
+    (1, 7, 7, 32, 0, False),      # one output
+    (1, 1, 1, 32, 3, True),       # one pixel
+    (15, 9, 8, 32, 3, False),     # 15 windows
+    (16, 9, 8, 64, 3, True),      # 16
+    (17, 9, 8, 32, 3, False),     # 17: a second, nearly empty group
+    (3, 30, 57, 96, 3, False),    # 8 windows per row, one column in the last
+    (2, 12, 130, 32, 6, True),    # a row longer than a group of windows, padding of a whole filter
+    (5, 8, 23, 160, 2, False),
+    (40, 15, 15, 32, 4, False),   # block ranges that start and end inside a strip
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=["x".join(map(str, c[:4])) + f"_p{c[4]}" for c in CASES])
+def test_depthwise7_at_the_edges_of_its_tiles(case):
+    N, H, W, C, pad, relu = case
+    g = torch.Generator().manual_seed(synth.SEED_BASE + 7100 + CASES.index(case))
+    x = torch.randn((N, H, W, C), generator=g).to(torch.bfloat16)
+    w = (torch.randn((7, 7, C), generator=g) / 7).to(torch.bfloat16)
+    bias = torch.randn((C,), generator=g) * 0.1
+    desc = api.make_desc(N, H, W, C, C, 7, 7, 1, pad, bias=True, relu=relu)
+    Ho, Wo = api.ssconv_out_shape(desc)
+    band = 256
+    buf = torch.full((N * Ho * Wo * C + 2 * band,), -5.0, dtype=torch.bfloat16, device=DEV)
+    y = buf[band:band + N * Ho * Wo * C].view(N, Ho, Wo, C)
+    api.ssconv_depthwise(desc, x.to(DEV), w.to(DEV), bias.to(DEV), y=y)
+    torch.cuda.synchronize()
+    assert bool((buf[:band] == -5.0).all()) and bool((buf[-band:] == -5.0).all())
+    shape = ConvShape(N, H, W, C, C, 7, 7, (1, 1), (pad, pad), (1, 1), relu=False)
+    ref = blocks.depthwise_conv2d_f64(shape, synth.bf16_bits(x), synth.bf16_bits(w), bias=bias.numpy())
+    if relu:
+        ref = np.maximum(ref, 0.0)
+    rel, mx = parity.errors(parity.bf16_tensor_to_f64(y), ref)
+    assert rel <= parity.REL_FRO_TOL and mx <= parity.MAX_ABS_TOL, (case, rel, mx)
+
+
+def test_depthwise7_non_finite_pixels_reach_their_own_windows_only():
+    N, H, W, C = 2, 20, 19, 64
+    g = torch.Generator().manual_seed(synth.SEED_BASE + 7200)
+    x = torch.randn((N, H, W, C), generator=g).to(torch.bfloat16)
+    w = (torch.rand((7, 7, C), generator=g) * 0.1 + 0.05).to(torch.bfloat16)   # positive: an infinity keeps its sign
+    bad = [(0, 5, 6, 3, float("inf")), (1, 10, 0, 7, float("nan")), (1, 19, 18, 40, float("-inf"))]
+    clean = x.clone()
+    for n, h, c0, c, v in bad:
+        x[n, h, c0, c] = v
+        clean[n, h, c0, c] = 0.0
+    desc = api.make_desc(N, H, W, C, C, 7, 7, 1, 3, bias=False)
+    y = api.ssconv_depthwise(desc, x.to(DEV), w.to(DEV)).cpu()
+    y_clean = api.ssconv_depthwise(desc, clean.to(DEV), w.to(DEV)).cpu()
+    touched = torch.zeros(y.shape, dtype=torch.bool)
+    for n, h, c0, c, v in bad:
+        box = (n, slice(max(0, h - 3), h + 4), slice(max(0, c0 - 3), c0 + 4), c)
+        touched[box] = True
+        assert bool(torch.isnan(y[box]).all()) if v != v else bool((y[box] == v).all())
+    # outputs next to them are computed again on fp32 pipes in another order of summation: one bf16 rounding apart
+    err = (y.float() - y_clean.float()).abs()[~touched]
+    assert bool((err <= 2.0 ** -7 * y_clean.float().abs()[~touched] + 1e-5).all())
