@@ -48,6 +48,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <type_traits>
 
 #include "layout.cuh"
@@ -62,6 +63,9 @@ constexpr int kGroupCols = kBN / kGroups;
 constexpr int kPiece = 40;               // positions per epilogue piece (one staging buffer)
 constexpr int kFirstExtraProducerWarp = 2 + 4 * kGroups;  // warps 10 and 11: two more TMA producers
 constexpr int kThreads = 64 + 128 * kGroups + 64;
+// With `sets` sets of epilogue groups (one-block kernel; see kWideMaxKBlocks) the producers follow the last group.
+__host__ __device__ constexpr int threads_with(int sets) { return 64 + 128 * kGroups * sets + 64; }
+__host__ __device__ constexpr int first_extra_producer_with(int sets) { return 2 + 4 * kGroups * sets; }
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAccCol1 = 256;       // second accumulator; the first starts at column 0
 constexpr uint32_t kMetaCol = kBN;       // metadata: 2 slots x 4 columns in [240, 248)
@@ -100,7 +104,8 @@ struct FwdParams {
   int pieces;               // epilogue pieces per group: ceil(BN / 2 / kPiece)
   int tail_cols;            // positions in a group's last piece (a multiple of 8, at most kPiece)
   int ring_groups;          // groups in the shared-memory ring
-  int stage_bufs;           // staging buffers per epilogue group: 2, or 4 when residual pieces are prefetched
+  int stage_bufs;           // staging buffers per half of a tile's positions: 2, or 4 (residual pieces prefetched, or
+                            // two sets of epilogue groups)
   int small_c;              // dense layers with C_in == 8: a k-block is 8 filter taps (see producer_role)
   uint32_t a_grp_bytes;     // bytes of weights (and metadata) at the head of a ring group; 0: weights resident
   uint32_t a_res_bytes;     // dense layers of one channel tile and at most four k-blocks: the whole weight
@@ -203,15 +208,17 @@ __device__ __forceinline__ size_t region_index(int c, bool tile_starts_here) {
   return 2 * (size_t)c + (tile_starts_here ? 1 : 0);
 }
 
-// Named barriers: 1 and 2 for the epilogue groups, 3 for the setup (warp 0 arrives without waiting).
+// Named barriers: 1 to 4 for the epilogue groups, 5 for the setup (warp 0 arrives without waiting).
 __device__ __forceinline__ void epilogue_bar_sync(int group) {
   asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory");
 }
+template <int THREADS>
 __device__ __forceinline__ void setup_bar_arrive() {
   __threadfence_block();
-  asm volatile("bar.arrive 3, %0;" ::"n"(kThreads) : "memory");
+  asm volatile("bar.arrive 5, %0;" ::"n"(THREADS) : "memory");
 }
-__device__ __forceinline__ void setup_bar_sync() { asm volatile("bar.sync 3, %0;" ::"n"(kThreads) : "memory"); }
+template <int THREADS>
+__device__ __forceinline__ void setup_bar_sync() { asm volatile("bar.sync 5, %0;" ::"n"(THREADS) : "memory"); }
 // One epilogue piece of this warp's 32 lanes x 40 columns in fragment layout: register
 // r[20 h + 4 k + 2 s + e] = lane (16 h + 8 s + t/4), column (8 k + 2 (t%4) + e).  No wait.
 __device__ __forceinline__ void tc_ld_piece(uint32_t taddr, uint32_t (&r)[kPiece]) {
@@ -229,22 +236,19 @@ __device__ __forceinline__ void tc_ld_piece(uint32_t taddr, uint32_t (&r)[kPiece
 // rounding, and overwritten in place (a warp only touches its own 16-byte columns).
 // ACT: 0 identity, 1 ReLU (inside the bf16 conversion), 2 GELU in its erf form x Phi(x) =
 // 0.5 x (1 + erf(x / sqrt 2)), evaluated in fp32 before the rounding.
-// erf without branches: erf(z) = 1 - 2^R(z) for z >= 0 with R a degree-6 polynomial (no constant term)
-// fitted to log2(erfc(z)) on [0, 4] (beyond 4, erfc < 2e-8 and z is clamped), odd extension by the sign of
-// x; the factor 1 / sqrt 2 of z = |x| / sqrt 2 is folded into the coefficients, so the polynomial takes
-// |x| clamped at 4 sqrt 2.  The difference 1 - 2^R loses relative accuracy near 0, which x Phi(x) does not
-// need.  Against fp64 over every bf16 input up to 8: |R - log2 erfc| <= 4.8e-5, i.e. 3.3e-5 relative in
-// exact arithmetic; evaluated in fp32 the result is within 5.1e-6 absolute, and within 3e-4 relative
-// wherever |x Phi(x)| > 1e-4 (the largest ratio sits in the far negative tail, where 0.5 x and |x| t
-// cancel), a seventh of the rounding to bf16 that follows (2^-9).  A degree-8 fit bought nothing after that
-// rounding and cost two more multiply-adds per value, which matters because shallow layers with this
-// activation are bound by the epilogue's arithmetic.
+// With Phi(-|x|) = 0.5 erfc(|x| / sqrt 2) the activation is max(x, 0) - |x| Phi(-|x|) on both sides of zero:
+// no sign to carry, and nothing cancels.  log2 erfc(z) is a degree-6 polynomial R (no constant term) fitted on
+// [0, 4] (beyond 4, erfc < 2e-8 and z is clamped); the factor 1 / sqrt 2 of z is folded into its coefficients,
+// the 0.5 into the exponent, and the polynomial takes n = -|x|, the factor of the last multiply-add.  Fitted to
+// |R - log2 erfc| <= 4.8e-5, i.e. 3.3e-5 relative; in fp32 over every bf16 input up to 8 the result is within 5.1e-6 absolute
+// and 3.3e-5 relative, a sixtieth of the rounding to bf16 that follows (2^-9).  A degree-8 fit bought nothing after that rounding and cost two more multiply-adds per value,
+// which matters because shallow layers with this activation are bound by the epilogue's arithmetic: eight
+// instructions of the FMA pipe (half rate for pairs) and two exponentials per pair of values.
 constexpr int kActNone = 0, kActRelu = 1, kActGelu = 2;
 constexpr float kGeluClamp = 5.656854152679443f;  // 4 sqrt 2
-constexpr float kGeluC1 = -1.1506847143173218f, kGeluC2 = -0.46029916405677795f, kGeluC3 = -0.05191940814256668f,
-                kGeluC4 = 0.00745233241468668f, kGeluC5 = -0.0006528479279950261f, kGeluC6 = 2.5540923161315732e-05f;
-// Two values at once, the polynomial on fp32 pairs (fma.rn.f32x2); the result is formed as
-// x (0.5 + sign(x) (0.5 - 0.5 e)) = 0.5 x + |x| (0.5 - 0.5 e) with e = 2^R.
+constexpr float kGeluC1 = 1.1506847143173218f, kGeluC2 = -0.46029916405677795f, kGeluC3 = 0.05191940814256668f,
+                kGeluC4 = 0.00745233241468668f, kGeluC5 = 0.0006528479279950261f, kGeluC6 = 2.5540923161315732e-05f;
+// Two values at once, the polynomial on fp32 pairs (fma.rn.f32x2).
 __device__ __forceinline__ unsigned long long f32x2(float lo, float hi) {
   unsigned long long r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -257,32 +261,26 @@ __device__ __forceinline__ unsigned long long horner2(unsigned long long r, unsi
 __device__ __forceinline__ void split2(unsigned long long v, float& lo, float& hi) {
   asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
 }
-// GELU of the pair x, returned as a pair; everything that has a paired form is done on pairs (the polynomial,
-// 0.5 - 0.5 e, 0.5 x and the final multiply-add), so that the eight epilogue warps issue as few instructions as
-// possible: the result is x s + 0.5 x with s = sign(x) (0.5 - 0.5 e).
 __device__ __forceinline__ unsigned long long gelu_f32x2(unsigned long long x) {
   float lo, hi;
   split2(x, lo, hi);
-  const unsigned long long a = f32x2(fminf(fabsf(lo), kGeluClamp), fminf(fabsf(hi), kGeluClamp));
+  const unsigned long long n = f32x2(fmaxf(-fabsf(lo), -kGeluClamp), fmaxf(-fabsf(hi), -kGeluClamp));
+  float p0, p1;  // max(x, 0); a NaN stays one
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(p0) : "f"(lo));
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(p1) : "f"(hi));
+  unsigned long long y = f32x2(p0, p1);
   unsigned long long r = f32x2(kGeluC6, kGeluC6);
-  r = horner2(r, a, kGeluC5);
-  r = horner2(r, a, kGeluC4);
-  r = horner2(r, a, kGeluC3);
-  r = horner2(r, a, kGeluC2);
-  r = horner2(r, a, kGeluC1);
-  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(r) : "l"(a));
+  r = horner2(r, n, kGeluC5);
+  r = horner2(r, n, kGeluC4);
+  r = horner2(r, n, kGeluC3);
+  r = horner2(r, n, kGeluC2);
+  r = horner2(r, n, kGeluC1);
+  r = horner2(r, n, -1.0f);
   float r0, r1, e0, e1;
   split2(r, r0, r1);
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(r0));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(r1));
-  unsigned long long t = f32x2(e0, e1);
-  asm("fma.rn.f32x2 %0, %0, %1, %2;" : "+l"(t) : "l"(f32x2(-0.5f, -0.5f)), "l"(f32x2(0.5f, 0.5f)));
-  float t0, t1;
-  split2(t, t0, t1);
-  const unsigned long long sgn = f32x2(copysignf(t0, lo), copysignf(t1, hi));
-  unsigned long long y;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(y) : "l"(x), "l"(f32x2(0.5f, 0.5f)));
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(y) : "l"(x), "l"(sgn));
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(y) : "l"(n), "l"(f32x2(e0, e1)));
   return y;
 }
 template <int ACT>
@@ -477,15 +475,18 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
 }
 
 // RES: a residual tensor is added in the epilogue (its own instantiation, so that the plain kernel's
-// epilogue loop carries none of that code).
-template <bool SPARSE, bool RES, bool FP8 = false>
-__global__ void __launch_bounds__(kThreads, 1)
+// epilogue loop carries none of that code).  EPI_SETS: sets of epilogue groups; with two, each serves one of the
+// two accumulators, i.e. every other tile.
+template <bool SPARSE, bool RES, bool FP8 = false, int EPI_SETS = 1>
+__global__ void __launch_bounds__(threads_with(EPI_SETS), 1)
 ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                   const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_y_tail,
                   const __grid_constant__ CUtensorMap tm_r, const __grid_constant__ CUtensorMap tm_r_tail,
                   const FwdParams p) {
   using C = Cfg<SPARSE, FP8>;
   static_assert(!(FP8 && RES), "the residual epilogue is not built for 8-bit operands");
+  static_assert(EPI_SETS == 1 || (EPI_SETS == 2 && !RES), "one set of epilogue groups, or one per accumulator");
+  constexpr int kThreadsHere = threads_with(EPI_SETS), kExtraProducer = first_extra_producer_with(EPI_SETS);
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -530,15 +531,15 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       fence_proxy_async_smem();
     }
     __syncwarp();
-    setup_bar_arrive();
+    setup_bar_arrive<kThreadsHere>();
   } else {
     if (warp == 1) {
       tmem_alloc(tmem_slot, kTmemCols);
       tmem_relinquish();
     }
     if (lane == 0) {  // tensor maps are fetched while thread 0 initialises the barriers
-      if (warp == kFirstExtraProducerWarp) prefetch_tensormap(&tm_b);
-      if (warp == kFirstExtraProducerWarp + 1) prefetch_tensormap(&tm_a);
+      if (warp == kExtraProducer) prefetch_tensormap(&tm_b);
+      if (warp == kExtraProducer + 1) prefetch_tensormap(&tm_a);
       if (warp == 2) {
         prefetch_tensormap(&tm_y);
         prefetch_tensormap(&tm_y_tail);
@@ -549,12 +550,12 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       }
     }
     tc_fence_before();
-    setup_bar_sync();
+    setup_bar_sync<kThreadsHere>();
     tc_fence_after();
   }
   const uint32_t tmem_base = (warp == 0) ? 0u : *tmem_slot;
 
-  if (warp == 0 || warp >= kFirstExtraProducerWarp) {
+  if (warp == 0 || warp >= kExtraProducer) {
     // ------------------------------------------------------------------ TMA producers
     // (each a whole warp in lock step, one elected lane issuing: see the warp-wide forms)
     {
@@ -563,7 +564,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
         producer_role<SPARSE, kRoleActFirst, FP8>(&tm_a, &tm_b, p, full0,
                                              p.ring_groups == 2 ? smem_u32(bar_empty_first) : empty0, ring0,
                                              smem_u32(bar_res), abort_flag);
-      else if (warp == kFirstExtraProducerWarp)
+      else if (warp == kExtraProducer)
         producer_role<SPARSE, kRoleActSecond, FP8>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res), abort_flag);
       else
         producer_role<SPARSE, kRoleWeights, FP8>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res), abort_flag);
@@ -718,18 +719,19 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
         if (ok) tc_commit_w(smem_u32(&bar_acc_full[buf]));
       }
     }
-  } else if (warp < kFirstExtraProducerWarp) {
+  } else if (warp < kExtraProducer) {
     // ------------------------------------------------------------------ epilogue
     // Two independent groups of four warps; group g owns positions [g BN/2, (g + 1) BN/2) of every
     // tile, with its own staging buffers and named barrier, and handles them 40 at a time (the last
     // piece of a group may hold fewer).
     const int grp = (warp - 2) >> 2;
+    const int half = EPI_SETS == 1 ? grp : (grp & (kGroups - 1));  // of the positions
     const int q = warp & 3;  // TMEM lane quadrant this warp may read: channels [32 q, 32 q + 32) of the tile
     const int gtid = q * 32 + lane;
     const bool leader = (q == 2 && lane == 0);  // first warp of each group
     const int act = activation_of(p.flags);
-    const int col_base = grp * (p.BN >> 1);
-    const uint32_t nbuf = (uint32_t)p.stage_bufs;  // 2 or 4
+    const int col_base = half * (p.BN >> 1);
+    const uint32_t nbuf = (uint32_t)p.stage_bufs / EPI_SETS;  // 2 or 4
     const uint32_t nbuf_shift = nbuf == 4 ? 2u : 1u;
     uint8_t* my_stage = out_stage + grp * nbuf * kPieceBytes;
     volatile int* my_go = epi_go + 2 * grp;
@@ -775,12 +777,15 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       const int m = seg.tile - pt * p.m_tiles;
       const uint32_t buf = tcount & 1u;
       const uint32_t aph = (tcount >> 1) & 1u;
+      // (two sets: each serves one accumulator, so that it has two tiles' time for its tiles)
+      if (EPI_SETS == 2 && buf != (uint32_t)(grp / kGroups)) continue;
+      const uint32_t verdict = (EPI_SETS == 2 ? tcount >> 1 : tcount) & 1u;
       const bool got = mbar_wait_bounded(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
       // All threads of a group must take the same branch (they meet at named barriers below):
       // the leader publishes one verdict, everybody reads it after the barrier.
-      if (leader) my_go[tcount & 1u] = (got && *abort_flag == 0) ? 1 : 0;
+      if (leader) my_go[verdict] = (got && *abort_flag == 0) ? 1 : 0;
       epilogue_bar_sync(grp);
-      if (my_go[tcount & 1u] == 0) break;
+      if (my_go[verdict] == 0) break;
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + buf * kAccCol1 + col_base;
       const bool whole = (seg.a0 == 0 && seg.a1 == p.a_tiles);
@@ -795,7 +800,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
           tc_wait_ld();
 #pragma unroll
           for (int j = 0; j < kPiece / 4; ++j)
-            __stcg(mine + region_vec(grp, piece, j, gtid),
+            __stcg(mine + region_vec(half, piece, j, gtid),
                    make_float4(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]),
                                __uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3])));
         }
@@ -1482,6 +1487,7 @@ constexpr double kLoadLatencyCycles = 1000.0;
 constexpr double kIssueSparse = 365.0, kIssueDense = 480.0;
 constexpr double kEpiloguePieceCycles = 900.0;
 constexpr double kCyclesPerParkedTile = 90.0;
+constexpr double kWideTileCycles = 500.0, kWidePieceCycles = 1775.0;  // GELU epilogue on two sets of groups, per tile
 constexpr double kSplitAdvantage = 1.1;  // split only if the model predicts at least this gain
 
 static int ring_groups_for(uint32_t a_group_bytes, int BN, int stage_bufs) {
@@ -1547,10 +1553,11 @@ struct Plan {
   double cost = 0.0;  // the model's cycles for the layer
   bool pair = false;  // 256-channel tiles on CTA pairs (ssconv_fwd_pair_kernel)
   bool dual = false;  // ... with two position tiles per work item
+  bool wide = false;  // one-CTA tiles with two sets of epilogue groups
 };
 template <bool SPARSE>
 static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force_split, int max_bn = kBN,
-                       int stage_bufs = 2, bool allow_split = true) {
+                       int stage_bufs = 2, bool allow_split = true, bool wide_epilogue = false) {
   if (force_split) return Plan{kBN, true};
   int min_bn = 48;
   if (g_tune_bn != 0 && g_tune_bn <= max_bn) max_bn = min_bn = g_tune_bn;
@@ -1562,8 +1569,9 @@ static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force
     const int pieces = (BN / 2 + kPiece - 1) / kPiece;
     // (with at most three groups per tile the ring never reaches its steady state: such layers are paced
     // by their output stream, and measured fastest at the width the other terms choose)
-    const double cost = (double)per_cta * geo.kblocks * kblock_cycles<SPARSE>(BN, stage_bufs, geo.stages >= 4) +
-                        pieces * kEpiloguePieceCycles;
+    double tile = geo.kblocks * kblock_cycles<SPARSE>(BN, stage_bufs, geo.stages >= 4);
+    if (wide_epilogue) tile = fmax(tile, kWideTileCycles + pieces * kWidePieceCycles);
+    const double cost = (double)per_cta * tile + pieces * kEpiloguePieceCycles;
     if (BN == max_bn || cost < 0.97 * best_cost) {  // a narrower tile has to earn its extra weight traffic
       best_cost = cost;
       best.BN = BN;
@@ -1678,6 +1686,7 @@ size_t workspace_bytes() { return scratch_bytes(kMaxWorkers); }
 
 static int g_sm_count[64] = {0};
 static bool g_attr_set[64][2][2] = {{{false}}};
+static bool g_wide_attr_set[64][2] = {{false}};
 static bool g_pair_attr_set[64][2] = {{false}};
 static bool g_pair_res_attr_set[64][2] = {{false}};
 static bool g_fp8_attr_set[64][2] = {{false}};
@@ -1719,14 +1728,37 @@ static int widest_tile(uint32_t a_group_bytes, int stage_bufs) {
   return BN;
 }
 
+// Two sets of epilogue groups (16 epilogue warps instead of 8, each set on its own accumulator).  With GELU a
+// shallow layer is bound by its epilogue, whose eight warps wait on one another's arithmetic, on TMEM and on the
+// staging buffers more than they issue (48 % of the issue slots used, no pipe above 44 %).  Taken for GELU layers of
+// at most six k-blocks whose tiles give every CTA more than one (a CTA with a single tile has no work for the
+// second set).  Measured (us, one set -> two, layers of n x h x h x c_in -> c_out): 128 x 56 x 56 x 96 -> 384
+// 113 -> 98, 128 x 28 x 28 x 192 -> 768 62.5 -> 56.3, 128 x 14 x 14 x 384 -> 1536 38.9 -> 35.3, 64 x 56 x 56 x 64 ->
+// 64 25.1 -> 21.5; beyond the line 8 k-blocks 14.8 -> 14.8, 12 19.4 -> 19.9, 16 26.6 -> 27.1, and one tile per CTA
+// (3 x 14 x 14 x 384 -> 1536) 6.1 -> 6.6.  Without GELU the layers are bound by their output stream: no gain (64 ->
+// 256 at 56 x 56 91 -> 91, 128 -> 512 at 28 x 28 52 -> 53).
+constexpr int kWideMaxKBlocks = 6;
+constexpr int kWideStageBufs = 4;  // staging buffers per half of a tile: two for each set
 // The plan for a layer without a residual: one-CTA tiles (whole or K split) or the pair kernel.
 template <bool SPARSE>
 static Plan choose_plan(const ssconv_desc_t& d, long long Q, const Geometry& geo, int workers, bool force_split,
-                        bool allow_split = true) {
+                        bool allow_split = true, bool allow_wide = true) {
   const Plan plan = plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, allow_split);
-  if (force_split || small_channel_mode(d, SPARSE) || g_tune_pair == 0) return plan;
-  const Plan pair = plan_pair<SPARSE>(Q, geo, workers, g_tune_pair == 1);
-  if (pair.BN != 0 && (g_tune_pair == 1 || plan.cost > kPairAdvantage * pair.cost)) return pair;
+  if (force_split || small_channel_mode(d, SPARSE)) return plan;
+  if (g_tune_pair != 0) {
+    const Plan pair = plan_pair<SPARSE>(Q, geo, workers, g_tune_pair == 1);
+    if (pair.BN != 0 && (g_tune_pair == 1 || plan.cost > kPairAdvantage * pair.cost)) return pair;
+  }
+  // (dense layers of one channel tile and at most four k-blocks keep their weights resident instead)
+  if (allow_wide && !plan.split && activation_of(d.flags) == kActGelu && geo.kblocks <= kWideMaxKBlocks &&
+      (SPARSE || geo.m_tiles > 1 || geo.kblocks > 4)) {
+    Plan wide = plan_layer<SPARSE>(Q, geo, workers, false, widest_tile(Cfg<SPARSE>::kAGroupBytes, kWideStageBufs),
+                                   kWideStageBufs, false, true);
+    if (((Q + wide.BN - 1) / wide.BN) * geo.m_tiles > workers) {
+      wide.wide = true;
+      return wide;
+    }
+  }
   return plan;
 }
 
@@ -1765,7 +1797,7 @@ int32_t plan_query_sms(const ssconv_desc_t& d, bool sparse, int sm_count, int32_
   const long long work = do_split ? tiles * geo.stages : tiles;
   if (split) *split = do_split ? 1 : 0;
   if (ctas) *ctas = (int32_t)(work < workers ? work : workers);
-  if (ring_groups) *ring_groups = ring_groups_for(a_group_bytes, plan.BN, 2);
+  if (ring_groups) *ring_groups = ring_groups_for(a_group_bytes, plan.BN, plan.wide ? kWideStageBufs : 2);
   return SSCONV_OK;
 }
 
@@ -1796,6 +1828,12 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
     if (e != cudaSuccess) return SSCONV_ERR_CUDA;
     g_attr_set[dev][SPARSE ? 1 : 0][res] = true;
   }
+  if (!FP8 && !g_wide_attr_set[dev][SPARSE ? 1 : 0]) {
+    if (cudaFuncSetAttribute(ssconv_fwd_kernel<SPARSE, false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kMaxSmemBytes) != cudaSuccess)
+      return SSCONV_ERR_CUDA;
+    g_wide_attr_set[dev][SPARSE ? 1 : 0] = true;
+  }
   if (FP8 && !g_fp8_attr_set[dev][SPARSE ? 1 : 0]) {
     if (cudaFuncSetAttribute(ssconv_fwd_kernel<SPARSE, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kMaxSmemBytes) != cudaSuccess)
@@ -1820,7 +1858,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   if (force_split && !have_ws) return SSCONV_ERR_WORKSPACE;
   // (8-bit operands: the pair kernel exists for the 2:4 form only; the dense counterpart stays on one-block tiles)
   Plan plan = (residual != nullptr || (FP8 && !SPARSE)) ? plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, have_ws)
-                                                        : choose_plan<SPARSE>(d, Q, geo, workers, force_split, have_ws);
+                                                        : choose_plan<SPARSE>(d, Q, geo, workers, force_split, have_ws, !FP8);
   int stage_bufs = 2;
   if (residual != nullptr && !plan.split) {
     stage_bufs = 4;
@@ -1840,6 +1878,8 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
       }
     }
   }
+  const bool wide_epilogue = plan.wide;
+  if (wide_epilogue) stage_bufs = kWideStageBufs;
   const int BN = plan.BN;
   const int pieces = (BN / 2 + kPiece - 1) / kPiece;
   const int tail_cols = BN / 2 - (pieces - 1) * kPiece;
@@ -1848,7 +1888,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   // channels): every tile needs the same 16-64 KB of weights, which then stay in shared memory for the
   // life of the CTA instead of travelling through the ring with every tile; the groups hold activations
   // only, and more of them fit.
-  const bool resident = !SPARSE && !FP8 && !small_c && !pair && !plan.split && residual == nullptr && geo.m_tiles == 1 &&
+  const bool resident = !wide_epilogue && !SPARSE && !FP8 && !small_c && !pair && !plan.split && residual == nullptr && geo.m_tiles == 1 &&
                         geo.kblocks <= 4 && g_tune_resident != 0;
   const uint32_t a_grp_bytes = resident ? 0u : C::kAGroupBytes;
   const uint32_t a_res_bytes = resident ? (uint32_t)geo.stages * 2u * kATileBytes : 0u;
@@ -2044,7 +2084,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   // waits for that kernel's completion before it touches global memory.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)kThreads);
+  cfg.blockDim = dim3((unsigned)threads_with(wide_epilogue ? 2 : 1));
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -2066,6 +2106,8 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
       : pair ? cudaLaunchKernelEx(&cfg, ssconv_fwd_pair_kernel<SPARSE>, tm_a, tm_b, tm_meta, tm_y, tm_y_tail, tm_r, tm_r_tail, p)
       : residual != nullptr
           ? cudaLaunchKernelEx(&cfg, ssconv_fwd_kernel<SPARSE, true>, tm_a, tm_b, tm_y, tm_y_tail, tm_r, tm_r_tail, p)
+      : wide_epilogue
+          ? cudaLaunchKernelEx(&cfg, ssconv_fwd_kernel<SPARSE, false, false, 2>, tm_a, tm_b, tm_y, tm_y_tail, tm_r, tm_r_tail, p)
           : cudaLaunchKernelEx(&cfg, ssconv_fwd_kernel<SPARSE, false>, tm_a, tm_b, tm_y, tm_y_tail, tm_r, tm_r_tail, p);
   if (launched != cudaSuccess) return SSCONV_ERR_CUDA;
   count_launch();

@@ -1,0 +1,79 @@
+"""The GELU epilogue: its values over every bf16 number, and the form with two sets of epilogue groups at the edges of
+its tiles (odd numbers of tiles, a short last tile, ragged channels, every staged width, slices of a wider tensor)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import blocks
+from oracle.conv import ConvShape
+from paper_2411_00288_b200 import api, synth
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def test_gelu_of_every_bf16_value():
+    bits = torch.arange(0, 65536, dtype=torch.int32).to(torch.uint16)
+    v = bits.view(torch.bfloat16)
+    v = v[~(torch.isfinite(v) & (v.abs() > 1e30))]            # (x 0.5 x stays finite)
+    pad = (-v.numel()) % 64
+    v = torch.cat([v, torch.zeros(pad, dtype=torch.bfloat16)])
+    x = torch.zeros((1, v.numel() // 64, 64, 16), dtype=torch.bfloat16)
+    x[0, :, :, 0] = v.view(-1, 64)
+    w = torch.zeros((16, 1, 1, 16), dtype=torch.bfloat16)
+    w[:, 0, 0, 0] = 1.0
+    desc = api.make_desc(1, x.shape[1], 64, 16, 16, 1, 1, bias=False, gelu=True)
+    pat = api.ssconv_select_mask(api.MASK_MAGNITUDE_BF16, w.to(DEV), w.numel() // 4)
+    comp = api.ssconv_compress(desc, w.to(DEV), pat)
+    y = api.ssconv_forward(desc, x.to(DEV), *comp).cpu()
+    for c in (0, 7, 15):
+        got = y[0, :, :, c].reshape(-1)
+        nan = torch.isnan(v)
+        assert bool(torch.isnan(got[nan]).all())
+        assert bool((got[v == float("inf")] == float("inf")).all())
+        fin = torch.isfinite(v)
+        ref = parity.gelu_f64(v[fin].double().numpy())
+        err = np.abs(got[fin].double().numpy() - ref)
+        # one rounding to bf16 (half a unit in the last of 8 bits: at most 2^-8 of the value), 3.3e-5 of the fp32
+        # evaluation, and the clamp's 2e-8 x 5.7 far below zero
+        assert (err <= (2.0 ** -8 + 5e-5) * np.abs(ref) + 2e-7).all(), float((err - 2.0 ** -8 * np.abs(ref)).max())
+
+
+LAYERS = [  # N, H, W, C_in, C_out, k, pad
+    (16, 56, 56, 96, 384, 1, 0),
+    (1, 160, 150, 16, 128, 1, 0),      # about one tile per thread block and a few with two
+    (3, 97, 83, 40, 136, 1, 0),        # ragged channels, an odd number of tiles, a short last one
+    (5, 57, 41, 64, 72, 1, 0),         # half a channel tile
+    (2, 120, 117, 24, 256, 2, 1),      # four taps
+]
+
+
+@pytest.mark.parametrize("layer", LAYERS, ids=["x".join(map(str, v[:5])) for v in LAYERS])
+@pytest.mark.parametrize("width", [0, 48, 112, 160, 208])
+def test_two_epilogue_sets_match_oracle(layer, width):
+    N, H, W, ci, co, k, pad = layer
+    spec = synth.LayerSpec("gelu2", N, H, W, ci, co, k, k, 1, pad, 1, gelu=True, w_std="fan_in", mask_source="magnitude",
+                           config=8, index=300 + LAYERS.index(layer))
+    api.ssconv_tune(api.TUNE_TILE_POSITIONS, width)
+    try:
+        for sparse in (True, False):
+            rel, mx = parity.check_layer(spec, DEV, sparse=sparse, sample=20000)
+            assert rel <= parity.REL_FRO_TOL and mx <= parity.MAX_ABS_TOL, (sparse, rel, mx)
+    finally:
+        api.ssconv_tune(api.TUNE_TILE_POSITIONS, 0)
+
+
+def test_two_epilogue_sets_on_channel_slices():
+    N, H, W, ci, co, groups = 4, 90, 77, 64, 288, 2
+    g = torch.Generator().manual_seed(synth.SEED_BASE + 7300)
+    x = torch.randn((N, H, W, ci), generator=g).to(torch.bfloat16)
+    w = (torch.randn((co, 1, 1, ci // groups), generator=g) / (ci // groups) ** 0.5).to(torch.bfloat16)
+    bias = torch.randn((co,), generator=g) * 0.1
+    desc = api.make_desc(N, H, W, ci, co, 1, 1, bias=True, gelu=True)
+    y = api.ssconv_forward_dense_grouped(desc, groups, x.to(DEV), w.to(DEV), bias.to(DEV))
+    torch.cuda.synchronize()
+    shape = ConvShape(N, H, W, ci, co, 1, 1, (1, 1), (0, 0), (1, 1), relu=False)
+    ref = parity.gelu_f64(blocks.grouped_conv2d_f64(shape, groups, synth.bf16_bits(x), synth.bf16_bits(w), bias=bias.numpy()))
+    rel, mx = parity.errors(parity.bf16_tensor_to_f64(y), ref)
+    assert rel <= parity.REL_FRO_TOL and mx <= parity.MAX_ABS_TOL, (rel, mx)
