@@ -7,6 +7,7 @@ is raised.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from dataclasses import dataclass
 from typing import Optional, Tuple
@@ -67,6 +68,68 @@ def desc_from_spec(spec) -> Desc:
 _lib = None
 
 
+def _prototypes():
+    """{entry point: (result, arguments)} as in include/ssconv.h.  Pointers (tensors, streams, descriptors and results
+    alike) are passed as addresses."""
+    vp, i32, i64, sz = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_size_t
+    f32, f64 = ctypes.c_float, ctypes.c_double
+    return {
+        "ssconv_version": (i32, []),
+        "ssconv_launch_count": (ctypes.c_uint64, []),
+        "ssconv_status_string": (ctypes.c_char_p, [i32]),
+        "ssconv_out_shape": (i32, [vp] * 3),
+        "ssconv_sizes": (i32, [vp] * 6),
+        "ssconv_plan": (i32, [vp, i32] + [vp] * 5),
+        "ssconv_plan_for_sms": (i32, [vp, i32, i32] + [vp] * 5),
+        "ssconv_tune": (i32, [i32, i32]),
+        "ssconv_window_extent": (i32, [i32] * 5),
+        "ssconv_selftest_wait_timeout": (i32, [i64, vp, vp]),
+        "ssconv_select_mask": (i32, [i32, vp, i64, vp, vp]),
+        "ssconv_nm_patterns": (i32, [i32, i32]),
+        "ssconv_select_mask_nm": (i32, [i32, vp, i64, i32, i32, vp, vp]),
+        "ssconv_apply_mask_nm": (i32, [vp, vp, i64, i32, i32, vp, vp]),
+        "ssconv_compress": (i32, [vp] * 6),
+        "ssconv_decompress": (i32, [vp] * 6),
+        "ssconv_maxpool": (i32, [vp, vp] + [i32] * 7 + [vp]),
+        "ssconv_pad_channels": (i32, [vp, vp, i64, i32, i32, vp]),
+        "ssconv_space_to_depth": (i32, [vp, vp] + [i32] * 9 + [vp]),
+        "ssconv_unfold_w": (i32, [vp, vp, i64] + [i32] * 7 + [vp]),
+        "ssconv_fold_factor": (i32, [vp]),
+        "ssconv_fold_desc": (i32, [vp, i32, vp]),
+        "ssconv_fold_weights": (i32, [vp, i32, vp, vp, i64, vp, vp, vp]),
+        "ssconv_forward": (i32, [vp] * 7 + [sz, vp, vp]),
+        "ssconv_forward_res": (i32, [vp] * 8 + [sz, vp, vp]),
+        "ssconv_forward_dense": (i32, [vp] * 6 + [sz, vp, vp]),
+        "ssconv_forward_dense_res": (i32, [vp] * 7 + [sz, vp, vp]),
+        "ssconv_forward_dense_strided": (i32, [vp, vp, i64, i64, i64, vp, vp, vp, vp, sz, vp, vp]),
+        "ssconv_forward_static_ws": (i32, [vp] * 8),
+        "ssconv_mask_norms": (i32, [vp, vp, i32, i64, vp, vp]),
+        "ssconv_absmax": (i32, [vp, i64, vp, vp]),
+        "ssconv_stability_threshold": (f64, [i32, f64, vp, i32, i32, f64, f64]),
+        "ssconv_soft_mask": (i32, [vp, vp, f32, vp, i64, vp, vp, vp]),
+        "ssconv_mask_grad": (i32, [vp, f32, vp, vp, i64, vp, vp]),
+        "ssconv_adamw": (i32, [vp] * 4 + [i64, i32] + [f32] * 5 + [vp]),
+        "ssconv_dgrad_prepare": (i32, [vp] * 5),
+        "ssconv_dgrad_spread": (i32, [vp] * 4),
+        "ssconv_wgrad": (i32, [vp] * 5 + [sz, vp, vp]),
+        "ssconv_wgrad_ws_bytes": (i32, [vp, vp]),
+        "ssconv_dgrad": (i32, [vp] * 5 + [sz, vp, vp]),
+        "ssconv_dgrad_ws_bytes": (i32, [vp, vp]),
+        "ssconv_sizes_grouped": (i32, [vp, i32, vp, vp, vp]),
+        "ssconv_compress_grouped": (i32, [vp, i32] + [vp] * 5),
+        "ssconv_forward_grouped": (i32, [vp, i32] + [vp] * 6 + [sz, vp, vp]),
+        "ssconv_forward_dense_grouped": (i32, [vp, i32] + [vp] * 5 + [sz, vp, vp]),
+        "ssconv_depthwise": (i32, [vp] * 6),
+        "ssconv_layernorm": (i32, [vp, vp, vp, f32, vp, i64, i32, vp]),
+        "ssconv_quantize_e4m3": (i32, [vp, vp, i64, f32, vp]),
+        "ssconv_sizes_fp8": (i32, [vp] * 4),
+        "ssconv_compress_fp8": (i32, [vp] * 6),
+        "ssconv_decompress_fp8": (i32, [vp] * 6),
+        "ssconv_forward_fp8": (i32, [vp] * 5 + [f32] + [vp] * 3),
+        "ssconv_forward_dense_fp8": (i32, [vp] * 4 + [f32] + [vp] * 3),
+    }
+
+
 def lib():
     """Load libssconv.so once; raise if it has not been built."""
     global _lib
@@ -76,30 +139,9 @@ def lib():
                 f"{_LIB_PATH} is missing: build it with `python -m paper_2411_00288_b200.build` "
                 "(there is no fallback path)")
         L = ctypes.CDLL(_LIB_PATH)
-        vp, i32, i64, sz = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_size_t
-        dp = ctypes.POINTER(Desc)
-        L.ssconv_version.restype = i32
-        L.ssconv_version.argtypes = []
-        L.ssconv_launch_count.restype = ctypes.c_uint64
-        L.ssconv_launch_count.argtypes = []
-        L.ssconv_status_string.restype = ctypes.c_char_p
-        L.ssconv_status_string.argtypes = [i32]
-        L.ssconv_out_shape.restype = i32
-        L.ssconv_out_shape.argtypes = [dp, ctypes.POINTER(i32), ctypes.POINTER(i32)]
-        L.ssconv_sizes.restype = i32
-        L.ssconv_sizes.argtypes = [dp, ctypes.POINTER(i64)] + [ctypes.POINTER(sz)] * 4
-        L.ssconv_select_mask.restype = i32
-        L.ssconv_select_mask.argtypes = [i32, vp, i64, vp, vp]
-        L.ssconv_compress.restype = i32
-        L.ssconv_compress.argtypes = [dp, vp, vp, vp, vp, vp]
-        L.ssconv_decompress.restype = i32
-        L.ssconv_decompress.argtypes = [dp, vp, vp, vp, vp, vp]
-        L.ssconv_forward.restype = i32
-        L.ssconv_forward.argtypes = [dp, vp, vp, vp, vp, vp, vp, sz, vp, vp]
-        L.ssconv_forward_dense.restype = i32
-        L.ssconv_forward_dense.argtypes = [dp, vp, vp, vp, vp, vp, sz, vp, vp]
-        L.ssconv_forward_static_ws.restype = i32
-        L.ssconv_forward_static_ws.argtypes = [dp, vp, vp, vp, vp, vp, vp, vp]
+        for name, (restype, argtypes) in _prototypes().items():
+            f = getattr(L, name)
+            f.restype, f.argtypes = restype, argtypes
         _lib = L
     return _lib
 
@@ -114,12 +156,17 @@ def _check(fn: str, status: int):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    """The raw handle of a stream, or of the current device's current one (without a Stream object around it, which
+    takes 3 us to make)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _need_cuda(*tensors):
@@ -138,7 +185,13 @@ def ssconv_launch_count() -> int:
 
 
 def ssconv_out_shape(desc: Desc) -> Tuple[int, int]:
-    h, w = ctypes.c_int32(), ctypes.c_int32()
+    return _out_shape(bytes(desc))
+
+
+# (by the descriptor's content: host arithmetic of the library, the same at every call)
+@functools.lru_cache(maxsize=1024)
+def _out_shape(desc_bytes: bytes) -> Tuple[int, int]:
+    desc, h, w = Desc.from_buffer_copy(desc_bytes), ctypes.c_int32(), ctypes.c_int32()
     _check("ssconv_out_shape", lib().ssconv_out_shape(ctypes.byref(desc), ctypes.byref(h), ctypes.byref(w)))
     return int(h.value), int(w.value)
 
@@ -153,7 +206,12 @@ class Sizes:
 
 
 def ssconv_sizes(desc: Desc) -> Sizes:
-    G = ctypes.c_int64()
+    return _sizes(bytes(desc))
+
+
+@functools.lru_cache(maxsize=1024)
+def _sizes(desc_bytes: bytes) -> Sizes:
+    desc, G = Desc.from_buffer_copy(desc_bytes), ctypes.c_int64()
     a, b, c, d = (ctypes.c_size_t() for _ in range(4))
     _check("ssconv_sizes", lib().ssconv_sizes(ctypes.byref(desc), ctypes.byref(G), ctypes.byref(a), ctypes.byref(b),
                                               ctypes.byref(c), ctypes.byref(d)))
@@ -165,7 +223,7 @@ def ssconv_select_mask(mode: int, scores: torch.Tensor, G: int, pattern: Optiona
     """pattern uint8 [G] from fp32 scores [G,6] (mode LOGITS) or bf16 weights (mode MAGNITUDE)."""
     _need_cuda(scores, pattern)
     if pattern is None:
-        pattern = torch.empty((G,), dtype=torch.uint8, device=scores.device)
+        pattern = torch.empty(G, dtype=torch.uint8, device=scores.device)
     _check("ssconv_select_mask", lib().ssconv_select_mask(mode, _ptr(scores), G, _ptr(pattern), _stream(stream)))
     return pattern
 
@@ -173,19 +231,14 @@ def ssconv_select_mask(mode: int, scores: torch.Tensor, G: int, pattern: Optiona
 def ssconv_nm_patterns(N: int, M: int) -> int:
     """n = C(M, N), the number of N:M patterns (0 if N, M are out of the supported range)."""
     f = lib().ssconv_nm_patterns
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_int32, ctypes.c_int32]
     return int(f(int(N), int(M)))
 
 
 def ssconv_select_mask_nm(mode: int, scores: torch.Tensor, G: int, N: int, M: int, stream=None) -> torch.Tensor:
     """pattern uint8 [G] for N:M blocks from fp32 scores [G, n] (mode LOGITS) or bf16 weights [G, M] (MAGNITUDE)."""
     _need_cuda(scores)
-    pattern = torch.empty((G,), dtype=torch.uint8, device=scores.device)
+    pattern = torch.empty(G, dtype=torch.uint8, device=scores.device)
     f = lib().ssconv_select_mask_nm
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_int32, ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p,
-                  ctypes.c_void_p]
     _check("ssconv_select_mask_nm", f(mode, _ptr(scores), G, N, M, _ptr(pattern), _stream(stream)))
     return pattern
 
@@ -195,9 +248,6 @@ def ssconv_apply_mask_nm(w: torch.Tensor, pattern: torch.Tensor, N: int, M: int,
     _need_cuda(w, pattern)
     out = torch.empty_like(w)
     f = lib().ssconv_apply_mask_nm
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p,
-                  ctypes.c_void_p]
     _check("ssconv_apply_mask_nm", f(_ptr(w), _ptr(pattern), pattern.numel(), N, M, _ptr(out), _stream(stream)))
     return out
 
@@ -206,8 +256,8 @@ def ssconv_compress(desc: Desc, w: torch.Tensor, pattern: torch.Tensor, stream=N
     """(w_comp, meta) uint8 blobs from bf16 weights [C_out,KH,KW,C_in] and pattern [G]."""
     _need_cuda(w, pattern)
     sz = ssconv_sizes(desc)
-    w_comp = torch.empty((sz.w_comp_bytes,), dtype=torch.uint8, device=w.device)
-    meta = torch.empty((sz.meta_bytes,), dtype=torch.uint8, device=w.device)
+    w_comp = torch.empty(sz.w_comp_bytes, dtype=torch.uint8, device=w.device)
+    meta = torch.empty(sz.meta_bytes, dtype=torch.uint8, device=w.device)
     _check("ssconv_compress", lib().ssconv_compress(ctypes.byref(desc), _ptr(w), _ptr(pattern), _ptr(w_comp),
                                                     _ptr(meta), _stream(stream)))
     return w_comp, meta
@@ -218,7 +268,7 @@ def ssconv_decompress(desc: Desc, w_comp: torch.Tensor, meta: torch.Tensor, want
     _need_cuda(w_comp, meta)
     sz = ssconv_sizes(desc)
     w_out = torch.empty((desc.C_out, desc.KH, desc.KW, desc.C_in), dtype=torch.bfloat16, device=w_comp.device)
-    pat = torch.empty((sz.G,), dtype=torch.uint8, device=w_comp.device) if want_pattern else None
+    pat = torch.empty(sz.G, dtype=torch.uint8, device=w_comp.device) if want_pattern else None
     _check("ssconv_decompress", lib().ssconv_decompress(ctypes.byref(desc), _ptr(w_comp), _ptr(meta), _ptr(w_out),
                                                         _ptr(pat), _stream(stream)))
     return w_out, pat
@@ -230,8 +280,6 @@ _workspaces = {}
 def ssconv_window_extent(n: int, k: int, stride: int = 1, pad: int = 0, dil: int = 1) -> int:
     """Placements of a k-tap window along an axis of n elements, as the library computes them."""
     f = lib().ssconv_window_extent
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_int32] * 5
     return int(f(int(n), int(k), int(stride), int(pad), int(dil)))
 
 
@@ -239,8 +287,6 @@ def ssconv_plan_for_sms(desc: Desc, sparse: bool, sm_count: int) -> dict:
     """ssconv_plan for a device with `sm_count` SMs; host arithmetic only, no GPU needed."""
     out = [ctypes.c_int32(0) for _ in range(5)]
     f = lib().ssconv_plan_for_sms
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_int32, ctypes.c_int32] + [ctypes.POINTER(ctypes.c_int32)] * 5
     _check("ssconv_plan_for_sms", f(ctypes.byref(desc), 1 if sparse else 0, int(sm_count), *[ctypes.byref(o) for o in out]))
     return dict(tile_positions=out[0].value, split=bool(out[1].value), ctas=out[2].value, ring_groups=out[3].value,
                 pair=bool(out[4].value))
@@ -250,8 +296,6 @@ def ssconv_selftest_wait_timeout(limit_cycles: int, dev_status: torch.Tensor, st
     """Launch the one-block kernel whose bounded wait runs out; it stores ERR_TIMEOUT to dev_status."""
     _need_cuda(dev_status)
     f = lib().ssconv_selftest_wait_timeout
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_selftest_wait_timeout", f(int(limit_cycles), _ptr(dev_status), _stream(stream)))
 
 
@@ -259,8 +303,6 @@ def ssconv_plan(desc: Desc, sparse: bool = True) -> dict:
     """Tile width, K split, thread blocks and ring depth the forward call would use on the current device."""
     out = [ctypes.c_int32(0) for _ in range(5)]
     f = lib().ssconv_plan
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_int32] + [ctypes.POINTER(ctypes.c_int32)] * 5
     _check("ssconv_plan", f(ctypes.byref(desc), 1 if sparse else 0, *[ctypes.byref(o) for o in out]))
     return dict(tile_positions=out[0].value, split=bool(out[1].value), ctas=out[2].value, ring_groups=out[3].value,
                 pair=bool(out[4].value))
@@ -274,8 +316,6 @@ def ssconv_tune(option: int, value: int) -> None:
     TUNE_PAIR (-1 automatic, 0 never, 1 wherever thread-block pairs apply), TUNE_PAIR_TILES (-1 automatic, 0 one
     position tile per work item of the pair kernel, 1 two wherever they fit), the others as the header says."""
     f = lib().ssconv_tune
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_int32, ctypes.c_int32]
     _check("ssconv_tune", f(int(option), int(value)))
 
 
@@ -283,17 +323,17 @@ def default_workspace(device) -> torch.Tensor:
     """One scratch buffer per device, shared by calls that pass ws=None.  It needs no initialisation
     (the kernels write every part before reading it), so stream-ordered calls can share it; calls
     on different streams that may overlap must pass their own."""
-    dev = torch.device(device)
+    dev = device if isinstance(device, torch.device) else torch.device(device)
     key = dev.index if dev.index is not None else torch.cuda.current_device()
     if key not in _workspaces:
         nbytes = ssconv_sizes(make_desc(1, 8, 8, 8, 8, 1, 1)).ws_bytes_sparse
-        _workspaces[key] = torch.empty((nbytes,), dtype=torch.uint8, device=torch.device("cuda", key))
+        _workspaces[key] = torch.empty(nbytes, dtype=torch.uint8, device=torch.device("cuda", key))
     return _workspaces[key]
 
 
 def _alloc_y(desc: Desc, x: torch.Tensor) -> torch.Tensor:
     ho, wo = ssconv_out_shape(desc)
-    return torch.empty((desc.N, ho, wo, desc.C_out), dtype=torch.bfloat16, device=x.device)
+    return torch.empty(desc.N, ho, wo, desc.C_out, dtype=torch.bfloat16, device=x.device)
 
 
 def ssconv_forward(desc: Desc, x: torch.Tensor, w_comp: torch.Tensor, meta: torch.Tensor,
@@ -307,7 +347,7 @@ def ssconv_forward(desc: Desc, x: torch.Tensor, w_comp: torch.Tensor, meta: torc
         y = _alloc_y(desc, x)
     if ws is None:
         ws = default_workspace(x.device)
-    ws_bytes = 0 if ws is None else ws.numel() * ws.element_size()
+    ws_bytes = ws.nbytes
     if residual is None:
         _check("ssconv_forward", lib().ssconv_forward(
             ctypes.byref(desc), _ptr(x), _ptr(w_comp), _ptr(meta), _ptr(bias), _ptr(y), _ptr(ws), ws_bytes,
@@ -315,9 +355,6 @@ def ssconv_forward(desc: Desc, x: torch.Tensor, w_comp: torch.Tensor, meta: torc
     else:
         assert residual.shape == y.shape and residual.dtype == torch.bfloat16 and residual.is_contiguous()
         f = lib().ssconv_forward_res
-        f.restype = ctypes.c_int32
-        f.argtypes = [ctypes.POINTER(Desc)] + [ctypes.c_void_p] * 7 + [ctypes.c_size_t, ctypes.c_void_p,
-                                                                     ctypes.c_void_p]
         _check("ssconv_forward_res", f(ctypes.byref(desc), _ptr(x), _ptr(w_comp), _ptr(meta), _ptr(bias),
                                        _ptr(residual), _ptr(y), _ptr(ws), ws_bytes, _ptr(dev_status),
                                        _stream(stream)))
@@ -334,7 +371,7 @@ def ssconv_forward_dense(desc: Desc, x: torch.Tensor, w: torch.Tensor, bias: Opt
         y = _alloc_y(desc, x)
     if ws is None:
         ws = default_workspace(x.device)
-    ws_bytes = 0 if ws is None else ws.numel() * ws.element_size()
+    ws_bytes = ws.nbytes
     if residual is None:
         _check("ssconv_forward_dense", lib().ssconv_forward_dense(
             ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(y), _ptr(ws), ws_bytes, _ptr(dev_status),
@@ -342,9 +379,6 @@ def ssconv_forward_dense(desc: Desc, x: torch.Tensor, w: torch.Tensor, bias: Opt
     else:
         assert residual.shape == y.shape and residual.dtype == torch.bfloat16 and residual.is_contiguous()
         f = lib().ssconv_forward_dense_res
-        f.restype = ctypes.c_int32
-        f.argtypes = [ctypes.POINTER(Desc)] + [ctypes.c_void_p] * 6 + [ctypes.c_size_t, ctypes.c_void_p,
-                                                                     ctypes.c_void_p]
         _check("ssconv_forward_dense_res", f(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(residual),
                                              _ptr(y), _ptr(ws), ws_bytes, _ptr(dev_status), _stream(stream)))
     return y
@@ -359,8 +393,6 @@ def ssconv_maxpool(x: torch.Tensor, k: int = 3, stride: int = 2, pad: int = 1, y
         y = torch.empty((n, ssconv_window_extent(h, k, stride, pad), ssconv_window_extent(w, k, stride, pad), c),
                         dtype=torch.bfloat16, device=x.device)
     f = lib().ssconv_maxpool
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p] + [ctypes.c_int32] * 7 + [ctypes.c_void_p]
     _check("ssconv_maxpool", f(_ptr(x), _ptr(y), n, h, w, c, k, stride, pad, _stream(stream)))
     return y
 
@@ -374,8 +406,6 @@ def ssconv_space_to_depth(x: torch.Tensor, block: int, pad: int, Hb: int, Wb: in
     if y is None:
         y = torch.empty((n, Hb, Wb, C_pad), dtype=torch.bfloat16, device=x.device)
     f = lib().ssconv_space_to_depth
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p] + [ctypes.c_int32] * 9 + [ctypes.c_void_p]
     _check("ssconv_space_to_depth", f(_ptr(x), _ptr(y), n, h, w, c, block, pad, Hb, Wb, C_pad, _stream(stream)))
     return y
 
@@ -383,8 +413,6 @@ def ssconv_space_to_depth(x: torch.Tensor, block: int, pad: int, Hb: int, Wb: in
 def ssconv_fold_factor(desc: Desc) -> int:
     """The number of neighbouring output pixels (1 or 2) the planner suggests folding into the output channels."""
     f = lib().ssconv_fold_factor
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc)]
     return int(f(ctypes.byref(desc)))
 
 
@@ -392,8 +420,6 @@ def ssconv_fold_desc(desc: Desc, f: int) -> Desc:
     """Descriptor of the layer with f output pixels of a row folded into f * C_out output channels."""
     out = Desc()
     fn = lib().ssconv_fold_desc
-    fn.restype = ctypes.c_int32
-    fn.argtypes = [ctypes.POINTER(Desc), ctypes.c_int32, ctypes.POINTER(Desc)]
     _check("ssconv_fold_desc", fn(ctypes.byref(desc), int(f), ctypes.byref(out)))
     return out
 
@@ -416,11 +442,8 @@ def ssconv_fold_weights(desc: Desc, f: int, w: Optional[torch.Tensor] = None, bi
             w2 = w2.view(-1)
     if bias is not None:
         assert bias.dtype == torch.float32
-        b2 = torch.empty((folded.C_out,), dtype=torch.float32, device=bias.device)
+        b2 = torch.empty(folded.C_out, dtype=torch.float32, device=bias.device)
     fn = lib().ssconv_fold_weights
-    fn.restype = ctypes.c_int32
-    fn.argtypes = [ctypes.POINTER(Desc), ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64,
-                   ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_fold_weights", fn(ctypes.byref(desc), int(f), _ptr(w), _ptr(w2), tap, _ptr(bias), _ptr(b2),
                                      _stream(stream)))
     return w2, b2
@@ -437,13 +460,9 @@ def ssconv_forward_dense_strided(desc: Desc, x: torch.Tensor, strides, w: torch.
         y = _alloc_y(desc, x)
     if ws is None:
         ws = default_workspace(x.device)
-    ws_bytes = 0 if ws is None else ws.numel() * ws.element_size()
+    ws_bytes = ws.nbytes
     s_w, s_h, s_n = (int(v) for v in strides)
     f = lib().ssconv_forward_dense_strided
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_void_p, ctypes.c_int64, ctypes.c_int64, ctypes.c_int64,
-                  ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_size_t,
-                  ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_forward_dense_strided", f(ctypes.byref(desc), _ptr(x), s_w, s_h, s_n, _ptr(w), _ptr(bias), _ptr(y),
                                              _ptr(ws), ws_bytes, _ptr(dev_status), _stream(stream)))
     return y
@@ -459,8 +478,6 @@ def ssconv_pad_channels(x: torch.Tensor, C_pad: int, y: Optional[torch.Tensor] =
     if y is None:
         y = torch.empty((*lead, C_pad), dtype=torch.bfloat16, device=x.device)
     f = lib().ssconv_pad_channels
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p]
     _check("ssconv_pad_channels", f(_ptr(x), _ptr(y), pixels, c, C_pad, _stream(stream)))
     return y
 
@@ -483,9 +500,6 @@ def ssconv_sizes_grouped(desc: Desc, groups: int):
     G = ctypes.c_int64()
     a, b = ctypes.c_size_t(), ctypes.c_size_t()
     f = lib().ssconv_sizes_grouped
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_int32, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_size_t),
-                  ctypes.POINTER(ctypes.c_size_t)]
     _check("ssconv_sizes_grouped", f(ctypes.byref(desc), groups, ctypes.byref(G), ctypes.byref(a), ctypes.byref(b)))
     return int(G.value), int(a.value), int(b.value)
 
@@ -494,11 +508,9 @@ def ssconv_compress_grouped(desc: Desc, groups: int, w: torch.Tensor, pattern: t
     """(w_comp, meta) of a grouped layer: the per-group blobs one after another."""
     _need_cuda(w, pattern)
     _, nv, nm = ssconv_sizes_grouped(desc, groups)
-    w_comp = torch.empty((nv,), dtype=torch.uint8, device=w.device)
-    meta = torch.empty((nm,), dtype=torch.uint8, device=w.device)
+    w_comp = torch.empty(nv, dtype=torch.uint8, device=w.device)
+    meta = torch.empty(nm, dtype=torch.uint8, device=w.device)
     f = lib().ssconv_compress_grouped
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_int32] + [ctypes.c_void_p] * 5
     _check("ssconv_compress_grouped", f(ctypes.byref(desc), groups, _ptr(w), _ptr(pattern), _ptr(w_comp), _ptr(meta),
                                         _stream(stream)))
     return w_comp, meta
@@ -513,9 +525,6 @@ def ssconv_forward_grouped(desc: Desc, groups: int, x: torch.Tensor, w_comp: tor
         y = _alloc_y(desc, x)
     ws = default_workspace(x.device)
     f = lib().ssconv_forward_grouped
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_int32] + [ctypes.c_void_p] * 6 + [ctypes.c_size_t, ctypes.c_void_p,
-                                                                                  ctypes.c_void_p]
     _check("ssconv_forward_grouped", f(ctypes.byref(desc), groups, _ptr(x), _ptr(w_comp), _ptr(meta), _ptr(bias), _ptr(y),
                                        _ptr(ws), ws.numel(), _ptr(dev_status), _stream(stream)))
     return y
@@ -530,9 +539,6 @@ def ssconv_forward_dense_grouped(desc: Desc, groups: int, x: torch.Tensor, w: to
         y = _alloc_y(desc, x)
     ws = default_workspace(x.device)
     f = lib().ssconv_forward_dense_grouped
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_int32] + [ctypes.c_void_p] * 5 + [ctypes.c_size_t, ctypes.c_void_p,
-                                                                                  ctypes.c_void_p]
     _check("ssconv_forward_dense_grouped", f(ctypes.byref(desc), groups, _ptr(x), _ptr(w), _ptr(bias), _ptr(y), _ptr(ws),
                                              ws.numel(), _ptr(dev_status), _stream(stream)))
     return y
@@ -545,8 +551,6 @@ def ssconv_depthwise(desc: Desc, x: torch.Tensor, w: torch.Tensor, bias: Optiona
     if y is None:
         y = _alloc_y(desc, x)
     f = lib().ssconv_depthwise
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc)] + [ctypes.c_void_p] * 5
     _check("ssconv_depthwise", f(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(y), _stream(stream)))
     return y
 
@@ -559,9 +563,6 @@ def ssconv_layernorm(x: torch.Tensor, gamma: torch.Tensor, beta: torch.Tensor, e
     if y is None:
         y = torch.empty_like(x)
     f = lib().ssconv_layernorm
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_float, ctypes.c_void_p, ctypes.c_int64,
-                  ctypes.c_int32, ctypes.c_void_p]
     _check("ssconv_layernorm", f(_ptr(x), _ptr(gamma), _ptr(beta), float(eps), _ptr(y), x.numel() // c, c, _stream(stream)))
     return y
 
@@ -574,8 +575,6 @@ def ssconv_quantize_e4m3(x: torch.Tensor, scale: float = 1.0, y: Optional[torch.
     if y is None:
         y = torch.empty(x.shape, dtype=torch.uint8, device=x.device)
     f = lib().ssconv_quantize_e4m3
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_float, ctypes.c_void_p]
     _check("ssconv_quantize_e4m3", f(_ptr(x), _ptr(y), x.numel(), float(scale), _stream(stream)))
     return y
 
@@ -585,9 +584,6 @@ def ssconv_sizes_fp8(desc: Desc):
     G = ctypes.c_int64()
     a, b = ctypes.c_size_t(), ctypes.c_size_t()
     f = lib().ssconv_sizes_fp8
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_size_t),
-                  ctypes.POINTER(ctypes.c_size_t)]
     _check("ssconv_sizes_fp8", f(ctypes.byref(desc), ctypes.byref(G), ctypes.byref(a), ctypes.byref(b)))
     return int(G.value), int(a.value), int(b.value)
 
@@ -596,11 +592,9 @@ def ssconv_compress_fp8(desc: Desc, w: torch.Tensor, pattern: torch.Tensor, stre
     """(w_comp, meta) uint8 blobs from e4m3 weights [C_out,KH,KW,C_in] (uint8) and pattern [G]."""
     _need_cuda(w, pattern)
     _, nv, nm = ssconv_sizes_fp8(desc)
-    w_comp = torch.empty((nv,), dtype=torch.uint8, device=w.device)
-    meta = torch.empty((nm,), dtype=torch.uint8, device=w.device)
+    w_comp = torch.empty(nv, dtype=torch.uint8, device=w.device)
+    meta = torch.empty(nm, dtype=torch.uint8, device=w.device)
     f = lib().ssconv_compress_fp8
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc)] + [ctypes.c_void_p] * 5
     _check("ssconv_compress_fp8", f(ctypes.byref(desc), _ptr(w), _ptr(pattern), _ptr(w_comp), _ptr(meta), _stream(stream)))
     return w_comp, meta
 
@@ -610,10 +604,8 @@ def ssconv_decompress_fp8(desc: Desc, w_comp: torch.Tensor, meta: torch.Tensor, 
     _need_cuda(w_comp, meta)
     G, _, _ = ssconv_sizes_fp8(desc)
     w_out = torch.empty((desc.C_out, desc.KH, desc.KW, desc.C_in), dtype=torch.uint8, device=w_comp.device)
-    pat = torch.empty((G,), dtype=torch.uint8, device=w_comp.device)
+    pat = torch.empty(G, dtype=torch.uint8, device=w_comp.device)
     f = lib().ssconv_decompress_fp8
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc)] + [ctypes.c_void_p] * 5
     _check("ssconv_decompress_fp8", f(ctypes.byref(desc), _ptr(w_comp), _ptr(meta), _ptr(w_out), _ptr(pat), _stream(stream)))
     return w_out, pat
 
@@ -626,8 +618,6 @@ def ssconv_forward_fp8(desc: Desc, x: torch.Tensor, w_comp: torch.Tensor, meta: 
     if y is None:
         y = _alloc_y(desc, x)
     f = lib().ssconv_forward_fp8
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc)] + [ctypes.c_void_p] * 4 + [ctypes.c_float] + [ctypes.c_void_p] * 3
     _check("ssconv_forward_fp8", f(ctypes.byref(desc), _ptr(x), _ptr(w_comp), _ptr(meta), _ptr(bias), float(out_scale),
                                    _ptr(y), _ptr(dev_status), _stream(stream)))
     return y
@@ -641,8 +631,6 @@ def ssconv_forward_dense_fp8(desc: Desc, x: torch.Tensor, w: torch.Tensor, bias:
     if y is None:
         y = _alloc_y(desc, x)
     f = lib().ssconv_forward_dense_fp8
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc)] + [ctypes.c_void_p] * 3 + [ctypes.c_float] + [ctypes.c_void_p] * 3
     _check("ssconv_forward_dense_fp8", f(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), float(out_scale), _ptr(y),
                                          _ptr(dev_status), _stream(stream)))
     return y
@@ -660,9 +648,6 @@ def ssconv_soft_mask(logits: torch.Tensor, noise: Optional[torch.Tensor], tau: f
     if w_eff is None and want_w_eff:
         w_eff = torch.empty_like(w)
     f = lib().ssconv_soft_mask
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_float, ctypes.c_void_p, ctypes.c_int64,
-                  ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_soft_mask", f(_ptr(logits), _ptr(noise), float(tau), _ptr(w), G, _ptr(z), _ptr(w_eff),
                                  _stream(stream)))
     return z, w_eff
@@ -676,9 +661,6 @@ def ssconv_mask_grad(z: torch.Tensor, tau: float, w: torch.Tensor, g_w_eff: torc
     if g_logits is None:
         g_logits = torch.empty((G, 6), dtype=torch.float32, device=z.device)
     f = lib().ssconv_mask_grad
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_float, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64,
-                  ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_mask_grad", f(_ptr(z), float(tau), _ptr(w), _ptr(g_w_eff), G, _ptr(g_logits), _stream(stream)))
     return g_logits
 
@@ -686,8 +668,6 @@ def ssconv_mask_grad(z: torch.Tensor, tau: float, w: torch.Tensor, g_w_eff: torc
 def ssconv_wgrad_ws_bytes(desc: Desc) -> int:
     n = ctypes.c_size_t()
     f = lib().ssconv_wgrad_ws_bytes
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.POINTER(ctypes.c_size_t)]
     _check("ssconv_wgrad_ws_bytes", f(ctypes.byref(desc), ctypes.byref(n)))
     return int(n.value)
 
@@ -701,12 +681,9 @@ def ssconv_wgrad(desc: Desc, x: torch.Tensor, dy: torch.Tensor, dw: Optional[tor
         dw = torch.empty((desc.C_out, desc.KH, desc.KW, desc.C_in), dtype=torch.float32, device=x.device)
     if ws is None:
         need = ssconv_wgrad_ws_bytes(desc)
-        ws = torch.empty((need,), dtype=torch.uint8, device=x.device) if need else None
-    ws_bytes = 0 if ws is None else ws.numel() * ws.element_size()
+        ws = torch.empty(need, dtype=torch.uint8, device=x.device) if need else None
+    ws_bytes = 0 if ws is None else ws.nbytes
     f = lib().ssconv_wgrad
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
-                  ctypes.c_size_t, ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_wgrad", f(ctypes.byref(desc), _ptr(x), _ptr(dy), _ptr(dw), _ptr(ws), ws_bytes, _ptr(dev_status),
                              _stream(stream)))
     return dw
@@ -715,8 +692,6 @@ def ssconv_wgrad(desc: Desc, x: torch.Tensor, dy: torch.Tensor, dw: Optional[tor
 def ssconv_dgrad_ws_bytes(desc: Desc) -> int:
     n = ctypes.c_size_t()
     f = lib().ssconv_dgrad_ws_bytes
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.POINTER(ctypes.c_size_t)]
     _check("ssconv_dgrad_ws_bytes", f(ctypes.byref(desc), ctypes.byref(n)))
     return int(n.value)
 
@@ -731,9 +706,6 @@ def ssconv_dgrad(desc: Desc, dy: torch.Tensor, w: torch.Tensor, dx: Optional[tor
     if ws is None:
         ws = torch.empty((max(ssconv_dgrad_ws_bytes(desc), 16),), dtype=torch.uint8, device=dy.device)
     f = lib().ssconv_dgrad
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
-                  ctypes.c_size_t, ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_dgrad", f(ctypes.byref(desc), _ptr(dy), _ptr(w), _ptr(dx), _ptr(ws), ws.numel() * ws.element_size(),
                              _ptr(dev_status), _stream(stream)))
     return dx
@@ -747,8 +719,6 @@ def ssconv_adamw(theta: torch.Tensor, g: torch.Tensor, m: torch.Tensor, v: torch
     assert theta.dtype == g.dtype == m.dtype == v.dtype == torch.float32
     assert theta.numel() == g.numel() == m.numel() == v.numel()
     f = lib().ssconv_adamw
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p] * 4 + [ctypes.c_int64, ctypes.c_int32] + [ctypes.c_float] * 5 + [ctypes.c_void_p]
     _check("ssconv_adamw", f(_ptr(theta), _ptr(g), _ptr(m), _ptr(v), theta.numel(), int(step), float(lr),
                              float(beta1), float(beta2), float(eps), float(weight_decay), _stream(stream)))
     return theta
@@ -769,8 +739,6 @@ def ssconv_unfold_w(x: torch.Tensor, KW: int, stride: int = 1, pad: int = 0, dil
         y = torch.empty((*lead, ssconv_window_extent(w, KW, stride, pad, dil), C_pad), dtype=torch.bfloat16,
                         device=x.device)
     f = lib().ssconv_unfold_w
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64] + [ctypes.c_int32] * 7 + [ctypes.c_void_p]
     _check("ssconv_unfold_w", f(_ptr(x), _ptr(y), rows, w, c, KW, stride, pad, dil, C_pad, _stream(stream)))
     return y
 
@@ -788,8 +756,6 @@ def ssconv_mask_norms(w: torch.Tensor, pattern: torch.Tensor, out: Optional[torc
     if out is None:
         out = torch.empty((3,), dtype=torch.float32, device=w.device)
     f = lib().ssconv_mask_norms
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_mask_norms", f(_ptr(w), _ptr(pattern), c_out, k, _ptr(out), _stream(stream)))
     return out
 
@@ -800,8 +766,6 @@ def ssconv_absmax(x: torch.Tensor, out: Optional[torch.Tensor] = None, stream=No
     if out is None:
         out = torch.empty((1,), dtype=torch.float32, device=x.device)
     f = lib().ssconv_absmax
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_absmax", f(_ptr(x), x.numel(), _ptr(out), _stream(stream)))
     return out
 
@@ -811,9 +775,6 @@ def ssconv_stability_threshold(lemma: int, L: float, layer_norms, j: int, extra_
     n = len(layer_norms)
     arr = (ctypes.c_double * n)(*[float(v) for v in layer_norms])
     f = lib().ssconv_stability_threshold
-    f.restype = ctypes.c_double
-    f.argtypes = [ctypes.c_int32, ctypes.c_double, ctypes.POINTER(ctypes.c_double), ctypes.c_int32, ctypes.c_int32,
-                  ctypes.c_double, ctypes.c_double]
     v = float(f(lemma, float(L), arr, n, j, float(extra_norm), float(x_norm)))
     if v < 0:
         raise ValueError("bad arguments to ssconv_stability_threshold")
@@ -830,8 +791,6 @@ def ssconv_dgrad_prepare(desc: Desc, w: Optional[torch.Tensor], stream=None):
     if w is not None:
         w_t = torch.empty((desc.C_in, desc.KH, desc.KW, desc.C_out), dtype=torch.bfloat16, device=w.device)
     f = lib().ssconv_dgrad_prepare
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTER(Desc), ctypes.c_void_p]
     _check("ssconv_dgrad_prepare", f(ctypes.byref(desc), _ptr(w), _ptr(w_t), ctypes.byref(out), _stream(stream)))
     return out, w_t
 
@@ -844,7 +803,5 @@ def ssconv_dgrad_spread(desc: Desc, dy: torch.Tensor, stream=None) -> torch.Tens
     Wz = ssconv_window_extent(desc.W, desc.KW, 1, desc.pad_w, desc.dil_w)
     out = torch.empty((desc.N, Hz, Wz, desc.C_out), dtype=torch.bfloat16, device=dy.device)
     f = lib().ssconv_dgrad_spread
-    f.restype = ctypes.c_int32
-    f.argtypes = [ctypes.POINTER(Desc), ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
     _check("ssconv_dgrad_spread", f(ctypes.byref(desc), _ptr(dy), _ptr(out), _stream(stream)))
     return out
