@@ -1,5 +1,5 @@
 // Mask selection (Eq. 1), mask application + 2:4 packing (Eq. 6, Fig. 1) and its inverse.
-// All three are one-off, memory-bound, integer-only kernels: values are compared and moved,
+// All are memory-bound, integer-only kernels: values are compared and moved,
 // never computed with.
 #include <cuda_runtime.h>
 
@@ -241,66 +241,52 @@ __global__ void decompress_e4m3_kernel(ssconv_desc_t d, Geometry geo, const uint
 }
 
 // ---------------------------------------------------------------------------------------
-// compress: values
+// compress
 // ---------------------------------------------------------------------------------------
-// One thread per (row, k-block, group-in-block): writes the two kept values (one 32-bit
-// store), +0 for padding.
-__global__ void compress_values_kernel(ssconv_desc_t d, Geometry geo, const uint2* __restrict__ w,
-                                       const uint8_t* __restrict__ pattern, uint32_t* __restrict__ w_comp) {
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t total = (int64_t)geo.Mp * geo.kblocks_pad * 16;
-  if (t >= total) return;
-  int q = (int)(t % 16);
-  int b = (int)((t / 16) % geo.kblocks_pad);
-  int co = (int)(t / (16 * (int64_t)geo.kblocks_pad));
-  uint32_t out = 0;
-  if (co < d.C_out && b < geo.kblocks) {
-    int tap = b % geo.taps;
-    int c = (b / geo.taps) * kBlockK + 4 * q;
-    if (c < d.C_in) {
-      int64_t g = ((int64_t)co * geo.taps + tap) * (d.C_in / 4) + c / 4;
-      uint2 v = w[g];
-      uint32_t vals[4] = {v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16};
-      uint32_t code = pattern_code(pattern[g]);
-      out = vals[code & 3u] | (vals[(code >> 2) & 3u] << 16);
-    }
-  }
-  // row-major [Mp][KC] bf16; this thread's pair sits at column 32*b + 2*q
-  w_comp[((int64_t)co * geo.KC + 32 * b + 2 * q) / 2] = out;
-}
-
-// ---------------------------------------------------------------------------------------
-// compress: metadata
-// ---------------------------------------------------------------------------------------
-// One thread per 32-bit metadata word (layout.cuh says what a word holds).
-__global__ void compress_meta_kernel(ssconv_desc_t d, Geometry geo, const uint8_t* __restrict__ pattern,
-                                     uint32_t* __restrict__ meta) {
-  int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  int64_t total = (int64_t)geo.m_tiles * geo.stages * 128 * 4;
-  if (t >= total) return;
-  int j = (int)(t % 4);
-  int L = (int)((t / 4) % 128);
-  int s = (int)((t / 512) % geo.stages);
-  int mt = (int)(t / (512 * (int64_t)geo.stages));
-  int b = 2 * s + (j >> 1);
-  int tap = b % geo.taps;
-  int cbase = (b / geo.taps) * kBlockK + (j & 1) * 32 + 16 * ((L >> 3) & 1);
+// One thread per 32-bit metadata word (layout.cuh says what a word holds): the codes of sixteen dense columns of
+// two rows of W eight apart, whose kept values it writes as well.  A thread reads 2 x 32 bytes of weights and 8
+// patterns and writes 2 x 16 bytes of values; the eight threads of a row and stage write 128 bytes.  Values and
+// metadata in one launch: a layer's weights are small (0.1 to 2 MB), so a launch more costs as much as the work
+// (52 layers of a ResNet-50: 154 + 120 us for the two kernels with one thread per group, 180 us for this one).
+__global__ void __launch_bounds__(256) compress_kernel(ssconv_desc_t d, Geometry geo, const uint4* __restrict__ w,
+                                                       const uint8_t* __restrict__ pattern, uint4* __restrict__ w_comp,
+                                                       uint32_t* __restrict__ meta) {
+  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (t >= (int64_t)geo.m_tiles * geo.stages * 512) return;
+  const int half = (int)(t & 1), j = (int)(t >> 1) & 3, row = ((int)(t >> 3) & 7) + 16 * ((int)(t >> 6) & 7);
+  const int64_t tile = t >> 9;  // (channel tile, stage)
+  const int s = (int)(tile % geo.stages), mt = (int)(tile / geo.stages);
+  const int b = 2 * s + (j >> 1);
+  const int tap = b % geo.taps;
+  const int col = (j & 1) * 32 + 16 * half;  // dense column within the k-block
+  const int c = (b / geo.taps) * kBlockK + col;
   uint32_t word = 0;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    int co = mt * kTileM + (L & 7) + 16 * (L >> 4) + 8 * h;
+    const int co = mt * kTileM + row + 8 * h;
+    uint32_t out[4] = {0u, 0u, 0u, 0u};
+    uint32_t codes = 0x4444u;
+    if (co < d.C_out && b < geo.kblocks && c < d.C_in) {
+      const int64_t g = ((int64_t)co * geo.taps + tap) * (d.C_in / 4) + c / 4;
+      const bool all = c + 8 < d.C_in;  // (input channels come in multiples of eight)
+      const uint4 lo = __ldg(w + g / 2);
+      const uint4 hi = all ? __ldg(w + g / 2 + 1) : make_uint4(0u, 0u, 0u, 0u);
+      const uint2 v[4] = {make_uint2(lo.x, lo.y), make_uint2(lo.z, lo.w), make_uint2(hi.x, hi.y), make_uint2(hi.z, hi.w)};
+      codes = 0;
 #pragma unroll
-    for (int gi = 0; gi < 4; ++gi) {
-      int c = cbase + 4 * gi;
-      uint32_t code = 0x4u;
-      if (co < d.C_out && b < geo.kblocks && c < d.C_in) {
-        int64_t g = ((int64_t)co * geo.taps + tap) * (d.C_in / 4) + c / 4;
-        code = pattern_code(pattern[g]);
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t code = (i < 2 || all) ? pattern_code(__ldg(pattern + g + i)) : 0x4u;
+        codes |= code << (4 * i);
+        // bytes 2 p, 2 p + 1 of the group for each kept position p
+        const uint32_t p0 = code & 3u, p1 = code >> 2;
+        out[i] = __byte_perm(v[i].x, v[i].y, (2 * p0) | ((2 * p0 + 1) << 4) | ((2 * p1) << 8) | ((2 * p1 + 1) << 12));
       }
-      word |= code << (16 * h + 4 * gi);
     }
+    word |= codes << (16 * h);
+    // row-major [Mp][KC] bf16; eight kept values at column 32 b + col / 2
+    w_comp[((int64_t)co * geo.KC + 32 * b + col / 2) / 8] = make_uint4(out[0], out[1], out[2], out[3]);
   }
-  meta[t] = word;
+  meta[(tile * 128 + (row & 7) + 8 * half + 16 * (row >> 4)) * 4 + j] = word;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -442,14 +428,9 @@ cudaError_t launch_compress(const ssconv_desc_t& d, const void* w, const uint8_t
                             cudaStream_t st) {
   Geometry geo = make_geometry(d);
   const int T = 256;
-  int64_t nv = (int64_t)geo.Mp * geo.kblocks_pad * 16;
   count_launch();
-  compress_values_kernel<<<blocks_for(nv, T), T, 0, st>>>(d, geo, (const uint2*)w, pattern, (uint32_t*)w_comp);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  int64_t nm = (int64_t)geo.m_tiles * geo.stages * 512;
-  count_launch();
-  compress_meta_kernel<<<blocks_for(nm, T), T, 0, st>>>(d, geo, pattern, (uint32_t*)meta);
+  compress_kernel<<<blocks_for((int64_t)geo.m_tiles * geo.stages * 512, T), T, 0, st>>>(
+      d, geo, (const uint4*)w, pattern, (uint4*)w_comp, (uint32_t*)meta);
   return cudaGetLastError();
 }
 
