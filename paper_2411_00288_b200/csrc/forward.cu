@@ -115,6 +115,8 @@ struct FwdParams {
   int taps, cblocks, kblocks;
   int m_tiles, num_tiles;   // (pair kernel: m_tiles counts pairs of 128-channel tiles, m_real the tiles themselves)
   int m_real;
+  int groups, m_group;      // one-block kernel: channel groups in this launch (m_tiles counts all their tiles), tiles of
+                            // one; C_in and C_out are a group's
   int a_tiles;              // pairs of k-blocks (groups) per output tile
   int dual;                 // pair kernel: a work item is two neighbouring position tiles sharing the group's weights
   int split;                // 1: units dealt out evenly across CTAs (stream-K); 0: whole tiles per CTA
@@ -386,6 +388,10 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
     const Pos q0 = decode_pos(pt * p.BN, p.Wo, p.Ho);
     const int base_w = q0.c * p.stride_w - p.pad_w;
     const int base_h = q0.r * p.stride_h - p.pad_h;
+    const int grp = p.groups > 1 ? m / p.m_group : 0;
+    const int ch0 = grp * p.C_in;  // the group's first input channel
+    // (the compressed operands of the groups follow one another in whole tiles, dense weights do not)
+    const int a_row = SPARSE ? m * kTileM : grp * p.C_out + (m - grp * p.m_group) * kTileM;
     const uint8_t* meta_src = p.meta + ((size_t)m * p.a_tiles + seg.a0) * C::kMetaBytes;
     TapIter it;
     it.init(2 * seg.a0 + (ROLE == kRoleActSecond ? 1 : 0), p);
@@ -401,7 +407,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
         TapIter rit;
         rit.init(0, p);
         for (int b = 0; b < p.kblocks; ++b) {
-          tma_load_3d_w(res0 + (uint32_t)b * kATileBytes, tm_a, res_bar, rit.cc * kKb, rit.tap, m * kTileM);
+          tma_load_3d_w(res0 + (uint32_t)b * kATileBytes, tm_a, res_bar, rit.cc * kKb, rit.tap, a_row);
           rit.advance(p);
         }
       }
@@ -429,7 +435,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
         } else if (ROLE == kRoleWeights) {
           mbar_expect_tx_w(full, (uint32_t)chunks * 2048u);
           for (int j = 0; j < chunks; ++j) {  // chunks 8.. belong to the second k-block: 16 KB further on = 8 x 2048
-            tma_load_3d_w(dst + (uint32_t)j * 2048u, tm_a, full, it.cc * kKb, it.tap, m * kTileM);
+            tma_load_3d_w(dst + (uint32_t)j * 2048u, tm_a, full, it.cc * kKb, it.tap, a_row);
             it.advance(p);
           }
         } else {
@@ -447,20 +453,20 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
       } else if (ROLE == kRoleWeights) {
         if (SPARSE) {
           mbar_expect_tx_w(full, C::kAGroupBytes);
-          tma_load_2d_w(dst, tm_a, full, a * (FP8 ? 128 : 64), m * kTileM);  // 128 bytes of kept values per group
+          tma_load_2d_w(dst, tm_a, full, a * (FP8 ? 128 : 64), a_row);  // 128 bytes of kept values per group
           bulk_load_w(dst + kATileBytes, meta_src, C::kMetaBytes, full);
           meta_src += C::kMetaBytes;
         } else {
           mbar_expect_tx_w(full, has_second ? 2 * kATileBytes : kATileBytes);
-          tma_load_3d_w(dst, tm_a, full, it.cc * kKb, it.tap, m * kTileM);
+          tma_load_3d_w(dst, tm_a, full, it.cc * kKb, it.tap, a_row);
           it.advance(p);
-          if (has_second) tma_load_3d_w(dst + kATileBytes, tm_a, full, it.cc * kKb, it.tap, m * kTileM);
+          if (has_second) tma_load_3d_w(dst + kATileBytes, tm_a, full, it.cc * kKb, it.tap, a_row);
           it.advance(p);
         }
       } else if (ROLE == kRoleActFirst || has_second) {
         mbar_expect_tx_w(full, b_bytes);
         tma_load_im2col_4d_w(dst + p.a_grp_bytes + (ROLE == kRoleActSecond ? b_bytes : 0u), tm_b, full,
-                             it.cc * kKb, base_w, base_h, q0.n, (uint16_t)it.off_w, (uint16_t)it.off_h);
+                             ch0 + it.cc * kKb, base_w, base_h, q0.n, (uint16_t)it.off_w, (uint16_t)it.off_h);
         it.advance(p);
         it.advance(p);
       } else {
@@ -811,11 +817,12 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       }
       // ---- finish the tile: bias, activation, bf16, transposed staging, TMA stores ---------------
       // the four channels whose accumulators this thread receives: 8 i + lane / 4 of the warp's 32
+      const int cgrp = p.groups > 1 ? m / p.m_group : 0, c0 = (m - cgrp * p.m_group) * kTileM;  // channel group, channel in it
       float bias_v[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int co = m * kTileM + q * 32 + 8 * i + (lane >> 2);
-        bias_v[i] = ((p.flags & SSCONV_FLAG_BIAS) && co < p.C_out) ? p.bias[co] : 0.0f;
+        const int co = c0 + q * 32 + 8 * i + (lane >> 2);
+        bias_v[i] = ((p.flags & SSCONV_FLAG_BIAS) && co < p.C_out) ? p.bias[cgrp * p.C_out + co] : 0.0f;
       }
 #pragma unroll 1
       for (int piece = 0; piece < p.pieces; ++piece, ++piece_count) {
@@ -867,8 +874,14 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
             // positions beyond Q and channels beyond C_out fall outside the tensor map and are dropped;
             // a short last piece goes through the map whose box holds just its positions
             const CUtensorMap* map = (piece == p.pieces - 1 && p.tail_cols != kPiece) ? &tm_y_tail : &tm_y;
-            tma_store_2d(map, stage, m * kTileM, q_piece);
-            if (m * kTileM + 64 < p.C_out) tma_store_2d(map, stage + kHalfPieceBytes, m * kTileM + 64, q_piece);
+            const bool two = c0 + 64 < p.C_out;
+            if (p.groups > 1) {  // the map's third dimension is the group: its channels are clipped at the group's end
+              tma_store_3d(map, stage, c0, q_piece, cgrp);
+              if (two) tma_store_3d(map, stage + kHalfPieceBytes, c0 + 64, q_piece, cgrp);
+            } else {
+              tma_store_2d(map, stage, c0, q_piece);
+              if (two) tma_store_2d(map, stage + kHalfPieceBytes, c0 + 64, q_piece);
+            }
           }
           bulk_commit_group();
           if (RES) {
@@ -1742,10 +1755,10 @@ constexpr int kWideStageBufs = 4;  // staging buffers per half of a tile: two fo
 // The plan for a layer without a residual: one-CTA tiles (whole or K split) or the pair kernel.
 template <bool SPARSE>
 static Plan choose_plan(const ssconv_desc_t& d, long long Q, const Geometry& geo, int workers, bool force_split,
-                        bool allow_split = true, bool allow_wide = true) {
+                        bool allow_split = true, bool allow_wide = true, bool allow_pair = true) {
   const Plan plan = plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, allow_split);
   if (force_split || small_channel_mode(d, SPARSE)) return plan;
-  if (g_tune_pair != 0) {
+  if (allow_pair && g_tune_pair != 0) {
     const Plan pair = plan_pair<SPARSE>(Q, geo, workers, g_tune_pair == 1);
     if (pair.BN != 0 && (g_tune_pair == 1 || plan.cost > kPairAdvantage * pair.cost)) return pair;
   }
@@ -1806,7 +1819,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
                                    const float* bias, const void* residual, void* y, void* ws, size_t ws_bytes,
                                    int32_t* dev_status, cudaStream_t stream, int worker_cap = kMaxWorkers,
                                    bool force_split = false, const int64_t* x_strides = nullptr,
-                                   float out_scale = 1.0f, int64_t y_pitch = 0) {
+                                   float out_scale = 1.0f, int64_t y_pitch = 0, int groups = 1) {
   using C = Cfg<SPARSE, FP8>;
   constexpr int kKb = C::kKbChannels;
   constexpr size_t kElem = FP8 ? 1 : 2;  // bytes per operand element
@@ -1840,7 +1853,9 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
       return SSCONV_ERR_CUDA;
     g_fp8_attr_set[dev][SPARSE ? 1 : 0] = true;
   }
-  const Geometry geo = layer_geometry(d, SPARSE, FP8);
+  Geometry geo = layer_geometry(d, SPARSE, FP8);
+  const int m_group = geo.m_tiles;
+  geo.m_tiles *= groups;  // (groups > 1: one launch for all channel groups, whole tiles of the one-block kernel)
   const bool small_c = !FP8 && small_channel_mode(d, SPARSE);
   const int Ho = out_extent(d.H, d.KH, d.stride_h, d.pad_h, d.dil_h);
   const int Wo = out_extent(d.W, d.KW, d.stride_w, d.pad_w, d.dil_w);
@@ -1857,7 +1872,8 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   if (have_ws && (reinterpret_cast<uintptr_t>(ws) & 15u)) return SSCONV_ERR_ALIGNMENT;
   if (force_split && !have_ws) return SSCONV_ERR_WORKSPACE;
   // (8-bit operands: the pair kernel exists for the 2:4 form only; the dense counterpart stays on one-block tiles)
-  Plan plan = (residual != nullptr || (FP8 && !SPARSE)) ? plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, have_ws)
+  Plan plan = groups > 1 ? choose_plan<SPARSE>(d, Q, geo, workers, false, false, true, false)
+              : (residual != nullptr || (FP8 && !SPARSE)) ? plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, have_ws)
                                                         : choose_plan<SPARSE>(d, Q, geo, workers, force_split, have_ws, !FP8);
   int stage_bufs = 2;
   if (residual != nullptr && !plan.split) {
@@ -1928,7 +1944,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   // activations: NHWC seen as (c, w, h, n), im2col mode; elements outside the image read as zero
   // (= the zero padding of Eq. 4); base pixels are the filter placements, each load adds a tap offset
   {
-    cuuint64_t dims[4] = {(cuuint64_t)d.C_in, (cuuint64_t)d.W, (cuuint64_t)d.H, (cuuint64_t)d.N};
+    cuuint64_t dims[4] = {(cuuint64_t)d.C_in * groups, (cuuint64_t)d.W, (cuuint64_t)d.H, (cuuint64_t)d.N};
     cuuint64_t strides[3] = {(cuuint64_t)d.C_in * kElem, (cuuint64_t)d.W * d.C_in * kElem,
                              (cuuint64_t)d.H * d.W * d.C_in * kElem};
     if (x_strides != nullptr)  // a strided (possibly overlapping) view: element strides of w, h, n
@@ -1951,7 +1967,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   }
   if (SPARSE) {
     // kept values: 64 bytes per row and k-block (KC counts 2-byte units); a box is 128 rows x 128 bytes
-    cuuint64_t dims[2] = {(cuuint64_t)geo.KC * 2 / kElem, (cuuint64_t)geo.Mp};
+    cuuint64_t dims[2] = {(cuuint64_t)geo.KC * 2 / kElem, (cuuint64_t)geo.Mp * groups};
     cuuint64_t strides[1] = {(cuuint64_t)geo.KC * 2};
     cuuint32_t box[2] = {(cuuint32_t)(128 / kElem), (cuuint32_t)kTileM};
     cuuint32_t estr[2] = {1, 1};
@@ -1962,7 +1978,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   } else {
     // dense weights [C_out][taps][C_in] seen as (c, tap, output channel); 8-channel mode: one tap's
     // 8 channels of 128 rows per load, unswizzled
-    cuuint64_t dims[3] = {(cuuint64_t)d.C_in, (cuuint64_t)geo.taps, (cuuint64_t)d.C_out};
+    cuuint64_t dims[3] = {(cuuint64_t)d.C_in, (cuuint64_t)geo.taps, (cuuint64_t)d.C_out * groups};
     cuuint64_t strides[2] = {(cuuint64_t)d.C_in * kElem, (cuuint64_t)geo.taps * d.C_in * kElem};
     cuuint32_t box[3] = {small_c ? 8u : (cuuint32_t)kKb, 1, (cuuint32_t)kTileM};
     cuuint32_t estr[3] = {1, 1, 1};
@@ -1989,17 +2005,19 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   }
   // output: NHWC seen as (c, position); a box is one staging half piece, 64 channels x 40 positions
   {
-    cuuint64_t dims[2] = {(cuuint64_t)d.C_out, (cuuint64_t)Q};
-    cuuint64_t strides[1] = {(cuuint64_t)y_pitch_el * 2};  // (channels beyond C_out are clipped: a slice stays a slice)
-    cuuint32_t box[2] = {64, (cuuint32_t)kPiece};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = g_encode_tiled(&tm_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, y, dims, strides, box, estr,
+    cuuint64_t dims[3] = {(cuuint64_t)d.C_out, (cuuint64_t)Q, (cuuint64_t)groups};
+    // (channels beyond C_out are clipped: a slice stays a slice)
+    cuuint64_t strides[2] = {(cuuint64_t)y_pitch_el * 2, (cuuint64_t)d.C_out * 2};
+    cuuint32_t box[3] = {64, (cuuint32_t)kPiece, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    const cuuint32_t rank = groups > 1 ? 3 : 2;
+    CUresult r = g_encode_tiled(&tm_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, y, dims, strides, box, estr,
                                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                 CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
     // the last piece of a group may hold fewer positions: same view, shorter box
     box[1] = (cuuint32_t)tail_cols;
-    r = g_encode_tiled(&tm_y_tail, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, y, dims, strides, box, estr,
+    r = g_encode_tiled(&tm_y_tail, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, y, dims, strides, box, estr,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
@@ -2046,6 +2064,8 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   p.cblocks = geo.cblocks;
   p.kblocks = geo.kblocks;
   p.m_real = geo.m_tiles;
+  p.groups = groups;
+  p.m_group = m_group;
   p.m_tiles = pair ? (geo.m_tiles + 1) / 2 : geo.m_tiles;
   const long long q_tiles = (Q + BN - 1) / BN;
   p.dual = dual ? 1 : 0;
@@ -2149,9 +2169,29 @@ int32_t launch_forward_dense(const ssconv_desc_t& d, const void* x, const void* 
                                     false, x_strides);
 }
 
+// Groups of a grouped convolution in one launch: what the model says of all groups' tiles dealt out together
+// against one launch per group (each of which may split K or use pairs, and starts and drains by itself).  A group's last
+// MMA takes up to 32 (2:4) or 16 (dense) channels, which have to be its own: the neighbouring group's would meet zero
+// weights, but an infinity among them would not vanish.  64 x 14 x 14 x 256 -> 288 in 4 groups, 3 x 3: four launches
+// 25 us, one GROUPED_US.
+constexpr double kLaunchCycles = 4000.0;
+template <bool SPARSE>
+static bool groups_in_one_launch(const ssconv_desc_t& g, int groups) {
+  if (groups < 2 || g.C_in % (SPARSE ? 32 : 16) != 0) return false;
+  int dev = 0;
+  if (current_device(&dev) != SSCONV_OK) return false;
+  const int workers = g_sm_count[dev] < kMaxWorkers ? g_sm_count[dev] : kMaxWorkers;
+  const long long Q = (long long)g.N * out_extent(g.H, g.KH, g.stride_h, g.pad_h, g.dil_h) *
+                      out_extent(g.W, g.KW, g.stride_w, g.pad_w, g.dil_w);
+  Geometry geo = layer_geometry(g, SPARSE);
+  const double each = choose_plan<SPARSE>(g, Q, geo, workers, false).cost;
+  geo.m_tiles *= groups;
+  return choose_plan<SPARSE>(g, Q, geo, workers, false, false, true, false).cost <= groups * each + (groups - 1) * kLaunchCycles;
+}
+
 // Grouped convolution: `groups` independent convolutions on channel slices, group g reading input
-// channels [g C_in/groups, ...) and writing output channels [g C_out/groups, ...); one launch per group
-// on strided views of x and y.  The compressed operand of a grouped layer is the concatenation of the
+// channels [g C_in/groups, ...) and writing output channels [g C_out/groups, ...), in one launch or in one launch per
+// group on strided views of x and y.  The compressed operand of a grouped layer is the concatenation of the
 // groups' blobs (each of the size ssconv_sizes reports for the per-group layer).
 int32_t launch_forward_grouped(const ssconv_desc_t& d, int groups, bool sparse, const void* x, const void* weights,
                                const void* meta, const float* bias, void* y, void* ws, size_t ws_bytes,
@@ -2163,16 +2203,18 @@ int32_t launch_forward_grouped(const ssconv_desc_t& d, int groups, bool sparse, 
   const size_t w_step = sparse ? (size_t)geo.Mp * geo.KC * 2 : (size_t)g.C_out * geo.taps * g.C_in * 2;
   const size_t m_step = (size_t)geo.m_tiles * geo.stages * kMetaImageBytes;
   const int64_t xs[3] = {d.C_in, (int64_t)d.W * d.C_in, (int64_t)d.H * d.W * d.C_in};
-  for (int i = 0; i < groups; ++i) {
+  const bool together = sparse ? groups_in_one_launch<true>(g, groups) : groups_in_one_launch<false>(g, groups);
+  for (int i = 0; i < (together ? 1 : groups); ++i) {
     const char* xg = static_cast<const char*>(x) + (size_t)i * g.C_in * 2;
     char* yg = static_cast<char*>(y) + (size_t)i * g.C_out * 2;
     const float* bg = bias ? bias + (size_t)i * g.C_out : nullptr;
     const char* wg = static_cast<const char*>(weights) + (size_t)i * w_step;
-    const int32_t rc =
-        sparse ? launch_forward_impl<true>(g, xg, wg, static_cast<const char*>(meta) + (size_t)i * m_step, bg, nullptr, yg,
-                                           ws, ws_bytes, dev_status, stream, kMaxWorkers, false, xs, 1.0f, d.C_out)
-               : launch_forward_impl<false>(g, xg, wg, nullptr, bg, nullptr, yg, ws, ws_bytes, dev_status, stream,
-                                            kMaxWorkers, false, xs, 1.0f, d.C_out);
+    const char* mg = sparse ? static_cast<const char*>(meta) + (size_t)i * m_step : nullptr;
+    const int n = together ? groups : 1;
+    const int32_t rc = sparse ? launch_forward_impl<true>(g, xg, wg, mg, bg, nullptr, yg, ws, ws_bytes, dev_status, stream,
+                                                          kMaxWorkers, false, xs, 1.0f, d.C_out, n)
+                              : launch_forward_impl<false>(g, xg, wg, nullptr, bg, nullptr, yg, ws, ws_bytes, dev_status,
+                                                           stream, kMaxWorkers, false, xs, 1.0f, d.C_out, n);
     if (rc != SSCONV_OK) return rc;
   }
   return SSCONV_OK;
