@@ -115,8 +115,8 @@ struct FwdParams {
   int taps, cblocks, kblocks;
   int m_tiles, num_tiles;   // (pair kernel: m_tiles counts pairs of 128-channel tiles, m_real the tiles themselves)
   int m_real;
-  int groups, m_group;      // one-block kernel: channel groups in this launch (m_tiles counts all their tiles), tiles of
-                            // one; C_in and C_out are a group's
+  int m_group;              // grouped launch: channel tiles of one group (m_tiles counts all groups' tiles; C_in and
+                            // C_out are a group's)
   int a_tiles;              // pairs of k-blocks (groups) per output tile
   int dual;                 // pair kernel: a work item is two neighbouring position tiles sharing the group's weights
   int split;                // 1: units dealt out evenly across CTAs (stream-K); 0: whole tiles per CTA
@@ -368,7 +368,7 @@ struct TapIter {
 // weights (with their metadata).  A TMA instruction occupies its issuing thread for a few hundred
 // cycles, so one thread issuing everything cannot keep up with the tensor pipe; three can.
 constexpr int kRoleActFirst = 0, kRoleActSecond = 1, kRoleWeights = 2;
-template <bool SPARSE, int ROLE, bool FP8 = false>
+template <bool SPARSE, int ROLE, bool FP8 = false, bool GROUPED = false>
 __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUtensorMap* tm_b, const FwdParams& p,
                                               uint32_t full0, uint32_t empty0, uint32_t ring0, uint32_t res_bar,
                                               volatile int* abort_flag) {
@@ -388,10 +388,10 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
     const Pos q0 = decode_pos(pt * p.BN, p.Wo, p.Ho);
     const int base_w = q0.c * p.stride_w - p.pad_w;
     const int base_h = q0.r * p.stride_h - p.pad_h;
-    const int grp = p.groups > 1 ? m / p.m_group : 0;
-    const int ch0 = grp * p.C_in;  // the group's first input channel
+    const int grp = GROUPED ? m / p.m_group : 0;
+    const int ch0 = GROUPED ? grp * p.C_in : 0;  // the group's first input channel
     // (the compressed operands of the groups follow one another in whole tiles, dense weights do not)
-    const int a_row = SPARSE ? m * kTileM : grp * p.C_out + (m - grp * p.m_group) * kTileM;
+    const int a_row = (SPARSE || !GROUPED) ? m * kTileM : grp * p.C_out + (m - grp * p.m_group) * kTileM;
     const uint8_t* meta_src = p.meta + ((size_t)m * p.a_tiles + seg.a0) * C::kMetaBytes;
     TapIter it;
     it.init(2 * seg.a0 + (ROLE == kRoleActSecond ? 1 : 0), p);
@@ -482,8 +482,9 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
 
 // RES: a residual tensor is added in the epilogue (its own instantiation, so that the plain kernel's
 // epilogue loop carries none of that code).  EPI_SETS: sets of epilogue groups; with two, each serves one of the
-// two accumulators, i.e. every other tile.
-template <bool SPARSE, bool RES, bool FP8 = false, int EPI_SETS = 1>
+// two accumulators, i.e. every other tile.  GROUPED: several channel groups in one launch (an instantiation of its own: as
+// run-time branches its few instructions cost the issuing lane of the plain epilogue 5 % on write-bound layers).
+template <bool SPARSE, bool RES, bool FP8 = false, int EPI_SETS = 1, bool GROUPED = false>
 __global__ void __launch_bounds__(threads_with(EPI_SETS), 1)
 ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                   const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_y_tail,
@@ -567,13 +568,13 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
     {
       const uint32_t full0 = smem_u32(bar_full), empty0 = smem_u32(bar_empty), ring0 = smem_u32(ring);
       if (warp == 0)
-        producer_role<SPARSE, kRoleActFirst, FP8>(&tm_a, &tm_b, p, full0,
+        producer_role<SPARSE, kRoleActFirst, FP8, GROUPED>(&tm_a, &tm_b, p, full0,
                                              p.ring_groups == 2 ? smem_u32(bar_empty_first) : empty0, ring0,
                                              smem_u32(bar_res), abort_flag);
       else if (warp == kExtraProducer)
-        producer_role<SPARSE, kRoleActSecond, FP8>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res), abort_flag);
+        producer_role<SPARSE, kRoleActSecond, FP8, GROUPED>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res), abort_flag);
       else
-        producer_role<SPARSE, kRoleWeights, FP8>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res), abort_flag);
+        producer_role<SPARSE, kRoleWeights, FP8, GROUPED>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res), abort_flag);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -817,7 +818,8 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       }
       // ---- finish the tile: bias, activation, bf16, transposed staging, TMA stores ---------------
       // the four channels whose accumulators this thread receives: 8 i + lane / 4 of the warp's 32
-      const int cgrp = p.groups > 1 ? m / p.m_group : 0, c0 = (m - cgrp * p.m_group) * kTileM;  // channel group, channel in it
+      const int cgrp = GROUPED ? m / p.m_group : 0;  // channel group; the tile's first channel in it
+      const int c0 = (GROUPED ? m - cgrp * p.m_group : m) * kTileM;
       float bias_v[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -874,13 +876,12 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
             // positions beyond Q and channels beyond C_out fall outside the tensor map and are dropped;
             // a short last piece goes through the map whose box holds just its positions
             const CUtensorMap* map = (piece == p.pieces - 1 && p.tail_cols != kPiece) ? &tm_y_tail : &tm_y;
-            const bool two = c0 + 64 < p.C_out;
-            if (p.groups > 1) {  // the map's third dimension is the group: its channels are clipped at the group's end
+            if (GROUPED) {  // the map's third dimension is the group: its channels are clipped at the group's end
               tma_store_3d(map, stage, c0, q_piece, cgrp);
-              if (two) tma_store_3d(map, stage + kHalfPieceBytes, c0 + 64, q_piece, cgrp);
+              if (c0 + 64 < p.C_out) tma_store_3d(map, stage + kHalfPieceBytes, c0 + 64, q_piece, cgrp);
             } else {
               tma_store_2d(map, stage, c0, q_piece);
-              if (two) tma_store_2d(map, stage + kHalfPieceBytes, c0 + 64, q_piece);
+              if (c0 + 64 < p.C_out) tma_store_2d(map, stage + kHalfPieceBytes, c0 + 64, q_piece);
             }
           }
           bulk_commit_group();
@@ -1500,8 +1501,19 @@ constexpr double kLoadLatencyCycles = 1000.0;
 constexpr double kIssueSparse = 365.0, kIssueDense = 480.0;
 constexpr double kEpiloguePieceCycles = 900.0;
 constexpr double kCyclesPerParkedTile = 90.0;
-constexpr double kWideTileCycles = 500.0, kWidePieceCycles = 1775.0;  // GELU epilogue on two sets of groups, per tile
+// What an epilogue that paces its layer takes per tile: fixed + per piece, whatever the piece's fill (a piece of 40
+// columns is processed whole).  Fitted to forced widths: GELU on two sets of groups; residual epilogues (128 -> 512 at
+// 28 x 28, batch 256: 80 / 112 / 144 / 160 / 176 / 208 positions 119 / 130 / 107 / 95 / 116 / 100 us: 160 positions are two
+// whole pieces per group, 208 are three with a sixth of them empty).
+struct EpilogueCycles {
+  double tile, piece;
+};
+constexpr EpilogueCycles kEpilogueHidden = {0.0, 0.0}, kEpilogueWide = {500.0, 1775.0}, kEpilogueResidual = {1314.0, 1927.0};
 constexpr double kSplitAdvantage = 1.1;  // split only if the model predicts at least this gain
+// ... and only a deep K: the finishing kernel is a launch of its own (3 us of the caller's time, 2 to 3 us on the GPU when
+// the one before it is short).  Whole tiles against split ones, one to eight images: 8 k-blocks 4.0 / 4.8 us, 16 5.0 / 5.0
+// and 5.3 / 5.9, 18 5.5 / 5.6 and 5.6 / 6.9; 24 9.7 / 6.0 and 6.3 / 6.7, 36 7.8 / 6.5, 72 12.5 / 9.2.
+constexpr int kSplitMinKBlocks = 20;
 
 static int ring_groups_for(uint32_t a_group_bytes, int BN, int stage_bufs) {
   // as many groups in the ring as fit beside the staging buffers, at most kMaxGroups
@@ -1570,7 +1582,7 @@ struct Plan {
 };
 template <bool SPARSE>
 static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force_split, int max_bn = kBN,
-                       int stage_bufs = 2, bool allow_split = true, bool wide_epilogue = false) {
+                       int stage_bufs = 2, bool allow_split = true, EpilogueCycles epilogue = kEpilogueHidden) {
   if (force_split) return Plan{kBN, true};
   int min_bn = 48;
   if (g_tune_bn != 0 && g_tune_bn <= max_bn) max_bn = min_bn = g_tune_bn;
@@ -1583,7 +1595,7 @@ static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force
     // (with at most three groups per tile the ring never reaches its steady state: such layers are paced
     // by their output stream, and measured fastest at the width the other terms choose)
     double tile = geo.kblocks * kblock_cycles<SPARSE>(BN, stage_bufs, geo.stages >= 4);
-    if (wide_epilogue) tile = fmax(tile, kWideTileCycles + pieces * kWidePieceCycles);
+    tile = fmax(tile, epilogue.tile + pieces * epilogue.piece);
     const double cost = (double)per_cta * tile + pieces * kEpiloguePieceCycles;
     if (BN == max_bn || cost < 0.97 * best_cost) {  // a narrower tile has to earn its extra weight traffic
       best_cost = cost;
@@ -1594,7 +1606,7 @@ static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force
   // Even split of K ("stream-K"), when many SMs would still idle and K is deep: every CTA gets the
   // same number of groups; parked partial tiles cost L2 traffic in proportion to the tile width.
   const int a_tiles = geo.stages;
-  if (a_tiles > 1 && allow_split) {
+  if (a_tiles > 1 && geo.kblocks >= kSplitMinKBlocks && allow_split) {
     Plan best_split{kBN, true};
     double best_split_cost = 0.0;
     for (int BN = max_bn; BN >= min_bn; BN -= 16) {
@@ -1766,7 +1778,7 @@ static Plan choose_plan(const ssconv_desc_t& d, long long Q, const Geometry& geo
   if (allow_wide && !plan.split && activation_of(d.flags) == kActGelu && geo.kblocks <= kWideMaxKBlocks &&
       (SPARSE || geo.m_tiles > 1 || geo.kblocks > 4)) {
     Plan wide = plan_layer<SPARSE>(Q, geo, workers, false, widest_tile(Cfg<SPARSE>::kAGroupBytes, kWideStageBufs),
-                                   kWideStageBufs, false, true);
+                                   kWideStageBufs, false, kEpilogueWide);
     if (((Q + wide.BN - 1) / wide.BN) * geo.m_tiles > workers) {
       wide.wide = true;
       return wide;
@@ -1843,6 +1855,8 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   }
   if (!FP8 && !g_wide_attr_set[dev][SPARSE ? 1 : 0]) {
     if (cudaFuncSetAttribute(ssconv_fwd_kernel<SPARSE, false, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kMaxSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(ssconv_fwd_kernel<SPARSE, false, false, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kMaxSmemBytes) != cudaSuccess)
       return SSCONV_ERR_CUDA;
     g_wide_attr_set[dev][SPARSE ? 1 : 0] = true;
@@ -1872,23 +1886,22 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   if (have_ws && (reinterpret_cast<uintptr_t>(ws) & 15u)) return SSCONV_ERR_ALIGNMENT;
   if (force_split && !have_ws) return SSCONV_ERR_WORKSPACE;
   // (8-bit operands: the pair kernel exists for the 2:4 form only; the dense counterpart stays on one-block tiles)
-  Plan plan = groups > 1 ? choose_plan<SPARSE>(d, Q, geo, workers, false, false, true, false)
+  Plan plan = groups > 1 ? choose_plan<SPARSE>(d, Q, geo, workers, false, false, false, false)
               : (residual != nullptr || (FP8 && !SPARSE)) ? plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, have_ws)
                                                         : choose_plan<SPARSE>(d, Q, geo, workers, force_split, have_ws, !FP8);
   int stage_bufs = 2;
   if (residual != nullptr && !plan.split) {
     stage_bufs = 4;
-    plan = plan_layer<SPARSE>(Q, geo, workers, false, widest_tile(C::kAGroupBytes, 4), 4);
-    if (plan.split) {  // the narrower limit made splitting look better: stay unsplit at the limit
-      plan.split = false;
-      plan.BN = widest_tile(C::kAGroupBytes, 4);
-    }
+    const int widest = widest_tile(C::kAGroupBytes, 4);
+    plan = plan_layer<SPARSE>(Q, geo, workers, false, widest, 4, false, kEpilogueResidual);
     // The pair kernel takes a residual too (four staging buffers per group there as well): where its model
     // wins and the ring still holds two groups, one work item is one tile.
-    if (!FP8 && !force_split && !small_c && g_tune_pair != 0) {
+    // (both costs without what their epilogues take)
+    if (!FP8 && !force_split && !small_c && g_tune_pair != 0 && (g_tune_pair == 1 || geo.kblocks >= kPairMinKBlocks)) {
       Plan pp = plan_pair<SPARSE>(Q, geo, workers, g_tune_pair == 1);
       if (pp.BN != 0 && pair_ring_groups_with(C::kAGroupBytes, pp.BN, 4) >= 2 &&
-          (g_tune_pair == 1 || plan.cost > kPairAdvantage * pp.cost)) {
+          (g_tune_pair == 1 ||
+           plan_layer<SPARSE>(Q, geo, workers, false, widest, 4, false).cost > kPairAdvantage * pp.cost)) {
         pp.dual = false;
         plan = pp;
       }
@@ -2064,7 +2077,6 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   p.cblocks = geo.cblocks;
   p.kblocks = geo.kblocks;
   p.m_real = geo.m_tiles;
-  p.groups = groups;
   p.m_group = m_group;
   p.m_tiles = pair ? (geo.m_tiles + 1) / 2 : geo.m_tiles;
   const long long q_tiles = (Q + BN - 1) / BN;
@@ -2126,6 +2138,9 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
       : pair ? cudaLaunchKernelEx(&cfg, ssconv_fwd_pair_kernel<SPARSE>, tm_a, tm_b, tm_meta, tm_y, tm_y_tail, tm_r, tm_r_tail, p)
       : residual != nullptr
           ? cudaLaunchKernelEx(&cfg, ssconv_fwd_kernel<SPARSE, true>, tm_a, tm_b, tm_y, tm_y_tail, tm_r, tm_r_tail, p)
+      : groups > 1
+          ? cudaLaunchKernelEx(&cfg, ssconv_fwd_kernel<SPARSE, false, false, 1, true>, tm_a, tm_b, tm_y, tm_y_tail, tm_r, tm_r_tail,
+                               p)
       : wide_epilogue
           ? cudaLaunchKernelEx(&cfg, ssconv_fwd_kernel<SPARSE, false, false, 2>, tm_a, tm_b, tm_y, tm_y_tail, tm_r, tm_r_tail, p)
           : cudaLaunchKernelEx(&cfg, ssconv_fwd_kernel<SPARSE, false>, tm_a, tm_b, tm_y, tm_y_tail, tm_r, tm_r_tail, p);
@@ -2173,7 +2188,7 @@ int32_t launch_forward_dense(const ssconv_desc_t& d, const void* x, const void* 
 // against one launch per group (each of which may split K or use pairs, and starts and drains by itself).  A group's last
 // MMA takes up to 32 (2:4) or 16 (dense) channels, which have to be its own: the neighbouring group's would meet zero
 // weights, but an infinity among them would not vanish.  64 x 14 x 14 x 256 -> 288 in 4 groups, 3 x 3: four launches
-// 25 us, one GROUPED_US.
+// 25 us, one 10.8 us by events of eight calls (22.0 before).
 constexpr double kLaunchCycles = 4000.0;
 template <bool SPARSE>
 static bool groups_in_one_launch(const ssconv_desc_t& g, int groups) {
@@ -2186,7 +2201,7 @@ static bool groups_in_one_launch(const ssconv_desc_t& g, int groups) {
   Geometry geo = layer_geometry(g, SPARSE);
   const double each = choose_plan<SPARSE>(g, Q, geo, workers, false).cost;
   geo.m_tiles *= groups;
-  return choose_plan<SPARSE>(g, Q, geo, workers, false, false, true, false).cost <= groups * each + (groups - 1) * kLaunchCycles;
+  return choose_plan<SPARSE>(g, Q, geo, workers, false, false, false, false).cost <= groups * each + (groups - 1) * kLaunchCycles;
 }
 
 // Grouped convolution: `groups` independent convolutions on channel slices, group g reading input
