@@ -410,8 +410,9 @@ double ssconv_stability_threshold(int32_t lemma, double L, const double* layer_n
  * pattern array follows the weight order, and the compressed operand is the concatenation of the
  * per-group blobs (ssconv_sizes_grouped gives the totals; each part is what ssconv_sizes reports for the
  * per-group layer and can be read back with ssconv_decompress).  Needs (C_in/groups) % 8 == 0 and
- * (C_out/groups) % 8 == 0; one launch per group on strided views of x and y.  ws as for
- * ssconv_forward (NULL allowed). */
+ * (C_out/groups) % 8 == 0; all groups in one launch where a group's last MMA stays inside its channels ((C_in/groups) %
+ * 32 == 0 for 2:4, % 16 for dense) and the model prefers it, else one launch per group on strided views of x and y.  ws
+ * as for ssconv_forward (NULL allowed). */
 int32_t ssconv_sizes_grouped(const ssconv_desc_t* desc, int32_t groups, int64_t* G, size_t* w_comp_bytes,
                              size_t* meta_bytes);
 int32_t ssconv_compress_grouped(const ssconv_desc_t* desc, int32_t groups, const void* w_bf16, const uint8_t* pattern,

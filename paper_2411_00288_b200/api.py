@@ -519,7 +519,7 @@ def ssconv_compress_grouped(desc: Desc, groups: int, w: torch.Tensor, pattern: t
 def ssconv_forward_grouped(desc: Desc, groups: int, x: torch.Tensor, w_comp: torch.Tensor, meta: torch.Tensor,
                            bias: Optional[torch.Tensor] = None, y: Optional[torch.Tensor] = None,
                            dev_status: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
-    """2:4 masked grouped convolution (one launch per group on channel slices)."""
+    """2:4 masked grouped convolution (one launch, or one per group on channel slices)."""
     _need_cuda(x, w_comp, meta, bias, y, dev_status)
     if y is None:
         y = _alloc_y(desc, x)

@@ -18,7 +18,9 @@
 //
 // Warp roles: warps 0, 10 and 11 TMA producers (one thread each: the activations of a group's
 // first k-block, of its second, the weights), warp 1 MMA issuer (one thread; owns TMEM), warps 2-9
-// epilogue in two groups of four warps that each own half of a tile's positions.  The accumulator
+// epilogue in two groups of four warps that each own half of a tile's positions; where a residual is added
+// or a tile's two accumulators have epilogue groups of their own, two more warps (one thread each) issue the
+// output's stores.  The accumulator
 // has channels on TMEM lanes and positions on columns, NHWC wants the transpose: the epilogue reads
 // TMEM in the MMA-fragment layout (tcgen05.ld 16x256b), adds the bias, converts pairs to bf16
 // (with ReLU in the conversion), and stmatrix.trans writes 8x8 blocks transposed into a 128-byte
@@ -64,8 +66,14 @@ constexpr int kPiece = 40;               // positions per epilogue piece (one st
 constexpr int kFirstExtraProducerWarp = 2 + 4 * kGroups;  // warps 10 and 11: two more TMA producers
 constexpr int kThreads = 64 + 128 * kGroups + 64;
 // With `sets` sets of epilogue groups (one-block kernel; see kWideMaxKBlocks) the producers follow the last group.
-__host__ __device__ constexpr int threads_with(int sets) { return 64 + 128 * kGroups * sets + 64; }
+// Two more warps follow those in the forms with store warps, one per half of a tile's positions.
+__host__ __device__ constexpr bool has_store_warps(bool residual, int sets) { return residual || sets == 2; }
+__host__ __device__ constexpr int threads_with(int sets, bool residual) {
+  return 64 + 128 * kGroups * sets + 64 + (has_store_warps(residual, sets) ? 32 * kGroups : 0);
+}
 __host__ __device__ constexpr int first_extra_producer_with(int sets) { return 2 + 4 * kGroups * sets; }
+constexpr int kPairStoreWarp = kFirstExtraProducerWarp + 2;  // pair kernel with a residual: warps 12 and 13 issue the stores
+__host__ __device__ constexpr int pair_threads(bool residual) { return kThreads + (residual ? 32 * kGroups : 0); }
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kAccCol1 = 256;       // second accumulator; the first starts at column 0
 constexpr uint32_t kMetaCol = kBN;       // metadata: 2 slots x 4 columns in [240, 248)
@@ -74,7 +82,7 @@ constexpr uint32_t kATileBytes = 128 * 128;          // 128 rows x 128 B
 constexpr uint32_t kHalfPieceBytes = kPiece * 128;    // 40 positions x 64 channels bf16, 128-byte swizzled
 constexpr uint32_t kPieceBytes = 2 * kHalfPieceBytes; // channels [0,64) then [64,128) of the tile
 __host__ __device__ constexpr uint32_t staging_bytes(int bufs) { return (uint32_t)bufs * kGroups * kPieceBytes; }  // per group 2 or 4 buffers
-constexpr uint32_t kBarrierBytes = 256;
+constexpr uint32_t kBarrierBytes = 384;
 
 // The ring's unit is a group: the operands of one pair of k-blocks (128 dense columns of K).
 // Layout of a group in shared memory: weights (sparse: one 128 x 128 B tile of kept values, which
@@ -210,7 +218,8 @@ __device__ __forceinline__ size_t region_index(int c, bool tile_starts_here) {
   return 2 * (size_t)c + (tile_starts_here ? 1 : 0);
 }
 
-// Named barriers: 1 to 4 for the epilogue groups, 5 for the setup (warp 0 arrives without waiting).
+// Named barriers: 1 and 2 for the epilogue groups (forms without store warps), 5 for the setup (warp 0 arrives without
+// waiting).
 __device__ __forceinline__ void epilogue_bar_sync(int group) {
   asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory");
 }
@@ -485,15 +494,18 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
 // two accumulators, i.e. every other tile.  GROUPED: several channel groups in one launch (an instantiation of its own: as
 // run-time branches its few instructions cost the issuing lane of the plain epilogue 5 % on write-bound layers).
 template <bool SPARSE, bool RES, bool FP8 = false, int EPI_SETS = 1, bool GROUPED = false>
-__global__ void __launch_bounds__(threads_with(EPI_SETS), 1)
+__global__ void __launch_bounds__(threads_with(EPI_SETS, RES), 1)
 ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                   const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_y_tail,
                   const __grid_constant__ CUtensorMap tm_r, const __grid_constant__ CUtensorMap tm_r_tail,
                   const FwdParams p) {
   using C = Cfg<SPARSE, FP8>;
   static_assert(!(FP8 && RES), "the residual epilogue is not built for 8-bit operands");
+  static_assert(!GROUPED || (!RES && EPI_SETS == 1), "channel groups: the plain epilogue");
   static_assert(EPI_SETS == 1 || (EPI_SETS == 2 && !RES), "one set of epilogue groups, or one per accumulator");
-  constexpr int kThreadsHere = threads_with(EPI_SETS), kExtraProducer = first_extra_producer_with(EPI_SETS);
+  constexpr int kThreadsHere = threads_with(EPI_SETS, RES), kExtraProducer = first_extra_producer_with(EPI_SETS);
+  constexpr bool kStoreWarps = has_store_warps(RES, EPI_SETS);
+  constexpr int kStoreWarp = kExtraProducer + 2;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -502,7 +514,8 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
   uint8_t* out_stage = ring + p.ring_groups * (p.a_grp_bytes + 2u * (uint32_t)p.BN * 128u) + p.a_res_bytes;
   // barrier slots: [0,4) group full, [4,8) group empty, [8,10) accumulator full, [10,12) accumulator empty,
   // [12,20) residual piece landed (per epilogue group and staging buffer), [20,24) first k-block of a
-  // group consumed (two-slot rings only: its activation tile may be refilled ahead of the rest)
+  // group consumed (two-slot rings only: its activation tile may be refilled ahead of the rest), [24,32) piece
+  // written to its staging buffer, [32,40) buffer free again (both per epilogue group and staging buffer)
   uint64_t* bars = reinterpret_cast<uint64_t*>(out_stage + staging_bytes(p.stage_bufs));
   uint64_t* bar_full = bars;
   uint64_t* bar_empty = bars + 4;
@@ -510,7 +523,9 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
   uint64_t* bar_acc_empty = bars + 10;
   uint64_t* bar_res = bars + 12;
   uint64_t* bar_empty_first = bars + 20;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 24);
+  uint64_t* bar_staged = bars + 24;
+  uint64_t* bar_stage_free = bars + 32;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 40);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* epi_go = abort_flag + 1;         // per group two slots: the leader's go/stop verdict per tile
 
@@ -522,11 +537,11 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
   if (warp == 0) {
     // barrier slots in memory order: 4 group full (3 arrivals: the three producers), 4 group empty (one
     // commit by the MMA thread), 2 accumulator full, 2 accumulator empty (one arrival per epilogue
-    // warp), 8 residual (one arrival with bytes), 4 first-k-block empty (one commit); lane i
-    // initialises slot i
-    if (lane < 24) {
-      const uint32_t count = (lane < 4) ? 3u : (lane < 10) ? 1u : (lane < 12) ? (uint32_t)(4 * kGroups) : 1u;
-      mbar_init(&bars[lane], count);
+    // warp), 8 residual (one arrival with bytes), 4 first-k-block empty (one commit), 8 piece staged (one
+    // arrival per warp of the epilogue group), 8 staging buffer free (one); lane i initialises slots i and 32 + i
+    for (int i = lane; i < 40; i += 32) {
+      const uint32_t count = (i < 4) ? 3u : (i < 10) ? 1u : (i < 12) ? (uint32_t)(4 * kGroups) : (i < 24 || i >= 32) ? 1u : 4u;
+      mbar_init(&bars[i], count);
     }
     if (lane == 0) {
       grid_launch_dependents();  // the next grid in the stream may set itself up as SMs become free
@@ -562,7 +577,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
   }
   const uint32_t tmem_base = (warp == 0) ? 0u : *tmem_slot;
 
-  if (warp == 0 || warp >= kExtraProducer) {
+  if (warp == 0 || (warp >= kExtraProducer && warp < kExtraProducer + 2)) {
     // ------------------------------------------------------------------ TMA producers
     // (each a whole warp in lock step, one elected lane issuing: see the warp-wide forms)
     {
@@ -729,7 +744,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
   } else if (warp < kExtraProducer) {
     // ------------------------------------------------------------------ epilogue
     // Two independent groups of four warps; group g owns positions [g BN/2, (g + 1) BN/2) of every
-    // tile, with its own staging buffers and named barrier, and handles them 40 at a time (the last
+    // tile, with its own staging buffers, and handles them 40 at a time (the last
     // piece of a group may hold fewer).
     const int grp = (warp - 2) >> 2;
     const int half = EPI_SETS == 1 ? grp : (grp & (kGroups - 1));  // of the positions
@@ -749,34 +764,8 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
                                ((((uint32_t)(q & 1) * 4u + (uint32_t)(lane >> 3)) ^ (uint32_t)(lane & 7)) << 4);
     uint32_t tcount = 0;
     uint32_t piece_count = 0;
+    bool ok = true;
     grid_dependency_wait();  // before the first access to global memory (bias, scratch, output)
-    // Residual pieces are brought into the staging buffers by TMA, nbuf - 1 pieces ahead of the
-    // epilogue (they come from HBM: one piece of latency would be exposed on every piece).  The
-    // leader walks the same sequence of pieces with an iterator of its own.
-    PieceAhead ahead(p);
-    auto load_residual = [&](uint32_t count) {  // leader only; count = running number of the piece to load
-      int tile_a, piece_a;
-      if (!ahead.next(tile_a, piece_a)) return;  // no such piece: nobody will wait for it
-      const uint32_t b = count & (nbuf - 1u);
-      const uint32_t bar = smem_u32(&bar_res[4 * grp + b]);
-      const int pt_a = tile_a / p.m_tiles;
-      const int m_a = tile_a - pt_a * p.m_tiles;
-      const int q_piece = pt_a * p.BN + col_base + piece_a * kPiece;
-      if (q_piece >= p.Q) {  // nothing of this piece is stored: only keep the barrier's phases in step
-        mbar_arrive_a(bar);
-        return;
-      }
-      const bool tail = (piece_a == p.pieces - 1 && p.tail_cols != kPiece);
-      const CUtensorMap* map = tail ? &tm_r_tail : &tm_r;
-      const uint32_t half_bytes = (uint32_t)(tail ? p.tail_cols : kPiece) * 128u;
-      const bool two = m_a * kTileM + 64 < p.C_out;
-      const uint32_t dst = smem_u32(my_stage + b * kPieceBytes);
-      mbar_expect_tx_a(bar, two ? 2u * half_bytes : half_bytes);
-      tma_load_2d_a(dst, map, bar, m_a * kTileM, q_piece);
-      if (two) tma_load_2d_a(dst + kHalfPieceBytes, map, bar, m_a * kTileM + 64, q_piece);
-    };
-    if (RES && leader)
-      for (uint32_t c = 0; c + 1 < nbuf; ++c) load_residual(c);
     WorkIter work(p);
     Segment seg;
     for (; work.next(seg); ++tcount) {
@@ -786,13 +775,16 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       const uint32_t aph = (tcount >> 1) & 1u;
       // (two sets: each serves one accumulator, so that it has two tiles' time for its tiles)
       if (EPI_SETS == 2 && buf != (uint32_t)(grp / kGroups)) continue;
-      const uint32_t verdict = (EPI_SETS == 2 ? tcount >> 1 : tcount) & 1u;
       const bool got = mbar_wait_bounded(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
-      // All threads of a group must take the same branch (they meet at named barriers below):
-      // the leader publishes one verdict, everybody reads it after the barrier.
-      if (leader) my_go[verdict] = (got && *abort_flag == 0) ? 1 : 0;
-      epilogue_bar_sync(grp);
-      if (my_go[verdict] == 0) break;
+      if (kStoreWarps) {
+        if (!got) break;
+      } else {
+        // All threads of a group must take the same branch (they meet at named barriers below):
+        // the leader publishes one verdict, everybody reads it after the barrier.
+        if (leader) my_go[tcount & 1u] = (got && *abort_flag == 0) ? 1 : 0;
+        epilogue_bar_sync(grp);
+        if (my_go[tcount & 1u] == 0) break;
+      }
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + buf * kAccCol1 + col_base;
       const bool whole = (seg.a0 == 0 && seg.a1 == p.a_tiles);
@@ -840,17 +832,25 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
           __syncwarp();
           if (lane == 0) mbar_arrive(&bar_acc_empty[buf]);
         }
-        // The buffer was last the source of the store issued two pieces ago; the leader saw that
-        // store finish reading before it entered the barrier of the previous piece.
+        // The store that last read the buffer, nbuf pieces ago, is through (with a residual: the piece that replaced
+        // its source has landed, below; without store warps: the leader saw that store finish reading before it
+        // entered the barrier of the previous piece).
+        if (kStoreWarps && !RES &&
+            !mbar_wait_bounded(&bar_stage_free[nbuf * grp + sbuf], ((piece_count >> nbuf_shift) & 1u) ^ 1u, abort_flag, kWaitLimitCycles)) {
+          ok = false;
+          break;
+        }
         const uint32_t st_addr = smem_u32(stage) + st_offset;
         if (FP8) {  // the accumulators are sums of products of quantised values: undo the operands' scales
 #pragma unroll
           for (int i = 0; i < kPiece; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * p.out_scale);
         }
         if (RES) {
-          // the residual piece has landed in this buffer (a wait that runs out raises the abort flag;
-          // the group still goes on to its barrier and stops at the next tile)
-          mbar_wait_bounded(&bar_res[4 * grp + sbuf], (piece_count >> nbuf_shift) & 1u, abort_flag, kWaitLimitCycles);
+          // the residual piece has landed in this buffer
+          if (!mbar_wait_bounded(&bar_res[4 * grp + sbuf], (piece_count >> nbuf_shift) & 1u, abort_flag, kWaitLimitCycles)) {
+            ok = false;
+            break;
+          }
           if (act == kActRelu)
             stage_piece<kActRelu, true>(r, bias_v, st_addr);
           else if (act == kActGelu)
@@ -865,10 +865,13 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
           stage_piece<kActNone, false>(r, bias_v, st_addr);
         }
         fence_proxy_async_smem();  // generic-proxy writes -> visible to the TMA store
-        // Without a residual the next piece overwrites the other buffer: its store (the previous
-        // piece's) must have read it.  With one, the buffers are refilled by the residual loads
-        // below, which wait for the stores themselves.
-        if (leader && !RES) bulk_wait_group_read0();
+        if (kStoreWarps) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bar_staged[nbuf * grp + sbuf]);
+          continue;
+        }
+        // The next piece overwrites the other buffer: its store (the previous piece's) must have read it.
+        if (leader) bulk_wait_group_read0();
         epilogue_bar_sync(grp);
         if (leader) {
           const int q_piece = pt * p.BN + col_base + piece * kPiece;
@@ -885,17 +888,101 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
             }
           }
           bulk_commit_group();
-          if (RES) {
-            // refill the buffer the previous piece's store read: residual piece (count + nbuf - 1)
-            bulk_wait_group_read1();
-            load_residual(piece_count + nbuf - 1u);
-          }
         }
       }
+      if (!ok) break;
     }
     // the stores have read their staging buffers before shared memory is released; the writes
     // themselves complete with the grid
-    if (leader) bulk_wait_group_read0();
+    if (!kStoreWarps && leader) bulk_wait_group_read0();
+  } else if (kStoreWarps && lane == 0) {
+    // ------------------------------------------------------------------ output stores (and residual loads)
+    // One thread per epilogue group: it waits for the group's four warps to have written a piece, stores it, and
+    // hands the buffer back once the store has read it, or has it filled with a residual piece.  A TMA instruction
+    // holds its thread for 100-250 cycles: issued by a thread of the epilogue, two stores, the wait and two residual
+    // loads per piece were its longest chain, and every warp of the group waited for it at the piece's barrier.
+    // Batch 256, us, leader of the epilogue -> store warps: 64 -> 256 at 56 x 56 with a residual 175 -> 148, 128 ->
+    // 512 at 28 x 28 91 -> 81, 256 -> 1024 at 14 x 14 51 -> 45, 512 -> 2048 at 7 x 7 33 -> 30.5; GELU on two sets 98 -> 92 (96
+    // -> 384, batch 128).  Plain one-set epilogues gain 2 % where the output stream paces them (64 -> 256 91 -> 89)
+    // and lose 1 to 4 % elsewhere (3 x 3 64 -> 64 88 -> 90, 27 images 13.8 -> 14.3): they keep their leader, as do
+    // pairs without a residual.
+    // With two sets it serves both, tile by tile: their tiles alternate, and a set's buffers hold what it finishes
+    // meanwhile.
+    const int half = warp - kStoreWarp;
+    const int col_base = half * (p.BN >> 1);
+    const uint32_t nbuf = (uint32_t)p.stage_bufs / EPI_SETS;  // 2 or 4
+    const uint32_t nbuf_shift = nbuf == 4 ? 2u : 1u;
+    int grp = half;                                // (the current tile's epilogue group)
+    uint8_t* my_stage = out_stage + grp * nbuf * kPieceBytes;
+    uint32_t piece_count = 0, other_count = 0;     // pieces of the current tile's set and of the other one so far
+    uint32_t tcount = 0;
+    grid_dependency_wait();  // before the first access to global memory
+    // Residual pieces are brought into the staging buffers by TMA, nbuf pieces ahead of the
+    // epilogue (they come from HBM: one piece of latency would be exposed on every piece).
+    PieceAhead ahead(p);
+    auto load_residual = [&](uint32_t count) {  // count = running number of the piece to load
+      int tile_a, piece_a;
+      if (!ahead.next(tile_a, piece_a)) return;  // no such piece: nobody will wait for it
+      const uint32_t b = count & (nbuf - 1u);
+      const uint32_t bar = smem_u32(&bar_res[4 * grp + b]);
+      const int pt_a = tile_a / p.m_tiles;
+      const int m_a = tile_a - pt_a * p.m_tiles;
+      const int q_piece = pt_a * p.BN + col_base + piece_a * kPiece;
+      if (q_piece >= p.Q) {  // nothing of this piece is stored: only keep the barrier's phases in step
+        mbar_arrive_a(bar);
+        return;
+      }
+      const bool tail = (piece_a == p.pieces - 1 && p.tail_cols != kPiece);
+      const CUtensorMap* map = tail ? &tm_r_tail : &tm_r;
+      const uint32_t half_bytes = (uint32_t)(tail ? p.tail_cols : kPiece) * 128u;
+      const bool two = m_a * kTileM + 64 < p.C_out;
+      const uint32_t dst = smem_u32(my_stage + b * kPieceBytes);
+      mbar_expect_tx_a(bar, two ? 2u * half_bytes : half_bytes);
+      tma_load_2d_a(dst, map, bar, m_a * kTileM, q_piece);
+      if (two) tma_load_2d_a(dst + kHalfPieceBytes, map, bar, m_a * kTileM + 64, q_piece);
+    };
+    if (RES)
+      for (uint32_t c = 0; c < nbuf; ++c) load_residual(c);
+    WorkIter work(p);
+    Segment seg;
+    bool ok = true;
+    for (; ok && work.next(seg); ++tcount) {
+      if (EPI_SETS == 2) {
+        if (tcount != 0) {
+          const uint32_t c = piece_count;
+          piece_count = other_count;
+          other_count = c;
+        }
+        grp = half + kGroups * (int)(tcount & 1u);
+        my_stage = out_stage + grp * nbuf * kPieceBytes;
+      }
+      if (seg.a0 != 0 || seg.a1 != p.a_tiles) continue;  // (parked in scratch by the epilogue)
+      const int pt = seg.tile / p.m_tiles;
+      const int m = seg.tile - pt * p.m_tiles;
+      const int c0 = m * kTileM;
+      for (int piece = 0; piece < p.pieces; ++piece, ++piece_count) {
+        const uint32_t sbuf = piece_count & (nbuf - 1u);
+        uint8_t* stage = my_stage + sbuf * kPieceBytes;
+        const int q_piece = pt * p.BN + col_base + piece * kPiece;
+        if (!mbar_wait_bounded(&bar_staged[nbuf * grp + sbuf], (piece_count >> nbuf_shift) & 1u, abort_flag, kWaitLimitCycles)) {
+          ok = false;
+          break;
+        }
+        if (q_piece < p.Q) {
+          // positions beyond Q and channels beyond C_out fall outside the tensor map and are dropped;
+          // a short last piece goes through the map whose box holds just its positions
+          const CUtensorMap* map = (piece == p.pieces - 1 && p.tail_cols != kPiece) ? &tm_y_tail : &tm_y;
+          tma_store_2d(map, stage, c0, q_piece);
+          if (c0 + 64 < p.C_out) tma_store_2d(map, stage + kHalfPieceBytes, c0 + 64, q_piece);
+          bulk_commit_group();
+          bulk_wait_group_read0();
+        }
+        if (RES)
+          load_residual(piece_count + nbuf);
+        else
+          mbar_arrive(&bar_stage_free[nbuf * grp + sbuf]);
+      }
+    }
   }
 
   // ------------------------------------------------------------------ teardown
@@ -1113,7 +1200,7 @@ __device__ __forceinline__ void pair_producer_role(const CUtensorMap* tm_a, cons
 }
 
 template <bool SPARSE, bool FP8 = false, bool RES = false>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(pair_threads(RES), 1)
 ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                        const __grid_constant__ CUtensorMap tm_meta, const __grid_constant__ CUtensorMap tm_y,
                        const __grid_constant__ CUtensorMap tm_y_tail, const __grid_constant__ CUtensorMap tm_r,
@@ -1128,15 +1215,16 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
   uint8_t* ring = smem;
   uint8_t* out_stage = ring + p.ring_groups * grp_bytes;
   // barrier slots: [0,4) group full (used in the leader), [4,8) group empty, [8,10) accumulator full,
-  // [10,12) accumulator empty (used in the leader), [12,20) residual piece landed (per epilogue group and
-  // staging buffer, each block its own)
+  // [10,12) accumulator empty (used in the leader); per epilogue group and staging buffer, each block its own:
+  // [12,20) residual piece landed, [20,28) piece written (with a residual)
   uint64_t* bars = reinterpret_cast<uint64_t*>(out_stage + staging_bytes(p.stage_bufs));
   uint64_t* bar_full = bars;
   uint64_t* bar_empty = bars + 4;
   uint64_t* bar_acc_full = bars + 8;
   uint64_t* bar_acc_empty = bars + 10;
   uint64_t* bar_res = bars + 12;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 20);
+  uint64_t* bar_staged = bars + 20;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 28);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* epi_go = abort_flag + 1;
 
@@ -1147,10 +1235,10 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
   const bool leader_cta = rank == 0;
 
   if (warp == 0) {
-    if (lane < 20) {
+    if (lane < 28) {
       // full: the leader's three producers; empty, accumulator full: one commit; accumulator empty: the
-      // epilogue warps of both CTAs; residual: one arrival with bytes
-      const uint32_t count = (lane < 4) ? 3u : (lane < 10) ? 1u : (lane < 12) ? (uint32_t)(2 * 4 * kGroups) : 1u;
+      // epilogue warps of both CTAs; residual: one arrival with bytes; staged: the group's warps
+      const uint32_t count = (lane < 4) ? 3u : (lane < 10) ? 1u : (lane < 12) ? (uint32_t)(2 * 4 * kGroups) : (lane < 20) ? 1u : 4u;
       mbar_init(&bars[lane], count);
     }
     if (lane == 0) {
@@ -1188,7 +1276,7 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 0 || warp >= kFirstExtraProducerWarp) {
+  if (warp == 0 || (warp >= kFirstExtraProducerWarp && warp < kPairStoreWarp)) {
     // ------------------------------------------------------------------ TMA producers (whole warps)
     const uint32_t full0_local = smem_u32(bar_full);
     const uint32_t full0_leader = map_to_cta(full0_local, 0);
@@ -1297,7 +1385,7 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
         if (ok && dual) tc2_commit_both_w(accf0 + 8u);
       }
     }
-  } else {
+  } else if (warp < kFirstExtraProducerWarp) {
     // ------------------------------------------------------------------ epilogue (as in the one-CTA kernel)
     const int grp = (warp - 2) >> 2;
     const int q = warp & 3;
@@ -1305,9 +1393,8 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
     const int act = activation_of(p.flags);
     const int col_base = grp * (p.BN >> 1);
     // one or two staging buffers per group (one where the K loop is long enough to hide the wait for the
-    // previous piece's store, which then leaves room for another ring group)
-    const bool one_buffer = p.stage_bufs == 1;
-    const uint32_t nbuf = (uint32_t)p.stage_bufs;  // 1 or 2; 4 with a residual (pieces prefetched three ahead)
+    // previous piece's store, which then leaves room for another ring group); 4 with a residual
+    const uint32_t nbuf = (uint32_t)p.stage_bufs, nbuf_shift = nbuf >> 1;  // (1, 2, 4 -> 0, 1, 2)
     uint8_t* my_stage = out_stage + grp * p.stage_bufs * kPieceBytes;
     volatile int* my_go = epi_go + 2 * grp;
     const uint32_t acc_empty0_leader = map_to_cta(smem_u32(bar_acc_empty), 0);
@@ -1317,10 +1404,105 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
     const uint32_t tiles_per = p.dual ? 2u : 1u;
     bool go_on = true;
     grid_dependency_wait();
-    // Residual pieces come into the staging buffers by TMA, nbuf - 1 pieces ahead of the epilogue, as in the
-    // one-block kernel; each block loads its own channels' pieces on its own barriers.
+    WorkIter work(p, pair);
+    Segment seg;
+    for (; go_on && work.next(seg); ++icount)
+    for (uint32_t t = 0; t < tiles_per; ++t, ++tcount) {  // the item's tiles, one accumulator each
+      const int pu = seg.tile / p.m_tiles;
+      const int pt = pu * (int)tiles_per + (int)t;
+      const int m = 2 * (seg.tile - pu * p.m_tiles) + (int)rank;
+      const uint32_t buf = p.dual ? t : (icount & 1u);
+      const uint32_t aph = p.dual ? (icount & 1u) : ((icount >> 1) & 1u);
+      const bool got = mbar_wait_bounded(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
+      if (!RES) {
+        if (leader) my_go[tcount & 1u] = (got && *abort_flag == 0) ? 1 : 0;
+        epilogue_bar_sync(grp);
+      }
+      if (RES ? !got : my_go[tcount & 1u] == 0) {
+        go_on = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + buf * kAccCol1 + col_base;
+      float bias_v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int co = m * kTileM + q * 32 + 8 * i + (lane >> 2);
+        bias_v[i] = ((p.flags & SSCONV_FLAG_BIAS) && co < p.C_out) ? p.bias[co] : 0.0f;
+      }
+#pragma unroll 1
+      for (int piece = 0; piece < p.pieces; ++piece, ++piece_count) {
+        const uint32_t sbuf = piece_count & (nbuf - 1u), use = (piece_count >> nbuf_shift) & 1u;
+        uint8_t* stage = my_stage + sbuf * kPieceBytes;
+        uint32_t r[kPiece];
+        tc_ld_piece(t_row + piece * kPiece, r);
+        tc_wait_ld();
+        if (piece == p.pieces - 1) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(acc_empty0_leader + 8u * buf);
+        }
+        if (FP8) {
+#pragma unroll
+          for (int i = 0; i < kPiece; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * p.out_scale);
+        }
+        if (!RES && nbuf == 1u) {  // the previous piece's store has read the buffer before anyone overwrites it
+          if (leader) bulk_wait_group_read0();
+          epilogue_bar_sync(grp);
+        }
+        const uint32_t st_addr = smem_u32(stage) + st_offset;
+        if (RES) {
+          // the residual piece has landed in this buffer
+          if (!mbar_wait_bounded(&bar_res[4 * grp + sbuf], use, abort_flag, kWaitLimitCycles)) {
+            go_on = false;
+            break;
+          }
+          if (act == kActRelu)
+            stage_piece<kActRelu, true>(r, bias_v, st_addr);
+          else if (act == kActGelu)
+            stage_piece<kActGelu, true>(r, bias_v, st_addr);
+          else
+            stage_piece<kActNone, true>(r, bias_v, st_addr);
+        } else if (act == kActRelu) {
+          stage_piece<kActRelu, false>(r, bias_v, st_addr);
+        } else if (act == kActGelu) {
+          stage_piece<kActGelu, false>(r, bias_v, st_addr);
+        } else {
+          stage_piece<kActNone, false>(r, bias_v, st_addr);
+        }
+        fence_proxy_async_smem();
+        if (RES) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bar_staged[4 * grp + sbuf]);
+          continue;
+        }
+        if (leader) bulk_wait_group_read0();
+        epilogue_bar_sync(grp);
+        if (leader) {
+          const int q_piece = pt * p.BN + col_base + piece * kPiece;
+          if (m < p.m_real && q_piece < p.Q) {  // (the odd CTA of the last pair may have no channels at all)
+            const CUtensorMap* map = (piece == p.pieces - 1 && p.tail_cols != kPiece) ? &tm_y_tail : &tm_y;
+            tma_store_2d(map, stage, m * kTileM, q_piece);
+            if (m * kTileM + 64 < p.C_out) tma_store_2d(map, stage + kHalfPieceBytes, m * kTileM + 64, q_piece);
+          }
+          bulk_commit_group();
+        }
+      }
+      if (!go_on) break;
+    }
+    if (!RES && leader) bulk_wait_group_read0();
+  } else if (RES && lane == 0) {
+    // ------------------------------------------------------------------ output stores (and residual loads)
+    // (one thread per epilogue group, as in the one-CTA kernel; each block stores its own channels)
+    const int grp = warp - kPairStoreWarp;
+    const int col_base = grp * (p.BN >> 1);
+    const uint32_t nbuf = (uint32_t)p.stage_bufs, nbuf_shift = nbuf >> 1;
+    uint8_t* my_stage = out_stage + grp * p.stage_bufs * kPieceBytes;
+    uint32_t piece_count = 0;
+    const uint32_t tiles_per = p.dual ? 2u : 1u;
+    grid_dependency_wait();
     PieceAhead ahead(p, pair);
-    auto load_residual = [&](uint32_t count) {  // leader only; count = running number of the piece to load
+    auto load_residual = [&](uint32_t count) {  // count = running number of the piece to load
       int tile_a, piece_a;
       if (!ahead.next(tile_a, piece_a)) return;
       const uint32_t b = count & (nbuf - 1u);
@@ -1341,91 +1523,35 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
       tma_load_2d_a(dst, map, bar, m_a * kTileM, q_piece);
       if (two) tma_load_2d_a(dst + kHalfPieceBytes, map, bar, m_a * kTileM + 64, q_piece);
     };
-    if (RES && leader)
-      for (uint32_t c = 0; c + 1 < nbuf; ++c) load_residual(c);
+    for (uint32_t c = 0; c < nbuf; ++c) load_residual(c);
     WorkIter work(p, pair);
     Segment seg;
-    for (; go_on && work.next(seg); ++icount)
-    for (uint32_t t = 0; t < tiles_per; ++t, ++tcount) {  // the item's tiles, one accumulator each
+    bool ok = true;
+    while (ok && work.next(seg)) {
       const int pu = seg.tile / p.m_tiles;
-      const int pt = pu * (int)tiles_per + (int)t;
       const int m = 2 * (seg.tile - pu * p.m_tiles) + (int)rank;
-      const uint32_t buf = p.dual ? t : (icount & 1u);
-      const uint32_t aph = p.dual ? (icount & 1u) : ((icount >> 1) & 1u);
-      const bool got = mbar_wait_bounded(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
-      if (leader) my_go[tcount & 1u] = (got && *abort_flag == 0) ? 1 : 0;
-      epilogue_bar_sync(grp);
-      if (my_go[tcount & 1u] == 0) {
-        go_on = false;
-        break;
-      }
-      tc_fence_after();
-      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + buf * kAccCol1 + col_base;
       const bool real = m < p.m_real;  // (the odd CTA of the last pair may have no channels at all)
-      float bias_v[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int co = m * kTileM + q * 32 + 8 * i + (lane >> 2);
-        bias_v[i] = ((p.flags & SSCONV_FLAG_BIAS) && co < p.C_out) ? p.bias[co] : 0.0f;
-      }
-#pragma unroll 1
-      for (int piece = 0; piece < p.pieces; ++piece, ++piece_count) {
-        const uint32_t sbuf = RES ? (piece_count & (nbuf - 1u)) : (one_buffer ? 0u : (piece_count & 1u));
-        uint8_t* stage = my_stage + sbuf * kPieceBytes;
-        uint32_t r[kPiece];
-        tc_ld_piece(t_row + piece * kPiece, r);
-        tc_wait_ld();
-        if (piece == p.pieces - 1) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(acc_empty0_leader + 8u * buf);
-        }
-        if (FP8) {
-#pragma unroll
-          for (int i = 0; i < kPiece; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * p.out_scale);
-        }
-        if (!RES && one_buffer) {  // the previous piece's store has read the buffer before anyone overwrites it
-          if (leader) bulk_wait_group_read0();
-          epilogue_bar_sync(grp);
-        }
-        const uint32_t st_addr = smem_u32(stage) + st_offset;
-        if (RES) {
-          // the residual piece has landed in this buffer (a wait that runs out raises the abort flag; the
-          // group still goes on to its barrier and stops at the next tile)
-          mbar_wait_bounded(&bar_res[4 * grp + sbuf], (piece_count >> 2) & 1u, abort_flag, kWaitLimitCycles);
-          if (act == kActRelu)
-            stage_piece<kActRelu, true>(r, bias_v, st_addr);
-          else if (act == kActGelu)
-            stage_piece<kActGelu, true>(r, bias_v, st_addr);
-          else
-            stage_piece<kActNone, true>(r, bias_v, st_addr);
-        } else if (act == kActRelu) {
-          stage_piece<kActRelu, false>(r, bias_v, st_addr);
-        } else if (act == kActGelu) {
-          stage_piece<kActGelu, false>(r, bias_v, st_addr);
-        } else {
-          stage_piece<kActNone, false>(r, bias_v, st_addr);
-        }
-        fence_proxy_async_smem();
-        if (leader && !RES) bulk_wait_group_read0();
-        epilogue_bar_sync(grp);
-        if (leader) {
+      for (uint32_t t = 0; ok && t < tiles_per; ++t) {
+        const int pt = pu * (int)tiles_per + (int)t;
+        for (int piece = 0; piece < p.pieces; ++piece, ++piece_count) {
+          const uint32_t sbuf = piece_count & (nbuf - 1u);
+          uint8_t* stage = my_stage + sbuf * kPieceBytes;
           const int q_piece = pt * p.BN + col_base + piece * kPiece;
+          if (!mbar_wait_bounded(&bar_staged[4 * grp + sbuf], (piece_count >> nbuf_shift) & 1u, abort_flag, kWaitLimitCycles)) {
+            ok = false;
+            break;
+          }
           if (real && q_piece < p.Q) {
             const CUtensorMap* map = (piece == p.pieces - 1 && p.tail_cols != kPiece) ? &tm_y_tail : &tm_y;
             tma_store_2d(map, stage, m * kTileM, q_piece);
             if (m * kTileM + 64 < p.C_out) tma_store_2d(map, stage + kHalfPieceBytes, m * kTileM + 64, q_piece);
+            bulk_commit_group();
+            bulk_wait_group_read0();
           }
-          bulk_commit_group();
-          if (RES) {
-            // refill the buffer the previous piece's store read: residual piece (count + nbuf - 1)
-            bulk_wait_group_read1();
-            load_residual(piece_count + nbuf - 1u);
-          }
+          load_residual(piece_count + nbuf);
         }
       }
     }
-    if (leader) bulk_wait_group_read0();
   }
 
   // ------------------------------------------------------------------ teardown
@@ -2116,7 +2242,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   // waits for that kernel's completion before it touches global memory.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads_with(wide_epilogue ? 2 : 1));
+  cfg.blockDim = dim3((unsigned)(pair ? pair_threads(residual != nullptr) : threads_with(wide_epilogue ? 2 : 1, residual != nullptr)));
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
