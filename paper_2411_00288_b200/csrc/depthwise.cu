@@ -195,7 +195,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
   int pos = blk * p.work_quot + min(blk, p.work_rem);
   const int end = pos + p.work_quot + (blk < p.work_rem ? 1 : 0);
   grid_launch_dependents();
-  grid_dependency_wait();
+  grid_dependency_wait();  // (loads below it are plain ones: read-only loads could be moved above it)
   __syncthreads();
 
   // Every role walks the block's segments; three block barriers per segment: tables written, outputs stored, done.
@@ -214,7 +214,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
                           ? (uint32_t)((((long long)n * p.Ho + sg.h0) * p.Wo + wo) * (p.C / kDw7Channels) + sg.z)
                           : ~0u;
       }
-      if (tid < kDw7Channels) bias_s[tid] = (p.flags & SSCONV_FLAG_BIAS) ? __ldg(p.bias + sg.z * kDw7Channels + tid) : 0.0f;
+      if (tid < kDw7Channels) bias_s[tid] = (p.flags & SSCONV_FLAG_BIAS) ? p.bias[sg.z * kDw7Channels + tid] : 0.0f;
       // the two channels' band matrices: B[k][n] = tap k - n of the filter row, n = g
       uint32_t band[2][kDw7K][2];
       {
@@ -226,7 +226,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const int kw = 2 * t + (e & 1) + 8 * (e >> 1) - g;
-            v[e] = (kw >= 0 && kw < kDw7K) ? __ldg(w + (kh * kDw7K + kw) * C2) : 0u;
+            v[e] = (kw >= 0 && kw < kDw7K) ? w[(kh * kDw7K + kw) * C2] : 0u;
           }
 #pragma unroll
           for (int half = 0; half < 2; ++half) {

@@ -11,9 +11,27 @@
 #include <cstdint>
 
 #include "layout.cuh"
+#include "sm100_ptx.cuh"
 #include "ssconv.h"
 
 namespace ssconv {
+
+// Launch with programmatic stream serialisation, for kernels that call grid_dependency_wait() before their first access
+// to global memory (by plain loads: read-only ones could be moved above the wait): the launch and the index arithmetic
+// overlap the tail of the grid before.
+template <class... Params, class... Args>
+static cudaError_t launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned threads, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
 
 __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
   __nv_bfloat162 x = *reinterpret_cast<__nv_bfloat162*>(&a);
@@ -60,8 +78,9 @@ constexpr int kPoolRows = 8;
 __device__ __forceinline__ uint4 max4(uint4 a, uint4 b) {
   return make_uint4(max_bf16x2(a.x, b.x), max_bf16x2(a.y, b.y), max_bf16x2(a.z, b.z), max_bf16x2(a.w, b.w));
 }
-__global__ void __launch_bounds__(256) maxpool3s2_nhwc_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, int N,
+__global__ void __launch_bounds__(256) maxpool3s2_nhwc_kernel(const uint4* x, uint4* y, int N,
                                                               int H, int W, int C8, int Ho, int Wo, int strips) {
+  grid_launch_dependents();
   const long long total = (long long)N * strips * Wo * C8;
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total) return;
@@ -80,12 +99,13 @@ __global__ void __launch_bounds__(256) maxpool3s2_nhwc_kernel(const uint4* __res
   auto row_max = [&](int h) -> uint4 {
     if (h < 0 || h >= H) return lowest;
     const uint4* centre = img + ((long long)h * W + w0 + 1) * C8;
-    uint4 m = __ldg(centre);
-    if (left) m = max4(m, __ldg(centre - C8));
-    if (right) m = max4(m, __ldg(centre + C8));
+    uint4 m = *centre;
+    if (left) m = max4(m, centre[-C8]);
+    if (right) m = max4(m, centre[C8]);
     return m;
   };
   const int ho0 = strip * kPoolRows;
+  grid_dependency_wait();
   uint4 prev = row_max(2 * ho0 - 1);
   uint4* out = y + (((long long)n * Ho + ho0) * Wo + wo) * C8 + c;
 #pragma unroll 2
@@ -639,21 +659,23 @@ __global__ void __launch_bounds__(256) layernorm_kernel(const __nv_bfloat16* __r
 // a lane holding V 16-byte pieces of it in registers: one read and one write of the tensor, 16 bytes at
 // a time, statistics by shuffles within the group.
 template <int V>
-__global__ void __launch_bounds__(256) layernorm_vec_kernel(const uint4* __restrict__ x, const float* __restrict__ gamma,
-                                                            const float* __restrict__ beta, uint4* __restrict__ y,
+__global__ void __launch_bounds__(256) layernorm_vec_kernel(const uint4* x, const float* gamma,
+                                                            const float* beta, uint4* y,
                                                             long long pixels, int C8, int G, float eps) {
+  grid_launch_dependents();
   const int lane = threadIdx.x & 31;
   const int sub = lane & (G - 1);
   const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const long long pix = warp * (32 / G) + lane / G;
   const bool live = pix < pixels;
+  grid_dependency_wait();
   float f[V][8];
   float sum = 0.0f;
 #pragma unroll
   for (int k = 0; k < V; ++k) {
     const int idx = sub + k * G;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (live && idx < C8) v = __ldg(x + pix * C8 + idx);
+    if (live && idx < C8) v = x[pix * C8 + idx];
     const uint32_t a[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -682,10 +704,10 @@ __global__ void __launch_bounds__(256) layernorm_vec_kernel(const uint4* __restr
   for (int k = 0; k < V; ++k) {
     const int idx = sub + k * G;
     if (!live || idx >= C8) continue;
-    const float4 g0 = __ldg(reinterpret_cast<const float4*>(gamma) + 2 * idx);
-    const float4 g1 = __ldg(reinterpret_cast<const float4*>(gamma) + 2 * idx + 1);
-    const float4 b0 = __ldg(reinterpret_cast<const float4*>(beta) + 2 * idx);
-    const float4 b1 = __ldg(reinterpret_cast<const float4*>(beta) + 2 * idx + 1);
+    const float4 g0 = reinterpret_cast<const float4*>(gamma)[2 * idx];
+    const float4 g1 = reinterpret_cast<const float4*>(gamma)[2 * idx + 1];
+    const float4 b0 = reinterpret_cast<const float4*>(beta)[2 * idx];
+    const float4 b1 = reinterpret_cast<const float4*>(beta)[2 * idx + 1];
     const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
     const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
     uint32_t o[4];
@@ -722,14 +744,12 @@ cudaError_t launch_layernorm(const void* x, const float* gamma, const float* bet
     const uint4* xp = static_cast<const uint4*>(x);
     uint4* yp = static_cast<uint4*>(y);
     if (V == 1)
-      layernorm_vec_kernel<1><<<grid, T, 0, st>>>(xp, gamma, beta, yp, pixels, C8, G, eps);
-    else if (V == 2)
-      layernorm_vec_kernel<2><<<grid, T, 0, st>>>(xp, gamma, beta, yp, pixels, C8, G, eps);
-    else if (V == 3)
-      layernorm_vec_kernel<3><<<grid, T, 0, st>>>(xp, gamma, beta, yp, pixels, C8, G, eps);
-    else
-      layernorm_vec_kernel<4><<<grid, T, 0, st>>>(xp, gamma, beta, yp, pixels, C8, G, eps);
-    return cudaGetLastError();
+      return launch_dependent(layernorm_vec_kernel<1>, grid, T, st, xp, gamma, beta, yp, pixels, C8, G, eps);
+    if (V == 2)
+      return launch_dependent(layernorm_vec_kernel<2>, grid, T, st, xp, gamma, beta, yp, pixels, C8, G, eps);
+    if (V == 3)
+      return launch_dependent(layernorm_vec_kernel<3>, grid, T, st, xp, gamma, beta, yp, pixels, C8, G, eps);
+    return launch_dependent(layernorm_vec_kernel<4>, grid, T, st, xp, gamma, beta, yp, pixels, C8, G, eps);
   }
   layernorm_kernel<<<(unsigned)((pixels * 32 + T - 1) / T), T, 0, st>>>(static_cast<const __nv_bfloat16*>(x), gamma, beta,
                                                                         static_cast<__nv_bfloat16*>(y), pixels, C, eps);
@@ -769,9 +789,8 @@ cudaError_t launch_maxpool(const void* x, void* y, int N, int H, int W, int C, i
   if (k == 3 && stride == 2 && pad == 1 && W >= 2) {
     const int strips = (Ho + kPoolRows - 1) / kPoolRows;
     const long long threads = (long long)N * strips * Wo * (C / 8);
-    maxpool3s2_nhwc_kernel<<<(unsigned)((threads + T - 1) / T), T, 0, st>>>(
-        static_cast<const uint4*>(x), static_cast<uint4*>(y), N, H, W, C / 8, Ho, Wo, strips);
-    return cudaGetLastError();
+    return launch_dependent(maxpool3s2_nhwc_kernel, (unsigned)((threads + T - 1) / T), T, st, static_cast<const uint4*>(x),
+                            static_cast<uint4*>(y), N, H, W, C / 8, Ho, Wo, strips);
   }
   maxpool_nhwc_kernel<<<(unsigned)((total + T - 1) / T), T, 0, st>>>(static_cast<const uint4*>(x),
                                                                      static_cast<uint4*>(y), N, H, W, C / 8, Ho, Wo,
