@@ -1628,9 +1628,11 @@ constexpr double kIssueSparse = 365.0, kIssueDense = 480.0;
 constexpr double kEpiloguePieceCycles = 900.0;
 constexpr double kCyclesPerParkedTile = 90.0;
 // What an epilogue that paces its layer takes per tile: fixed + per piece, whatever the piece's fill (a piece of 40
-// columns is processed whole).  Fitted to forced widths: GELU on two sets of groups; residual epilogues (128 -> 512 at
-// 28 x 28, batch 256: 80 / 112 / 144 / 160 / 176 / 208 positions 119 / 130 / 107 / 95 / 116 / 100 us: 160 positions are two
-// whole pieces per group, 208 are three with a sixth of them empty).
+// columns is processed whole).  Fitted to forced widths: GELU on two sets of groups; residual epilogues, while a
+// thread of theirs issued the stores (128 -> 512 at 28 x 28, batch 256: 80 / 112 / 144 / 160 / 176 / 208 positions 119 / 130 /
+// 107 / 95 / 116 / 100 us: 160 positions are two whole pieces per group, 208 are three with a sixth of them empty).  With
+// store warps the order is the same where it matters: 112 / 144 / 160 / 176 / 192 / 208 positions 97 / 81 / 83 / 89 / 85 / 81 us
+// there, 55 / 47 / 45 / 53 / 50 / 48 for 256 -> 1024 at 14 x 14.
 struct EpilogueCycles {
   double tile, piece;
 };
