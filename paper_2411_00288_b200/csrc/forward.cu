@@ -905,7 +905,8 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
     // 512 at 28 x 28 91 -> 81, 256 -> 1024 at 14 x 14 51 -> 45, 512 -> 2048 at 7 x 7 33 -> 30.5; GELU on two sets 98 -> 92 (96
     // -> 384, batch 128).  Plain one-set epilogues gain 2 % where the output stream paces them (64 -> 256 91 -> 89)
     // and lose 1 to 4 % elsewhere (3 x 3 64 -> 64 88 -> 90, 27 images 13.8 -> 14.3): they keep their leader, as do
-    // pairs without a residual.
+    // pairs without a residual.  Residual layers of few tiles pay about 0.3 us for the longer way of their last pieces
+    // (8 x 28 x 28 x 256, 3 x 3: 10.6 -> 10.9); sleeping instead of polling in the store warps changes nothing.
     // With two sets it serves both, tile by tile: their tiles alternate, and a set's buffers hold what it finishes
     // meanwhile.
     const int half = warp - kStoreWarp;
