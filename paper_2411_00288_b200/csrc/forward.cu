@@ -247,18 +247,19 @@ __device__ __forceinline__ void tc_ld_piece(uint32_t taddr, uint32_t (&r)[kPiece
 // rounding, and overwritten in place (a warp only touches its own 16-byte columns).
 // ACT: 0 identity, 1 ReLU (inside the bf16 conversion), 2 GELU in its erf form x Phi(x) =
 // 0.5 x (1 + erf(x / sqrt 2)), evaluated in fp32 before the rounding.
-// With Phi(-|x|) = 0.5 erfc(|x| / sqrt 2) the activation is max(x, 0) - |x| Phi(-|x|) on both sides of zero:
-// no sign to carry, and nothing cancels.  log2 erfc(z) is a degree-6 polynomial R (no constant term) fitted on
-// [0, 4] (beyond 4, erfc < 2e-8 and z is clamped); the factor 1 / sqrt 2 of z is folded into its coefficients,
-// the 0.5 into the exponent, and the polynomial takes n = -|x|, the factor of the last multiply-add.  Fitted to
-// |R - log2 erfc| <= 4.8e-5, i.e. 3.3e-5 relative; in fp32 over every bf16 input up to 8 the result is within 5.1e-6 absolute
-// and 3.3e-5 relative, a sixtieth of the rounding to bf16 that follows (2^-9).  A degree-8 fit bought nothing after that rounding and cost two more multiply-adds per value,
-// which matters because shallow layers with this activation are bound by the epilogue's arithmetic: eight
-// instructions of the FMA pipe (half rate for pairs) and two exponentials per pair of values.
+// With n = -|x| and e = Phi(n) the activation is n (e - 1) from zero on and n e below it: no sign to carry, nothing that
+// cancels, and the ends come out of the arithmetic itself (infinity at infinity, NaN at minus infinity, as x Phi(x) gives
+// there, and at a NaN).  log2 e is a degree-7 polynomial R in n, -1 at zero and fitted on [-5.54, 0] to 5.5e-6; its
+// leading term takes it to minus infinity below that (R < log2 Phi(n) + 7e-4 there), so that n needs no clamp.
+// Evaluated in fp32 the result is within 5.1e-6 relative from -5.54 up (a four-hundredth of the rounding to bf16 that
+// follows), 6.5e-7 absolute everywhere, 6.1e-13 below -5.54.  The degree-6 fit before it, with n clamped at -4 sqrt 2
+// (3.3e-5 relative down to there; the constant -4.4e-8 below, at minus infinity as well), took two instructions of the
+// FMA pipe fewer per pair: 96 -> 384 at 56 x 56, batch 128 90.2 -> 92.7 us, 384 -> 1536 at 14 x 14 34.8 -> 34.9, 3 x 3
+// 256 -> 256 at 28 x 28, batch 32 23.2 -> 22.8.  A clamp on the positive side alone (for the NaN) costs more: 98.9 us.
 constexpr int kActNone = 0, kActRelu = 1, kActGelu = 2;
-constexpr float kGeluClamp = 5.656854152679443f;  // 4 sqrt 2
-constexpr float kGeluC1 = 1.1506847143173218f, kGeluC2 = -0.46029916405677795f, kGeluC3 = 0.05191940814256668f,
-                kGeluC4 = 0.00745233241468668f, kGeluC5 = 0.0006528479279950261f, kGeluC6 = 2.5540923161315732e-05f;
+constexpr float kGeluC1 = 1.1512105857193118f, kGeluC2 = -0.4585589426410932f, kGeluC3 = 0.05386546609966522f,
+                kGeluC4 = 0.008460201316438069f, kGeluC5 = 0.0009178260683469985f, kGeluC6 = 5.989503356838717e-05f,
+                kGeluC7 = 1.7442654864735877e-06f;
 // Two values at once, the polynomial on fp32 pairs (fma.rn.f32x2).
 __device__ __forceinline__ unsigned long long f32x2(float lo, float hi) {
   unsigned long long r;
@@ -275,12 +276,12 @@ __device__ __forceinline__ void split2(unsigned long long v, float& lo, float& h
 __device__ __forceinline__ unsigned long long gelu_f32x2(unsigned long long x) {
   float lo, hi;
   split2(x, lo, hi);
-  const unsigned long long n = f32x2(fmaxf(-fabsf(lo), -kGeluClamp), fmaxf(-fabsf(hi), -kGeluClamp));
-  float p0, p1;  // max(x, 0); a NaN stays one
-  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(p0) : "f"(lo));
-  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(p1) : "f"(hi));
-  unsigned long long y = f32x2(p0, p1);
-  unsigned long long r = f32x2(kGeluC6, kGeluC6);
+  const unsigned long long n = f32x2(-fabsf(lo), -fabsf(hi));
+  float m0, m1;  // 1 from zero on, 0 below it
+  asm("set.ge.f32.f32 %0, %1, 0f00000000;" : "=f"(m0) : "f"(lo));
+  asm("set.ge.f32.f32 %0, %1, 0f00000000;" : "=f"(m1) : "f"(hi));
+  unsigned long long r = f32x2(kGeluC7, kGeluC7);
+  r = horner2(r, n, kGeluC6);
   r = horner2(r, n, kGeluC5);
   r = horner2(r, n, kGeluC4);
   r = horner2(r, n, kGeluC3);
@@ -291,7 +292,9 @@ __device__ __forceinline__ unsigned long long gelu_f32x2(unsigned long long x) {
   split2(r, r0, r1);
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(r0));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(r1));
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(y) : "l"(n), "l"(f32x2(e0, e1)));
+  unsigned long long t = f32x2(m0, m1), y;
+  asm("fma.rn.f32x2 %0, %0, %1, %2;" : "+l"(t) : "l"(f32x2(-1.0f, -1.0f)), "l"(f32x2(e0, e1)));
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(y) : "l"(n), "l"(t));
   return y;
 }
 template <int ACT>

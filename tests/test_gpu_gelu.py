@@ -1,5 +1,7 @@
 """The GELU epilogue: its values over every bf16 number, and the form with two sets of epilogue groups at the edges of
 its tiles (odd numbers of tiles, a short last tile, ragged channels, every staged width, slices of a wider tensor)."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -38,6 +40,27 @@ def test_gelu_of_every_bf16_value():
         # one rounding to bf16 (half a unit in the last of 8 bits: at most 2^-8 of the value), 3.3e-5 of the fp32
         # evaluation, and the clamp's 2e-8 x 5.7 far below zero
         assert (err <= (2.0 ** -8 + 5e-5) * np.abs(ref) + 2e-7).all(), float((err - 2.0 ** -8 * np.abs(ref)).max())
+
+
+def test_gelu_far_below_zero_and_at_minus_infinity():
+    bits = torch.arange(0x8000, 0x10000, dtype=torch.int32).to(torch.uint16)       # every bf16 number below zero
+    v = bits.view(torch.bfloat16)
+    x = torch.zeros((1, v.numel() // 64, 64, 16), dtype=torch.bfloat16)
+    x[0, :, :, 0] = v.view(-1, 64)
+    w = torch.zeros((16, 1, 1, 16), dtype=torch.bfloat16)
+    w[:, 0, 0, 0] = 1.0
+    desc = api.make_desc(1, x.shape[1], 64, 16, 16, 1, 1, bias=False, gelu=True)
+    pat = api.ssconv_select_mask(api.MASK_MAGNITUDE_BF16, w.to(DEV), w.numel() // 4)
+    comp = api.ssconv_compress(desc, w.to(DEV), pat)
+    got = api.ssconv_forward(desc, x.to(DEV), *comp).cpu()[0, :, :, 5].reshape(-1)
+    assert bool(torch.isnan(got[v == float("-inf")]).all())                        # as x Phi(x) in fp64
+    fin = torch.isfinite(v)
+    z = v[fin].double().numpy()
+    ref = z * 0.5 * np.vectorize(math.erfc)(-z / math.sqrt(2.0))                   # (no cancellation below zero)
+    err = np.abs(got[fin].double().numpy() - ref)
+    # one rounding to bf16 (half a unit in the last of 8 bits), the evaluation's 5.1e-6, and 6.1e-13 below -5.54, where the
+    # polynomial is not fitted
+    assert (err <= (2.0 ** -8 + 1e-5) * np.abs(ref) + 1e-12).all(), float((err - 2.0 ** -8 * np.abs(ref)).max())
 
 
 LAYERS = [  # N, H, W, C_in, C_out, k, pad
