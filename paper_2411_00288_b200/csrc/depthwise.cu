@@ -8,6 +8,12 @@
 // them, one per filter row, reuse the same A fragment for the seven output rows the image row contributes
 // to.  tcgen05.mma has no use here: every channel is a matrix product of its own, with N = 8.
 //
+// Rounding, before the one to bf16: rms error in units of 2^-24 times the sum of the products' magnitudes, on normal /
+// widely spread / positive data, against fp64: a chain of 49 fp32 FMAs .163 / .744 / .801, all rows through one
+// accumulator .235 / 1.230 / 1.435 (the last with a mean of -1.23: what an MMA drops, it drops towards zero), rows three
+// to seven added in fp32 as here .156 / .617 / .730, rows two to seven .147 / .535 / .687.  The additions take 8 % of the
+// kernel's time (128 x 56 x 56 x 96: 55.8 -> 60.5 us, all rows added 63.5; 14 x 14 x 384 28.1 -> 29.9).
+//
 // What bounds it and why: on fp32 FMA pipes the 1.9 G multiply-adds of a 128 x 56 x 56 x 96 tensor take at
 // least 52 us, twice what moving the tensor takes (23 us); as band matrices they are 2.3 M instructions, 16 us
 // at the 8.4 cycles per scheduler that one takes.  What is left is bringing channels that are neighbours in
@@ -59,6 +65,10 @@ constexpr int kDw7ChannelWords = kDw7Slots * 4;     // a channel's staged row, i
 // eight words between channels 8 apart: the four lanes that hold a pixel's channels write to different banks
 constexpr int kDw7StageWords = kDw7Channels * kDw7ChannelWords + 3 * 8;
 constexpr int kDw7OutWords = kDw7Windows * 8 * 17 + 4;
+// An MMA aligns its products to the accumulator it adds them to and drops what falls below, so a long chain through
+// the accumulator loses more than fp32 additions do.  Filter rows past this one are therefore multiplied by
+// themselves and added in fp32, rounded to nearest.
+constexpr int kDw7ChainedRows = 2;
 constexpr int kDw7StageBufs = 3, kDw7OutBufs = 2;
 constexpr int kDw7StageBytes = 4 * kDw7StageWords, kDw7OutBytes = 4 * kDw7OutWords;
 // image rows as TMA brings them in: kDw7RawRows rows of every 8-pixel piece per copy, 64 bytes per pixel
@@ -114,6 +124,16 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// d += r, each sum rounded to nearest, two at a time.
+__device__ __forceinline__ void add4(float (&d)[4], const float (&r)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; e += 2)
+    asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%0, %1};\n\tmov.b64 b, {%2, %3};\n\tadd.rn.f32x2 a, a, b;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(d[e]), "+f"(d[e + 1])
+        : "f"(r[e]), "f"(r[e + 1]));
 }
 
 // One output of channel pair c2 from its own window's pixels only.
@@ -265,8 +285,16 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             for (int ch = 0; ch < 2; ++ch) {
               // (the row's oldest output first: the epilogue below waits for it)
 #pragma unroll
-              for (int kh = kDw7K - 1; kh > 0; --kh)
-                mma_bf16_16816<false>(acc[ch][(ph - kh + kDw7K) % kDw7K], a[ch], band[ch][kh][0], band[ch][kh][1]);
+              for (int kh = kDw7K - 1; kh > 0; --kh) {
+                float(&d)[4] = acc[ch][(ph - kh + kDw7K) % kDw7K];
+                if (kh <= kDw7ChainedRows) {
+                  mma_bf16_16816<false>(d, a[ch], band[ch][kh][0], band[ch][kh][1]);
+                } else {
+                  float row[4];
+                  mma_bf16_16816<true>(row, a[ch], band[ch][kh][0], band[ch][kh][1]);
+                  add4(d, row);
+                }
+              }
               mma_bf16_16816<true>(acc[ch][ph], a[ch], band[ch][0][0], band[ch][0][1]);
             }
             if (++sbuf == kDw7StageBufs) {
