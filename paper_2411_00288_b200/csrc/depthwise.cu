@@ -69,6 +69,7 @@ constexpr int kDw7OutWords = kDw7Windows * 8 * 17 + 4;
 // the accumulator loses more than fp32 additions do.  Filter rows past this one are therefore multiplied by
 // themselves and added in fp32, rounded to nearest.
 constexpr int kDw7ChainedRows = 2;
+constexpr int kDw7RunRows = 8;                      // (see launch_depthwise7)
 constexpr int kDw7StageBufs = 3, kDw7OutBufs = 2;
 constexpr int kDw7StageBytes = 4 * kDw7StageWords, kDw7OutBytes = 4 * kDw7OutWords;
 // image rows as TMA brings them in: kDw7RawRows rows of every 8-pixel piece per copy, 64 bytes per pixel
@@ -96,6 +97,7 @@ struct Dw7Params {
   long long y_row;          // bytes per output row
   int nblk;                 // windows per output row
   int groups;               // groups of 16 windows (of N nblk)
+  int parts;                // thread blocks per unit (a group's 32 channels), each with one run of its rows; or 0:
   int work_quot, work_rem;  // output rows per thread block (of groups * C / 32 * Ho): quotient and remainder
   uint32_t flags;
 };
@@ -212,8 +214,15 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     prefetch_tensormap(&tm_x);
   }
   const int blk = (int)blockIdx.x;
-  int pos = blk * p.work_quot + min(blk, p.work_rem);
-  const int end = pos + p.work_quot + (blk < p.work_rem ? 1 : 0);
+  int pos, end;
+  if (p.parts != 0) {
+    const int unit = blk / p.parts, part = blk - unit * p.parts;
+    pos = unit * p.Ho + part * p.Ho / p.parts;
+    end = unit * p.Ho + (part + 1) * p.Ho / p.parts;
+  } else {
+    pos = blk * p.work_quot + min(blk, p.work_rem);
+    end = pos + p.work_quot + (blk < p.work_rem ? 1 : 0);
+  }
   grid_launch_dependents();
   grid_dependency_wait();  // (loads below it are plain ones: read-only loads could be moved above it)
   __syncthreads();
@@ -516,11 +525,26 @@ cudaError_t launch_depthwise7(const void* x, const void* w, const float* bias, v
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) sm_count[dev][relu] = sms;
   }
-  // output rows are dealt out evenly: a block walks a contiguous range of (32 channels, group of windows, row)
-  const long long work = (long long)p.groups * (C / kDw7Channels) * Ho;
-  const int blocks = (int)(work < sms ? work : sms);
-  p.work_quot = (int)(work / blocks);
-  p.work_rem = (int)(work % blocks);
+  // Output rows are dealt out evenly, a block walking a contiguous range of (32 channels, group of windows, row) that may
+  // cross from one unit into the next; or, where there are no more units than SMs, every unit is cut into the same
+  // number of runs and a block has one of them.  A run starts with six image rows for its first output row and with
+  // filling the pipeline, together worth about kDw7RunRows output rows, so that two short runs in a block cost more than
+  // a longer one.  us, dealt out evenly -> in runs: 3 x 7 x 7 x 768 12.5 -> 7.9, 12 x 14 x 14 x 384 13.3 -> 9.6,
+  // 24 x 28 x 28 x 192 15.5 -> 12.8, 96 x 14 x 14 x 384 21.2 -> 15.9; 64 x 56 x 56 x 96 stays with even ranges (35.3; 57 %
+  // of the SMs would have a run).
+  const int units = p.groups * (C / kDw7Channels);
+  const long long work = (long long)units * Ho;
+  const int even = (int)(work < sms ? work : sms);
+  p.work_quot = (int)(work / even);
+  p.work_rem = (int)(work % even);
+  p.parts = 0;
+  if (units <= sms) {
+    const int rows = p.work_quot + (p.work_rem != 0 ? 1 : 0);
+    const int runs = (rows == 1 || (p.work_rem == 0 && Ho % rows == 0)) ? 1 : (rows - 2) / Ho + 2;  // at most, of a block
+    const int parts = sms / units < Ho ? sms / units : Ho;
+    if ((Ho + parts - 1) / parts + kDw7RunRows < rows + runs * kDw7RunRows) p.parts = parts;
+  }
+  const int blocks = p.parts != 0 ? units * p.parts : even;
   CUtensorMap tm_x;
   {
     static EncodeFn encode = nullptr;  // (every thread finds the same function)

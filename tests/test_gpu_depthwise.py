@@ -25,6 +25,12 @@ CASES = [  # N, H, W, C, pad, relu
     (5, 8, 23, 160, 2, False),
     (40, 15, 15, 32, 4, False),   # block ranges that start and end inside a strip
 ]
+CASES += [
+    (12, 14, 14, 384, 3, True),   # units of rows cut into runs of two and three
+    (9, 27, 30, 160, 3, False),   # (15 units of 27 rows: nine runs of three)
+    (17, 9, 8, 2560, 3, False),   # 160 units of nine rows: ranges that cross from one into the next
+    (96, 5, 7, 256, 3, False),    # 48 units of five rows: runs of one and two
+]
 
 
 @pytest.mark.parametrize("case", CASES, ids=["x".join(map(str, c[:4])) + f"_p{c[4]}" for c in CASES])
