@@ -112,7 +112,8 @@ int32_t ssconv_plan(const ssconv_desc_t* desc, int32_t sparse, int32_t* tile_pos
  * at most four k-blocks in shared memory, 0 sends them through the ring like every other layer's.
  * SSCONV_TUNE_PAIR_TILES: -1 lets the planner choose (default) whether a work item of the pair kernel is two
  * neighbouring position tiles that share every group's weights, 0 never, 1 wherever the ring still holds two
- * groups (tiles of at most 192 positions keep three).  Not
+ * groups (tiles of at most 192 positions keep three).  SSCONV_TUNE_DEPTHWISE_MMA: -1 (default) runs 7 x 7 depthwise
+ * layers on the tensor cores where that is the faster way, 0 never (the fp32 kernels take them).  Not
  * thread-safe against concurrent calls.  Returns SSCONV_ERR_BAD_DESC for an unknown option or a value
  * out of range. */
 enum {
@@ -121,7 +122,8 @@ enum {
   SSCONV_TUNE_WGRAD_RANGES = 3,
   SSCONV_TUNE_WGRAD_PAIR = 4,
   SSCONV_TUNE_RESIDENT_WEIGHTS = 5,
-  SSCONV_TUNE_PAIR_TILES = 6
+  SSCONV_TUNE_PAIR_TILES = 6,
+  SSCONV_TUNE_DEPTHWISE_MMA = 7
 };
 int32_t ssconv_tune(int32_t option, int32_t value);
 

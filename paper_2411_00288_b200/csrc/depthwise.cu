@@ -39,6 +39,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 
 #include "layout.cuh"
@@ -480,19 +481,54 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
   }
 }
 
-// False: not a layer for this kernel (the caller goes on to the general ones).
-bool depthwise7_applies(int N, int H, int W, int C, int Ho, int Wo, int KH, int KW, int stride, int dil) {
-  return KH == kDw7K && KW == kDw7K && stride == 1 && dil == 1 && C % kDw7Channels == 0 &&
-         (long long)N * Ho * Wo * (C / kDw7Channels) < 0xFFFFFFFFll && (long long)H * W * C < (1ll << 38) &&
+static int g_tune_mma = -1;  // ssconv_tune: -1 automatic, 0 never this kernel
+int32_t set_depthwise_tuning(int32_t value) {
+  if (value != -1 && value != 0) return SSCONV_ERR_BAD_DESC;
+  g_tune_mma = value;
+  return SSCONV_OK;
+}
+
+// Layers for this kernel; for the others the caller goes on to the fp32 kernels.
+static bool depthwise7_applies(int N, int H, int W, int C, int Ho, int Wo, int KH, int KW, int stride, int dil) {
+  if (KH != kDw7K || KW != kDw7K || stride != 1 || dil != 1 || C % kDw7Channels != 0 || g_tune_mma == 0) return false;
+  return (long long)N * Ho * Wo * (C / kDw7Channels) < 0xFFFFFFFFll && (long long)H * W * C < (1ll << 38) &&
          (long long)N * ((Wo + 7) / 8) * (C / kDw7Channels) * Ho < 0x7FFFFFF0ll / 2;
+}
+
+// The kernel's SM count on the current device, after it has been made ready there; 0 in *sms: not to be run, because this
+// build of it was given another number of registers than its split between the roles counts on (a debug build, another
+// compiler).
+static cudaError_t depthwise7_ready(bool relu, int* sms) {
+  const auto kernel = relu ? depthwise7_mma_kernel<true> : depthwise7_mma_kernel<false>;
+  static std::atomic<int> known[64][2];  // SM count + 1 per device and form, 0: not looked at yet
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool keep = dev >= 0 && dev < 64;
+  const int k = keep ? known[dev][relu].load(std::memory_order_relaxed) : 0;
+  if (k != 0) {
+    *sms = k - 1;
+    return cudaSuccess;
+  }
+  cudaFuncAttributes fa;
+  e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  *sms = 0;
+  if (fa.numRegs == kDw7LaunchRegs) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDw7SmemBytes);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+  }
+  if (keep) known[dev][relu].store(*sms + 1, std::memory_order_relaxed);
+  return cudaSuccess;
 }
 
 typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-cudaError_t launch_depthwise7(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho,
-                              int Wo, int pad, uint32_t flags, cudaStream_t st) {
+static cudaError_t launch_depthwise7_on(int sms, const void* x, const void* w, const float* bias, void* y, int N, int H, int W,
+                                        int C, int Ho, int Wo, int pad, uint32_t flags, cudaStream_t st) {
   Dw7Params p;
   p.x = static_cast<const uint32_t*>(x);
   p.w = static_cast<const uint32_t*>(w);
@@ -509,22 +545,7 @@ cudaError_t launch_depthwise7(const void* x, const void* w, const float* bias, v
   p.nblk = (Wo + 7) / 8;
   p.groups = (N * p.nblk + kDw7Windows - 1) / kDw7Windows;
   p.flags = flags;
-  const bool relu = (flags & SSCONV_FLAG_RELU) != 0;
-  const auto kernel = relu ? depthwise7_mma_kernel<true> : depthwise7_mma_kernel<false>;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  static int sm_count[64][2] = {{0}};  // (set once per device and form, after the kernel has been made ready there)
-  int sms = (dev >= 0 && dev < 64) ? sm_count[dev][relu] : 0;
-  if (sms == 0) {
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, kernel);
-    if (e == cudaSuccess && fa.numRegs != kDw7LaunchRegs) return cudaErrorInvalidConfiguration;  // (the register split counts on it)
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDw7SmemBytes);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) sm_count[dev][relu] = sms;
-  }
+  const auto kernel = (flags & SSCONV_FLAG_RELU) ? depthwise7_mma_kernel<true> : depthwise7_mma_kernel<false>;
   // Output rows are dealt out evenly, a block walking a contiguous range of (32 channels, group of windows, row) that may
   // cross from one unit into the next; or, where there are no more units than SMs, every unit is cut into the same
   // number of runs and a block has one of them.  A run starts with six image rows for its first output row and with
@@ -551,7 +572,7 @@ cudaError_t launch_depthwise7(const void* x, const void* w, const float* bias, v
     if (encode == nullptr) {
       void* f = nullptr;
       cudaDriverEntryPointQueryResult q;
-      e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q);
+      const cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &f, cudaEnableDefault, &q);
       if (e != cudaSuccess) return e;
       if (q != cudaDriverEntryPointSuccess || f == nullptr) return cudaErrorNotSupported;
       encode = reinterpret_cast<EncodeFn>(f);
@@ -576,6 +597,19 @@ cudaError_t launch_depthwise7(const void* x, const void* w, const float* bias, v
   cfg.numAttrs = 1;
   count_launch();
   return cudaLaunchKernelEx(&cfg, kernel, tm_x, p);
+}
+
+// False: not a layer for this kernel, nothing has been launched.
+bool launch_depthwise7(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho, int Wo,
+                       int KH, int KW, int stride, int pad, int dil, uint32_t flags, cudaStream_t st, cudaError_t* result) {
+  if (!depthwise7_applies(N, H, W, C, Ho, Wo, KH, KW, stride, dil)) return false;
+  const bool relu = (flags & SSCONV_FLAG_RELU) != 0;
+  int sms = 0;
+  *result = depthwise7_ready(relu, &sms);
+  if (*result != cudaSuccess) return true;
+  if (sms == 0) return false;
+  *result = launch_depthwise7_on(sms, x, w, bias, y, N, H, W, C, Ho, Wo, pad, flags, st);
+  return true;
 }
 
 }  // namespace ssconv

@@ -488,24 +488,24 @@ __global__ void __launch_bounds__(128, 4) depthwise_run_kernel(const uint2* __re
   }
 }
 
-// Unit stride, no dilation, square 3 x 3 or 5 x 5 filter, C a multiple of 32 (7 x 7: depthwise.cu, where the
-// tensor cores win; their band matrices hold 3 or 5 taps in 16 columns here): a thread computes a tile of
-// kDwTileH x kDwTileW output pixels for one pair of channels, so that an image pixel is loaded and widened once
+// Unit stride, no dilation, square 3 x 3, 5 x 5 or 7 x 7 filter, C a multiple of 32 (7 x 7 only where the tensor cores
+// of depthwise.cu are not faster or not to be had; for 3 x 3 and 5 x 5 their band matrices would hold 3 or 5 taps in 16
+// columns): a thread computes a tile of kDwTileH x TW output pixels for one pair of channels (TW = 8, or 7 where that
+// divides the output width and 8 does not), so that an image pixel is loaded and widened once
 // for all the (up to K per direction) outputs of the tile it meets.  Sixteen lanes hold sixteen neighbouring
 // channel pairs of one tile (64 contiguous bytes per pixel); a block's eight tiles share the same 32 channels,
 // whose filter it keeps in shared memory as fp32 pairs.  The loop over image rows stays rolled (the filter row
 // under which image row r meets output row o is r - o, looked up at run time): unrolled, the kernel waited on
 // instruction fetch.  Output rows beyond the map's last are skipped.
-constexpr int kDwTileH = 4, kDwTileW = 8;
+constexpr int kDwTileH = 4;
 __device__ __forceinline__ float2 widen_f2(uint32_t v) {
   return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xFFFF0000u));
 }
-template <int K>
+template <int K, int TW>
 __global__ void __launch_bounds__(128, 4) depthwise_tile_kernel(const uint32_t* __restrict__ x, const uint32_t* __restrict__ w,
                                                                 const float* __restrict__ bias, uint32_t* __restrict__ y,
                                                                 int H, int W, int C2, int Ho, int Wo, int pad, int tiles_h,
                                                                 int tiles_w, long long tiles, uint32_t flags) {
-  constexpr int TW = kDwTileW;
   __shared__ float2 w_s[K * K][16];
   const int sub = threadIdx.x & 15;
   const int c2 = blockIdx.y * 16 + sub;
@@ -582,29 +582,29 @@ __global__ void __launch_bounds__(128, 4) depthwise_tile_kernel(const uint32_t* 
   }
 }
 
-bool depthwise7_applies(int N, int H, int W, int C, int Ho, int Wo, int KH, int KW, int stride, int dil);  // (depthwise.cu)
-cudaError_t launch_depthwise7(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho,
-                              int Wo, int pad, uint32_t flags, cudaStream_t st);
+bool launch_depthwise7(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho, int Wo,
+                       int KH, int KW, int stride, int pad, int dil, uint32_t flags, cudaStream_t st,
+                       cudaError_t* result);  // (depthwise.cu)
 
 cudaError_t launch_depthwise(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho,
                              int Wo, int KH, int KW, int stride, int pad, int dil, uint32_t flags, cudaStream_t st) {
   const long long total = (long long)N * Ho * Wo * (C / 8);
   if (total == 0) return cudaSuccess;
-  if (depthwise7_applies(N, H, W, C, Ho, Wo, KH, KW, stride, dil))
-    return launch_depthwise7(x, w, bias, y, N, H, W, C, Ho, Wo, pad, flags, st);
+  cudaError_t e;
+  if (launch_depthwise7(x, w, bias, y, N, H, W, C, Ho, Wo, KH, KW, stride, pad, dil, flags, st, &e)) return e;
   const int T = 256;
   count_launch();
-  if (stride == 1 && dil == 1 && KH == KW && (KW == 3 || KW == 5) && C % 32 == 0) {
-    const int tiles_h = (Ho + kDwTileH - 1) / kDwTileH, tiles_w = (Wo + kDwTileW - 1) / kDwTileW;
+  if (stride == 1 && dil == 1 && KH == KW && (KW == 3 || KW == 5 || KW == 7) && C % 32 == 0) {
+    const int tw = (KW == 7 && Wo % 7 == 0 && Wo % 8 != 0) ? 7 : 8;
+    const int tiles_h = (Ho + kDwTileH - 1) / kDwTileH, tiles_w = (Wo + tw - 1) / tw;
     const long long tiles = (long long)N * tiles_h * tiles_w;
     const dim3 grid((unsigned)((tiles + 7) / 8), (unsigned)(C / 32));
-    const uint32_t* xp = static_cast<const uint32_t*>(x);
-    const uint32_t* wp = static_cast<const uint32_t*>(w);
-    uint32_t* yp = static_cast<uint32_t*>(y);
-    if (KW == 3)
-      depthwise_tile_kernel<3><<<grid, 128, 0, st>>>(xp, wp, bias, yp, H, W, C / 2, Ho, Wo, pad, tiles_h, tiles_w, tiles, flags);
-    else
-      depthwise_tile_kernel<5><<<grid, 128, 0, st>>>(xp, wp, bias, yp, H, W, C / 2, Ho, Wo, pad, tiles_h, tiles_w, tiles, flags);
+    const auto kernel = KW == 3   ? depthwise_tile_kernel<3, 8>
+                        : KW == 5 ? depthwise_tile_kernel<5, 8>
+                        : tw == 7 ? depthwise_tile_kernel<7, 7>
+                                  : depthwise_tile_kernel<7, 8>;
+    kernel<<<grid, 128, 0, st>>>(static_cast<const uint32_t*>(x), static_cast<const uint32_t*>(w), bias,
+                                 static_cast<uint32_t*>(y), H, W, C / 2, Ho, Wo, pad, tiles_h, tiles_w, tiles, flags);
     return cudaGetLastError();
   }
   if (stride == 1 && dil == 1 && (KW == 3 || KW == 5 || KW == 7)) {

@@ -30,11 +30,26 @@ CASES += [
     (9, 27, 30, 160, 3, False),   # (15 units of 27 rows: nine runs of three)
     (17, 9, 8, 2560, 3, False),   # 160 units of nine rows: ranges that cross from one into the next
     (96, 5, 7, 256, 3, False),    # 48 units of five rows: runs of one and two
+    (3, 7, 21, 32, 3, True),      # (the fp32 kernel's tiles of 7 columns)
 ]
 
 
 @pytest.mark.parametrize("case", CASES, ids=["x".join(map(str, c[:4])) + f"_p{c[4]}" for c in CASES])
 def test_depthwise7_at_the_edges_of_its_tiles(case):
+    _check_case(case)
+
+
+@pytest.mark.parametrize("case", CASES, ids=["x".join(map(str, c[:4])) + f"_p{c[4]}" for c in CASES])
+def test_depthwise7_on_the_fp32_kernels(case):
+    # where the tensor-core kernel is not run (another register count than its roles' split needs, maps too small)
+    api.ssconv_tune(api.TUNE_DEPTHWISE_MMA, 0)
+    try:
+        _check_case(case)
+    finally:
+        api.ssconv_tune(api.TUNE_DEPTHWISE_MMA, -1)
+
+
+def _check_case(case):
     N, H, W, C, pad, relu = case
     g = torch.Generator().manual_seed(synth.SEED_BASE + 7100 + CASES.index(case))
     x = torch.randn((N, H, W, C), generator=g).to(torch.bfloat16)
