@@ -31,6 +31,11 @@ CASES += [
     (17, 9, 8, 2560, 3, False),   # 160 units of nine rows: ranges that cross from one into the next
     (96, 5, 7, 256, 3, False),    # 48 units of five rows: runs of one and two
     (3, 7, 21, 32, 3, True),      # (the fp32 kernel's tiles of 7 columns)
+    (4, 4, 4, 32, 3, False),      # 64 pixels, and on the other side of that line
+    (5, 4, 4, 32, 3, True),
+    (30, 3, 8, 64, 3, False),     # three rows of one window, and on the other sides of that line
+    (30, 3, 9, 64, 3, False),
+    (30, 4, 8, 64, 3, True),
 ]
 
 
@@ -96,21 +101,23 @@ def test_depthwise7_non_finite_pixels_reach_their_own_windows_only():
 
 @pytest.mark.parametrize("data", ["normal", "spread", "positive"])
 def test_depthwise7_sums_are_as_exact_as_fp32_ones(data):
-    # One output per channel; the bias (added last) is minus the exact sum, so that what is left is the error of the sum.
+    # The bias (added last) is minus the exact sum of one output per channel, so that what is left there is the error of
+    # the sum.  (17 maps of 4 x 1 outputs: fewer, or flatter ones, would go to the fp32 kernel.)
     C, units = 4096, []
     for seed in range(8):
         g = torch.Generator().manual_seed(synth.SEED_BASE + 7900 + seed)
-        x, w = torch.randn((7, 7, C), generator=g), torch.randn((7, 7, C), generator=g) / 7
+        x, w = torch.randn((17, 10, 7, C), generator=g), torch.randn((7, 7, C), generator=g) / 7
         if data == "spread":
             x = x * torch.exp(2.0 * torch.randn(x.shape, generator=g))
         if data == "positive":
             x, w = x.abs(), w.abs()
         x, w = x.to(torch.bfloat16), w.to(torch.bfloat16)
-        products = x.double() * w.double()
+        n, row = 2 * seed, seed % 4
+        products = x[n, row:row + 7].double() * w.double()
         total = products.sum((0, 1))
         bias = (-total).float()
-        desc = api.make_desc(1, 7, 7, C, C, 7, 7, 1, 0, bias=True)
-        y = api.ssconv_depthwise(desc, x[None].to(DEV), w.to(DEV), bias.to(DEV)).cpu().double().view(-1)
+        desc = api.make_desc(17, 10, 7, C, C, 7, 7, 1, 0, bias=True)
+        y = api.ssconv_depthwise(desc, x.to(DEV), w.to(DEV), bias.to(DEV))[n, row, 0].cpu().double()
         units.append((y - (total + bias.double())) / products.abs().sum((0, 1)) * 2.0 ** 24)
     err = torch.cat(units)
     # what a chain of 49 fused multiply-adds leaves on these data (0.163, 0.744, 0.801 over 131072 sums; a fortieth more for
