@@ -425,7 +425,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
       }
     }
     for (int a = seg.a0; a < seg.a1; ++a) {
-      if (!mbar_wait_a(empty0 + 8u * g, ph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
+      if (!mbar_wait_warp_a(empty0 + 8u * g, ph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
       const uint32_t full = full0 + 8u * g;
       const uint32_t dst = ring0 + g * grp_bytes;
       const bool has_second = 2 * a + 1 < p.kblocks;
@@ -611,7 +611,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       const bool resident = !SPARSE && !FP8 && p.a_res_bytes != 0;
       const uint32_t res_lo0 = ring_lo0 + (uint32_t)p.ring_groups * grp_desc;
       bool ok = true;
-      if (resident && !mbar_wait_bounded(&bar_res[0], 0u, abort_flag, kWaitLimitCycles)) ok = false;
+      if (resident && !mbar_wait_warp(&bar_res[0], 0u, abort_flag, kWaitLimitCycles)) ok = false;
       const uint32_t full0 = smem_u32(bar_full), empty0 = smem_u32(bar_empty);
       // With two ring slots the ring's depth bounds the main loop: the first k-block's activation
       // tile is then released on its own, so that its reload starts one k-block earlier.
@@ -633,7 +633,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       for (; ok && work.next(seg); ++tcount) {
         const uint32_t buf = tcount & 1u;
         const uint32_t aph = (tcount >> 1) & 1u;
-        if (!mbar_wait_bounded(&bar_acc_empty[buf], aph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
+        if (!mbar_wait_warp(&bar_acc_empty[buf], aph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * kAccCol1;
         uint32_t accumulate = 0;
@@ -644,7 +644,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
         auto run_groups = [&](auto early_tag) {
           constexpr bool kEarly = decltype(early_tag)::value;
           for (int a = seg.a0; a < seg.a1; ++a) {
-            if (!mbar_wait_a(full0 + 8u * g, ph, abort_flag, kWaitLimitCycles)) { ok = false; break; }
+            if (!mbar_wait_warp_a(full0 + 8u * g, ph, abort_flag, kWaitLimitCycles)) { ok = false; break; }
             const uint32_t grp_lo = ring_lo0 + g * grp_desc;
             const uint32_t a_lo = resident ? res_lo0 + (uint32_t)a * ((2u * kATileBytes) >> 4) : grp_lo;
             const uint32_t b0_lo = grp_lo + a_off_desc;
@@ -778,7 +778,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       const uint32_t aph = (tcount >> 1) & 1u;
       // (two sets: each serves one accumulator, so that it has two tiles' time for its tiles)
       if (EPI_SETS == 2 && buf != (uint32_t)(grp / kGroups)) continue;
-      const bool got = mbar_wait_bounded(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
+      const bool got = mbar_wait_warp(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
       if (kStoreWarps) {
         if (!got) break;
       } else {
@@ -839,7 +839,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
         // its source has landed, below; without store warps: the leader saw that store finish reading before it
         // entered the barrier of the previous piece).
         if (kStoreWarps && !RES &&
-            !mbar_wait_bounded(&bar_stage_free[nbuf * grp + sbuf], ((piece_count >> nbuf_shift) & 1u) ^ 1u, abort_flag, kWaitLimitCycles)) {
+            !mbar_wait_warp(&bar_stage_free[nbuf * grp + sbuf], ((piece_count >> nbuf_shift) & 1u) ^ 1u, abort_flag, kWaitLimitCycles)) {
           ok = false;
           break;
         }
@@ -850,7 +850,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
         }
         if (RES) {
           // the residual piece has landed in this buffer
-          if (!mbar_wait_bounded(&bar_res[4 * grp + sbuf], (piece_count >> nbuf_shift) & 1u, abort_flag, kWaitLimitCycles)) {
+          if (!mbar_wait_warp(&bar_res[4 * grp + sbuf], (piece_count >> nbuf_shift) & 1u, abort_flag, kWaitLimitCycles)) {
             ok = false;
             break;
           }
@@ -1167,7 +1167,7 @@ __device__ __forceinline__ void pair_producer_role(const CUtensorMap* tm_a, cons
       first_segment = false;
     }
     for (int a = 0; a < p.a_tiles; ++a) {
-      if (!mbar_wait_a(empty0 + 8u * g, ph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
+      if (!mbar_wait_warp_a(empty0 + 8u * g, ph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
       const uint32_t full = full0_leader + 8u * g;  // cluster address of the leader's barrier
       const uint32_t dst = ring0 + g * grp_bytes;
       const bool has_second = 2 * a + 1 < p.kblocks;
@@ -1322,18 +1322,18 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
         // one accumulator per tile: alternating between the two buffers, or (two tiles per item) both at once
         const uint32_t buf = dual ? 0u : (tcount & 1u);
         const uint32_t aph = dual ? (tcount & 1u) : ((tcount >> 1) & 1u);
-        if (!mbar_wait_bounded(&bar_acc_empty[buf], aph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
-        if (dual && !mbar_wait_bounded(&bar_acc_empty[1], aph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
+        if (!mbar_wait_warp(&bar_acc_empty[buf], aph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
+        if (dual && !mbar_wait_warp(&bar_acc_empty[1], aph ^ 1u, abort_flag, kWaitLimitCycles)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * kAccCol1;
         const uint32_t d_tmem1 = tmem_base + kAccCol1;
         uint32_t accumulate = 0;
         for (int a = 0; a < p.a_tiles; ++a) {
-          if (!ready && !mbar_wait_a(full0 + 8u * g, ph, abort_flag, kWaitLimitCycles)) { ok = false; break; }
+          if (!ready && !mbar_wait_warp_a(full0 + 8u * g, ph, abort_flag, kWaitLimitCycles)) { ok = false; break; }
           {  // look ahead at the next group's barrier (the ring runs on across tiles) while this group's
              // MMAs are issued; the answer is used at the top of the next iteration
             const uint32_t g_next = (g + 1u == (uint32_t)p.ring_groups) ? 0u : g + 1u;
-            ready = mbar_test_a(full0 + 8u * g_next, g_next == 0u ? ph ^ 1u : ph);
+            ready = __all_sync(0xFFFFFFFFu, mbar_test_a(full0 + 8u * g_next, g_next == 0u ? ph ^ 1u : ph));
           }
           tc_fence_after();
           const uint32_t a_lo = ring_lo0 + g * grp_desc;
@@ -1417,7 +1417,7 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
       const int m = 2 * (seg.tile - pu * p.m_tiles) + (int)rank;
       const uint32_t buf = p.dual ? t : (icount & 1u);
       const uint32_t aph = p.dual ? (icount & 1u) : ((icount >> 1) & 1u);
-      const bool got = mbar_wait_bounded(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
+      const bool got = mbar_wait_warp(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
       if (!RES) {
         if (leader) my_go[tcount & 1u] = (got && *abort_flag == 0) ? 1 : 0;
         epilogue_bar_sync(grp);
@@ -1457,7 +1457,7 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
         const uint32_t st_addr = smem_u32(stage) + st_offset;
         if (RES) {
           // the residual piece has landed in this buffer
-          if (!mbar_wait_bounded(&bar_res[4 * grp + sbuf], use, abort_flag, kWaitLimitCycles)) {
+          if (!mbar_wait_warp(&bar_res[4 * grp + sbuf], use, abort_flag, kWaitLimitCycles)) {
             go_on = false;
             break;
           }

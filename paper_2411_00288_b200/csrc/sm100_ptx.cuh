@@ -76,6 +76,19 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return mbar_wait_a(smem_u32(bar), parity, abort_flag, limit_cycles, backoff_ns);
 }
 
+// The same for a warp that goes on in lock step (tcgen05, ldmatrix, stmatrix, elect and the like take all 32 lanes):
+// one verdict for the whole warp.  Lanes poll the barrier and read the flag each for itself, so that around the limit
+// some may find the phase complete and others the flag raised.  The votes are not to be seen in any layer's time.
+__device__ __forceinline__ bool mbar_wait_warp_a(uint32_t bar_addr, uint32_t parity, volatile int* abort_flag,
+                                                 long long limit_cycles, uint32_t backoff_ns = 0) {
+  if (__all_sync(0xFFFFFFFFu, mbar_spin_a(bar_addr, parity, kFastSpins))) return true;
+  return __all_sync(0xFFFFFFFFu, mbar_wait_slow(bar_addr, parity, abort_flag, limit_cycles, backoff_ns));
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                               long long limit_cycles, uint32_t backoff_ns = 0) {
+  return mbar_wait_warp_a(smem_u32(bar), parity, abort_flag, limit_cycles, backoff_ns);
+}
+
 // ---------------------------------------------------------------- proxies / fences
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

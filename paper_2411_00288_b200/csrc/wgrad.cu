@@ -210,8 +210,7 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
     // ------------------------------------------------------------------ epilogue
     const int qd = warp & 3;  // TMEM lane quadrant of this warp
     // the TMEM loads below are warp-wide: the warp goes on only if every lane saw the barrier complete
-    const bool got =
-        __all_sync(0xFFFFFFFFu, mbar_wait_bounded(bar_acc, 0u, abort_flag, kWgWaitLimitCycles, 64) ? 1 : 0) != 0;
+    const bool got = mbar_wait_warp(bar_acc, 0u, abort_flag, kWgWaitLimitCycles, 64);
     if (got) {
       tc_fence_after();
       const size_t K = (size_t)p.taps * p.C_in;
@@ -366,7 +365,7 @@ ssconv_wgrad_pair_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid
     }
     grid_dependency_wait();   // everything above may overlap the tail of the kernel before this one
     for (int ks = ks0; ks < ks1; ++ks) {
-      if (!mbar_wait_a(empty0 + 8u * s, ph ^ 1u, abort_flag, kWgWaitLimitCycles)) break;
+      if (!mbar_wait_warp_a(empty0 + 8u * s, ph ^ 1u, abort_flag, kWgWaitLimitCycles)) break;
       const uint32_t full = full0_leader + 8u * s;
       const uint32_t dst = ring0 + s * kWpStageBytes;
       const int q0 = ks * kWpPos;
@@ -400,7 +399,7 @@ ssconv_wgrad_pair_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid
       uint32_t s = 0, ph = 0, accumulate = 0;
       bool ok = true;
       for (int ks = ks0; ks < ks1; ++ks) {
-        if (!mbar_wait_a(full0_local + 8u * s, ph, abort_flag, kWgWaitLimitCycles)) { ok = false; break; }
+        if (!mbar_wait_warp_a(full0_local + 8u * s, ph, abort_flag, kWgWaitLimitCycles)) { ok = false; break; }
         tc_fence_after();
         const uint32_t a_lo = wp_desc_lo(ring0 + s * kWpStageBytes);
         const uint32_t b_lo = a_lo + ((2u * kWpTileBytes) >> 4);
@@ -421,8 +420,7 @@ ssconv_wgrad_pair_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid
   } else if (warp >= 4) {
     // ------------------------------------------------------------------ epilogue
     const int qd = warp & 3;  // TMEM lane quadrant of this warp
-    const bool got =
-        __all_sync(0xFFFFFFFFu, mbar_wait_bounded(bar_acc, 0u, abort_flag, kWgWaitLimitCycles, 64) ? 1 : 0) != 0;
+    const bool got = mbar_wait_warp(bar_acc, 0u, abort_flag, kWgWaitLimitCycles, 64);
     if (got) {
       tc_fence_after();
       // Lane row 32 qd + lane of this CTA = channel (32 qd + lane) % 64 of its k-block (32 qd + lane) / 64.
