@@ -433,6 +433,13 @@ int32_t ssconv_forward_dense_grouped(const ssconv_desc_t* desc, int32_t groups, 
 int32_t ssconv_depthwise(const ssconv_desc_t* desc, const void* x, const void* w_bf16, const float* bias, void* y,
                          void* stream);
 
+/* ssconv_depthwise on the tensor-core kernel with a limit of `polls` polls (0 to 2^20) on its waits, which then run out
+ * (0: every one of them).  The blocks end their copies and compute their outputs again by themselves: y is what
+ * ssconv_depthwise gives but for the order of summation.  For tests.  SSCONV_ERR_UNSUPPORTED_SHAPE: not a layer for
+ * that kernel. */
+int32_t ssconv_selftest_depthwise_give_up(const ssconv_desc_t* desc, const void* x, const void* w_bf16, const float* bias,
+                                          void* y, int32_t polls, void* stream);
+
 /* Layer normalisation over the channels of each pixel, y = (x - mean) / sqrt(var + eps) * gamma + beta
  * (biased variance; fp32 arithmetic, one rounding to bf16): the normalisation between the depthwise and
  * the point-wise convolutions of a ConvNeXt block (Sec. 4 evaluates on ConvNeXt); no counterpart in the

@@ -25,7 +25,7 @@ ERR_TIMEOUT = 8
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libssconv.so")
 EXPORTS = ("ssconv_version", "ssconv_launch_count", "ssconv_status_string", "ssconv_out_shape", "ssconv_sizes",
-           "ssconv_plan", "ssconv_plan_for_sms", "ssconv_tune", "ssconv_window_extent", "ssconv_selftest_wait_timeout",
+           "ssconv_plan", "ssconv_plan_for_sms", "ssconv_tune", "ssconv_window_extent", "ssconv_selftest_wait_timeout", "ssconv_selftest_depthwise_give_up",
            "ssconv_select_mask", "ssconv_nm_patterns", "ssconv_select_mask_nm", "ssconv_apply_mask_nm",
            "ssconv_compress", "ssconv_decompress", "ssconv_maxpool", "ssconv_pad_channels", "ssconv_space_to_depth", "ssconv_unfold_w",
            "ssconv_fold_factor", "ssconv_fold_desc", "ssconv_fold_weights", "ssconv_forward", "ssconv_forward_res",
@@ -120,6 +120,7 @@ def _prototypes():
         "ssconv_forward_grouped": (i32, [vp, i32] + [vp] * 6 + [sz, vp, vp]),
         "ssconv_forward_dense_grouped": (i32, [vp, i32] + [vp] * 5 + [sz, vp, vp]),
         "ssconv_depthwise": (i32, [vp] * 6),
+        "ssconv_selftest_depthwise_give_up": (i32, [vp] * 5 + [i32, vp]),
         "ssconv_layernorm": (i32, [vp, vp, vp, f32, vp, i64, i32, vp]),
         "ssconv_quantize_e4m3": (i32, [vp, vp, i64, f32, vp]),
         "ssconv_sizes_fp8": (i32, [vp] * 4),
@@ -553,6 +554,16 @@ def ssconv_depthwise(desc: Desc, x: torch.Tensor, w: torch.Tensor, bias: Optiona
         y = _alloc_y(desc, x)
     f = lib().ssconv_depthwise
     _check("ssconv_depthwise", f(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(y), _stream(stream)))
+    return y
+
+
+def ssconv_selftest_depthwise_give_up(desc: Desc, x: torch.Tensor, w: torch.Tensor, bias: Optional[torch.Tensor],
+                                      polls: int, stream=None) -> torch.Tensor:
+    """ssconv_depthwise with waits that run out after `polls` polls; the outputs are then computed again and come out whole."""
+    _need_cuda(x, w, bias)
+    y = _alloc_y(desc, x)
+    _check("ssconv_selftest_depthwise_give_up", lib().ssconv_selftest_depthwise_give_up(
+        ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(y), int(polls), _stream(stream)))
     return y
 
 

@@ -27,10 +27,12 @@
 //   16 warps of two channels each keep the band matrices (28 registers) and the accumulators of the seven
 //     output rows in flight (56) and write each finished row to shared memory;
 //   4 warps store finished rows, 64 bytes per pixel.
-// The roles meet at mbarriers only.  Measured on that tensor under ncu: 61 us (the fp32 kernel with 4 x 8
-// outputs per thread before it: 122-127 us; one set of helper warps 65 us; no roles and one row of loads ahead
-// 72 us).  By events around one launch: 131 -> 64 us, 128 x 28 x 28 x 192 74 -> 47, 14 x 14 x 384 44 -> 33,
-// 7 x 7 x 768 33 -> 27 us.  The shared-memory pipe is 59 % busy, the tensor pipe 31 %.
+// The roles meet at mbarriers only.  A warp that gives up on one (after kDw7Polls polls) ends its part, the others run
+// into their own limits, and the block computes its outputs again from the image alone.
+// Measured on that tensor (us): the fp32 kernel with tiles of outputs per thread 122; without roles and one row of
+// loads ahead 72 under ncu, with one set of helper warps 65, as here 61 before the additions above and the votes on
+// the waits (1.5).  Now 61.8 between other launches, 128 x 28 x 28 x 192 44.5 (65 in fp32), 14 x 14 x 384 30.4 (36), 7 x 7 x
+// 768 22.9 (25).
 //
 // Zero entries of the band matrix meet pixels outside an output's window.  An infinity or NaN among those
 // would turn the output into a NaN, so a block that meets a non-finite accumulator looks at its outputs again at
@@ -58,7 +60,7 @@ constexpr int kDw7LaunchRegs = 80, kDw7MainRegs = 96, kDw7HelperRegs = 48;
 static_assert(kDw7MainWarps * kDw7MainRegs + 2 * kDw7HelperWarps * kDw7HelperRegs <=
                   (kDw7MainWarps + 2 * kDw7HelperWarps) * kDw7LaunchRegs,
               "a register split above the launch's total never ends");
-constexpr uint32_t kDw7Spins = 1u << 20;            // polls of a barrier before a warp gives up on it
+constexpr uint32_t kDw7Polls = 1u << 20;            // of a barrier, before a warp gives up on it
 constexpr int kDw7Channels = 32;                    // per block
 constexpr int kDw7Windows = 16;                     // per block: the rows of the MMA
 constexpr int kDw7Slots = 2 * kDw7Windows;          // most 8-pixel pieces of a row they touch
@@ -100,9 +102,31 @@ struct Dw7Params {
   int groups;               // groups of 16 windows (of N nblk)
   int parts;                // thread blocks per unit (a group's 32 channels), each with one run of its rows; or 0:
   int work_quot, work_rem;  // output rows per thread block (of groups * C / 32 * Ho): quotient and remainder
+  uint32_t polls;           // kDw7Polls, or fewer in the self-test (0: every wait gives up)
   uint32_t flags;
 };
 
+// Polls a phase of an mbarrier at most `polls` times (0: not at all).  Every lane has an answer of its own; the roles go on
+// in lock step (ldmatrix, mma, shuffles) and so only branch on what __all_sync makes of it.
+__device__ __forceinline__ bool dw7_poll(uint32_t bar, uint32_t parity, uint32_t polls) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\t"
+      "mov.u32 n, %3;\n\t"
+      "setp.ne.u32 p, 0, 0;\n"
+      "SPIN:\n\t"
+      "setp.eq.u32 q, n, 0;\n\t"
+      "@q bra DONE;\n\t"
+      "sub.u32 n, n, 1;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@!p bra SPIN;\n"
+      "DONE:\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(polls)
+      : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
@@ -283,10 +307,11 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
         for (int ph = 0; ph < kDw7K; ++ph) {  // (unrolled: the accumulator of output row o is o mod 7)
           const int r = r0 + ph;
           if (r >= rows || !ok) break;
+          bool got = true;
           // Image row r under filter row kh is output row r - kh.  (Rows before the segment's first are dropped
           // below, rows past its last never leave the accumulators.)
           if (r >= row0 && r < row1) {
-            ok = mbar_spin_a(full0 + 8u * sbuf, sphase, kDw7Spins);
+            got = dw7_poll(full0 + 8u * sbuf, sphase, p.polls);  // (if it gives up: every output is computed again below)
             uint32_t a[2][4];
             ldmatrix_x4(a_addr + sbuf * kDw7StageBytes, a[0]);
             ldmatrix_x4(a_addr + sbuf * kDw7StageBytes + 4u * kDw7ChannelWords, a[1]);
@@ -319,7 +344,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             float(&d0)[4] = acc[0][(ph + 1) % kDw7K];
             float(&d1)[4] = acc[1][(ph + 1) % kDw7K];
             const float bias0 = __uint_as_float(lds32(bias_at)), bias1 = __uint_as_float(lds32(bias_at + 4u));
-            ok = mbar_spin_a(oempty0 + 8u * obuf, ophase ^ 1u, kDw7Spins) && ok;
+            got = dw7_poll(oempty0 + 8u * obuf, ophase ^ 1u, p.polls) && got;
             const uint32_t o = out_dst + obuf * kDw7OutBytes;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -337,6 +362,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
             const float sum = ((d0[0] + d0[1]) + (d0[2] + d0[3])) + ((d1[0] + d1[1]) + (d1[2] + d1[3]));
             if (!(fabsf(sum) <= 3.0e38f)) *again = 1;
           }
+          ok = __all_sync(0xFFFFFFFFu, got);
         }
       }
       if (!ok) *failed = 1;
@@ -362,6 +388,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kDw7HelperRegs));
     const int ht = tid - 32 * kDw7MainWarps, hw = warp - kDw7MainWarps;
     uint32_t rbuf = 0, rphase = 0;
+    uint32_t in_flight = 0;                                     // copies issued and not used up
     while (pos < end) {
       const Dw7Segment sg(p, pos, end);
       // A warp brings in pieces 2 hw, 2 hw + 1, 2 hw + 8, ... of the rows by itself: lane l < 8 copies piece
@@ -376,7 +403,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
       int row_next = sg.row0;                                   // first row of the next copy
       uint32_t cbuf = rbuf;
       auto copy_rows = [&]() {  // (all lanes; the buffer's last rows have been read)
-        if (row_next >= sg.row1) return;
+        if (row_next >= sg.row1 || !ok) return;
         const uint32_t bar = raw_bar0 + 8u * cbuf;
         if (lane == 0) mbar_expect_tx_a(bar, copies * kDw7RawSlotBytes);
         __syncwarp();
@@ -384,6 +411,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
           tma_load_4d_a(raw0 + cbuf * kDw7RawBytes + my_slot * kDw7RawSlotBytes, &tm_x, bar, sg.z * kDw7Channels, my_col,
                         sg.h0 - p.pad + row_next, my_n);
         row_next += kDw7RawRows;
+        ++in_flight;
         cbuf = (cbuf + 1 == kDw7RawBufs) ? 0u : cbuf + 1;
       };
       for (int k = 0; k < kDw7RawBufs; ++k) copy_rows();
@@ -397,8 +425,10 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
       __syncthreads();
       for (int r = sg.row0; r < sg.row1 && ok; ++r) {
         const int sub = (r - sg.row0) % kDw7RawRows;
-        if (sub == 0) ok = mbar_spin_a(raw_bar0 + 8u * rbuf, rphase, kDw7Spins);
-        ok = mbar_spin_a(empty0 + 8u * sbuf, sphase ^ 1u, kDw7Spins) && ok;
+        bool got = sub != 0 || dw7_poll(raw_bar0 + 8u * rbuf, rphase, p.polls);
+        got = dw7_poll(empty0 + 8u * sbuf, sphase ^ 1u, p.polls) && got;
+        ok = __all_sync(0xFFFFFFFFu, got);
+        if (!ok) break;
         const uint32_t src = raw_src + rbuf * kDw7RawBytes + sub * 512u;
 #pragma unroll
         for (int k2 = 0; k2 < 4; k2 += 2) {
@@ -427,6 +457,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
           sphase ^= 1u;
         }
         if (sub == kDw7RawRows - 1 || r + 1 == sg.row1) {  // the copy is used up
+          --in_flight;
           copy_rows();
           if (++rbuf == kDw7RawBufs) {
             rbuf = 0;
@@ -434,7 +465,18 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
           }
         }
       }
-      if (!ok) *failed = 1;
+      if (!ok) {
+        // Copies that are under way land before the block goes on (it may be at its end): no more are issued, and
+        // each of these is waited for, with the full limit, in the order of their buffers.
+        for (; in_flight != 0; --in_flight) {
+          dw7_poll(raw_bar0 + 8u * rbuf, rphase, kDw7Polls);
+          if (++rbuf == kDw7RawBufs) {
+            rbuf = 0;
+            rphase ^= 1u;
+          }
+        }
+        *failed = 1;
+      }
       __syncthreads();
       __syncthreads();
     }
@@ -451,7 +493,7 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
       char* y_row = reinterpret_cast<char*>(p.y + (lane & 15));
       __syncthreads();
       for (int o = 0; o < sg.S && ok; ++o) {
-        ok = mbar_spin_a(ofull0 + 8u * obuf, ophase, kDw7Spins);
+        ok = __all_sync(0xFFFFFFFFu, dw7_poll(ofull0 + 8u * obuf, ophase, p.polls));
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
           uint32_t to[8], w[8];
@@ -532,7 +574,7 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 static cudaError_t launch_depthwise7_on(int sms, const void* x, const void* w, const float* bias, void* y, int N, int H, int W,
-                                        int C, int Ho, int Wo, int pad, uint32_t flags, cudaStream_t st) {
+                                        int C, int Ho, int Wo, int pad, uint32_t flags, uint32_t polls, cudaStream_t st) {
   Dw7Params p;
   p.x = static_cast<const uint32_t*>(x);
   p.w = static_cast<const uint32_t*>(w);
@@ -548,6 +590,7 @@ static cudaError_t launch_depthwise7_on(int sms, const void* x, const void* w, c
   p.y_row = 2ll * Wo * C;
   p.nblk = (Wo + 7) / 8;
   p.groups = (N * p.nblk + kDw7Windows - 1) / kDw7Windows;
+  p.polls = polls;
   p.flags = flags;
   const auto kernel = (flags & SSCONV_FLAG_RELU) ? depthwise7_mma_kernel<true> : depthwise7_mma_kernel<false>;
   // Output rows are dealt out evenly, a block walking a contiguous range of (32 channels, group of windows, row) that may
@@ -603,16 +646,18 @@ static cudaError_t launch_depthwise7_on(int sms, const void* x, const void* w, c
   return cudaLaunchKernelEx(&cfg, kernel, tm_x, p);
 }
 
-// False: not a layer for this kernel, nothing has been launched.
+// False: not a layer for this kernel, nothing has been launched.  polls: of a barrier, -1 = kDw7Polls.
 bool launch_depthwise7(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho, int Wo,
-                       int KH, int KW, int stride, int pad, int dil, uint32_t flags, cudaStream_t st, cudaError_t* result) {
+                       int KH, int KW, int stride, int pad, int dil, uint32_t flags, int32_t polls, cudaStream_t st,
+                       cudaError_t* result) {
   if (!depthwise7_applies(N, H, W, C, Ho, Wo, KH, KW, stride, dil)) return false;
   const bool relu = (flags & SSCONV_FLAG_RELU) != 0;
   int sms = 0;
   *result = depthwise7_ready(relu, &sms);
   if (*result != cudaSuccess) return true;
   if (sms == 0) return false;
-  *result = launch_depthwise7_on(sms, x, w, bias, y, N, H, W, C, Ho, Wo, pad, flags, st);
+  *result = launch_depthwise7_on(sms, x, w, bias, y, N, H, W, C, Ho, Wo, pad, flags, polls < 0 ? kDw7Polls : (uint32_t)polls,
+                                 st);
   return true;
 }
 

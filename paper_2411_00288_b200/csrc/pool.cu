@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(128, 4) depthwise_tile_kernel(const uint32_t* 
 }
 
 bool launch_depthwise7(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho, int Wo,
-                       int KH, int KW, int stride, int pad, int dil, uint32_t flags, cudaStream_t st,
+                       int KH, int KW, int stride, int pad, int dil, uint32_t flags, int32_t polls, cudaStream_t st,
                        cudaError_t* result);  // (depthwise.cu)
 
 cudaError_t launch_depthwise(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho,
@@ -591,7 +591,7 @@ cudaError_t launch_depthwise(const void* x, const void* w, const float* bias, vo
   const long long total = (long long)N * Ho * Wo * (C / 8);
   if (total == 0) return cudaSuccess;
   cudaError_t e;
-  if (launch_depthwise7(x, w, bias, y, N, H, W, C, Ho, Wo, KH, KW, stride, pad, dil, flags, st, &e)) return e;
+  if (launch_depthwise7(x, w, bias, y, N, H, W, C, Ho, Wo, KH, KW, stride, pad, dil, flags, -1, st, &e)) return e;
   const int T = 256;
   count_launch();
   if (stride == 1 && dil == 1 && KH == KW && (KW == 3 || KW == 5 || KW == 7) && C % 32 == 0) {

@@ -76,6 +76,27 @@ def _check_case(case):
     assert rel <= parity.REL_FRO_TOL and mx <= parity.MAX_ABS_TOL, (case, rel, mx)
 
 
+@pytest.mark.parametrize("polls", [0, 1, 3, 40])
+@pytest.mark.parametrize("case", [(17, 9, 8, 2560, 3, False), (24, 28, 28, 64, 3, True), (9, 27, 30, 160, 3, False)])
+def test_depthwise7_computes_everything_again_when_waits_run_out(case, polls):
+    # (0: all waits give up; more: some warps of a block may give up and others not)
+    N, H, W, C, pad, relu = case
+    g = torch.Generator(device=DEV).manual_seed(synth.SEED_BASE + 7990)
+    x = torch.randn((N, H, W, C), generator=g, device=DEV).to(torch.bfloat16)
+    w = (torch.randn((7, 7, C), generator=g, device=DEV) / 7).to(torch.bfloat16)
+    bias = torch.randn(C, generator=g, device=DEV) * 0.1
+    desc = api.make_desc(N, H, W, C, C, 7, 7, 1, pad, bias=True, relu=relu)
+    ref = api.ssconv_depthwise(desc, x, w, bias)                                   # (compared with the oracle above)
+    y = api.ssconv_selftest_depthwise_give_up(desc, x, w, bias, polls)
+    again = api.ssconv_depthwise(desc, x, w, bias)
+    torch.cuda.synchronize()
+    assert torch.equal(again, ref)
+    # two fp32 sums of the same products: one rounding to bf16 apart, and near zero what they lose to cancellation
+    assert bool(((y.float() - ref.float()).abs() <= 2.0 ** -7 * ref.float().abs() + 1e-5).all())
+    if polls == 0:
+        assert not torch.equal(y, ref)                                             # (computed another way: some roundings differ)
+
+
 def test_depthwise7_non_finite_pixels_reach_their_own_windows_only():
     N, H, W, C = 2, 20, 19, 64
     g = torch.Generator().manual_seed(synth.SEED_BASE + 7200)

@@ -34,8 +34,7 @@ def _enclosing_heads(text, at):
 def test_waits_of_whole_warps_are_voted(name):
     text = _without_comments(open(os.path.join(CSRC, name)).read())
     uses = list(PER_LANE.finditer(text))
-    waits = uses + list(re.finditer(r"\bmbar_wait_warp(_a)?\s*\(", text))
-    assert len(waits) >= 5
+    assert len(uses) + len(re.findall(r"\b(?:mbar_wait_warp|mbar_wait_warp_a)\s*\(", text)) >= 5
     for use in uses:
         statement = text[max(text.rfind(c, 0, use.start()) for c in ";{}") + 1:use.start()]
         single = any(ONE_THREAD.search(h) for h in _enclosing_heads(text, use.start()))
