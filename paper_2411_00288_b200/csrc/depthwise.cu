@@ -531,12 +531,15 @@ int32_t set_depthwise_tuning(int32_t value) {
 }
 
 // Layers for this kernel; for the others the caller goes on to the fp32 kernels.  Maps of a few pixels are among the others:
-// their windows are mostly empty, and this kernel's start-up is longer than what the fp32 kernel takes for all of it
-// (us, this kernel / the fp32 tiles: 1 x 3 x 3 x 768 7.0 / 5.6, 60 x 2 x 2 x 768 6.5 / 5.5, 4 x 4 x 4 x 768 8.1 / 7.0,
-// 1 x 7 x 7 x 768 11.3 / 8.8; beyond the lines 8 x 4 x 4 x 768 7.0 / 7.0, 32 x 4 x 4 x 768 7.3 / 9.2, 2 x 7 x 7 x 768 8.0 / 8.8).
+// their windows are mostly empty, and this kernel's start-up is longer than what the fp32 kernel takes for all of it.
+// Up to 64 pixels the line is the number of blocks: from about half the SMs on, the copies of empty windows are slow.  us,
+// this kernel / the fp32 tiles: 1 x 3 x 3 x 768 7.0 / 5.6, 60 x 2 x 2 x 768 6.5 / 5.5; 84 blocks 1 x 7 x 7 x 384 10.2 / 8.8, 96
+// blocks 4 x 4 x 4 x 768 8.1 / 7.0, 144 blocks 1 x 7 x 7 x 768 11.3 / 8.8.  Beyond the lines: 72 blocks 1 x 6 x 6 x 384 8.0 / 9.4, 60
+// blocks 1 x 5 x 5 x 384 7.8 / 8.5, 98 pixels 2 x 7 x 7 x 768 8.0 / 8.8, 8 x 4 x 4 x 768 7.0 / 7.0, 32 x 4 x 4 x 768 7.3 / 9.2.
 static bool depthwise7_applies(int N, int H, int W, int C, int Ho, int Wo, int KH, int KW, int stride, int dil) {
   if (KH != kDw7K || KW != kDw7K || stride != 1 || dil != 1 || C % kDw7Channels != 0 || g_tune_mma == 0) return false;
-  if ((long long)N * Ho * Wo <= 64 || (Ho <= 3 && Wo <= 8)) return false;
+  if (Ho <= 3 && Wo <= 8) return false;
+  if ((long long)N * Ho * Wo <= 64 && (long long)Ho * (C / kDw7Channels) > 72) return false;
   return (long long)N * Ho * Wo * (C / kDw7Channels) < 0xFFFFFFFFll && (long long)H * W * C < (1ll << 38) &&
          (long long)N * ((Wo + 7) / 8) * (C / kDw7Channels) * Ho < 0x7FFFFFF0ll / 2;
 }

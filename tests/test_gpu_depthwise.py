@@ -31,8 +31,10 @@ CASES += [
     (17, 9, 8, 2560, 3, False),   # 160 units of nine rows: ranges that cross from one into the next
     (96, 5, 7, 256, 3, False),    # 48 units of five rows: runs of one and two
     (3, 7, 21, 32, 3, True),      # (the fp32 kernel's tiles of 7 columns)
-    (4, 4, 4, 32, 3, False),      # 64 pixels, and on the other side of that line
-    (5, 4, 4, 32, 3, True),
+    (4, 4, 4, 608, 3, False),     # 64 pixels and 76 runs of rows, and on the other sides of that line
+    (5, 4, 4, 608, 3, True),
+    (4, 4, 4, 576, 3, False),
+    (1, 5, 12, 96, 3, True),
     (30, 3, 8, 64, 3, False),     # three rows of one window, and on the other sides of that line
     (30, 3, 9, 64, 3, False),
     (30, 4, 8, 64, 3, True),
