@@ -1632,7 +1632,9 @@ constexpr double kIssueSparse = 365.0, kIssueDense = 480.0;
 constexpr double kEpiloguePieceCycles = 900.0;
 constexpr double kCyclesPerParkedTile = 90.0;
 // What an epilogue that paces its layer takes per tile: fixed + per piece, whatever the piece's fill (a piece of 40
-// columns is processed whole).  Fitted to forced widths: GELU on two sets of groups; residual epilogues, while a
+// columns is processed whole).  Fitted to forced widths, at 1.9 GHz: GELU on one set of groups (two groups of 96 -> 384 at
+// 56 x 56, batch 128, in one launch: 80 / 160 / 240 positions 324 / 249 / 223 us) and on two (96 -> 384: 80 / 160 / 208
+// positions 114 / 93 / 105 us); residual epilogues, while a
 // thread of theirs issued the stores (128 -> 512 at 28 x 28, batch 256: 80 / 112 / 144 / 160 / 176 / 208 positions 119 / 130 /
 // 107 / 95 / 116 / 100 us: 160 positions are two whole pieces per group, 208 are three with a sixth of them empty).  With
 // store warps the order is the same where it matters: 112 / 144 / 160 / 176 / 192 / 208 positions 97 / 81 / 83 / 89 / 85 / 81 us
@@ -1640,7 +1642,8 @@ constexpr double kCyclesPerParkedTile = 90.0;
 struct EpilogueCycles {
   double tile, piece;
 };
-constexpr EpilogueCycles kEpilogueHidden = {0.0, 0.0}, kEpilogueWide = {500.0, 1775.0}, kEpilogueResidual = {1314.0, 1927.0};
+constexpr EpilogueCycles kEpilogueHidden = {0.0, 0.0}, kEpilogueGelu = {1400.0, 1610.0}, kEpilogueWide = {700.0, 1420.0},
+                           kEpilogueResidual = {1314.0, 1927.0};
 constexpr double kSplitAdvantage = 1.1;  // split only if the model predicts at least this gain
 // ... and only a deep K: the finishing kernel is a launch of its own (3 us of the caller's time, 2 to 3 us on the GPU when
 // the one before it is short).  Whole tiles against split ones, one to eight images: 8 k-blocks 4.0 / 4.8 us, 16 5.0 / 5.0
@@ -2321,11 +2324,21 @@ int32_t launch_forward_dense(const ssconv_desc_t& d, const void* x, const void* 
 // Groups of a grouped convolution in one launch: what the model says of all groups' tiles dealt out together
 // against one launch per group (each of which may split K or use pairs, and starts and drains by itself).  A group's last
 // MMA takes up to 32 (2:4) or 16 (dense) channels, which have to be its own: the neighbouring group's would meet zero
-// weights, but an infinity among them would not vanish.  64 x 14 x 14 x 256 -> 288 in 4 groups, 3 x 3: four launches
-// 25 us, one 10.8 us by events of eight calls (22.0 before).
+// weights, but an infinity among them would not vanish.  Shallow GELU layers are paced by their epilogue, which has one set
+// of groups in a launch of all and may have two in launches of their own: each side is charged the one that it would run.
+// us, one launch / one per group: 64 x 14 x 14 x 256 -> 288 in 4 groups, 3 x 3 10.8 / 22.0; GELU 128 x 56 x 56 x 192 -> 768 in
+// 2 223 / 190, 128 x 28 x 28 x 384 -> 1536 in 2 119 / 110, 128 x 56 x 56 x 96 -> 384 in 3 115 / 105; 64 x 28 x 28 x 128 -> 256 in 2
+// 15.7 / 18.0, 64 x 28 x 28 x 768 -> 768 in 4 46.5 / 62.4.
 constexpr double kLaunchCycles = 4000.0;
 template <bool SPARSE>
-static bool groups_in_one_launch(const ssconv_desc_t& g, int groups) {
+static double grouped_cost(const ssconv_desc_t& g, long long Q, const Geometry& geo, int workers, bool together, bool have_ws) {
+  const Plan plan = together ? choose_plan<SPARSE>(g, Q, geo, workers, false, false, false, false)
+                             : choose_plan<SPARSE>(g, Q, geo, workers, false, have_ws);
+  if (plan.wide || activation_of(g.flags) != kActGelu || geo.kblocks > kWideMaxKBlocks) return plan.cost;
+  return plan_layer<SPARSE>(Q, geo, workers, false, kBN, 2, false, kEpilogueGelu).cost;
+}
+template <bool SPARSE>
+static bool groups_in_one_launch(const ssconv_desc_t& g, int groups, bool have_ws) {
   if (groups < 2 || g.C_in % (SPARSE ? 32 : 16) != 0) return false;
   int dev = 0;
   if (current_device(&dev) != SSCONV_OK) return false;
@@ -2333,9 +2346,9 @@ static bool groups_in_one_launch(const ssconv_desc_t& g, int groups) {
   const long long Q = (long long)g.N * out_extent(g.H, g.KH, g.stride_h, g.pad_h, g.dil_h) *
                       out_extent(g.W, g.KW, g.stride_w, g.pad_w, g.dil_w);
   Geometry geo = layer_geometry(g, SPARSE);
-  const double each = choose_plan<SPARSE>(g, Q, geo, workers, false).cost;
+  const double each = grouped_cost<SPARSE>(g, Q, geo, workers, false, have_ws);
   geo.m_tiles *= groups;
-  return choose_plan<SPARSE>(g, Q, geo, workers, false, false, false, false).cost <= groups * each + (groups - 1) * kLaunchCycles;
+  return grouped_cost<SPARSE>(g, Q, geo, workers, true, have_ws) <= groups * each + (groups - 1) * kLaunchCycles;
 }
 
 // Grouped convolution: `groups` independent convolutions on channel slices, group g reading input
@@ -2352,7 +2365,8 @@ int32_t launch_forward_grouped(const ssconv_desc_t& d, int groups, bool sparse, 
   const size_t w_step = sparse ? (size_t)geo.Mp * geo.KC * 2 : (size_t)g.C_out * geo.taps * g.C_in * 2;
   const size_t m_step = (size_t)geo.m_tiles * geo.stages * kMetaImageBytes;
   const int64_t xs[3] = {d.C_in, (int64_t)d.W * d.C_in, (int64_t)d.H * d.W * d.C_in};
-  const bool together = sparse ? groups_in_one_launch<true>(g, groups) : groups_in_one_launch<false>(g, groups);
+  const bool have_ws = ws != nullptr && ws_bytes >= workspace_bytes();
+  const bool together = sparse ? groups_in_one_launch<true>(g, groups, have_ws) : groups_in_one_launch<false>(g, groups, have_ws);
   for (int i = 0; i < (together ? 1 : groups); ++i) {
     const char* xg = static_cast<const char*>(x) + (size_t)i * g.C_in * 2;
     char* yg = static_cast<char*>(y) + (size_t)i * g.C_out * 2;

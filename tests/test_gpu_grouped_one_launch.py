@@ -1,6 +1,8 @@
 """All channel groups in one launch: against one launch per group on the same slices (bit for bit where both walk whole
 tiles of the same width order, so within the oracle's tolerance in general), at group widths on both sides of the
 rule, ragged output channels and several channel tiles per group; and infinities stay in their group."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -69,3 +71,39 @@ def test_an_infinite_pixel_stays_in_its_group(case):
     y, _ = _run(case, x.to(DEV), w.to(DEV), bias.to(DEV))
     assert torch.equal(y[..., :co], clean[..., :co]) and torch.equal(y[..., 2 * co:], clean[..., 2 * co:])
     assert not bool(torch.isfinite(y[..., co:2 * co].float()).all())
+
+
+PLANS = [  # N, H, C_in, C_out, groups, K, act, workspace, launches (2:4)
+    (32, 56, 192, 768, 2, 1, "gelu", True, 2),        # paced by the epilogue: two sets of epilogue groups in each launch
+    (32, 56, 192, 768, 2, 1, "relu", True, 1),
+    (16, 28, 128, 256, 2, 1, "gelu", True, 1),        # too few tiles to make up for a launch
+    (1, 7, 2048, 2048, 2, 3, "none", True, 4),        # K split in each launch, and a finishing kernel
+    (1, 7, 2048, 2048, 2, 3, "none", False, 1),       # no scratch, no split: all groups' tiles together
+]
+
+
+@pytest.mark.parametrize("plan", PLANS, ids=[f"{p[0]}x{p[1]}_{p[2]}to{p[3]}_g{p[4]}_{p[6]}_{'ws' if p[7] else 'no_ws'}" for p in PLANS])
+def test_launches_of_a_grouped_layer(plan):
+    N, H, ci, co, groups, K, act, with_ws, launches = plan
+    g = torch.Generator(device=DEV).manual_seed(synth.SEED_BASE + 7600)
+    x = torch.randn((N, H, H, ci), generator=g, device=DEV).to(torch.bfloat16)
+    w = (torch.randn((co, K, K, ci // groups), generator=g, device=DEV) / (K * K * ci / groups) ** 0.5).to(torch.bfloat16)
+    desc = api.make_desc(N, H, H, ci, co, K, K, 1, K // 2, bias=False, relu=act == "relu", gelu=act == "gelu")
+    pat = api.ssconv_select_mask(api.MASK_MAGNITUDE_BF16, w, w.numel() // 4)
+    w_comp, meta = api.ssconv_compress_grouped(desc, groups, w, pat)
+    y = torch.empty((N, H, H, co), dtype=torch.bfloat16, device=DEV)
+    ws = api.default_workspace(x.device)
+    c0 = api.ssconv_launch_count()
+    rc = api.lib().ssconv_forward_grouped(ctypes.byref(desc), groups, x.data_ptr(), w_comp.data_ptr(), meta.data_ptr(), None, y.data_ptr(),
+                                          ws.data_ptr() if with_ws else None, ws.numel() if with_ws else 0, None, None)
+    assert rc == api.OK and api.ssconv_launch_count() - c0 == launches
+    torch.cuda.synchronize()
+    # each group as a layer of its own on a copy of its channels
+    ci_g, co_g = ci // groups, co // groups
+    one = api.make_desc(N, H, H, ci_g, co_g, K, K, 1, K // 2, bias=False, relu=act == "relu", gelu=act == "gelu")
+    for i in range(groups):
+        wi = w[i * co_g:(i + 1) * co_g].contiguous()
+        comp = api.ssconv_compress(one, wi, api.ssconv_select_mask(api.MASK_MAGNITUDE_BF16, wi, wi.numel() // 4))
+        ref = api.ssconv_forward(one, x[..., i * ci_g:(i + 1) * ci_g].contiguous(), *comp).float()
+        err = (y[..., i * co_g:(i + 1) * co_g].float() - ref).abs()
+        assert bool((err <= 2.0 ** -7 * ref.abs() + 1e-3).all())   # (K split or not: another order of summation)
