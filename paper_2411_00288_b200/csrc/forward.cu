@@ -66,10 +66,13 @@ constexpr int kPiece = 40;               // positions per epilogue piece (one st
 constexpr int kFirstExtraProducerWarp = 2 + 4 * kGroups;  // warps 10 and 11: two more TMA producers
 constexpr int kThreads = 64 + 128 * kGroups + 64;
 // With `sets` sets of epilogue groups (one-block kernel; see kWideMaxKBlocks) the producers follow the last group.
-// Two more warps follow those in the forms with store warps, one per half of a tile's positions.
-__host__ __device__ constexpr bool has_store_warps(bool residual, int sets) { return residual || sets == 2; }
-__host__ __device__ constexpr int threads_with(int sets, bool residual) {
-  return 64 + 128 * kGroups * sets + 64 + (has_store_warps(residual, sets) ? 32 * kGroups : 0);
+// Two more warps follow those in the forms with store warps, one per half of a tile's positions: with two sets, and with a
+// residual unless a block has one tile at most (one_tile; see the epilogue).
+__host__ __device__ constexpr bool has_store_warps(bool residual, int sets, bool one_tile) {
+  return (residual && !one_tile) || sets == 2;
+}
+__host__ __device__ constexpr int threads_with(int sets, bool residual, bool one_tile) {
+  return 64 + 128 * kGroups * sets + 64 + (has_store_warps(residual, sets, one_tile) ? 32 * kGroups : 0);
 }
 __host__ __device__ constexpr int first_extra_producer_with(int sets) { return 2 + 4 * kGroups * sets; }
 constexpr int kPairStoreWarp = kFirstExtraProducerWarp + 2;  // pair kernel with a residual: warps 12 and 13 issue the stores
@@ -197,6 +200,25 @@ struct PieceAhead {
     return true;
   }
 };
+
+// Bring one piece of the residual tensor into a staging buffer (one thread): `bar` completes when it has landed.
+__device__ __forceinline__ void load_residual_piece(const FwdParams& p, const CUtensorMap* tm_r, const CUtensorMap* tm_r_tail, int tile,
+                                                    int piece, int col_base, uint32_t dst, uint32_t bar) {
+  const int pt = tile / p.m_tiles;
+  const int m = tile - pt * p.m_tiles;
+  const int q_piece = pt * p.BN + col_base + piece * kPiece;
+  if (q_piece >= p.Q) {  // nothing of this piece is stored: only keep the barrier's phases in step
+    mbar_arrive_a(bar);
+    return;
+  }
+  const bool tail = (piece == p.pieces - 1 && p.tail_cols != kPiece);
+  const CUtensorMap* map = tail ? tm_r_tail : tm_r;
+  const uint32_t half_bytes = (uint32_t)(tail ? p.tail_cols : kPiece) * 128u;
+  const bool two = m * kTileM + 64 < p.C_out;
+  mbar_expect_tx_a(bar, two ? 2u * half_bytes : half_bytes);
+  tma_load_2d_a(dst, map, bar, m * kTileM, q_piece);
+  if (two) tma_load_2d_a(dst + kHalfPieceBytes, map, bar, m * kTileM + 64, q_piece);
+}
 
 // CTA that owns work unit u under that dealing: inverse of start(c) = c q + min(c, r).
 __device__ __forceinline__ int unit_owner(uint32_t u, uint32_t q, uint32_t r) {
@@ -496,8 +518,9 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
 // epilogue loop carries none of that code).  EPI_SETS: sets of epilogue groups; with two, each serves one of the
 // two accumulators, i.e. every other tile.  GROUPED: several channel groups in one launch (an instantiation of its own: as
 // run-time branches its few instructions cost the issuing lane of the plain epilogue 5 % on write-bound layers).
-template <bool SPARSE, bool RES, bool FP8 = false, int EPI_SETS = 1, bool GROUPED = false>
-__global__ void __launch_bounds__(threads_with(EPI_SETS, RES), 1)
+// ONE_TILE: a block has one tile at most, all of whose residual pieces are brought in at its start.
+template <bool SPARSE, bool RES, bool FP8 = false, int EPI_SETS = 1, bool GROUPED = false, bool ONE_TILE = false>
+__global__ void __launch_bounds__(threads_with(EPI_SETS, RES, ONE_TILE), 1)
 ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                   const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_y_tail,
                   const __grid_constant__ CUtensorMap tm_r, const __grid_constant__ CUtensorMap tm_r_tail,
@@ -506,8 +529,9 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
   static_assert(!(FP8 && RES), "the residual epilogue is not built for 8-bit operands");
   static_assert(!GROUPED || (!RES && EPI_SETS == 1), "channel groups: the plain epilogue");
   static_assert(EPI_SETS == 1 || (EPI_SETS == 2 && !RES), "one set of epilogue groups, or one per accumulator");
-  constexpr int kThreadsHere = threads_with(EPI_SETS, RES), kExtraProducer = first_extra_producer_with(EPI_SETS);
-  constexpr bool kStoreWarps = has_store_warps(RES, EPI_SETS);
+  static_assert(!ONE_TILE || (RES && EPI_SETS == 1 && !GROUPED), "one tile per block: the residual epilogue");
+  constexpr int kThreadsHere = threads_with(EPI_SETS, RES, ONE_TILE), kExtraProducer = first_extra_producer_with(EPI_SETS);
+  constexpr bool kStoreWarps = has_store_warps(RES, EPI_SETS, ONE_TILE);
   constexpr int kStoreWarp = kExtraProducer + 2;
 
   extern __shared__ uint8_t smem_raw[];
@@ -769,6 +793,14 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
     uint32_t piece_count = 0;
     bool ok = true;
     grid_dependency_wait();  // before the first access to global memory (bias, scratch, output)
+    if (ONE_TILE && leader) {  // (at most as many pieces as buffers)
+      WorkIter first(p);
+      Segment its;
+      if (first.next(its))
+        for (int piece = 0; piece < p.pieces; ++piece)
+          load_residual_piece(p, &tm_r, &tm_r_tail, its.tile, piece, col_base, smem_u32(my_stage + piece * kPieceBytes),
+                              smem_u32(&bar_res[4 * grp + piece]));
+    }
     WorkIter work(p);
     Segment seg;
     for (; work.next(seg); ++tcount) {
@@ -849,8 +881,11 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
           for (int i = 0; i < kPiece; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * p.out_scale);
         }
         if (RES) {
-          // the residual piece has landed in this buffer
-          if (!mbar_wait_warp(&bar_res[4 * grp + sbuf], (piece_count >> nbuf_shift) & 1u, abort_flag, kWaitLimitCycles)) {
+          // the residual piece has landed in this buffer (without store warps a group whose wait runs out still meets at
+          // its barrier and stops at the next tile)
+          const bool landed =
+              mbar_wait_warp(&bar_res[4 * grp + sbuf], (piece_count >> nbuf_shift) & 1u, abort_flag, kWaitLimitCycles);
+          if (kStoreWarps && !landed) {
             ok = false;
             break;
           }
@@ -874,7 +909,7 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
           continue;
         }
         // The next piece overwrites the other buffer: its store (the previous piece's) must have read it.
-        if (leader) bulk_wait_group_read0();
+        if (!ONE_TILE && leader) bulk_wait_group_read0();
         epilogue_bar_sync(grp);
         if (leader) {
           const int q_piece = pt * p.BN + col_base + piece * kPiece;
@@ -908,8 +943,10 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
     // 512 at 28 x 28 91 -> 81, 256 -> 1024 at 14 x 14 51 -> 45, 512 -> 2048 at 7 x 7 33 -> 30.5; GELU on two sets 98 -> 92 (96
     // -> 384, batch 128).  Plain one-set epilogues gain 2 % where the output stream paces them (64 -> 256 91 -> 89)
     // and lose 1 to 4 % elsewhere (3 x 3 64 -> 64 88 -> 90, 27 images 13.8 -> 14.3): they keep their leader, as do
-    // pairs without a residual.  Residual layers of few tiles pay about 0.3 us for the longer way of their last pieces
-    // (8 x 28 x 28 x 256, 3 x 3: 10.6 -> 10.9); sleeping instead of polling in the store warps changes nothing.
+    // pairs without a residual.  A block with a single tile has nothing to gain and pays for the longer way of its last
+    // pieces, so that residual layers of one tile per block keep the leader too (ONE_TILE; us, store warps / leader:
+    // 1 x 56 x 56 x 64 -> 256 4.25 / 3.95, 4 x 28 x 28 x 64, 3 x 3 4.8 / 4.45, 8 x 28 x 28 x 256, 3 x 3 11.1 / 10.8; two tiles
+    // per block 5 x 56 x 56 x 64 -> 256 6.95 / 7.25).  Sleeping instead of polling in the store warps changes nothing.
     // With two sets it serves both, tile by tile: their tiles alternate, and a set's buffers hold what it finishes
     // meanwhile.
     const int half = warp - kStoreWarp;
@@ -928,22 +965,8 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       int tile_a, piece_a;
       if (!ahead.next(tile_a, piece_a)) return;  // no such piece: nobody will wait for it
       const uint32_t b = count & (nbuf - 1u);
-      const uint32_t bar = smem_u32(&bar_res[4 * grp + b]);
-      const int pt_a = tile_a / p.m_tiles;
-      const int m_a = tile_a - pt_a * p.m_tiles;
-      const int q_piece = pt_a * p.BN + col_base + piece_a * kPiece;
-      if (q_piece >= p.Q) {  // nothing of this piece is stored: only keep the barrier's phases in step
-        mbar_arrive_a(bar);
-        return;
-      }
-      const bool tail = (piece_a == p.pieces - 1 && p.tail_cols != kPiece);
-      const CUtensorMap* map = tail ? &tm_r_tail : &tm_r;
-      const uint32_t half_bytes = (uint32_t)(tail ? p.tail_cols : kPiece) * 128u;
-      const bool two = m_a * kTileM + 64 < p.C_out;
-      const uint32_t dst = smem_u32(my_stage + b * kPieceBytes);
-      mbar_expect_tx_a(bar, two ? 2u * half_bytes : half_bytes);
-      tma_load_2d_a(dst, map, bar, m_a * kTileM, q_piece);
-      if (two) tma_load_2d_a(dst + kHalfPieceBytes, map, bar, m_a * kTileM + 64, q_piece);
+      load_residual_piece(p, &tm_r, &tm_r_tail, tile_a, piece_a, col_base, smem_u32(my_stage + b * kPieceBytes),
+                          smem_u32(&bar_res[4 * grp + b]));
     };
     if (RES)
       for (uint32_t c = 0; c < nbuf; ++c) load_residual(c);
@@ -1988,6 +2011,9 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
                               : cudaFuncSetAttribute(ssconv_fwd_kernel<SPARSE, false>,
                                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemBytes);
     if (e != cudaSuccess) return SSCONV_ERR_CUDA;
+    if (res && cudaFuncSetAttribute(ssconv_fwd_kernel<SPARSE, true, false, 1, false, true>,
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemBytes) != cudaSuccess)
+      return SSCONV_ERR_CUDA;
     g_attr_set[dev][SPARSE ? 1 : 0][res] = true;
   }
   if (!FP8 && !g_wide_attr_set[dev][SPARSE ? 1 : 0]) {
@@ -2253,7 +2279,9 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   // waits for that kernel's completion before it touches global memory.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)(pair ? pair_threads(residual != nullptr) : threads_with(wide_epilogue ? 2 : 1, residual != nullptr)));
+  const bool one_tile = residual != nullptr && !pair && p.split == 0 && p.num_tiles <= workers;
+  cfg.blockDim = dim3((unsigned)(pair ? pair_threads(residual != nullptr)
+                                      : threads_with(wide_epilogue ? 2 : 1, residual != nullptr, one_tile)));
   cfg.dynamicSmemBytes = smem_bytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -2273,6 +2301,9 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
           ? cudaLaunchKernelEx(&cfg, ssconv_fwd_pair_kernel<SPARSE, false, true>, tm_a, tm_b, tm_meta, tm_y, tm_y_tail, tm_r,
                                tm_r_tail, p)
       : pair ? cudaLaunchKernelEx(&cfg, ssconv_fwd_pair_kernel<SPARSE>, tm_a, tm_b, tm_meta, tm_y, tm_y_tail, tm_r, tm_r_tail, p)
+      : one_tile
+          ? cudaLaunchKernelEx(&cfg, ssconv_fwd_kernel<SPARSE, true, false, 1, false, true>, tm_a, tm_b, tm_y, tm_y_tail, tm_r, tm_r_tail,
+                               p)
       : residual != nullptr
           ? cudaLaunchKernelEx(&cfg, ssconv_fwd_kernel<SPARSE, true>, tm_a, tm_b, tm_y, tm_y_tail, tm_r, tm_r_tail, p)
       : groups > 1
