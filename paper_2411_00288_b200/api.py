@@ -160,14 +160,26 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
+def _raw_stream_functions(module):
+    """(current raw stream of a device, current device) of a torch extension module, or None where this torch has not both:
+    they are not public names."""
+    names = ("_cuda_getCurrentRawStream", "_cuda_getDevice")
+    found = tuple(getattr(module, n, None) for n in names)
+    return None if None in found else found
+
+
+_RAW = _raw_stream_functions(torch._C)
+
+
 def _stream(stream=None):
     """The raw handle of a stream, or of the current device's current one (without a Stream object around it, which
-    takes 3 us to make)."""
+    takes 3 us to make, where torch lets one)."""
     if stream is not None:
         return stream.cuda_stream
-    if not torch.cuda.is_initialized():
+    if _RAW is None or not torch.cuda.is_initialized():
         return torch.cuda.current_stream().cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    current, device = _RAW
+    return current(device())
 
 
 def _need_cuda(*tensors):

@@ -75,3 +75,17 @@ def test_host_detectable_errors_return_before_any_launch(lib):
     assert lib.ssconv_forward(ctypes.byref(nob), 8, 16, 16, None, 16, None, 0, None, None) == 4
     # bias flag set but no bias
     assert lib.ssconv_forward(p, 16, 16, 16, None, 16, None, 0, None, None) == 1
+
+
+def test_current_stream_by_public_names(monkeypatch):
+    # (a torch without the two private functions behind the quick way)
+    import types
+
+    import torch
+    assert api._raw_stream_functions(types.SimpleNamespace()) is None
+    assert api._raw_stream_functions(types.SimpleNamespace(_cuda_getDevice=int)) is None
+    monkeypatch.setattr(api, "_RAW", None)
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=77))
+    assert api._stream() == 77
+    assert api._stream(types.SimpleNamespace(cuda_stream=5)) == 5
