@@ -147,3 +147,30 @@ def test_depthwise7_sums_are_as_exact_as_fp32_ones(data):
     # the sampling of a quarter as many)
     assert float(err.pow(2).mean().sqrt()) <= 1.025 * {"normal": 0.163, "spread": 0.744, "positive": 0.801}[data]
     assert abs(float(err.mean())) <= 0.3
+
+
+@pytest.mark.parametrize("relu", [False, True], ids=["none", "relu"])
+@pytest.mark.parametrize("with_bias", [False, True], ids=["no_bias", "bias"])
+def test_depthwise7_non_finite_outputs_are_those_of_the_fp32_kernel(relu, with_bias):
+    N, H, W, C = 3, 22, 25, 64
+    g = torch.Generator(device=DEV).manual_seed(synth.SEED_BASE + 7250)
+    x = torch.randn((N, H, W, C), generator=g, device=DEV).to(torch.bfloat16)
+    w = (torch.randn((7, 7, C), generator=g, device=DEV) / 7).to(torch.bfloat16)
+    bias = torch.randn(C, generator=g, device=DEV) if with_bias else None
+    for n, h, c0, c, v in [(0, 5, 6, 3, float("inf")), (0, 6, 9, 3, float("-inf")), (1, 10, 0, 7, float("nan")), (2, 21, 24, 40, float("-inf")),
+                           (1, 3, 3, 8, 3.0e38), (1, 3, 4, 8, 3.0e38)]:
+        x[n, h, c0, c] = v
+    desc = api.make_desc(N, H, W, C, C, 7, 7, 1, 3, bias=with_bias, relu=relu)
+    y = api.ssconv_depthwise(desc, x, w, bias)
+    api.ssconv_tune(api.TUNE_DEPTHWISE_MMA, 0)
+    try:
+        ref = api.ssconv_depthwise(desc, x, w, bias)
+    finally:
+        api.ssconv_tune(api.TUNE_DEPTHWISE_MMA, -1)
+    assert torch.equal(torch.isnan(y), torch.isnan(ref)) and torch.equal(y == float("inf"), ref == float("inf"))
+    assert torch.equal(y == float("-inf"), ref == float("-inf")) and not bool(torch.isfinite(ref).all())
+    fin = torch.isfinite(ref)
+    # (one bf16 rounding apart; the sums that meet 3e38 have lost everything below 2^-24 of it)
+    near = fin.clone()
+    near[1, :8, :9, 8] = False
+    assert bool(((y.float() - ref.float()).abs()[near] <= 2.0 ** -7 * ref.float().abs()[near] + 1e-5).all())

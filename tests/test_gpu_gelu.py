@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 import torch
 
-from oracle import blocks
+from oracle import blocks, masks
 from oracle.conv import ConvShape
 from paper_2411_00288_b200 import api, synth
 from tests import parity
@@ -87,16 +87,28 @@ def test_two_epilogue_sets_match_oracle(layer, width):
         api.ssconv_tune(api.TUNE_TILE_POSITIONS, 0)
 
 
-def test_two_epilogue_sets_on_channel_slices():
-    N, H, W, ci, co, groups = 4, 90, 77, 64, 288, 2
+@pytest.mark.parametrize("sparse,ci_g,co_g", [(False, 32, 144), (False, 24, 144), (True, 40, 136)], ids=["one_launch", "dense", "sparse"])
+def test_two_epilogue_sets_on_channel_slices(sparse, ci_g, co_g):
+    # 24 and 40 channels per group: the last MMA would reach into the next group, so that every group is a launch of its own, on
+    # strided views and with two sets of epilogue groups (350 tiles); 32 dense ones go in one launch with one set
+    N, H, W, groups = 4, 90, 77, 2
+    ci, co = groups * ci_g, groups * co_g
     g = torch.Generator().manual_seed(synth.SEED_BASE + 7300)
     x = torch.randn((N, H, W, ci), generator=g).to(torch.bfloat16)
-    w = (torch.randn((co, 1, 1, ci // groups), generator=g) / (ci // groups) ** 0.5).to(torch.bfloat16)
+    w = (torch.randn((co, 1, 1, ci_g), generator=g) / ci_g ** 0.5).to(torch.bfloat16)
     bias = torch.randn((co,), generator=g) * 0.1
     desc = api.make_desc(N, H, W, ci, co, 1, 1, bias=True, gelu=True)
-    y = api.ssconv_forward_dense_grouped(desc, groups, x.to(DEV), w.to(DEV), bias.to(DEV))
+    mask = None
+    if sparse:
+        pat = api.ssconv_select_mask(api.MASK_MAGNITUDE_BF16, w.to(DEV), w.numel() // 4)
+        comp = api.ssconv_compress_grouped(desc, groups, w.to(DEV), pat)
+        mask = masks.mask_from_pattern(masks.select_from_magnitude(synth.bf16_bits(w)), tuple(w.shape))
+    c0 = api.ssconv_launch_count()
+    y = (api.ssconv_forward_grouped(desc, groups, x.to(DEV), *comp, bias.to(DEV)) if sparse else
+         api.ssconv_forward_dense_grouped(desc, groups, x.to(DEV), w.to(DEV), bias.to(DEV)))
+    assert api.ssconv_launch_count() - c0 == (1 if ci_g == 32 else groups)
     torch.cuda.synchronize()
     shape = ConvShape(N, H, W, ci, co, 1, 1, (1, 1), (0, 0), (1, 1), relu=False)
-    ref = parity.gelu_f64(blocks.grouped_conv2d_f64(shape, groups, synth.bf16_bits(x), synth.bf16_bits(w), bias=bias.numpy()))
+    ref = parity.gelu_f64(blocks.grouped_conv2d_f64(shape, groups, synth.bf16_bits(x), synth.bf16_bits(w), mask=mask, bias=bias.numpy()))
     rel, mx = parity.errors(parity.bf16_tensor_to_f64(y), ref)
     assert rel <= parity.REL_FRO_TOL and mx <= parity.MAX_ABS_TOL, (rel, mx)

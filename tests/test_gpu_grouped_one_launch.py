@@ -24,6 +24,9 @@ CASES = [  # N, H, W, C_in per group, C_out per group, K, stride, pad, groups, s
     (3, 14, 14, 16, 72, 3, 1, 1, 3, False, "relu", True),
     (7, 30, 28, 80, 200, 3, 1, 1, 2, False, "gelu", True),
     (2, 9, 9, 24, 48, 3, 1, 1, 3, False, "relu", False),
+    # a full k-block followed by one that is partly the group's own
+    (4, 28, 28, 96, 264, 1, 1, 0, 4, True, "relu", True),
+    (7, 30, 28, 80, 200, 3, 1, 1, 2, False, "none", True),
 ]
 
 
