@@ -9,12 +9,13 @@ The reported value is dense-equivalent TFLOP/s (2*P*C_out*K per convolution, the
 its 3 real input channels) over all ranks; images per second, the dense counterpart, a per-layer
 table with each layer's roofline, the end-to-end figure with host buffers, the CPU oracle and
 short summaries of the three per-layer sweeps (ResNet-18 3x3 sweep, ResNet-50 bottleneck layers,
-ConvNeXt-T point-wise layers) ride in the same JSON line.
+ConvNeXt-T point-wise layers) are in the report.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                     [--workload-config 2|3|4|5] [--train]
 
-Prints exactly one JSON line on rank 0.  With --gpus N > 1 and no torchrun environment it starts N
+Prints exactly one JSON line on rank 0 (the figures, under 2000 characters) and the whole report, tables included, to
+standard error.  With --gpus N > 1 and no torchrun environment it starts N
 ranks itself (one per GPU; the ranks share nothing but the timing barrier).
 """
 from __future__ import annotations
@@ -84,6 +85,33 @@ def spread(values):
     n = len(v)
     return {"median": statistics.median(v), "min": v[0], "max": v[-1], "p10": v[int(0.1 * (n - 1))],
             "p90": v[int(round(0.9 * (n - 1)))], "regions": n}
+
+
+# ----------------------------------------------------------------------------- the line
+KEPT = {"config": ("workload", "layers", "batch_per_gpu", "l2"),
+        "roofline": ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic", "peak_source"),
+        "cpu_baseline": ("value", "unit", "cores", "kind", "sample"),
+        "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step"),
+        "clocks": None, "ms_per_step_spread": ("min", "max", "regions")}
+
+
+def short_line(line):
+    """The line's figures without the tables and explanations, short enough for a log that keeps a few thousand characters."""
+    def rounded(v):
+        return float(f"{v:.6g}") if isinstance(v, float) else v[:120] if isinstance(v, str) else v
+    out = {}
+    for key, v in line.items():
+        if not isinstance(v, (dict, list)):
+            out[key] = v
+        elif key in KEPT and isinstance(v, dict):
+            out[key] = {k: rounded(x) for k, x in v.items() if KEPT[key] is None or k in KEPT[key]}
+    return out
+
+
+def print_line(line):
+    """The whole report to standard error, its figures as the one JSON line of standard output."""
+    print(json.dumps({"report": line}), file=sys.stderr, flush=True)
+    print(json.dumps(short_line(line)), flush=True)
 
 
 # ----------------------------------------------------------------------------- clocks
@@ -964,7 +992,7 @@ def stack_arm(args):
         line.update(summaries)
         if cpu is not None:
             line["cpu_baseline"] = cpu
-        print(json.dumps(line))
+        print_line(line)
     if distributed:
         dist.destroy_process_group()
 
@@ -1127,7 +1155,7 @@ def sweep_arm(args):
         }
         if cpu is not None:
             line["cpu_baseline"] = cpu
-        print(json.dumps(line))
+        print_line(line)
     if distributed:
         dist.destroy_process_group()
 
