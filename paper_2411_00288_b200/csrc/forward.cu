@@ -810,7 +810,9 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       const uint32_t aph = (tcount >> 1) & 1u;
       // (two sets: each serves one accumulator, so that it has two tiles' time for its tiles)
       if (EPI_SETS == 2 && buf != (uint32_t)(grp / kGroups)) continue;
-      const bool got = mbar_wait_warp(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
+      // (without store warps the leader's answer counts, below)
+      const bool got = kStoreWarps ? mbar_wait_warp(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64)
+                                   : mbar_wait_bounded(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
       if (kStoreWarps) {
         if (!got) break;
       } else {
@@ -1440,7 +1442,8 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
       const int m = 2 * (seg.tile - pu * p.m_tiles) + (int)rank;
       const uint32_t buf = p.dual ? t : (icount & 1u);
       const uint32_t aph = p.dual ? (icount & 1u) : ((icount >> 1) & 1u);
-      const bool got = mbar_wait_warp(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
+      const bool got = RES ? mbar_wait_warp(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64)
+                           : mbar_wait_bounded(&bar_acc_full[buf], aph, abort_flag, kWaitLimitCycles, 64);
       if (!RES) {
         if (leader) my_go[tcount & 1u] = (got && *abort_flag == 0) ? 1 : 0;
         epilogue_bar_sync(grp);

@@ -78,7 +78,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 
 // The same for a warp that goes on in lock step (tcgen05, ldmatrix, stmatrix, elect and the like take all 32 lanes):
 // one verdict for the whole warp.  Lanes poll the barrier and read the flag each for itself, so that around the limit
-// some may find the phase complete and others the flag raised.  The votes are not to be seen in any layer's time.
+// some may find the phase complete and others the flag raised.  Costs 0 to 0.6 % of a layer's time.
 __device__ __forceinline__ bool mbar_wait_warp_a(uint32_t bar_addr, uint32_t parity, volatile int* abort_flag,
                                                  long long limit_cycles, uint32_t backoff_ns = 0) {
   if (__all_sync(0xFFFFFFFFu, mbar_spin_a(bar_addr, parity, kFastSpins))) return true;
