@@ -92,7 +92,7 @@ KEPT = {"config": ("workload", "layers", "batch_per_gpu", "l2"),
         "roofline": ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic", "peak_source"),
         "cpu_baseline": ("value", "unit", "cores", "kind", "sample"),
         "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step"),
-        "clocks": None, "ms_per_step_spread": ("min", "max", "regions")}
+        "clocks": ("sm_mhz", "sm_max_mhz", "samples_under_load", "reasons"), "ms_per_step_spread": ("min", "max", "regions")}
 
 
 def short_line(line):
@@ -104,7 +104,7 @@ def short_line(line):
         if not isinstance(v, (dict, list)):
             out[key] = v
         elif key in KEPT and isinstance(v, dict):
-            out[key] = {k: rounded(x) for k, x in v.items() if KEPT[key] is None or k in KEPT[key]}
+            out[key] = {k: rounded(x) for k, x in v.items() if k in KEPT[key]}
     return out
 
 

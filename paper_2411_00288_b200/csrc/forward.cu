@@ -18,9 +18,9 @@
 //
 // Warp roles: warps 0, 10 and 11 TMA producers (one thread each: the activations of a group's
 // first k-block, of its second, the weights), warp 1 MMA issuer (one thread; owns TMEM), warps 2-9
-// epilogue in two groups of four warps that each own half of a tile's positions; where a residual is added
-// or a tile's two accumulators have epilogue groups of their own, two more warps (one thread each) issue the
-// output's stores.  The accumulator
+// epilogue in two groups of four warps that each own half of a tile's positions; where a residual is added (and a
+// block has more than one tile) or the two accumulators have epilogue groups of their own, two more warps (one
+// thread each) issue the output's stores.  The accumulator
 // has channels on TMEM lanes and positions on columns, NHWC wants the transpose: the epilogue reads
 // TMEM in the MMA-fragment layout (tcgen05.ld 16x256b), adds the bias, converts pairs to bf16
 // (with ReLU in the conversion), and stmatrix.trans writes 8x8 blocks transposed into a 128-byte
@@ -202,8 +202,8 @@ struct PieceAhead {
 };
 
 // Bring one piece of the residual tensor into a staging buffer (one thread): `bar` completes when it has landed.
-__device__ __forceinline__ void load_residual_piece(const FwdParams& p, const CUtensorMap* tm_r, const CUtensorMap* tm_r_tail, int tile,
-                                                    int piece, int col_base, uint32_t dst, uint32_t bar) {
+__device__ __forceinline__ void load_residual_piece(const FwdParams& p, const CUtensorMap* tm_r, const CUtensorMap* tm_r_tail,
+                                                    int tile, int piece, int col_base, uint32_t dst, uint32_t bar) {
   const int pt = tile / p.m_tiles;
   const int m = tile - pt * p.m_tiles;
   const int q_piece = pt * p.BN + col_base + piece * kPiece;
@@ -873,7 +873,8 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
         // its source has landed, below; without store warps: the leader saw that store finish reading before it
         // entered the barrier of the previous piece).
         if (kStoreWarps && !RES &&
-            !mbar_wait_warp(&bar_stage_free[nbuf * grp + sbuf], ((piece_count >> nbuf_shift) & 1u) ^ 1u, abort_flag, kWaitLimitCycles)) {
+            !mbar_wait_warp(&bar_stage_free[nbuf * grp + sbuf], ((piece_count >> nbuf_shift) & 1u) ^ 1u, abort_flag,
+                            kWaitLimitCycles)) {
           ok = false;
           break;
         }
@@ -1669,7 +1670,8 @@ constexpr double kCyclesPerParkedTile = 90.0;
 struct EpilogueCycles {
   double tile, piece, position;
 };
-constexpr EpilogueCycles kEpilogueHidden = {0.0, 0.0, 0.0}, kEpilogueGelu = {1400.0, 1610.0, 0.0}, kEpilogueWide = {700.0, 1420.0, 0.0};
+constexpr EpilogueCycles kEpilogueHidden = {0.0, 0.0, 0.0}, kEpilogueGelu = {1400.0, 1610.0, 0.0},
+                         kEpilogueWide = {700.0, 1420.0, 0.0};
 constexpr int kStreamTiles = 4;
 constexpr double kMemoryBytesPerCycle = 22.9;  // of an SM: 6.45 TB/s, 148 SMs, 1.9 GHz
 // (an output and a residual element per position and channel, and the layer's input once, over its channel tiles)
@@ -1928,7 +1930,8 @@ static int widest_tile(uint32_t a_group_bytes, int stage_bufs) {
 // shallow layer is bound by its epilogue, whose eight warps wait on one another's arithmetic, on TMEM and on the
 // staging buffers more than they issue (48 % of the issue slots used, no pipe above 44 %).  Taken for GELU layers of
 // at most six k-blocks whose tiles give every CTA more than one (a CTA with a single tile has no work for the
-// second set).  Measured (us, one set -> two, layers of n x h x h x c_in -> c_out): 128 x 56 x 56 x 96 -> 384
+// second set).  Measured with the GELU and the stores of the time (us, one set -> two, layers of n x h x h x c_in -> c_out;
+// the first now takes 92.7, and two of it as groups of one launch, on one set, 223 instead of 189): 128 x 56 x 56 x 96 -> 384
 // 113 -> 98, 128 x 28 x 28 x 192 -> 768 62.5 -> 56.3, 128 x 14 x 14 x 384 -> 1536 38.9 -> 35.3, 64 x 56 x 56 x 64 ->
 // 64 25.1 -> 21.5; beyond the line 8 k-blocks 14.8 -> 14.8, 12 19.4 -> 19.9, 16 26.6 -> 27.1, and one tile per CTA
 // (3 x 14 x 14 x 384 -> 1536) 6.1 -> 6.6.  Without GELU the layers are bound by their output stream: no gain (64 ->
