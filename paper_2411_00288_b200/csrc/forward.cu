@@ -1659,30 +1659,23 @@ constexpr double kIssueSparse = 365.0, kIssueDense = 480.0;
 constexpr double kEpiloguePieceCycles = 900.0;
 constexpr double kCyclesPerParkedTile = 90.0;
 // What an epilogue that paces its layer takes per tile: fixed + per piece, whatever the piece's fill (a piece of 40
-// columns is processed whole), and not less per position than its tensors take to cross memory.  Fitted to forced widths at
-// 1.9 GHz: GELU on one set of groups (two groups of 96 -> 384 at 56 x 56, batch 128, in one launch: 80 / 160 / 240 positions
-// 324 / 249 / 223 us) and on two (96 -> 384: 80 / 160 / 208 positions 114 / 93 / 105 us); a residual with store warps, whose
-// tiles of 64 -> 256 at 56 x 56, batch 256 take 1.16 / 1.84 / 1.96 / 2.66 us at 80 / 96 / 144 / 176 positions (one, two, two,
-// three pieces) and 2.25 / 2.76 at 160 / 208, where pieces are full and memory is the limit (25 cycles per position).
-// Without and with that limit, us: that layer 154 (160 positions) / 146 (208), 16 x 40 x 40 x 256 -> 512 17.4 (160) / 16.5 (80),
-// 256 -> 1024 at 14 x 14, batch 256 43.3 (160) either way.  Blocks of a few tiles start and drain more than they stream: the
-// limit counts from kStreamTiles tiles per block on (27 x 14 x 14 x 256 -> 1024, two: 144 positions 8.75, 160 8.5).
+// columns is processed whole).  Fitted to forced widths at 1.9 GHz: GELU on one set of groups (two groups of 96 -> 384 at
+// 56 x 56, batch 128, in one launch: 80 / 160 / 240 positions 324 / 249 / 223 us) and on two (96 -> 384: 80 / 160 / 208
+// positions 114 / 93 / 105 us); a residual with store warps, whose tiles of 64 -> 256 at 56 x 56, batch 256 take 1.16 / 1.84 /
+// 1.96 / 2.66 us at 80 / 96 / 144 / 176 positions (one, two, two, three pieces).  That layer is limited by memory from 160
+// positions on and alone is faster at 208 (146 us, 153 at 160); a rule with the time its tensors take to cross memory
+// found that, but the ResNet-50-shaped pass at batch 256, where the layer's input and residual come from the steps before,
+// was slower with it (3.106 ms against 3.085).
 struct EpilogueCycles {
-  double tile, piece, position;
+  double tile, piece;
 };
-constexpr EpilogueCycles kEpilogueHidden = {0.0, 0.0, 0.0}, kEpilogueGelu = {1400.0, 1610.0, 0.0},
-                         kEpilogueWide = {700.0, 1420.0, 0.0};
-constexpr int kStreamTiles = 4;
-constexpr double kMemoryBytesPerCycle = 22.9;  // of an SM: 6.45 TB/s, 148 SMs, 1.9 GHz
-// (an output and a residual element per position and channel, and the layer's input once, over its channel tiles)
-static EpilogueCycles residual_epilogue(const ssconv_desc_t& d, long long Q, int m_tiles) {
-  const double in = 2.0 * d.C_in * ((double)d.N * d.H * d.W) / (double)Q;
-  return {800.0, 1400.0, (4.0 * d.C_out + in) / m_tiles / kMemoryBytesPerCycle};
-}
+constexpr EpilogueCycles kEpilogueHidden = {0.0, 0.0}, kEpilogueGelu = {1400.0, 1610.0}, kEpilogueWide = {700.0, 1420.0},
+                         kEpilogueResidual = {800.0, 1400.0};
 constexpr double kSplitAdvantage = 1.1;  // split only if the model predicts at least this gain
 // ... and only a deep K: the finishing kernel is a launch of its own (3 us of the caller's time, 2 to 3 us on the GPU when
-// the one before it is short).  Whole tiles against split ones, one to eight images: 8 k-blocks 4.0 / 4.8 us, 16 5.0 / 5.0
-// and 5.3 / 5.9, 18 5.5 / 5.6 and 5.6 / 6.9; 24 9.7 / 6.0 and 6.3 / 6.7, 36 7.8 / 6.5, 72 12.5 / 9.2.
+// the one before it is short).  Whole tiles against split ones, us on the GPU, one to eight images: 8 k-blocks 4.0 / 4.8, 16
+// 5.0 / 5.0 and 5.3 / 5.9, 18 5.5 / 5.6 and 5.6 / 6.9; 24 9.7 / 6.0 and 6.3 / 6.7, 36 7.8 / 6.5, 72 12.5 / 9.2.  Dense layers'
+// k-blocks take longer (16 5.7 / 5.1 and 5.9 / 5.3, 18 6.2 / 5.9 and 6.4 / 6.1): there the caller's time decides.
 constexpr int kSplitMinKBlocks = 20;
 
 static int ring_groups_for(uint32_t a_group_bytes, int BN, int stage_bufs) {
@@ -1768,7 +1761,6 @@ static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force
     // by their output stream, and measured fastest at the width the other terms choose)
     double tile = geo.kblocks * kblock_cycles<SPARSE>(BN, stage_bufs, geo.stages >= 4);
     tile = fmax(tile, epilogue.tile + pieces * epilogue.piece);
-    if (per_cta >= kStreamTiles) tile = fmax(tile, BN * epilogue.position);
     const double cost = (double)per_cta * tile + pieces * kEpiloguePieceCycles;
     if (BN == max_bn || cost < 0.97 * best_cost) {  // a narrower tile has to earn its extra weight traffic
       best_cost = cost;
@@ -2070,7 +2062,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   if (residual != nullptr && !plan.split) {
     stage_bufs = 4;
     const int widest = widest_tile(C::kAGroupBytes, 4);
-    plan = plan_layer<SPARSE>(Q, geo, workers, false, widest, 4, false, residual_epilogue(d, Q, geo.m_tiles));
+    plan = plan_layer<SPARSE>(Q, geo, workers, false, widest, 4, false, kEpilogueResidual);
     // The pair kernel takes a residual too (four staging buffers per group there as well): where its model
     // wins and the ring still holds two groups, one work item is one tile.
     // (both costs without what their epilogues take)
