@@ -131,6 +131,7 @@ struct FwdParams {
   int a_tiles;              // pairs of k-blocks (groups) per output tile
   int dual;                 // pair kernel: a work item is two neighbouring position tiles sharing the group's weights
   int split;                // 1: units dealt out evenly across CTAs (stream-K); 0: whole tiles per CTA
+  int csplit;               // cluster kernel: CTAs that share one tile's K
   int work_quot, work_rem;  // work items per CTA: quotient and remainder of (tiles or units) / grid
   float out_scale;          // 8-bit operands: factor applied to the accumulators before the bias
   float4* ws_regions;       // [2 * gridDim.x] regions of 128 x 240 fp32: a CTA's partial tiles
@@ -166,6 +167,16 @@ struct WorkIter {
       a0 = 0;
       left = count * A;
     }
+  }
+  // cluster kernel: this CTA's share of the groups of its cluster's tile
+  struct ClusterShare {};
+  __device__ WorkIter(const FwdParams& p, ClusterShare) {
+    A = p.a_tiles;
+    tile = (int)(blockIdx.x / (uint32_t)p.csplit);
+    const int rank = (int)blockIdx.x - tile * p.csplit;
+    const int quot = A / p.csplit, rem = A - quot * p.csplit;
+    a0 = rank * quot + (rank < rem ? rank : rem);
+    left = quot + (rank < rem ? 1 : 0);
   }
   __device__ bool next(Segment& s) {
     if (left <= 0) return false;
@@ -405,7 +416,7 @@ constexpr int kRoleActFirst = 0, kRoleActSecond = 1, kRoleWeights = 2;
 template <bool SPARSE, int ROLE, bool FP8 = false, bool GROUPED = false>
 __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUtensorMap* tm_b, const FwdParams& p,
                                               uint32_t full0, uint32_t empty0, uint32_t ring0, uint32_t res_bar,
-                                              volatile int* abort_flag) {
+                                              volatile int* abort_flag, WorkIter work) {
   using C = Cfg<SPARSE, FP8>;
   constexpr int kKb = C::kKbChannels;
   const uint32_t b_bytes = (uint32_t)p.BN * 128u;  // one activation tile: BN positions x 64 channels
@@ -414,7 +425,6 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
   uint32_t g = 0, ph = 0;  // group slot and its phase parity
   bool ok = true;
   bool first_segment = true;
-  WorkIter work(p);
   Segment seg;
   while (ok && work.next(seg)) {
     const int pt = seg.tile / p.m_tiles;
@@ -612,11 +622,13 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
       if (warp == 0)
         producer_role<SPARSE, kRoleActFirst, FP8, GROUPED>(&tm_a, &tm_b, p, full0,
                                              p.ring_groups == 2 ? smem_u32(bar_empty_first) : empty0, ring0,
-                                             smem_u32(bar_res), abort_flag);
+                                             smem_u32(bar_res), abort_flag, WorkIter(p));
       else if (warp == kExtraProducer)
-        producer_role<SPARSE, kRoleActSecond, FP8, GROUPED>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res), abort_flag);
+        producer_role<SPARSE, kRoleActSecond, FP8, GROUPED>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res),
+                                                            abort_flag, WorkIter(p));
       else
-        producer_role<SPARSE, kRoleWeights, FP8, GROUPED>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res), abort_flag);
+        producer_role<SPARSE, kRoleWeights, FP8, GROUPED>(&tm_a, &tm_b, p, full0, empty0, ring0, smem_u32(bar_res), abort_flag,
+                                                          WorkIter(p));
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -1055,9 +1067,59 @@ constexpr int kFinishThreads = 128;
 __host__ __device__ constexpr int finish_items_per_tile(int pieces) { return kGroups * pieces * (kPiece / 8); }
 constexpr int kFinishBatch = 8;  // contributors whose loads are in flight together
 
+// The summed accumulators of channel tile m at the 8 positions from q0 on -> bias, residual, activation, bf16, transposed
+// through `stage` (2 KB, [position][128 channels], 16-byte chunks permuted per row), NHWC.  128 threads (gtid); acc0 and
+// acc1 are the two float4s each holds in fragment layout; `sync` is a barrier of those threads.
+template <class Sync>
+__device__ __forceinline__ void finish_block(uint32_t flags, const float* bias, const __nv_bfloat16* residual, __nv_bfloat16* y,
+                                             int y_pitch, int C_out, int Q, int m, int q0, float4 acc0, float4 acc1,
+                                             uint8_t* stage, int gtid, Sync sync) {
+  const int lane = gtid & 31, q = gtid >> 5;
+  float bias_v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int co = m * kTileM + q * 32 + 8 * i + (lane >> 2);
+    bias_v[i] = ((flags & SSCONV_FLAG_BIAS) && co < C_out) ? bias[co] : 0.0f;
+  }
+  // thread 8 i + j of a warp addresses position j of channel block i of the warp's four
+  const uint32_t row = (uint32_t)(lane & 7);
+  const uint32_t chunk = (uint32_t)(4 * q + (lane >> 3));
+  const uint32_t st_addr = smem_u32(stage) + row * 256u + ((chunk ^ row) << 4);
+  const int pos = gtid >> 4, ch16 = gtid & 15;  // 16 threads cover the 256 contiguous bytes of one position
+  const int q_pos = q0 + pos;
+  const int co16 = m * kTileM + 8 * ch16;
+  const bool in_range = q_pos < Q && co16 < C_out;
+  if (residual != nullptr) {
+    // residual block -> staging buffer (same layout), read back in fragment layout, added in fp32
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (in_range) v = *reinterpret_cast<const uint4*>(residual + (size_t)q_pos * y_pitch + co16);
+    *reinterpret_cast<uint4*>(stage + pos * 256 + ((ch16 ^ pos) << 4)) = v;
+    sync();
+    uint32_t res[4];
+    ldmatrix_x4_trans(st_addr, res);
+    acc0.x += bf16_lo(res[0]); acc0.y += bf16_hi(res[0]); acc0.z += bf16_lo(res[1]); acc0.w += bf16_hi(res[1]);
+    acc1.x += bf16_lo(res[2]); acc1.y += bf16_hi(res[2]); acc1.z += bf16_lo(res[3]); acc1.w += bf16_hi(res[3]);
+  }
+  uint32_t w[4];
+  const float v[8] = {acc0.x + bias_v[0], acc0.y + bias_v[0], acc0.z + bias_v[1], acc0.w + bias_v[1],
+                      acc1.x + bias_v[2], acc1.y + bias_v[2], acc1.z + bias_v[3], acc1.w + bias_v[3]};
+  const int act = activation_of(flags);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    w[i] = (act == kActRelu)   ? activate_pack<kActRelu>(v[2 * i], v[2 * i + 1])
+           : (act == kActGelu) ? activate_pack<kActGelu>(v[2 * i], v[2 * i + 1])
+                               : activate_pack<kActNone>(v[2 * i], v[2 * i + 1]);
+  stmatrix_x4_trans(st_addr, w[0], w[1], w[2], w[3]);
+  sync();
+  if (in_range) {
+    const uint4 o = *reinterpret_cast<const uint4*>(stage + pos * 256 + ((ch16 ^ pos) << 4));
+    *reinterpret_cast<uint4*>(y + (size_t)q_pos * y_pitch + co16) = o;
+  }
+}
+
 __global__ void __launch_bounds__(kFinishThreads) ssconv_split_finish_kernel(const FinishParams f) {
   __shared__ __align__(128) uint8_t stage[8 * 256];  // [position][128 channels], 16-byte chunks permuted per row
-  const int gtid = threadIdx.x, lane = gtid & 31, q = gtid >> 5;
+  const int gtid = threadIdx.x;
   int item = blockIdx.x;
   const int k = item % (kPiece / 8);
   item /= (kPiece / 8);
@@ -1097,45 +1159,192 @@ __global__ void __launch_bounds__(kFinishThreads) ssconv_split_finish_kernel(con
       }
     }
   }
-  float bias_v[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int co = m * kTileM + q * 32 + 8 * i + (lane >> 2);
-    bias_v[i] = ((f.flags & SSCONV_FLAG_BIAS) && co < f.C_out) ? f.bias[co] : 0.0f;
+  finish_block(f.flags, f.bias, f.residual, f.y, f.y_pitch, f.C_out, f.Q, m, pt * f.BN + grp * (f.BN >> 1) + piece * kPiece + 8 * k,
+               acc0, acc1, stage, gtid, [] { __syncthreads(); });
+}
+
+
+// ---------------------------------------------------------------------------------------
+// Cluster kernel: the K of one tile on the CTAs of a cluster
+// ---------------------------------------------------------------------------------------
+// For layers of few tiles and a deep K (one or a few images, late stages).  Each of the 2, 4 or 8 CTAs of a cluster
+// multiplies its share of the tile's groups; the partial tiles meet in shared memory: a CTA puts its accumulators into its
+// own ring, which by then holds nothing that is still needed (every load has landed and every MMA has read it), as float4s
+// in fragment order, one cluster barrier, and then the tile's blocks of 8 positions are dealt out to the CTAs, each block
+// summed over the CTAs in rank order by 128 threads that read the peers' rings directly, and finished like a split tile.
+// Against the split over the whole grid there is no second launch (3 us of the caller's time, 2 us on the GPU) and no
+// scratch in global memory; against whole tiles the K loop is 2 to 8 times shorter.  Nothing waits for a CTA outside the
+// cluster, whose CTAs the hardware starts together.  The residual is read by the finishing threads.
+// Shared memory: ring, three 2-KB staging buffers (one per 128 threads), barriers.
+constexpr int kClusterThreads = kThreads;                          // 384: three sets of 128 finishing threads
+constexpr uint32_t kClusterStageBytes = 3u * 2048u;
+template <bool SPARSE>
+__global__ void __launch_bounds__(kClusterThreads, 1)
+ssconv_fwd_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
+                          const __nv_bfloat16* residual, const int y_pitch, const FwdParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const uint32_t b_bytes = (uint32_t)p.BN * 128u;
+  uint8_t* ring = smem;
+  uint8_t* stage = ring + p.ring_groups * (p.a_grp_bytes + 2u * b_bytes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(stage + kClusterStageBytes);
+  // barrier slots: [0,4) group full (the three producers), [4,8) group empty (one commit), [8] accumulator full
+  uint64_t* bar_acc_full = bars + 8;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 9);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  if (warp == 0) {
+    if (lane < 9) mbar_init(&bars[lane], lane < 4 ? 3u : 1u);
+    if (lane == 0) {
+      grid_launch_dependents();
+      *abort_flag = 0;
+    }
+    __syncwarp();
+    if (lane == 0) {
+      mbar_fence_init();
+      fence_proxy_async_smem();
+    }
+  } else if (warp == 1) {
+    tmem_alloc(tmem_slot, kTmemCols);
+    tmem_relinquish();
+  } else if (lane == 0) {
+    if (warp == kFirstExtraProducerWarp) prefetch_tensormap(&tm_b);
+    if (warp == kFirstExtraProducerWarp + 1) prefetch_tensormap(&tm_a);
   }
-  // thread 8 i + j of a warp addresses position j of channel block i of the warp's four
-  const uint32_t row = (uint32_t)(lane & 7);
-  const uint32_t chunk = (uint32_t)(4 * q + (lane >> 3));
-  const uint32_t st_addr = smem_u32(stage) + row * 256u + ((chunk ^ row) << 4);
-  const int pos = gtid >> 4, ch16 = gtid & 15;  // 16 threads cover the 256 contiguous bytes of one position
-  const int q_pos = pt * f.BN + grp * (f.BN >> 1) + piece * kPiece + 8 * k + pos;
-  const int co16 = m * kTileM + 8 * ch16;
-  const bool in_range = q_pos < f.Q && co16 < f.C_out;
-  if (f.residual != nullptr) {
-    // residual block -> staging buffer (same layout), read back in fragment layout, added in fp32
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (in_range) v = *reinterpret_cast<const uint4*>(f.residual + (size_t)q_pos * f.y_pitch + co16);
-    *reinterpret_cast<uint4*>(stage + pos * 256 + ((ch16 ^ pos) << 4)) = v;
-    __syncthreads();
-    uint32_t res[4];
-    ldmatrix_x4_trans(st_addr, res);
-    acc0.x += bf16_lo(res[0]); acc0.y += bf16_hi(res[0]); acc0.z += bf16_lo(res[1]); acc0.w += bf16_hi(res[1]);
-    acc1.x += bf16_lo(res[2]); acc1.y += bf16_hi(res[2]); acc1.z += bf16_lo(res[3]); acc1.w += bf16_hi(res[3]);
-  }
-  uint32_t w[4];
-  const float v[8] = {acc0.x + bias_v[0], acc0.y + bias_v[0], acc0.z + bias_v[1], acc0.w + bias_v[1],
-                      acc1.x + bias_v[2], acc1.y + bias_v[2], acc1.z + bias_v[3], acc1.w + bias_v[3]};
-  const int act = activation_of(f.flags);
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    w[i] = (act == kActRelu)   ? activate_pack<kActRelu>(v[2 * i], v[2 * i + 1])
-           : (act == kActGelu) ? activate_pack<kActGelu>(v[2 * i], v[2 * i + 1])
-                               : activate_pack<kActNone>(v[2 * i], v[2 * i + 1]);
-  stmatrix_x4_trans(st_addr, w[0], w[1], w[2], w[3]);
+  tc_fence_before();
   __syncthreads();
-  if (in_range) {
-    const uint4 v = *reinterpret_cast<const uint4*>(stage + pos * 256 + ((ch16 ^ pos) << 4));
-    *reinterpret_cast<uint4*>(f.y + (size_t)q_pos * f.y_pitch + co16) = v;
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t full0 = smem_u32(bars), empty0 = full0 + 32u, ring0 = smem_u32(ring);
+  const int rank = (int)cluster_ctarank();
+  const WorkIter share(p, WorkIter::ClusterShare{});
+
+  if (warp == 0) {
+    producer_role<SPARSE, kRoleActFirst>(&tm_a, &tm_b, p, full0, empty0, ring0, 0u, abort_flag, share);
+  } else if (warp == kFirstExtraProducerWarp) {
+    producer_role<SPARSE, kRoleActSecond>(&tm_a, &tm_b, p, full0, empty0, ring0, 0u, abort_flag, share);
+  } else if (warp == kFirstExtraProducerWarp + 1) {
+    producer_role<SPARSE, kRoleWeights>(&tm_a, &tm_b, p, full0, empty0, ring0, 0u, abort_flag, share);
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer (as in the one-CTA kernel)
+    const uint32_t idesc = make_idesc_bf16(kTileM, (uint32_t)p.BN, SPARSE);
+    const uint32_t grp_desc = (p.a_grp_bytes + 2u * b_bytes) >> 4, b_desc = b_bytes >> 4;
+    const uint32_t ring_lo0 = desc_lo(ring0);
+    const int tail_c = p.C_in - (p.cblocks - 1) * kBlockK;
+    const int mma_full = SPARSE ? 2 : 4;
+    const int mma_tail = SPARSE ? ((tail_c + 31) >> 5) : ((tail_c + 15) >> 4);
+    const int tail_start = (tail_c == kBlockK) ? p.kblocks : (p.cblocks - 1) * p.taps;  // first k-block of the tail
+    uint32_t g = 0, ph = 0, accumulate = 0, mslot = 0;
+    bool ok = true;
+    const int a_end = share.a0 + share.left;
+    for (int a = share.a0; a < a_end; ++a) {
+      if (!mbar_wait_warp_a(full0 + 8u * g, ph, abort_flag, kWaitLimitCycles)) { ok = false; break; }
+      const uint32_t a_lo = ring_lo0 + g * grp_desc;
+      const uint32_t b0_lo = a_lo + (p.a_grp_bytes >> 4);
+      const uint32_t b1_lo = b0_lo + b_desc;
+      const int n0 = (2 * a >= tail_start) ? mma_tail : mma_full;
+      const int n1 = (2 * a + 1 >= p.kblocks) ? 0 : ((2 * a + 1 >= tail_start) ? mma_tail : mma_full);
+      if (SPARSE) {
+        const uint32_t meta_tmem = tmem_base + kMetaCol + 4u * mslot;
+        mslot ^= 1u;
+        tc_cp_128x128b_w(meta_tmem, a_lo + (kATileBytes >> 4));
+        tc_mma_sparse_w(tmem_base, a_lo, b0_lo, meta_tmem, idesc, accumulate);
+        if (n0 > 1) tc_mma_sparse_w(tmem_base, a_lo + 2u, b0_lo + 4u, meta_tmem, idesc | 1u, 1u);
+        if (n1 > 0) tc_mma_sparse_w(tmem_base, a_lo + 4u, b1_lo, meta_tmem + 2u, idesc, 1u);
+        if (n1 > 1) tc_mma_sparse_w(tmem_base, a_lo + 6u, b1_lo + 4u, meta_tmem + 2u, idesc | 1u, 1u);
+      } else {
+        const uint32_t a1_lo = a_lo + (kATileBytes >> 4);
+        for (int kk = 0; kk < n0; ++kk)
+          tc_mma_dense_w(tmem_base, a_lo + 2u * kk, b0_lo + 2u * kk, idesc, (kk > 0) ? 1u : accumulate);
+        for (int kk = 0; kk < n1; ++kk) tc_mma_dense_w(tmem_base, a1_lo + 2u * kk, b1_lo + 2u * kk, idesc, 1u);
+      }
+      accumulate = 1;
+      tc_commit_w(empty0 + 8u * g);
+      if (++g == (uint32_t)p.ring_groups) {
+        g = 0;
+        ph ^= 1u;
+      }
+    }
+    if (ok) tc_commit_w(smem_u32(bar_acc_full));
+  } else {
+    // ------------------------------------------------------------------ accumulators -> ring
+    // (8 warps: two groups of four, each with half of the positions; block b of 8 positions, thread t of its group of
+    // four warps: float4s (2 b) 128 + t and (2 b + 1) 128 + t, 512 BN bytes in all: two groups' activation tiles)
+    const int half = (warp - 2) >> 2, q = warp & 3, gtid = q * 32 + lane;
+    const bool got = mbar_wait_warp(bar_acc_full, 0u, abort_flag, kWaitLimitCycles, 64);
+    if (got) {
+      tc_fence_after();
+      const int blocks = p.BN >> 4;  // of this half
+      const uint32_t t_row = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * (p.BN >> 1));
+      float4* part = reinterpret_cast<float4*>(ring) + 2 * (half * blocks) * 128 + gtid;
+      for (int piece = 0; piece < p.pieces; ++piece) {
+        uint32_t r[kPiece];
+        tc_ld_piece(t_row + piece * kPiece, r);
+        tc_wait_ld();
+#pragma unroll
+        for (int k = 0; k < kPiece / 8; ++k) {
+          const int b = piece * (kPiece / 8) + k;
+          if (b < blocks) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              part[(2 * b + h) * 128] = make_float4(__uint_as_float(r[20 * h + 4 * k]), __uint_as_float(r[20 * h + 4 * k + 1]),
+                                                    __uint_as_float(r[20 * h + 4 * k + 2]), __uint_as_float(r[20 * h + 4 * k + 3]));
+          }
+        }
+      }
+    }
+  }
+
+  // ------------------------------------------------------------------ sum and finish
+  // (a CTA whose waits ran out takes part with whatever its ring holds: its status word says so)
+  tc_fence_before();
+  __syncthreads();
+  cluster_arrive();
+  cluster_wait();
+  {
+    const int set = (int)threadIdx.x >> 7, gtid = (int)threadIdx.x & 127;
+    const int tile = share.tile, pt = tile / p.m_tiles, m = tile - pt * p.m_tiles;
+    grid_dependency_wait();
+    for (int b = rank + set * p.csplit; b < (p.BN >> 3); b += 3 * p.csplit) {
+      if (pt * p.BN + 8 * b >= p.Q) break;
+      const uint32_t at = ring0 + (uint32_t)(2 * b * 128 + gtid) * 16u;
+      float4 v0[8], v1[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        if (c < p.csplit) {
+          const uint32_t src = map_to_cta(at, (uint32_t)c);
+          v0[c] = ld_cluster_f4(src);
+          v1[c] = ld_cluster_f4(src + 2048u);
+        }
+      }
+      float4 acc0 = v0[0], acc1 = v1[0];
+#pragma unroll
+      for (int c = 1; c < 8; ++c) {
+        if (c < p.csplit) {
+          acc0.x += v0[c].x; acc0.y += v0[c].y; acc0.z += v0[c].z; acc0.w += v0[c].w;
+          acc1.x += v1[c].x; acc1.y += v1[c].y; acc1.z += v1[c].z; acc1.w += v1[c].w;
+        }
+      }
+      finish_block(p.flags, p.bias, residual, p.y, y_pitch, p.C_out, p.Q, m, pt * p.BN + 8 * b, acc0, acc1, stage + set * 2048,
+                   gtid, [set] { asm volatile("bar.sync %0, 128;" ::"r"(set + 1) : "memory"); });
+      asm volatile("bar.sync %0, 128;" ::"r"(set + 1) : "memory");  // (the buffer is free again)
+    }
+  }
+  // ------------------------------------------------------------------ teardown
+  __syncthreads();
+  cluster_arrive();  // no CTA leaves while another still reads its ring
+  cluster_wait();
+  if (*abort_flag != 0) {
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000LL) __nanosleep(1000);
+    if (threadIdx.x == 0 && p.dev_status != nullptr) atomicExch(p.dev_status, (int)SSCONV_ERR_TIMEOUT);
+    __syncthreads();
+  }
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, kTmemCols);
   }
 }
 
@@ -1711,7 +1920,13 @@ static int g_tune_bn = 0;
 static int g_tune_resident = 1;  // 0: weights always travel through the ring
 static int g_tune_pair = -1;  // -1: the model chooses; 0: never the pair kernel; 1: wherever it applies
 static int g_tune_pair_dual = -1;  // pair kernel, two position tiles per work item: -1 the model, 0 never, 1 always
+static int g_tune_cluster = -1;    // cluster kernel: -1 the model chooses; 0 never; 2, 4, 8: wherever that many CTAs fit
 int32_t set_tuning(int32_t option, int32_t value) {
+  if (option == SSCONV_TUNE_CLUSTER) {
+    if (value != -1 && value != 0 && value != 2 && value != 4 && value != 8) return SSCONV_ERR_BAD_DESC;
+    g_tune_cluster = value;
+    return SSCONV_OK;
+  }
   if (option == SSCONV_TUNE_PAIR) {
     if (value < -1 || value > 1) return SSCONV_ERR_BAD_DESC;
     g_tune_pair = value;
@@ -1744,6 +1959,7 @@ struct Plan {
   bool pair = false;  // 256-channel tiles on CTA pairs (ssconv_fwd_pair_kernel)
   bool dual = false;  // ... with two position tiles per work item
   bool wide = false;  // one-CTA tiles with two sets of epilogue groups
+  int cluster = 0;    // CTAs of a cluster that share each tile's K (ssconv_fwd_cluster_kernel); 0: none
 };
 template <bool SPARSE>
 static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force_split, int max_bn = kBN,
@@ -1869,6 +2085,52 @@ static Plan plan_pair(long long Q, const Geometry& geo, int workers, bool forced
 }
 constexpr double kPairAdvantage = 1.05;  // the pair kernel only if the model predicts at least this gain
 
+// Plan for the cluster kernel (the K of a tile on the CTAs of a cluster), or cluster = 0 where it does not apply.
+// The exchange costs 1.6 us on the GPU and 0.015 us per position of a tile's width beyond 64, so that narrow tiles and a
+// deep K are what it is for.  Measured in us, 2:4 / dense, whole tiles or the split over the grid -> clusters (images x
+// height x channels, filter; stride in brackets):
+//   8 CTAs, 64 positions   1 x 14 x 256 -> 256, 3   6.6 / 6.9 -> 5.4 / 6.0    1 x 7 x 512 -> 512, 3     9.6 / 9.6 -> 5.9 / 6.8
+//                          1 x 7 x 2048 -> 512, 1   5.6 / 6.0 -> 5.0 / 5.4    1 x 7 x 1024 -> 1024, 3   9.3 / 9.3 -> 7.6 / 9.1
+//     beyond the line      1 x 20 x 2048 -> 256, 3 (18 groups of k-blocks per CTA)  10.0 / 11.1 -> 11.1 / 13.8
+//   4 CTAs                 1 x 14 x 1024 -> 256, 1  4.9 / 5.7 -> 4.6 / 5.2    1 x 28 x 128 -> 128, 3    5.3 / 6.2 -> 5.0 / 5.7
+//                          3 x 14 x 384 -> 768, 2 (2)  6.6 / 7.2 -> 5.3 / 6.0   3 x 14 x 1536 -> 384, 1   6.4 / 7.7 -> 6.0 / 6.8
+//                          3 x 7 x 3072 -> 768, 1   6.9 / 7.4 -> 6.2 / 7.4
+//     beyond the line      8 x 7 x 512 -> 264, 3 (9 groups per CTA)  7.8 / 8.1 -> 7.6 / 9.1,  1 x 28 x 512 -> 128, 1 (4 groups in
+//                          all)  3.9 / 4.6 -> 4.4 / 4.9
+//   2 CTAs                 8 x 14 x 256 -> 256, 3  7.7 / 9.0 -> 7.4 / 9.1,  27 x 7 x 512 -> 512, 3  11.6 / 13.5 -> 11.2 / 14.0,
+//                          27 x 7 x 2048 -> 512, 1  7.6 / 10.2 -> 8.0 / 9.4: not worth a rule
+// (groups = pairs of k-blocks).  Of the widths, 48 where it covers the positions with fewer columns.
+constexpr int kClusterMinGroups = 8, kCluster8MinGroups = 16, kCluster8MaxGroups = 72, kCluster4MaxGroups = 24;
+// Clusters that the chip holds at once: its SMs come in groups that are no multiple of the cluster, so that a few stay out.
+static int max_clusters(int workers, int size) { return workers / size - (size == 8 ? 4 : size == 4 ? 3 : 2); }
+static int cluster_ring_groups(uint32_t a_group_bytes, int BN) {
+  const int n = (int)((kMaxSmemBytes - 1024 - kBarrierBytes - kClusterStageBytes) / group_bytes(a_group_bytes, BN));
+  return n > kMaxGroups ? kMaxGroups : n;
+}
+static Plan plan_cluster(long long Q, const Geometry& geo, int workers) {
+  Plan none{0, false};
+  // (an override of the width or of the pairs asks for the kernels that it is about)
+  if (g_tune_cluster == 0 || (g_tune_cluster < 0 && (g_tune_bn != 0 || g_tune_pair != -1))) return none;
+  const long long tiles48 = ((Q + 47) / 48) * geo.m_tiles, tiles64 = ((Q + 63) / 64) * geo.m_tiles;
+  Plan c{64, false};
+  if (g_tune_cluster > 0) {
+    c.cluster = g_tune_cluster;
+    if (g_tune_bn != 0) c.BN = g_tune_bn;
+    return geo.stages < c.cluster || ((Q + c.BN - 1) / c.BN) * geo.m_tiles > max_clusters(workers, c.cluster) ? none : c;
+  }
+  if (geo.stages >= kCluster8MinGroups && geo.stages <= kCluster8MaxGroups && tiles64 <= max_clusters(workers, 8)) {
+    c.cluster = 8;
+    return c;
+  }
+  if (48 * tiles48 < 64 * tiles64) c.BN = 48;
+  if (geo.stages >= kClusterMinGroups && geo.stages <= kCluster4MaxGroups &&
+      (c.BN == 48 ? tiles48 : tiles64) <= max_clusters(workers, 4)) {
+    c.cluster = 4;
+    return c;
+  }
+  return none;
+}
+
 constexpr size_t scratch_bytes(int workers) {
   return 2 * (size_t)workers * kRegionBytes;
 }
@@ -1880,6 +2142,7 @@ static bool g_wide_attr_set[64][2] = {{false}};
 static bool g_pair_attr_set[64][2] = {{false}};
 static bool g_pair_res_attr_set[64][2] = {{false}};
 static bool g_fp8_attr_set[64][2] = {{false}};
+static bool g_cluster_attr_set[64][2] = {{false}};
 static bool g_pair_fp8_attr_set[64] = {false};
 
 // Dense layers with 8 input channels (a channel-padded RGB stem): a k-block of 64 K-elements is 8
@@ -1933,7 +2196,11 @@ constexpr int kWideStageBufs = 4;  // staging buffers per half of a tile: two fo
 // The plan for a layer without a residual: one-CTA tiles (whole or K split) or the pair kernel.
 template <bool SPARSE>
 static Plan choose_plan(const ssconv_desc_t& d, long long Q, const Geometry& geo, int workers, bool force_split,
-                        bool allow_split = true, bool allow_wide = true, bool allow_pair = true) {
+                        bool allow_split = true, bool allow_wide = true, bool allow_pair = true, bool allow_cluster = true) {
+  if (allow_cluster && !force_split && !small_channel_mode(d, SPARSE)) {
+    const Plan c = plan_cluster(Q, geo, workers);
+    if (c.cluster != 0) return c;
+  }
   const Plan plan = plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, allow_split);
   if (force_split || small_channel_mode(d, SPARSE)) return plan;
   if (allow_pair && g_tune_pair != 0) {
@@ -1984,6 +2251,12 @@ int32_t plan_query_sms(const ssconv_desc_t& d, bool sparse, int sm_count, int32_
     return SSCONV_OK;
   }
   const long long tiles = q_tiles * geo.m_tiles;
+  if (plan.cluster != 0) {  // (K is split, over the CTAs of a cluster each)
+    if (split) *split = 1;
+    if (ctas) *ctas = (int32_t)(tiles * plan.cluster);
+    if (ring_groups) *ring_groups = cluster_ring_groups(a_group_bytes, plan.BN);
+    return SSCONV_OK;
+  }
   const bool do_split = plan.split && geo.stages > 1;
   const long long work = do_split ? tiles * geo.stages : tiles;
   if (split) *split = do_split ? 1 : 0;
@@ -2055,11 +2328,17 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   if (have_ws && (reinterpret_cast<uintptr_t>(ws) & 15u)) return SSCONV_ERR_ALIGNMENT;
   if (force_split && !have_ws) return SSCONV_ERR_WORKSPACE;
   // (8-bit operands: the pair kernel exists for the 2:4 form only; the dense counterpart stays on one-block tiles)
-  Plan plan = groups > 1 ? choose_plan<SPARSE>(d, Q, geo, workers, false, false, false, false)
-              : (residual != nullptr || (FP8 && !SPARSE)) ? plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, have_ws)
-                                                        : choose_plan<SPARSE>(d, Q, geo, workers, force_split, have_ws, !FP8);
+  // (a grouped layer's own launches per group keep the split over the grid)
+  const bool allow_cluster = !FP8 && !force_split && !small_c && groups == 1 && y_pitch == 0;
+  Plan plan{0, false};
+  if (allow_cluster) plan = plan_cluster(Q, geo, workers);
+  if (plan.cluster == 0)
+    plan = groups > 1 ? choose_plan<SPARSE>(d, Q, geo, workers, false, false, false, false, false)
+           : (residual != nullptr || (FP8 && !SPARSE))
+               ? plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, have_ws)
+               : choose_plan<SPARSE>(d, Q, geo, workers, force_split, have_ws, !FP8, true, false);
   int stage_bufs = 2;
-  if (residual != nullptr && !plan.split) {
+  if (residual != nullptr && !plan.split && plan.cluster == 0) {
     stage_bufs = 4;
     const int widest = widest_tile(C::kAGroupBytes, 4);
     plan = plan_layer<SPARSE>(Q, geo, workers, false, widest, 4, false, kEpilogueResidual);
@@ -2086,8 +2365,9 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   // channels): every tile needs the same 16-64 KB of weights, which then stay in shared memory for the
   // life of the CTA instead of travelling through the ring with every tile; the groups hold activations
   // only, and more of them fit.
-  const bool resident = !wide_epilogue && !SPARSE && !FP8 && !small_c && !pair && !plan.split && residual == nullptr && geo.m_tiles == 1 &&
-                        geo.kblocks <= 4 && g_tune_resident != 0;
+  const int cluster = plan.cluster;
+  const bool resident = !wide_epilogue && !SPARSE && !FP8 && !small_c && !pair && !plan.split && cluster == 0 && residual == nullptr &&
+                        geo.m_tiles == 1 && geo.kblocks <= 4 && g_tune_resident != 0;
   const uint32_t a_grp_bytes = resident ? 0u : C::kAGroupBytes;
   const uint32_t a_res_bytes = resident ? (uint32_t)geo.stages * 2u * kATileBytes : 0u;
   if (pair) stage_bufs = residual != nullptr ? 4 : pair_stage_bufs(geo.kblocks);
@@ -2101,8 +2381,15 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
     ring_groups = (int)((kMaxSmemBytes - 1024 - kBarrierBytes - staging_bytes(stage_bufs) - a_res_bytes) / grp_bytes);
     if (ring_groups > kMaxGroups) ring_groups = kMaxGroups;
   }
-  const uint32_t smem_bytes =
-      1024 + (uint32_t)ring_groups * grp_bytes + a_res_bytes + staging_bytes(stage_bufs) + kBarrierBytes;
+  if (cluster != 0) ring_groups = cluster_ring_groups(C::kAGroupBytes, BN);
+  const uint32_t smem_bytes = 1024 + (uint32_t)ring_groups * grp_bytes + a_res_bytes +
+                              (cluster != 0 ? kClusterStageBytes : staging_bytes(stage_bufs)) + kBarrierBytes;
+  if (cluster != 0 && !g_cluster_attr_set[dev][SPARSE ? 1 : 0]) {
+    if (cudaFuncSetAttribute(ssconv_fwd_cluster_kernel<SPARSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kMaxSmemBytes) != cudaSuccess)
+      return SSCONV_ERR_CUDA;
+    g_cluster_attr_set[dev][SPARSE ? 1 : 0] = true;
+  }
   if (pair && !FP8 && !g_pair_attr_set[dev][SPARSE ? 1 : 0]) {
     if (cudaFuncSetAttribute(ssconv_fwd_pair_kernel<SPARSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kMaxSmemBytes) != cudaSuccess)
@@ -2186,7 +2473,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
     if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
   }
   // output: NHWC seen as (c, position); a box is one staging half piece, 64 channels x 40 positions
-  {
+  if (cluster == 0) {  // (the cluster kernel stores from registers)
     cuuint64_t dims[3] = {(cuuint64_t)d.C_out, (cuuint64_t)Q, (cuuint64_t)groups};
     // (channels beyond C_out are clipped: a slice stays a slice)
     cuuint64_t strides[2] = {(cuuint64_t)y_pitch_el * 2, (cuuint64_t)d.C_out * 2};
@@ -2262,8 +2549,12 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   const long long units = q_tiles * geo.m_tiles * geo.stages;
   if (units >= (1LL << 31)) return SSCONV_ERR_UNSUPPORTED_SHAPE;  // 32-bit work indices on the device
   p.split = (plan.split && p.a_tiles > 1) ? 1 : 0;
+  p.csplit = cluster;
   int grid;
-  if (p.split) {
+  if (cluster != 0) {
+    grid = p.num_tiles * cluster;
+    p.ws_regions = nullptr;
+  } else if (p.split) {
     grid = units < workers ? (int)units : workers;
     p.ws_regions = static_cast<float4*>(ws);
   } else if (pair) {
@@ -2294,11 +2585,19 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;  // pair kernel: clusters of two CTAs
-  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.x = cluster != 0 ? (unsigned)cluster : 2u;
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pair ? 2 : 1;
+  cfg.numAttrs = pair || cluster != 0 ? 2 : 1;
+  if (cluster != 0) {
+    cfg.blockDim = dim3((unsigned)kClusterThreads);
+    if (cudaLaunchKernelEx(&cfg, ssconv_fwd_cluster_kernel<SPARSE>, tm_a, tm_b, static_cast<const __nv_bfloat16*>(residual),
+                           (int)y_pitch_el, p) != cudaSuccess)
+      return SSCONV_ERR_CUDA;
+    count_launch();
+    return SSCONV_OK;
+  }
   const cudaError_t launched =
       (FP8 && pair) ? cudaLaunchKernelEx(&cfg, ssconv_fwd_pair_kernel<true, true>, tm_a, tm_b, tm_meta, tm_y, tm_y_tail, tm_r,
                                          tm_r_tail, p)
@@ -2369,8 +2668,8 @@ int32_t launch_forward_dense(const ssconv_desc_t& d, const void* x, const void* 
 constexpr double kLaunchCycles = 4000.0;
 template <bool SPARSE>
 static double grouped_cost(const ssconv_desc_t& g, long long Q, const Geometry& geo, int workers, bool together, bool have_ws) {
-  const Plan plan = together ? choose_plan<SPARSE>(g, Q, geo, workers, false, false, false, false)
-                             : choose_plan<SPARSE>(g, Q, geo, workers, false, have_ws);
+  const Plan plan = together ? choose_plan<SPARSE>(g, Q, geo, workers, false, false, false, false, false)
+                             : choose_plan<SPARSE>(g, Q, geo, workers, false, have_ws, true, true, false);
   if (plan.wide || activation_of(g.flags) != kActGelu || geo.kblocks > kWideMaxKBlocks) return plan.cost;
   return plan_layer<SPARSE>(Q, geo, workers, false, kBN, 2, false, kEpilogueGelu).cost;
 }
