@@ -10,7 +10,7 @@ ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libssconv.so")
 SOURCES = ["api.cu", "mask.cu", "pool.cu", "depthwise.cu", "train.cu", "wgrad.cu", "forward.cu"]
-HEADERS = ["layout.cuh", "sm100_ptx.cuh"]
+HEADERS = ["launch.cuh", "layout.cuh", "sm100_ptx.cuh"]
 
 
 def _newest_source_mtime() -> float:

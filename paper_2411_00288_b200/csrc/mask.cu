@@ -3,7 +3,9 @@
 // never computed with.
 #include <cuda_runtime.h>
 
+#include "launch.cuh"
 #include "layout.cuh"
+#include "sm100_ptx.cuh"
 #include "ssconv.h"
 
 namespace ssconv {
@@ -13,8 +15,10 @@ namespace ssconv {
 // ---------------------------------------------------------------------------------------
 
 // Eq. 1 without the one-hot: first maximum of the six scores of each group.
-__global__ void select_logits_kernel(const float2* __restrict__ scores, int64_t G, uint8_t* __restrict__ pattern) {
+__global__ void select_logits_kernel(const float2* scores, int64_t G, uint8_t* pattern) {
+  grid_launch_dependents();
   int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  grid_dependency_wait();
   if (g >= G) return;
   float2 a = scores[3 * g], b = scores[3 * g + 1], c = scores[3 * g + 2];
   float v[6] = {a.x, a.y, b.x, b.y, c.x, c.y};
@@ -57,16 +61,20 @@ __device__ __forceinline__ uint32_t magnitude_pattern(uint32_t lo, uint32_t hi) 
   return magnitude_pattern4(a);
 }
 
-__global__ void select_magnitude_kernel(const uint2* __restrict__ w, int64_t G, uint8_t* __restrict__ pattern) {
+__global__ void select_magnitude_kernel(const uint2* w, int64_t G, uint8_t* pattern) {
+  grid_launch_dependents();
   int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  grid_dependency_wait();
   if (g >= G) return;
   uint2 v = w[g];
   pattern[g] = (uint8_t)magnitude_pattern(v.x, v.y);
 }
 
 // The same for e4m3 weights: a group is four bytes, a magnitude the 7 bits below the sign bit.
-__global__ void select_magnitude_e4m3_kernel(const uint32_t* __restrict__ w, int64_t G, uint8_t* __restrict__ pattern) {
+__global__ void select_magnitude_e4m3_kernel(const uint32_t* w, int64_t G, uint8_t* pattern) {
+  grid_launch_dependents();
   int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  grid_dependency_wait();
   if (g >= G) return;
   const uint32_t v = w[g];
   const uint32_t a[4] = {v & 0x7Fu, (v >> 8) & 0x7Fu, (v >> 16) & 0x7Fu, (v >> 24) & 0x7Fu};
@@ -83,11 +91,13 @@ __device__ __forceinline__ uint32_t e4m3_pair(uint32_t v, float scale) {
   asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(out) : "f"(hi), "f"(lo));
   return out;
 }
-__global__ void __launch_bounds__(256) quantize_e4m3_kernel(const uint32_t* __restrict__ x, uint16_t* __restrict__ y,
-                                                            int64_t vectors, int64_t pairs, float scale) {
+__global__ void __launch_bounds__(256) quantize_e4m3_kernel(const uint32_t* x, uint16_t* y, int64_t vectors,
+                                                            int64_t pairs, float scale) {
+  grid_launch_dependents();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  grid_dependency_wait();
   if (i < vectors) {
-    const uint4 a = __ldg(reinterpret_cast<const uint4*>(x) + 2 * i), b = __ldg(reinterpret_cast<const uint4*>(x) + 2 * i + 1);
+    const uint4 a = reinterpret_cast<const uint4*>(x)[2 * i], b = reinterpret_cast<const uint4*>(x)[2 * i + 1];
     uint4 o;
     o.x = e4m3_pair(a.x, scale) | (e4m3_pair(a.y, scale) << 16);
     o.y = e4m3_pair(a.z, scale) | (e4m3_pair(a.w, scale) << 16);
@@ -248,10 +258,11 @@ __global__ void decompress_e4m3_kernel(ssconv_desc_t d, Geometry geo, const uint
 // patterns and writes 2 x 16 bytes of values; the eight threads of a row and stage write 128 bytes.  Values and
 // metadata in one launch: a layer's weights are small (0.1 to 2 MB), so a launch more costs as much as the work
 // (52 layers of a ResNet-50: 154 + 120 us for the two kernels with one thread per group, 180 us for this one).
-__global__ void __launch_bounds__(256) compress_kernel(ssconv_desc_t d, Geometry geo, const uint4* __restrict__ w,
-                                                       const uint8_t* __restrict__ pattern, uint4* __restrict__ w_comp,
-                                                       uint32_t* __restrict__ meta) {
+__global__ void __launch_bounds__(256) compress_kernel(ssconv_desc_t d, Geometry geo, const uint4* w, const uint8_t* pattern,
+                                                       uint4* w_comp, uint32_t* meta) {
+  grid_launch_dependents();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  grid_dependency_wait();
   if (t >= (int64_t)geo.m_tiles * geo.stages * 512) return;
   const int half = (int)(t & 1), j = (int)(t >> 1) & 3, row = ((int)(t >> 3) & 7) + 16 * ((int)(t >> 6) & 7);
   const int64_t tile = t >> 9;  // (channel tile, stage)
@@ -269,13 +280,13 @@ __global__ void __launch_bounds__(256) compress_kernel(ssconv_desc_t d, Geometry
     if (co < d.C_out && b < geo.kblocks && c < d.C_in) {
       const int64_t g = ((int64_t)co * geo.taps + tap) * (d.C_in / 4) + c / 4;
       const bool all = c + 8 < d.C_in;  // (input channels come in multiples of eight)
-      const uint4 lo = __ldg(w + g / 2);
-      const uint4 hi = all ? __ldg(w + g / 2 + 1) : make_uint4(0u, 0u, 0u, 0u);
+      const uint4 lo = w[g / 2];
+      const uint4 hi = all ? w[g / 2 + 1] : make_uint4(0u, 0u, 0u, 0u);
       const uint2 v[4] = {make_uint2(lo.x, lo.y), make_uint2(lo.z, lo.w), make_uint2(hi.x, hi.y), make_uint2(hi.z, hi.w)};
       codes = 0;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const uint32_t code = (i < 2 || all) ? pattern_code(__ldg(pattern + g + i)) : 0x4u;
+        const uint32_t code = (i < 2 || all) ? pattern_code(pattern[g + i]) : 0x4u;
         codes |= code << (4 * i);
         // bytes 2 p, 2 p + 1 of the group for each kept position p
         const uint32_t p0 = code & 3u, p1 = code >> 2;
@@ -332,12 +343,10 @@ cudaError_t launch_select(int mode, const void* scores, int64_t G, uint8_t* patt
   const int T = 256;
   count_launch();
   if (mode == SSCONV_MASK_LOGITS_F32)
-    select_logits_kernel<<<blocks_for(G, T), T, 0, st>>>((const float2*)scores, G, pattern);
-  else if (mode == SSCONV_MASK_MAGNITUDE_E4M3)
-    select_magnitude_e4m3_kernel<<<blocks_for(G, T), T, 0, st>>>((const uint32_t*)scores, G, pattern);
-  else
-    select_magnitude_kernel<<<blocks_for(G, T), T, 0, st>>>((const uint2*)scores, G, pattern);
-  return cudaGetLastError();
+    return launch_dependent(select_logits_kernel, blocks_for(G, T), T, st, (const float2*)scores, G, pattern);
+  if (mode == SSCONV_MASK_MAGNITUDE_E4M3)
+    return launch_dependent(select_magnitude_e4m3_kernel, blocks_for(G, T), T, st, (const uint32_t*)scores, G, pattern);
+  return launch_dependent(select_magnitude_kernel, blocks_for(G, T), T, st, (const uint2*)scores, G, pattern);
 }
 
 // All N-subsets of {0..M-1} in lexicographic order of the kept positions, as bitmasks.
@@ -393,9 +402,8 @@ cudaError_t launch_quantize_e4m3(const void* x, void* y, int64_t n, float scale,
   count_launch();
   const bool wide = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u) == 0;
   const int64_t pairs = n / 2, vectors = wide ? n / 16 : 0;
-  quantize_e4m3_kernel<<<blocks_for(vectors + (pairs - 8 * vectors), T), T, 0, st>>>((const uint32_t*)x, (uint16_t*)y, vectors,
-                                                                                    pairs, scale);
-  return cudaGetLastError();
+  return launch_dependent(quantize_e4m3_kernel, blocks_for(vectors + (pairs - 8 * vectors), T), T, st, (const uint32_t*)x,
+                          (uint16_t*)y, vectors, pairs, scale);
 }
 
 cudaError_t launch_compress_e4m3(const ssconv_desc_t& d, const void* w, const uint8_t* pattern, void* w_comp, void* meta,
@@ -429,9 +437,8 @@ cudaError_t launch_compress(const ssconv_desc_t& d, const void* w, const uint8_t
   Geometry geo = make_geometry(d);
   const int T = 256;
   count_launch();
-  compress_kernel<<<blocks_for((int64_t)geo.m_tiles * geo.stages * 512, T), T, 0, st>>>(
-      d, geo, (const uint4*)w, pattern, (uint4*)w_comp, (uint32_t*)meta);
-  return cudaGetLastError();
+  return launch_dependent(compress_kernel, blocks_for((int64_t)geo.m_tiles * geo.stages * 512, T), T, st, d, geo, (const uint4*)w,
+                          pattern, (uint4*)w_comp, (uint32_t*)meta);
 }
 
 cudaError_t launch_decompress(const ssconv_desc_t& d, const void* w_comp, const void* meta, void* w_out,

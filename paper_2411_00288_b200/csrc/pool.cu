@@ -10,28 +10,12 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "layout.cuh"
 #include "sm100_ptx.cuh"
 #include "ssconv.h"
 
 namespace ssconv {
-
-// Launch with programmatic stream serialisation, for kernels that call grid_dependency_wait() before their first access
-// to global memory (by plain loads: read-only ones could be moved above the wait): the launch and the index arithmetic
-// overlap the tail of the grid before.
-template <class... Params, class... Args>
-static cudaError_t launch_dependent(void (*kernel)(Params...), unsigned grid, unsigned threads, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(threads);
-  cfg.stream = st;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
-}
 
 __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
   __nv_bfloat162 x = *reinterpret_cast<__nv_bfloat162*>(&a);

@@ -2,10 +2,13 @@
 // group (Eq. 3), the soft mask block b = D z (Eq. 2 with that z), the effective weights
 // M .* W (Eq. 6 with the soft mask) that the dense convolution then uses, and the gradient
 // from dL/dW_eff back to the choice weights.  One thread per group of four weights; both
-// kernels move 70-90 bytes per group and do a handful of flops: HBM-bound.
+// kernels move 70-90 bytes per group and do a handful of flops: HBM-bound, or, on most layers, too short to be bound by
+// anything but their launches: the kernels of a step start while the one before them finishes (launch_dependent).
 #include <cuda_runtime.h>
 
+#include "launch.cuh"
 #include "layout.cuh"
+#include "sm100_ptx.cuh"
 #include "ssconv.h"
 
 namespace ssconv {
@@ -39,10 +42,11 @@ __device__ __forceinline__ uint32_t f32_pair_to_bf16(float lo, float hi) {
 
 // Eq. 3 in fp32: z = softmax((logits + noise) / tau), evaluated with the maximum subtracted
 // (which cancels in the quotient); then b = D z and W_eff = b .* W rounded once to bf16.
-__global__ void soft_mask_kernel(const float* __restrict__ logits, const float* __restrict__ noise, float inv_tau,
-                                 const uint2* __restrict__ w, int64_t G, float* __restrict__ z_out,
-                                 uint2* __restrict__ w_eff) {
+__global__ void soft_mask_kernel(const float* logits, const float* noise, float inv_tau, const uint2* w, int64_t G,
+                                 float* z_out, uint2* w_eff) {
+  grid_launch_dependents();
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  grid_dependency_wait();
   if (g >= G) return;
   float s[6];
   load6(logits, g, s);
@@ -78,9 +82,11 @@ __global__ void soft_mask_kernel(const float* __restrict__ logits, const float* 
 
 // Chain rule from G = dL/dW_eff to the choice weights: dL/db_j = G_j W_j, dL/dz_i = the sum of
 // dL/db over the two positions pattern i keeps, dL/dlogit_i = z_i (dL/dz_i - sum_k z_k dL/dz_k) / tau.
-__global__ void mask_grad_kernel(const float* __restrict__ z_in, float inv_tau, const uint2* __restrict__ w,
-                                 const float4* __restrict__ g_w_eff, int64_t G, float* __restrict__ g_logits) {
+__global__ void mask_grad_kernel(const float* z_in, float inv_tau, const uint2* w, const float4* g_w_eff, int64_t G,
+                                 float* g_logits) {
+  grid_launch_dependents();
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  grid_dependency_wait();
   if (g >= G) return;
   float z[6];
   load6(z_in, g, z);
@@ -108,11 +114,12 @@ __device__ __forceinline__ void adamw_one(float& t, float g, float& m, float& v,
   t = t - lr * (m * c1 / (sqrtf(v * c2) + eps) + wd * t);
 }
 // Four elements per thread (16-byte accesses); the last n % 4 elements are handled one by one.
-__global__ void adamw_kernel(float* __restrict__ theta, const float* __restrict__ g, float* __restrict__ m,
-                             float* __restrict__ v, int64_t n, float lr, float beta1, float beta2, float eps,
-                             float wd, float c1, float c2) {
+__global__ void adamw_kernel(float* theta, const float* g, float* m, float* v, int64_t n, float lr, float beta1, float beta2,
+                             float eps, float wd, float c1, float c2) {
+  grid_launch_dependents();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t n4 = n >> 2;
+  grid_dependency_wait();
   if (i < n4) {
     float4 t = reinterpret_cast<float4*>(theta)[i];
     const float4 gi = reinterpret_cast<const float4*>(g)[i];
@@ -138,10 +145,9 @@ cudaError_t launch_adamw(float* theta, const float* g, float* m, float* v, int64
                          float beta2, float eps, float wd, float c1, float c2, cudaStream_t st) {
   const int threads = 256;
   const int64_t work = (n >> 2) + (n & 3);
-  adamw_kernel<<<(unsigned)((work + threads - 1) / threads), threads, 0, st>>>(theta, g, m, v, n, lr, beta1, beta2,
-                                                                                 eps, wd, c1, c2);
   count_launch();
-  return cudaGetLastError();
+  return launch_dependent(adamw_kernel, (unsigned)((work + threads - 1) / threads), threads, st, theta, g, m, v, n, lr, beta1,
+                          beta2, eps, wd, c1, c2);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -318,11 +324,12 @@ __global__ void __launch_bounds__(256) dgrad_class_weights_kernel(const uint16_t
 //   w_all[k C_in + ci][u_h][u_w][co] = w[co][a + (Jh - 1 - u_h) s_h][b + (Jw - 1 - u_w) s_w][ci]  (0 past KH, KW).
 // One launch instead of s_h s_w small ones; the zero taps cost multiply-adds (16 tap-classes for the 9
 // taps of a 3x3 stride-2 layer, against 36 for the zero-spread form).
-__global__ void __launch_bounds__(256) dgrad_fused_weights_kernel(const uint16_t* __restrict__ w, uint16_t* __restrict__ w_all,
+__global__ void __launch_bounds__(256) dgrad_fused_weights_kernel(const uint16_t* w, uint16_t* w_all,
                                                                   int C_out, int KH, int KW, int C_in, int Jh, int Jw,
                                                                   int sh, int sw) {
   // A block transposes one 32 (ci) x 32 (co) tile of one (class, tap): reads run along ci, writes along co.
   __shared__ uint16_t tile[32][33];
+  grid_launch_dependents();
   int z = blockIdx.z;
   const int uw = z % Jw;
   z /= Jw;
@@ -333,6 +340,7 @@ __global__ void __launch_bounds__(256) dgrad_fused_weights_kernel(const uint16_t
   const bool tap = kh < KH && kw < KW;
   const int ci0 = blockIdx.x * 32, co0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
+  grid_dependency_wait();
 #pragma unroll
   for (int r = ty; r < 32; r += 8) {
     const int co = co0 + r, ci = ci0 + tx;
@@ -351,10 +359,9 @@ cudaError_t launch_dgrad_fused_weights(const void* w, void* w_all, int C_out, in
                                        int sh, int sw, cudaStream_t st) {
   if (C_in == 0 || C_out == 0) return cudaSuccess;
   const dim3 grid((unsigned)((C_in + 31) / 32), (unsigned)((C_out + 31) / 32), (unsigned)(sh * sw * Jh * Jw));
-  dgrad_fused_weights_kernel<<<grid, 256, 0, st>>>((const uint16_t*)w, (uint16_t*)w_all, C_out, KH, KW, C_in, Jh, Jw, sh,
-                                                   sw);
   count_launch();
-  return cudaGetLastError();
+  return launch_dependent(dgrad_fused_weights_kernel, grid, 256, st, (const uint16_t*)w, (uint16_t*)w_all, C_out, KH, KW, C_in,
+                          Jh, Jw, sh, sw);
 }
 
 cudaError_t launch_dgrad_class_weights(const void* w, void* w_c, int C_out, int KH, int KW, int C_in, int a, int b,
@@ -371,9 +378,11 @@ cudaError_t launch_dgrad_class_weights(const void* w, void* w_c, int C_out, int 
 // padded position; zero for a class without taps and beyond a class tensor's extent (no filter placement
 // reaches those pixels).  `pitch8` = 16-byte units between pixels of a class tensor (C_in / 8, or the
 // channels of all classes when they share one tensor).  One thread per 16 bytes of dx.
-__global__ void __launch_bounds__(256) dgrad_gather_kernel(DgradClasses cls, uint4* __restrict__ dx, long long total, int H,
+__global__ void __launch_bounds__(256) dgrad_gather_kernel(DgradClasses cls, uint4* dx, long long total, int H,
                                                            int W, int C8, int pitch8, int sh, int sw, int ph, int pw) {
+  grid_launch_dependents();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  grid_dependency_wait();
   if (i >= total) return;
   const int c = (int)(i % C8);
   long long r = i / C8;
@@ -387,7 +396,7 @@ __global__ void __launch_bounds__(256) dgrad_gather_kernel(DgradClasses cls, uin
   uint4 v = make_uint4(0u, 0u, 0u, 0u);
   const uint4* t = static_cast<const uint4*>(cls.t[k]);
   if (t != nullptr && ih < cls.rows[k] && iw < cls.cols[k])
-    v = __ldg(t + ((n * cls.rows[k] + ih) * cls.cols[k] + iw) * pitch8 + c);
+    v = t[((n * cls.rows[k] + ih) * cls.cols[k] + iw) * pitch8 + c];
   dx[i] = v;
 }
 
@@ -395,30 +404,27 @@ cudaError_t launch_dgrad_gather(const DgradClasses& cls, void* dx, int N, int H,
                                 int ph, int pw, cudaStream_t st) {
   const long long total = (long long)N * H * W * (C / 8);
   if (total == 0) return cudaSuccess;
-  dgrad_gather_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(cls, (uint4*)dx, total, H, W, C / 8, pitch / 8, sh,
-                                                                       sw, ph, pw);
   count_launch();
-  return cudaGetLastError();
+  return launch_dependent(dgrad_gather_kernel, (unsigned)((total + 255) / 256), 256, st, cls, (uint4*)dx, total, H, W, C / 8,
+                          pitch / 8, sh, sw, ph, pw);
 }
 
 cudaError_t launch_soft_mask(const float* logits, const float* noise, float tau, const void* w, int64_t G, float* z,
                              void* w_eff, cudaStream_t st) {
   const int threads = 256;
   const int64_t blocks = (G + threads - 1) / threads;
-  soft_mask_kernel<<<(unsigned)blocks, threads, 0, st>>>(logits, noise, 1.0f / tau, (const uint2*)w, G, z,
-                                                         (uint2*)w_eff);
   count_launch();
-  return cudaGetLastError();
+  return launch_dependent(soft_mask_kernel, (unsigned)blocks, threads, st, logits, noise, 1.0f / tau, (const uint2*)w, G, z,
+                          (uint2*)w_eff);
 }
 
 cudaError_t launch_mask_grad(const float* z, float tau, const void* w, const float* g_w_eff, int64_t G,
                              float* g_logits, cudaStream_t st) {
   const int threads = 256;
   const int64_t blocks = (G + threads - 1) / threads;
-  mask_grad_kernel<<<(unsigned)blocks, threads, 0, st>>>(z, 1.0f / tau, (const uint2*)w, (const float4*)g_w_eff, G,
-                                                         g_logits);
   count_launch();
-  return cudaGetLastError();
+  return launch_dependent(mask_grad_kernel, (unsigned)blocks, threads, st, z, 1.0f / tau, (const uint2*)w,
+                          (const float4*)g_w_eff, G, g_logits);
 }
 
 }  // namespace ssconv

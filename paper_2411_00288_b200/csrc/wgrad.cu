@@ -27,6 +27,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "launch.cuh"
 #include "layout.cuh"
 #include "sm100_ptx.cuh"
 #include "ssconv.h"
@@ -122,6 +123,7 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
       fence_proxy_async_smem();
       prefetch_tensormap(&tm_dy);
       prefetch_tensormap(&tm_x);
+      grid_launch_dependents();   // (the adding kernel waits for this grid's completion itself)
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -142,6 +144,7 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
     const int role = (warp == 0) ? 0 : warp - 5;
     if (lane == 0 && role < (int)producers) {
       uint32_t s = 0, ph = 0;
+      grid_dependency_wait();   // everything above may overlap the tail of the kernel before this one
       for (int ks = item.ks0; ks < item.ks1; ++ks) {
         if (!mbar_wait_a(empty0 + 8u * s, ph ^ 1u, abort_flag, kWgWaitLimitCycles)) break;
         const uint32_t full = full0 + 8u * s;
@@ -213,6 +216,7 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
     const bool got = mbar_wait_warp(bar_acc, 0u, abort_flag, kWgWaitLimitCycles, 64);
     if (got) {
       tc_fence_after();
+      grid_dependency_wait();
       const size_t K = (size_t)p.taps * p.C_in;
       float* out = p.out + ((size_t)item.split * p.m_tiles + item.m) * K * kTileM + qd * 32 + lane;
       for (int t = 0; t < item.nb; ++t) {
@@ -484,8 +488,8 @@ ssconv_wgrad_pair_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid
 }
 
 // dW = the sum, in slice order, of `splits` slices of the same layout (four elements per thread).
-__global__ void __launch_bounds__(256) wgrad_sum_kernel(const float4* __restrict__ slices, int splits, size_t slice_vec,
-                                                        float4* __restrict__ dw) {
+__global__ void __launch_bounds__(256) wgrad_sum_kernel(const float4* slices, int splits, size_t slice_vec, float4* dw) {
+  grid_launch_dependents();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   grid_dependency_wait();   // launched while the kernel that writes the slices is still running
   if (i >= slice_vec) return;
@@ -504,12 +508,13 @@ __global__ void __launch_bounds__(256) wgrad_sum_kernel(const float4* __restrict
 // of 32 x 8 threads handles 32 output channels x 8 columns of K, one element per thread: reads are
 // contiguous along the output channels, writes go out as 32-byte runs along K.  With many slices
 // the sums are latency-bound, hence the small tiles (many blocks) and eight loads in flight.
-__global__ void wgrad_reduce_kernel(const float* __restrict__ slices, int splits, int K, int C_out, int m_tiles,
-                                    float* __restrict__ dw) {
+__global__ void wgrad_reduce_kernel(const float* slices, int splits, int K, int C_out, int m_tiles, float* dw) {
   __shared__ float tile[8][33];
+  grid_launch_dependents();
   const int k0 = blockIdx.x * 8, c0 = blockIdx.y * 32;
   const size_t slice = (size_t)m_tiles * K * kTileM;
   const int c = c0 + threadIdx.x, k = k0 + threadIdx.y;
+  grid_dependency_wait();
   float acc = 0.0f;
   if (k < K && c < C_out) {
     const float* src = slices + ((size_t)(c / kTileM) * K + k) * kTileM + (c % kTileM);
@@ -867,16 +872,16 @@ int32_t launch_wgrad(const ssconv_desc_t& d, const void* x, const void* dy, floa
   p.dev_status = dev_status;
 
   const unsigned grid = (unsigned)(w.splits * w.m_tiles * w.items_b);
-  ssconv_wgrad_kernel<<<grid, kWgThreads, kWgSmemBytes, stream>>>(tm_dy, tm_x, p);
   count_launch();
-  if (cudaGetLastError() != cudaSuccess) return SSCONV_ERR_CUDA;
+  if (launch_dependent_smem(ssconv_wgrad_kernel, grid, kWgThreads, kWgSmemBytes, stream, tm_dy, tm_x, p) != cudaSuccess)
+    return SSCONV_ERR_CUDA;
   {
     const int K = w.taps * d.C_in;
     const dim3 rgrid((unsigned)((K + 7) / 8), (unsigned)((d.C_out + 31) / 32));
-    wgrad_reduce_kernel<<<rgrid, dim3(32, 8), 0, stream>>>(static_cast<const float*>(ws), w.splits, K, d.C_out,
-                                                           w.m_tiles, dw);
     count_launch();
-    if (cudaGetLastError() != cudaSuccess) return SSCONV_ERR_CUDA;
+    if (launch_dependent(wgrad_reduce_kernel, rgrid, dim3(32, 8), stream, static_cast<const float*>(ws), w.splits, K, d.C_out,
+                         w.m_tiles, dw) != cudaSuccess)
+      return SSCONV_ERR_CUDA;
   }
   return SSCONV_OK;
 }
