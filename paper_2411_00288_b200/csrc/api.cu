@@ -16,7 +16,8 @@ int32_t launch_forward_sparse(const ssconv_desc_t& d, const void* x, const void*
                               int32_t* dev_status, cudaStream_t stream);
 int32_t launch_forward_dense(const ssconv_desc_t& d, const void* x, const void* w, const float* bias,
                              const void* residual, void* y, void* ws, size_t ws_bytes, int32_t* dev_status,
-                             cudaStream_t stream, const int64_t* x_strides = nullptr);
+                             cudaStream_t stream, const int64_t* x_strides = nullptr, bool gradient_weights = false);
+bool takes_gradient_weights(const ssconv_desc_t& d);
 cudaError_t launch_space_to_depth(const void* x, void* y, int N, int H, int W, int C, int s, int pad, int Hb, int Wb,
                                   int C_pad, cudaStream_t st);
 int32_t plan_query_sms(const ssconv_desc_t& d, bool sparse, int sm_count, int32_t* bn, int32_t* split, int32_t* ctas,
@@ -892,6 +893,9 @@ int32_t ssconv_dgrad(const ssconv_desc_t* desc, const void* dy, const void* w_bf
     c.pad_w = d.dil_w * (d.KW - 1) - d.pad_w;
     rc = check_desc(&c, true);
     if (rc != SSCONV_OK) return rc;
+    if (ssconv::takes_gradient_weights(c))
+      return ssconv::launch_forward_dense(c, dy, w_bf16, nullptr, nullptr, dx, base + p.fwd_off, p.fwd_bytes, dev_status, st,
+                                          nullptr, true);
     // (the reversed, channel-exchanged filter = the one class of a unit stride, written by the tiled transpose)
     if (ssconv::launch_dgrad_fused_weights(w_bf16, base, d.C_out, d.KH, d.KW, d.C_in, d.KH, d.KW, 1, 1, st) != cudaSuccess)
       return SSCONV_ERR_CUDA;
@@ -904,13 +908,15 @@ int32_t ssconv_dgrad(const ssconv_desc_t* desc, const void* dy, const void* w_bf
     c.pad_w = d.dil_w * (d.KW - 1) - d.pad_w;
     rc = check_desc(&c, true);
     if (rc != SSCONV_OK) return rc;
-    if (ssconv::launch_dgrad_fused_weights(w_bf16, base, d.C_out, d.KH, d.KW, d.C_in, d.KH, d.KW, 1, 1, st) != cudaSuccess)
+    const bool as_they_are = ssconv::takes_gradient_weights(c);
+    if (!as_they_are &&
+        ssconv::launch_dgrad_fused_weights(w_bf16, base, d.C_out, d.KH, d.KW, d.C_in, d.KH, d.KW, 1, 1, st) != cudaSuccess)
       return SSCONV_ERR_CUDA;
     if (ssconv::launch_dgrad_spread(dy, base + p.spread_off, d.N, p.Ho, p.Wo, d.C_out, p.Hz, p.Wz, d.stride_h, d.stride_w,
                                     st) != cudaSuccess)
       return SSCONV_ERR_CUDA;
-    return ssconv::launch_forward_dense(c, base + p.spread_off, base, nullptr, nullptr, dx, base + p.fwd_off, p.fwd_bytes,
-                                        dev_status, st);
+    return ssconv::launch_forward_dense(c, base + p.spread_off, as_they_are ? w_bf16 : base, nullptr, nullptr, dx,
+                                        base + p.fwd_off, p.fwd_bytes, dev_status, st, nullptr, as_they_are);
   }
   ssconv::DgradClasses cls;
   for (int k = 0; k < ssconv::kMaxDgradClasses; ++k) {

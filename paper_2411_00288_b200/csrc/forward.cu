@@ -119,6 +119,9 @@ struct FwdParams {
                             // two sets of epilogue groups)
   int small_c;              // dense layers with C_in == 8: a k-block is 8 filter taps (see producer_role)
   uint32_t a_grp_bytes;     // bytes of weights (and metadata) at the head of a ring group; 0: weights resident
+  int a_mn;                 // dense: the weights are those of the layer whose input gradient this convolution computes,
+                            // w[input channel][reversed tap][output channel]: tiles with the output channels in rows
+                            // of 128 bytes (MN-major), 64 input channels deep
   uint32_t a_res_bytes;     // dense layers of one channel tile and at most four k-blocks: the whole weight
                             // tile stays in shared memory after the ring (loaded once per CTA), groups hold
                             // activations only
@@ -408,6 +411,29 @@ struct TapIter {
   }
 };
 
+// One k-block of dense weights (64 input channels at one tap, 128 output channels from a_row on) -> 16 KB at dst.
+// As stored for this layer: 128 rows of 64 input channels.  Read from the weights of the layer whose input gradient this
+// is (a_mn): two blocks of 64 output channels, each 64 rows (input channels), which the MMAs take as a transposed operand.
+// That saves writing the exchanged and reversed weights first: 3 x 3 training step at 256 channels, batch 64 69.7 -> 64.7 us.
+__device__ __forceinline__ void load_dense_weights(const CUtensorMap* tm_a, const FwdParams& p, uint32_t dst, uint32_t full,
+                                                   int c0, int tap, int a_row) {
+  if (p.a_mn) {
+    tma_load_3d_w(dst, tm_a, full, a_row, p.taps - 1 - tap, c0);
+    tma_load_3d_w(dst + kATileBytes / 2, tm_a, full, a_row + 64, p.taps - 1 - tap, c0);
+  } else {
+    tma_load_3d_w(dst, tm_a, full, c0, tap, a_row);
+  }
+}
+// What an MN-major A tile changes for the issuing warp: the distance of the two blocks of 64 output channels in the
+// descriptor (K-major tiles have 1 there), the step of 16 input channels (16 rows of 128 bytes instead of 32 bytes along
+// a row) and a bit of the instruction descriptor.
+struct DenseA {
+  uint32_t lo_add, step, idesc_bits;
+  __device__ explicit DenseA(const FwdParams& p)
+      : lo_add(p.a_mn ? (((kATileBytes / 2) >> 4) - 1u) << 16 : 0u), step(p.a_mn ? 2048u >> 4 : 2u),
+        idesc_bits(p.a_mn ? 1u << 15 : 0u) {}
+};
+
 // One of the three TMA producer warps.  All of them walk the same sequence of groups; role 0
 // loads the activation tile of each group's first k-block, role 1 that of the second, role 2 the
 // weights (with their metadata).  A TMA instruction occupies its issuing thread for a few hundred
@@ -451,7 +477,7 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
         TapIter rit;
         rit.init(0, p);
         for (int b = 0; b < p.kblocks; ++b) {
-          tma_load_3d_w(res0 + (uint32_t)b * kATileBytes, tm_a, res_bar, rit.cc * kKb, rit.tap, a_row);
+          load_dense_weights(tm_a, p, res0 + (uint32_t)b * kATileBytes, res_bar, rit.cc * kKb, rit.tap, a_row);
           rit.advance(p);
         }
       }
@@ -502,9 +528,9 @@ __device__ __forceinline__ void producer_role(const CUtensorMap* tm_a, const CUt
           meta_src += C::kMetaBytes;
         } else {
           mbar_expect_tx_w(full, has_second ? 2 * kATileBytes : kATileBytes);
-          tma_load_3d_w(dst, tm_a, full, it.cc * kKb, it.tap, a_row);
+          load_dense_weights(tm_a, p, dst, full, it.cc * kKb, it.tap, a_row);
           it.advance(p);
-          if (has_second) tma_load_3d_w(dst + kATileBytes, tm_a, full, it.cc * kKb, it.tap, a_row);
+          if (has_second) load_dense_weights(tm_a, p, dst + kATileBytes, full, it.cc * kKb, it.tap, a_row);
           it.advance(p);
         }
       } else if (ROLE == kRoleActFirst || has_second) {
@@ -635,8 +661,9 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
     // All 32 lanes run this loop in lock step and wait on the barriers together; the tcgen05
     // instructions are issued by one elected lane (see the warp-wide forms in sm100_ptx.cuh).
     {
+      const DenseA da(p);
       const uint32_t idesc = FP8 ? make_idesc_e4m3(kTileM, (uint32_t)p.BN, SPARSE)
-                                 : make_idesc_bf16(kTileM, (uint32_t)p.BN, SPARSE);
+                                 : make_idesc_bf16(kTileM, (uint32_t)p.BN, SPARSE) | (SPARSE ? 0u : da.idesc_bits);
       constexpr int kKb = C::kKbChannels;
       // descriptor address units are 16 B
       const uint32_t grp_desc = (p.a_grp_bytes + 2u * (uint32_t)p.BN * 128u) >> 4;
@@ -748,24 +775,24 @@ ssconv_fwd_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constan
               if (kEarly) tc_commit_w(empty_first0 + 8u * g);
               for (int kk = 0; kk < n1; ++kk) tc_mma_f8_dense_w(d_tmem, a1_lo + 2u * kk, b1_lo + 2u * kk, idesc, 1u);
             } else {
-              const uint32_t a1_lo = a_lo + (kATileBytes >> 4);
+              const uint32_t w0_lo = a_lo + da.lo_add, a1_lo = w0_lo + (kATileBytes >> 4), st = da.step;
               if (a < a_lean_end) {
-                tc_mma_dense_w(d_tmem, a_lo, b0_lo, idesc, accumulate);
-                tc_mma_dense_w(d_tmem, a_lo + 2u, b0_lo + 2u, idesc, 1u);
-                tc_mma_dense_w(d_tmem, a_lo + 4u, b0_lo + 4u, idesc, 1u);
-                tc_mma_dense_w(d_tmem, a_lo + 6u, b0_lo + 6u, idesc, 1u);
+                tc_mma_dense_w(d_tmem, w0_lo, b0_lo, idesc, accumulate);
+                tc_mma_dense_w(d_tmem, w0_lo + st, b0_lo + 2u, idesc, 1u);
+                tc_mma_dense_w(d_tmem, w0_lo + 2u * st, b0_lo + 4u, idesc, 1u);
+                tc_mma_dense_w(d_tmem, w0_lo + 3u * st, b0_lo + 6u, idesc, 1u);
                 if (kEarly) tc_commit_w(empty_first0 + 8u * g);
                 tc_mma_dense_w(d_tmem, a1_lo, b1_lo, idesc, 1u);
-                tc_mma_dense_w(d_tmem, a1_lo + 2u, b1_lo + 2u, idesc, 1u);
-                tc_mma_dense_w(d_tmem, a1_lo + 4u, b1_lo + 4u, idesc, 1u);
-                tc_mma_dense_w(d_tmem, a1_lo + 6u, b1_lo + 6u, idesc, 1u);
+                tc_mma_dense_w(d_tmem, a1_lo + st, b1_lo + 2u, idesc, 1u);
+                tc_mma_dense_w(d_tmem, a1_lo + 2u * st, b1_lo + 4u, idesc, 1u);
+                tc_mma_dense_w(d_tmem, a1_lo + 3u * st, b1_lo + 6u, idesc, 1u);
               } else {
                 const int n0 = (2 * a >= tail_start) ? mma_tail : mma_full;
                 const int n1 = (2 * a + 1 >= p.kblocks) ? 0 : ((2 * a + 1 >= tail_start) ? mma_tail : mma_full);
                 for (int kk = 0; kk < n0; ++kk)
-                  tc_mma_dense_w(d_tmem, a_lo + 2u * kk, b0_lo + 2u * kk, idesc, (kk > 0) ? 1u : accumulate);
+                  tc_mma_dense_w(d_tmem, w0_lo + st * kk, b0_lo + 2u * kk, idesc, (kk > 0) ? 1u : accumulate);
                 if (kEarly) tc_commit_w(empty_first0 + 8u * g);
-                for (int kk = 0; kk < n1; ++kk) tc_mma_dense_w(d_tmem, a1_lo + 2u * kk, b1_lo + 2u * kk, idesc, 1u);
+                for (int kk = 0; kk < n1; ++kk) tc_mma_dense_w(d_tmem, a1_lo + st * kk, b1_lo + 2u * kk, idesc, 1u);
               }
             }
             accumulate = 1;
@@ -1229,7 +1256,8 @@ ssconv_fwd_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid
     producer_role<SPARSE, kRoleWeights>(&tm_a, &tm_b, p, full0, empty0, ring0, 0u, abort_flag, share);
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (as in the one-CTA kernel)
-    const uint32_t idesc = make_idesc_bf16(kTileM, (uint32_t)p.BN, SPARSE);
+    const DenseA da(p);
+    const uint32_t idesc = make_idesc_bf16(kTileM, (uint32_t)p.BN, SPARSE) | (SPARSE ? 0u : da.idesc_bits);
     const uint32_t grp_desc = (p.a_grp_bytes + 2u * b_bytes) >> 4, b_desc = b_bytes >> 4;
     const uint32_t ring_lo0 = desc_lo(ring0);
     const int tail_c = p.C_in - (p.cblocks - 1) * kBlockK;
@@ -1255,10 +1283,10 @@ ssconv_fwd_cluster_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid
         if (n1 > 0) tc_mma_sparse_w(tmem_base, a_lo + 4u, b1_lo, meta_tmem + 2u, idesc, 1u);
         if (n1 > 1) tc_mma_sparse_w(tmem_base, a_lo + 6u, b1_lo + 4u, meta_tmem + 2u, idesc | 1u, 1u);
       } else {
-        const uint32_t a1_lo = a_lo + (kATileBytes >> 4);
+        const uint32_t w0_lo = a_lo + da.lo_add, a1_lo = w0_lo + (kATileBytes >> 4);
         for (int kk = 0; kk < n0; ++kk)
-          tc_mma_dense_w(tmem_base, a_lo + 2u * kk, b0_lo + 2u * kk, idesc, (kk > 0) ? 1u : accumulate);
-        for (int kk = 0; kk < n1; ++kk) tc_mma_dense_w(tmem_base, a1_lo + 2u * kk, b1_lo + 2u * kk, idesc, 1u);
+          tc_mma_dense_w(tmem_base, w0_lo + da.step * kk, b0_lo + 2u * kk, idesc, (kk > 0) ? 1u : accumulate);
+        for (int kk = 0; kk < n1; ++kk) tc_mma_dense_w(tmem_base, a1_lo + da.step * kk, b1_lo + 2u * kk, idesc, 1u);
       }
       accumulate = 1;
       tc_commit_w(empty0 + 8u * g);
@@ -1413,10 +1441,17 @@ __device__ __forceinline__ void pair_producer_role(const CUtensorMap* tm_a, cons
           tma2_load_2d_w(dst + kATileBytes, tm_meta, full, 0, (m_meta * p.a_tiles + a) * (int)(C::kMetaBytes / kMetaImageBytes));
         } else {
           if (leader) mbar_expect_tx_w(full0_local + 8u * g, (has_second ? 4u : 2u) * kATileBytes);
-          tma2_load_3d_w(dst, tm_a, full, it.cc * kKb, it.tap, m * kTileM);
-          it.advance(p);
-          if (has_second) tma2_load_3d_w(dst + kATileBytes, tm_a, full, it.cc * kKb, it.tap, m * kTileM);
-          it.advance(p);
+          for (uint32_t b = 0; b < (has_second ? 2u : 1u); ++b) {
+            const uint32_t to = dst + b * kATileBytes;
+            if (p.a_mn) {
+              tma2_load_3d_w(to, tm_a, full, m * kTileM, p.taps - 1 - it.tap, it.cc * kKb);
+              tma2_load_3d_w(to + kATileBytes / 2, tm_a, full, m * kTileM + 64, p.taps - 1 - it.tap, it.cc * kKb);
+            } else {
+              tma2_load_3d_w(to, tm_a, full, it.cc * kKb, it.tap, m * kTileM);
+            }
+            it.advance(p);
+          }
+          if (!has_second) it.advance(p);
         }
       } else if (ROLE == kRoleActFirst || has_second) {
         if (leader) mbar_expect_tx_w(full0_local + 8u * g, 2u * tiles_per * half_bytes);
@@ -1532,8 +1567,9 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (leader CTA only)
     if (leader_cta) {
+      const DenseA da(p);
       const uint32_t idesc = FP8 ? make_idesc_e4m3(2 * kTileM, (uint32_t)p.BN, SPARSE)
-                                 : make_idesc_bf16(2 * kTileM, (uint32_t)p.BN, SPARSE);
+                                 : make_idesc_bf16(2 * kTileM, (uint32_t)p.BN, SPARSE) | (SPARSE ? 0u : da.idesc_bits);
       constexpr int kKb = C::kKbChannels;
       const uint32_t grp_desc = grp_bytes >> 4;
       const uint32_t half_desc = half_bytes >> 4;
@@ -1605,12 +1641,12 @@ ssconv_fwd_pair_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_co
               if (n1 > 1) tc2_mma_sparse_w(d_tmem1, a_lo + 6u, c1_lo + 4u, meta_tmem + 2u, idesc | 1u, 1u);
             }
           } else {
-            const uint32_t a1_lo = a_lo + (kATileBytes >> 4);
+            const uint32_t w0_lo = a_lo + da.lo_add, a1_lo = w0_lo + (kATileBytes >> 4);
             for (uint32_t t = 0; t < (dual ? 2u : 1u); ++t) {
               const uint32_t d = t ? d_tmem1 : d_tmem, tb = t * tile1_desc;
               for (int kk = 0; kk < n0; ++kk)
-                tc2_mma_dense_w(d, a_lo + 2u * kk, b0_lo + tb + 2u * kk, idesc, (kk > 0) ? 1u : accumulate);
-              for (int kk = 0; kk < n1; ++kk) tc2_mma_dense_w(d, a1_lo + 2u * kk, b1_lo + tb + 2u * kk, idesc, 1u);
+                tc2_mma_dense_w(d, w0_lo + da.step * kk, b0_lo + tb + 2u * kk, idesc, (kk > 0) ? 1u : accumulate);
+              for (int kk = 0; kk < n1; ++kk) tc2_mma_dense_w(d, a1_lo + da.step * kk, b1_lo + tb + 2u * kk, idesc, 1u);
             }
           }
           accumulate = 1;
@@ -2270,7 +2306,8 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
                                    const float* bias, const void* residual, void* y, void* ws, size_t ws_bytes,
                                    int32_t* dev_status, cudaStream_t stream, int worker_cap = kMaxWorkers,
                                    bool force_split = false, const int64_t* x_strides = nullptr,
-                                   float out_scale = 1.0f, int64_t y_pitch = 0, int groups = 1) {
+                                   float out_scale = 1.0f, int64_t y_pitch = 0, int groups = 1,
+                                   bool gradient_weights = false) {
   using C = Cfg<SPARSE, FP8>;
   constexpr int kKb = C::kKbChannels;
   constexpr size_t kElem = FP8 ? 1 : 2;  // bytes per operand element
@@ -2444,6 +2481,17 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
                                 box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                 CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
+  } else if (gradient_weights) {
+    // the weights [C_in][taps][C_out] of the layer whose input gradient this is, seen as (output channel, tap, input
+    // channel); two boxes of 64 output channels x 64 input channels per k-block (see load_dense_weights)
+    cuuint64_t dims[3] = {(cuuint64_t)d.C_out, (cuuint64_t)geo.taps, (cuuint64_t)d.C_in};
+    cuuint64_t strides[2] = {(cuuint64_t)d.C_out * 2, (cuuint64_t)geo.taps * d.C_out * 2};
+    cuuint32_t box[3] = {64, 1, 64};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = g_encode_tiled(&tm_a, kOperandType, 3, const_cast<void*>(weights), dims, strides, box, estr,
+                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
   } else {
     // dense weights [C_out][taps][C_in] seen as (c, tap, output channel); 8-channel mode: one tap's
     // 8 channels of 128 rows per load, unswizzled
@@ -2521,6 +2569,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   p.ring_groups = ring_groups;
   p.small_c = small_c ? 1 : 0;
   p.a_grp_bytes = a_grp_bytes;
+  p.a_mn = gradient_weights ? 1 : 0;
   p.a_res_bytes = a_res_bytes;
   p.stage_bufs = stage_bufs;
   p.stride_h = d.stride_h;
@@ -2653,10 +2702,13 @@ int32_t launch_forward_sparse(const ssconv_desc_t& d, const void* x, const void*
 }
 int32_t launch_forward_dense(const ssconv_desc_t& d, const void* x, const void* w, const float* bias,
                              const void* residual, void* y, void* ws, size_t ws_bytes, int32_t* dev_status,
-                             cudaStream_t stream, const int64_t* x_strides) {
+                             cudaStream_t stream, const int64_t* x_strides, bool gradient_weights) {
   return launch_forward_impl<false>(d, x, w, nullptr, bias, residual, y, ws, ws_bytes, dev_status, stream, kMaxWorkers,
-                                    false, x_strides);
+                                    false, x_strides, 1.0f, 0, 1, gradient_weights);
 }
+// Whether launch_forward_dense takes the weights of the layer whose input gradient `d` computes as they are (the 8-channel
+// mode cuts its k-blocks across taps).
+bool takes_gradient_weights(const ssconv_desc_t& d) { return !small_channel_mode(d, false); }
 
 // Groups of a grouped convolution in one launch: what the model says of all groups' tiles dealt out together
 // against one launch per group (each of which may split K or use pairs, and starts and drains by itself).  A group's last
