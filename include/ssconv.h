@@ -113,7 +113,8 @@ int32_t ssconv_plan(const ssconv_desc_t* desc, int32_t sparse, int32_t* tile_pos
  * SSCONV_TUNE_PAIR_TILES: -1 lets the planner choose (default) whether a work item of the pair kernel is two
  * neighbouring position tiles that share every group's weights, 0 never, 1 wherever the ring still holds two
  * groups (tiles of at most 192 positions keep three).  SSCONV_TUNE_DEPTHWISE_MMA: -1 (default) runs 7 x 7 depthwise
- * layers on the tensor cores where that is the faster way, 0 never (the fp32 kernels take them).
+ * layers on the tensor cores, or, on small maps, in the kernel made for those, where that is the faster way, 0 never (the
+ * fp32 kernels of other filters take them).  SSCONV_TUNE_DEPTHWISE_SMALL: 0 keeps small maps off the kernel made for them.
  * SSCONV_TUNE_CLUSTER: -1 lets the planner choose (default; with a tile width or pairs overridden: never) whether the CTAs
  * of a cluster share the K of each tile, 0 never, 2, 4 or 8 that many CTAs wherever the layer and the chip allow it.  Not
  * thread-safe against concurrent calls.  Returns SSCONV_ERR_BAD_DESC for an unknown option or a value
@@ -126,7 +127,8 @@ enum {
   SSCONV_TUNE_RESIDENT_WEIGHTS = 5,
   SSCONV_TUNE_PAIR_TILES = 6,
   SSCONV_TUNE_DEPTHWISE_MMA = 7,
-  SSCONV_TUNE_CLUSTER = 8
+  SSCONV_TUNE_CLUSTER = 8,
+  SSCONV_TUNE_DEPTHWISE_SMALL = 9
 };
 int32_t ssconv_tune(int32_t option, int32_t value);
 

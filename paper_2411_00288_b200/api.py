@@ -323,7 +323,7 @@ def ssconv_plan(desc: Desc, sparse: bool = True) -> dict:
 
 TUNE_TILE_POSITIONS, TUNE_PAIR, TUNE_WGRAD_RANGES, TUNE_WGRAD_PAIR, TUNE_RESIDENT_WEIGHTS, TUNE_PAIR_TILES = 1, 2, 3, 4, 5, 6
 TUNE_DEPTHWISE_MMA = 7
-TUNE_CLUSTER = 8
+TUNE_CLUSTER, TUNE_DEPTHWISE_SMALL = 8, 9
 
 
 def ssconv_tune(option: int, value: int) -> None:

@@ -44,6 +44,7 @@
 #include <atomic>
 #include <cstdint>
 
+#include "launch.cuh"
 #include "layout.cuh"
 #include "sm100_ptx.cuh"
 #include "ssconv.h"
@@ -523,10 +524,116 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
   }
 }
 
-static int g_tune_mma = -1;  // ssconv_tune: -1 automatic, 0 never this kernel
-int32_t set_depthwise_tuning(int32_t value) {
+// ---------------------------------------------------------------------------------------
+// Small maps
+// ---------------------------------------------------------------------------------------
+// A few images' maps give the kernel above one short run of rows per block: 9 us of start-up (six image rows before the first
+// output row, rows handed from role to role), whatever the map holds.  Here a block of 128 threads makes 4 x 8 outputs of 32
+// channels: all it needs, 10 x 14 pixels and the filter, is loaded at once (one latency), and a thread then computes four
+// neighbouring outputs of one pair of channels from shared memory with fp32 multiply-adds, a filter row at a time (each row a
+// chain of its own, added to the sum: rms error in the units above .109 / .469 / .448).  Bound by that one latency and 196
+// multiply-adds per thread while the blocks are resident at once; every pixel is loaded 4.4 times, so larger maps are not
+// for it.us between other
+// launches, tensor-core kernel / this one: 3 x 56 x 56 x 96 9.3 / 5.8, 3 x 28 x 28 x 192 8.8 / 4.5, 3 x 14 x 14 x 384 8.8 / 3.2,
+// 3 x 7 x 7 x 768 8.1 / 2.6; with 64 threads of eight outputs each 5.6, 4.5, 3.4, 3.3.
+constexpr int kDwSmallH = 4, kDwSmallW = 8, kDwSmallRun = 4;
+constexpr int kDwSmallThreads = 16 * kDwSmallH * (kDwSmallW / kDwSmallRun);
+constexpr int kDwSmallRows = kDwSmallH + kDw7K - 1, kDwSmallCols = kDwSmallW + kDw7K - 1;
+constexpr int kDwSmallPixel = 20;  // words from pixel to pixel: the two runs of a warp, four pixels apart, read different banks
+constexpr int kDwSmallSharedBytes = 4 * kDwSmallRows * kDwSmallCols * kDwSmallPixel + 8 * kDw7K * kDw7K * 16;
+template <bool RELU>
+__global__ void __launch_bounds__(kDwSmallThreads) depthwise7_small_kernel(const Dw7Params p, int tiles_h, int tiles_w) {
+  __shared__ __align__(16) uint32_t px[kDwSmallRows * kDwSmallCols * kDwSmallPixel];
+  __shared__ float2 w_s[kDw7K * kDw7K][16];
+  grid_launch_dependents();
+  const int t = threadIdx.x, C8 = p.C >> 3;
+  int tile = blockIdx.x;
+  const int tw = tile % tiles_w;
+  tile /= tiles_w;
+  const int th = tile % tiles_h;
+  const int n = tile / tiles_h;
+  const int h0 = th * kDwSmallH, w0 = tw * kDwSmallW;
+  const int c8 = blockIdx.y * (kDw7Channels / 8);
+  const uint4* x4 = reinterpret_cast<const uint4*>(p.x) + c8;
+  const uint4* w4 = reinterpret_cast<const uint4*>(p.w) + c8;
+  grid_dependency_wait();
+  constexpr int kVecs = kDwSmallRows * kDwSmallCols * 4, kLoads = (kVecs + kDwSmallThreads - 1) / kDwSmallThreads;
+  constexpr int kWVecs = kDw7K * kDw7K * 4, kWLoads = (kWVecs + kDwSmallThreads - 1) / kDwSmallThreads;
+  uint4 v[kLoads], wv[kWLoads];
+#pragma unroll
+  for (int j = 0; j < kLoads; ++j) {
+    const int i = t + j * kDwSmallThreads, pixel = i >> 2;
+    const int r = pixel / kDwSmallCols, h = h0 - p.pad + r, col = w0 - p.pad + pixel - r * kDwSmallCols;
+    v[j] = make_uint4(0u, 0u, 0u, 0u);
+    if (i < kVecs && h >= 0 && h < p.H && col >= 0 && col < p.W)
+      v[j] = x4[(((long long)n * p.H + h) * p.W + col) * C8 + (i & 3)];
+  }
+#pragma unroll
+  for (int j = 0; j < kWLoads; ++j) {
+    const int i = t + j * kDwSmallThreads;
+    wv[j] = i < kWVecs ? w4[(long long)(i >> 2) * C8 + (i & 3)] : make_uint4(0u, 0u, 0u, 0u);
+  }
+#pragma unroll
+  for (int j = 0; j < kLoads; ++j) {
+    const int i = t + j * kDwSmallThreads;
+    if (i < kVecs) *reinterpret_cast<uint4*>(px + (i >> 2) * kDwSmallPixel + 4 * (i & 3)) = v[j];
+  }
+#pragma unroll
+  for (int j = 0; j < kWLoads; ++j) {
+    const int i = t + j * kDwSmallThreads;
+    if (i < kWVecs) {
+      float2* dst = &w_s[i >> 2][4 * (i & 3)];
+      dst[0] = make_float2(bf16_lo(wv[j].x), bf16_hi(wv[j].x));
+      dst[1] = make_float2(bf16_lo(wv[j].y), bf16_hi(wv[j].y));
+      dst[2] = make_float2(bf16_lo(wv[j].z), bf16_hi(wv[j].z));
+      dst[3] = make_float2(bf16_lo(wv[j].w), bf16_hi(wv[j].w));
+    }
+  }
+  __syncthreads();
+  const int sub = t & 15, run = (t >> 4) & 1, o = t >> 5;
+  const int ho = h0 + o, wo0 = w0 + run * kDwSmallRun, c2 = blockIdx.y * 16 + sub;
+  if (ho >= p.Ho || wo0 >= p.Wo) return;
+  float2 acc[kDwSmallRun];
+  {
+    float2 b = make_float2(0.0f, 0.0f);
+    if (p.flags & SSCONV_FLAG_BIAS) b = make_float2(p.bias[2 * c2], p.bias[2 * c2 + 1]);
+#pragma unroll
+    for (int k = 0; k < kDwSmallRun; ++k) acc[k] = b;
+  }
+#pragma unroll 1
+  for (int kh = 0; kh < kDw7K; ++kh) {
+    const int h = ho - p.pad + kh;
+    if (h < 0 || h >= p.H) continue;
+    const uint32_t* row = px + ((o + kh) * kDwSmallCols + run * kDwSmallRun) * kDwSmallPixel + sub;
+    float2 xv[kDwSmallRun + kDw7K - 1], part[kDwSmallRun];
+#pragma unroll
+    for (int col = 0; col < kDwSmallRun + kDw7K - 1; ++col) {
+      const uint32_t u = row[col * kDwSmallPixel];
+      xv[col] = make_float2(bf16_lo(u), bf16_hi(u));
+    }
+#pragma unroll
+    for (int kw = 0; kw < kDw7K; ++kw) {
+      const float2 wk = w_s[kh * kDw7K + kw][sub];
+#pragma unroll
+      for (int k = 0; k < kDwSmallRun; ++k)
+        part[k] = kw == 0 ? __fmul2_rn(xv[k], wk) : __ffma2_rn(xv[k + kw], wk, part[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < kDwSmallRun; ++k) acc[k] = __fadd2_rn(acc[k], part[k]);
+  }
+  uint32_t* out = p.y + (((long long)n * p.Ho + ho) * p.Wo + wo0) * (p.C >> 1) + c2;
+#pragma unroll
+  for (int k = 0; k < kDwSmallRun; ++k)
+    if (wo0 + k < p.Wo)
+      out[(long long)k * (p.C >> 1)] =
+          RELU ? pack_bf16x2<false>(fmaxf(acc[k].x, 0.0f), fmaxf(acc[k].y, 0.0f)) : pack_bf16x2<false>(acc[k].x, acc[k].y);
+}
+
+static int g_tune_mma = -1;    // ssconv_tune: -1 automatic, 0 neither of the two kernels here
+static int g_tune_small = -1;  // -1 automatic, 0 never the small maps' kernel
+int32_t set_depthwise_tuning(int32_t option, int32_t value) {
   if (value != -1 && value != 0) return SSCONV_ERR_BAD_DESC;
-  g_tune_mma = value;
+  (option == SSCONV_TUNE_DEPTHWISE_SMALL ? g_tune_small : g_tune_mma) = value;
   return SSCONV_OK;
 }
 
@@ -575,6 +682,42 @@ static cudaError_t depthwise7_ready(bool relu, int* sms) {
 typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// Blocks of depthwise7_small_kernel for a map, and the most that it is used for.  us, tensor-core kernel /
+// small: 1152 blocks 12 x 14 x 14 x 384 9.7 / 6.9, 1536 blocks 32 x 7 x 7 x 768 8.5 / 8.3, 1764 blocks 6 x 56 x 56 x 96 10.0 /
+// 10.1, 2304 blocks 24 x 14 x 14 x 384 10.5 / 11.7.
+constexpr long long kDwSmallMaxBlocks = 10 * 148;
+static long long depthwise7_small_blocks(int N, int C, int Ho, int Wo) {
+  return (long long)N * ((Ho + kDwSmallH - 1) / kDwSmallH) * ((Wo + kDwSmallW - 1) / kDwSmallW) * (C / kDw7Channels);
+}
+// A grid that starts while the one before it drains puts its blocks where that one leaves first, as many as fit: up to a
+// dozen on some SMs and none on others.  So much shared memory per block that an even share of the blocks fits on an SM
+// spreads them.  us without it and with: 3 x 56 x 56 x 96 7.9 / 5.8, 3 x 28 x 28 x 192 6.8 / 4.5, 3 x 14 x 14 x 384 4.4 / 3.2.
+constexpr int kSmSharedBytes = 228 * 1024, kMaxBlockSharedBytes = 232448, kBlockReservedBytes = 1024;
+static cudaError_t launch_depthwise7_small(const Dw7Params& p, cudaStream_t st) {
+  const int tiles_h = (p.Ho + kDwSmallH - 1) / kDwSmallH, tiles_w = (p.Wo + kDwSmallW - 1) / kDwSmallW;
+  const dim3 grid((unsigned)(p.N * tiles_h * tiles_w), (unsigned)(p.C / kDw7Channels));
+  const bool relu = (p.flags & SSCONV_FLAG_RELU) != 0;
+  const auto kernel = relu ? depthwise7_small_kernel<true> : depthwise7_small_kernel<false>;
+  static std::atomic<int> known[64][2];  // per device and form: SM count, once the kernel may take all shared memory
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int sms = dev >= 0 && dev < 64 ? known[dev][relu].load(std::memory_order_relaxed) : 0;
+  if (sms == 0) {
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxBlockSharedBytes - kDwSmallSharedBytes);
+    if (e != cudaSuccess) return e;
+    if (dev >= 0 && dev < 64) known[dev][relu].store(sms, std::memory_order_relaxed);
+  }
+  const long long blocks = (long long)grid.x * grid.y;
+  const int per_sm = (int)((blocks + sms - 1) / sms);
+  int extra = kSmSharedBytes / per_sm - kBlockReservedBytes - kDwSmallSharedBytes;
+  if (extra > kMaxBlockSharedBytes - kDwSmallSharedBytes) extra = kMaxBlockSharedBytes - kDwSmallSharedBytes;
+  count_launch();
+  return launch_dependent_smem(kernel, grid, kDwSmallThreads, extra > 0 ? (size_t)(extra & ~127) : 0, st, p, tiles_h, tiles_w);
+}
 
 static cudaError_t launch_depthwise7_on(int sms, const void* x, const void* w, const float* bias, void* y, int N, int H, int W,
                                         int C, int Ho, int Wo, int pad, uint32_t flags, uint32_t polls, cudaStream_t st) {
@@ -653,6 +796,24 @@ static cudaError_t launch_depthwise7_on(int sms, const void* x, const void* w, c
 bool launch_depthwise7(const void* x, const void* w, const float* bias, void* y, int N, int H, int W, int C, int Ho, int Wo,
                        int KH, int KW, int stride, int pad, int dil, uint32_t flags, int32_t polls, cudaStream_t st,
                        cudaError_t* result) {
+  if (polls < 0 && KH == kDw7K && KW == kDw7K && stride == 1 && dil == 1 && C % kDw7Channels == 0 && g_tune_mma != 0 &&
+      g_tune_small != 0 && depthwise7_small_blocks(N, C, Ho, Wo) <= kDwSmallMaxBlocks) {
+    Dw7Params p{};
+    p.x = static_cast<const uint32_t*>(x);
+    p.w = static_cast<const uint32_t*>(w);
+    p.bias = bias;
+    p.y = static_cast<uint32_t*>(y);
+    p.N = N;
+    p.H = H;
+    p.W = W;
+    p.C = C;
+    p.Ho = Ho;
+    p.Wo = Wo;
+    p.pad = pad;
+    p.flags = flags;
+    *result = launch_depthwise7_small(p, st);
+    return true;
+  }
   if (!depthwise7_applies(N, H, W, C, Ho, Wo, KH, KW, stride, dil)) return false;
   const bool relu = (flags & SSCONV_FLAG_RELU) != 0;
   int sms = 0;

@@ -1951,7 +1951,7 @@ static double kblock_cycles(int BN, int stage_bufs, bool steady_ring = true) {
 // Process-wide overrides of the planner (ssconv_tune): tile width (0 lets the model choose) and the
 // use of the pair kernel.
 int32_t wgrad_set_tuning(int32_t option, int32_t value);  // (wgrad.cu)
-int32_t set_depthwise_tuning(int32_t value);               // (depthwise.cu)
+int32_t set_depthwise_tuning(int32_t option, int32_t value);  // (depthwise.cu)
 static int g_tune_bn = 0;
 static int g_tune_resident = 1;  // 0: weights always travel through the ring
 static int g_tune_pair = -1;  // -1: the model chooses; 0: never the pair kernel; 1: wherever it applies
@@ -1983,7 +1983,7 @@ int32_t set_tuning(int32_t option, int32_t value) {
     g_tune_bn = value;
     return SSCONV_OK;
   }
-  if (option == SSCONV_TUNE_DEPTHWISE_MMA) return set_depthwise_tuning(value);
+  if (option == SSCONV_TUNE_DEPTHWISE_MMA || option == SSCONV_TUNE_DEPTHWISE_SMALL) return set_depthwise_tuning(option, value);
   return wgrad_set_tuning(option, value);
 }
 

@@ -56,6 +56,31 @@ def test_depthwise7_on_the_fp32_kernels(case):
         api.ssconv_tune(api.TUNE_DEPTHWISE_MMA, -1)
 
 
+@pytest.mark.parametrize("case", CASES, ids=["x".join(map(str, c[:4])) + f"_p{c[4]}" for c in CASES])
+def test_depthwise7_without_the_kernel_for_small_maps(case):
+    # (most of the maps above are small: the tensor-core kernel at the edges of its own tiles)
+    api.ssconv_tune(api.TUNE_DEPTHWISE_SMALL, 0)
+    try:
+        _check_case(case)
+    finally:
+        api.ssconv_tune(api.TUNE_DEPTHWISE_SMALL, -1)
+
+
+@pytest.mark.parametrize("case", [
+    (1, 4, 8, 32, 3, False),      # one tile exactly
+    (2, 5, 9, 64, 3, True),       # one row and one column more
+    (1, 10, 14, 32, 0, False),    # no padding: the tile's pixels are the map
+    (3, 3, 23, 96, 5, False),     # wide padding, rows of three tiles
+    (2, 1, 1, 960, 6, True),      # many channels, windows mostly outside
+    (37, 14, 14, 160, 3, False),  # 1480 blocks: the most
+    (38, 14, 14, 160, 3, False),  # (one image more: the tensor-core kernel)
+], ids=lambda c: "x".join(map(str, c[:4])) + f"_p{c[4]}")
+def test_depthwise7_on_small_maps(case):
+    if case not in CASES:
+        CASES.append(case)        # (its index seeds the inputs)
+    _check_case(case)
+
+
 def _check_case(case):
     N, H, W, C, pad, relu = case
     g = torch.Generator().manual_seed(synth.SEED_BASE + 7100 + CASES.index(case))
@@ -174,3 +199,29 @@ def test_depthwise7_non_finite_outputs_are_those_of_the_fp32_kernel(relu, with_b
     near = fin.clone()
     near[1, :8, :9, 8] = False
     assert bool(((y.float() - ref.float()).abs()[near] <= 2.0 ** -7 * ref.float().abs()[near] + 1e-5).all())
+
+
+@pytest.mark.parametrize("data", ["normal", "spread", "positive"])
+def test_depthwise7_sums_on_small_maps_are_as_exact(data):
+    # as above, on the kernel for small maps (1360 blocks); the bias is the first thing its sums hold
+    C, units = 2560, []
+    for seed in range(13):
+        g = torch.Generator().manual_seed(synth.SEED_BASE + 7950 + seed)
+        x, w = torch.randn((17, 10, 7, C), generator=g), torch.randn((7, 7, C), generator=g) / 7
+        if data == "spread":
+            x = x * torch.exp(2.0 * torch.randn(x.shape, generator=g))
+        if data == "positive":
+            x, w = x.abs(), w.abs()
+        x, w = x.to(torch.bfloat16), w.to(torch.bfloat16)
+        n, row = seed, seed % 4
+        products = x[n, row:row + 7].double() * w.double()
+        total = products.sum((0, 1))
+        bias = (-total).float()
+        desc = api.make_desc(17, 10, 7, C, C, 7, 7, 1, 0, bias=True)
+        y = api.ssconv_depthwise(desc, x.to(DEV), w.to(DEV), bias.to(DEV))[n, row, 0].cpu().double()
+        units.append((y - (total + bias.double())) / products.abs().sum((0, 1)) * 2.0 ** 24)
+    err = torch.cat(units)
+    print("small maps", data, float(err.pow(2).mean().sqrt()), float(err.mean()))
+    # what the tensor-core kernel leaves on these data (a fortieth more for the sampling)
+    assert float(err.pow(2).mean().sqrt()) <= 1.025 * {"normal": 0.156, "spread": 0.617, "positive": 0.730}[data]
+    assert abs(float(err.mean())) <= 0.3
