@@ -1,7 +1,8 @@
-"""ctypes binding of libssconv.so: the same entry points as include/ssconv.h.
+"""Python binding of libssconv.so: the same entry points as include/ssconv.h.
 
 Only argument marshalling happens here; torch supplies device memory and the current
-stream.  There is no CPU path: if the library is missing or a call fails, an exception
+stream.  The calls that a network makes per layer and step go through _binding.so (csrc/binding.cpp), which converts and
+checks their arguments in native code; the others through ctypes.  There is no CPU path: if the library is missing or a call fails, an exception
 is raised.
 """
 from __future__ import annotations
@@ -147,6 +148,19 @@ def lib():
     return _lib
 
 
+_native = None
+
+
+def _binding():
+    """The native binding (csrc/binding.cpp), loaded once; raise if it has not been built."""
+    global _native
+    if _native is None:
+        lib()
+        from . import _binding as native
+        _native = native
+    return _native
+
+
 def status_string(status: int) -> str:
     return lib().ssconv_status_string(status).decode()
 
@@ -234,10 +248,11 @@ def _sizes(desc_bytes: bytes) -> Sizes:
 def ssconv_select_mask(mode: int, scores: torch.Tensor, G: int, pattern: Optional[torch.Tensor] = None,
                        stream=None) -> torch.Tensor:
     """pattern uint8 [G] from fp32 scores [G,6] (mode LOGITS) or bf16 weights (mode MAGNITUDE)."""
-    _need_cuda(scores, pattern)
+    b = _binding()
     if pattern is None:
-        pattern = torch.empty(G, dtype=torch.uint8, device=scores.device)
-    _check("ssconv_select_mask", lib().ssconv_select_mask(mode, _ptr(scores), G, _ptr(pattern), _stream(stream)))
+        _need_cuda(scores)
+        pattern = b.blob(G, scores)
+    _check("ssconv_select_mask", b.ssconv_select_mask(mode, scores, G, pattern, stream))
     return pattern
 
 
@@ -267,12 +282,11 @@ def ssconv_apply_mask_nm(w: torch.Tensor, pattern: torch.Tensor, N: int, M: int,
 
 def ssconv_compress(desc: Desc, w: torch.Tensor, pattern: torch.Tensor, stream=None):
     """(w_comp, meta) uint8 blobs from bf16 weights [C_out,KH,KW,C_in] and pattern [G]."""
-    _need_cuda(w, pattern)
+    b = _binding()
+    _need_cuda(w)
     sz = ssconv_sizes(desc)
-    w_comp = torch.empty(sz.w_comp_bytes, dtype=torch.uint8, device=w.device)
-    meta = torch.empty(sz.meta_bytes, dtype=torch.uint8, device=w.device)
-    _check("ssconv_compress", lib().ssconv_compress(ctypes.byref(desc), _ptr(w), _ptr(pattern), _ptr(w_comp),
-                                                    _ptr(meta), _stream(stream)))
+    w_comp, meta = b.blob(sz.w_comp_bytes, w), b.blob(sz.meta_bytes, w)
+    _check("ssconv_compress", b.ssconv_compress(desc, w, pattern, w_comp, meta, stream))
     return w_comp, meta
 
 
@@ -347,8 +361,19 @@ def default_workspace(device) -> torch.Tensor:
 
 
 def _alloc_y(desc: Desc, x: torch.Tensor) -> torch.Tensor:
-    ho, wo = ssconv_out_shape(desc)
-    return torch.empty(desc.N, ho, wo, desc.C_out, dtype=torch.bfloat16, device=x.device)
+    y = _binding().output(desc, x)
+    if type(y) is int:
+        _check("ssconv_out_shape", y)
+    return y
+
+
+def _scratch(x: torch.Tensor) -> torch.Tensor:
+    """default_workspace of x's device."""
+    ws = _workspaces.get(x.get_device())
+    if ws is None:
+        _need_cuda(x)
+        ws = default_workspace(x.device)
+    return ws
 
 
 def ssconv_forward(desc: Desc, x: torch.Tensor, w_comp: torch.Tensor, meta: torch.Tensor,
@@ -357,22 +382,16 @@ def ssconv_forward(desc: Desc, x: torch.Tensor, w_comp: torch.Tensor, meta: torc
                    stream=None, residual: Optional[torch.Tensor] = None) -> torch.Tensor:
     """2:4 masked convolution forward; returns y bf16 [N,H_out,W_out,C_out] (enqueued, not synchronised).
     With `residual` (bf16, the shape of y) the call is ssconv_forward_res: y = act(bias + conv + residual)."""
-    _need_cuda(x, w_comp, meta, bias, y, ws, dev_status, residual)
+    b = _binding()
+    if ws is None:
+        ws = _scratch(x)
     if y is None:
         y = _alloc_y(desc, x)
-    if ws is None:
-        ws = default_workspace(x.device)
-    ws_bytes = ws.nbytes
     if residual is None:
-        _check("ssconv_forward", lib().ssconv_forward(
-            ctypes.byref(desc), _ptr(x), _ptr(w_comp), _ptr(meta), _ptr(bias), _ptr(y), _ptr(ws), ws_bytes,
-            _ptr(dev_status), _stream(stream)))
+        _check("ssconv_forward", b.ssconv_forward(desc, x, w_comp, meta, bias, y, ws, ws, dev_status, stream))
     else:
-        assert residual.shape == y.shape and residual.dtype == torch.bfloat16 and residual.is_contiguous()
-        f = lib().ssconv_forward_res
-        _check("ssconv_forward_res", f(ctypes.byref(desc), _ptr(x), _ptr(w_comp), _ptr(meta), _ptr(bias),
-                                       _ptr(residual), _ptr(y), _ptr(ws), ws_bytes, _ptr(dev_status),
-                                       _stream(stream)))
+        assert residual.shape == y.shape and residual.dtype == torch.bfloat16
+        _check("ssconv_forward_res", b.ssconv_forward_res(desc, x, w_comp, meta, bias, residual, y, ws, ws, dev_status, stream))
     return y
 
 
@@ -381,34 +400,28 @@ def ssconv_forward_dense(desc: Desc, x: torch.Tensor, w: torch.Tensor, bias: Opt
                          dev_status: Optional[torch.Tensor] = None, stream=None,
                          residual: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Dense counterpart with bf16 weights [C_out,KH,KW,C_in]; `residual` as in ssconv_forward."""
-    _need_cuda(x, w, bias, y, ws, dev_status, residual)
+    b = _binding()
+    if ws is None:
+        ws = _scratch(x)
     if y is None:
         y = _alloc_y(desc, x)
-    if ws is None:
-        ws = default_workspace(x.device)
-    ws_bytes = ws.nbytes
     if residual is None:
-        _check("ssconv_forward_dense", lib().ssconv_forward_dense(
-            ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(y), _ptr(ws), ws_bytes, _ptr(dev_status),
-            _stream(stream)))
+        _check("ssconv_forward_dense", b.ssconv_forward_dense(desc, x, w, bias, y, ws, ws, dev_status, stream))
     else:
-        assert residual.shape == y.shape and residual.dtype == torch.bfloat16 and residual.is_contiguous()
-        f = lib().ssconv_forward_dense_res
-        _check("ssconv_forward_dense_res", f(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(residual),
-                                             _ptr(y), _ptr(ws), ws_bytes, _ptr(dev_status), _stream(stream)))
+        assert residual.shape == y.shape and residual.dtype == torch.bfloat16
+        _check("ssconv_forward_dense_res", b.ssconv_forward_dense_res(desc, x, w, bias, residual, y, ws, ws, dev_status, stream))
     return y
 
 
 def ssconv_maxpool(x: torch.Tensor, k: int = 3, stride: int = 2, pad: int = 1, y: Optional[torch.Tensor] = None,
                    stream=None) -> torch.Tensor:
     """k x k max-pooling of NHWC bf16 activations; returns y [N,H_out,W_out,C] (enqueued, not synchronised)."""
-    _need_cuda(x, y)
     n, h, w, c = x.shape
     if y is None:
+        _need_cuda(x)
         y = torch.empty((n, ssconv_window_extent(h, k, stride, pad), ssconv_window_extent(w, k, stride, pad), c),
                         dtype=torch.bfloat16, device=x.device)
-    f = lib().ssconv_maxpool
-    _check("ssconv_maxpool", f(_ptr(x), _ptr(y), n, h, w, c, k, stride, pad, _stream(stream)))
+    _check("ssconv_maxpool", _binding().ssconv_maxpool(x, y, n, h, w, c, k, stride, pad, stream))
     return y
 
 
@@ -416,12 +429,11 @@ def ssconv_space_to_depth(x: torch.Tensor, block: int, pad: int, Hb: int, Wb: in
                           y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """y [N,Hb,Wb,C_pad] with y[n,r,q,(bh*block+bw)*C+c] = x[n, block*r-pad+bh, block*q-pad+bw, c] (zeros outside
     the image and in the padding channels) from x [N,H,W,C] bf16."""
-    _need_cuda(x, y)
     n, h, w, c = x.shape
     if y is None:
+        _need_cuda(x)
         y = torch.empty((n, Hb, Wb, C_pad), dtype=torch.bfloat16, device=x.device)
-    f = lib().ssconv_space_to_depth
-    _check("ssconv_space_to_depth", f(_ptr(x), _ptr(y), n, h, w, c, block, pad, Hb, Wb, C_pad, _stream(stream)))
+    _check("ssconv_space_to_depth", _binding().ssconv_space_to_depth(x, y, n, h, w, c, block, pad, Hb, Wb, C_pad, stream))
     return y
 
 
@@ -470,16 +482,14 @@ def ssconv_forward_dense_strided(desc: Desc, x: torch.Tensor, strides, w: torch.
                                  stream=None) -> torch.Tensor:
     """ssconv_forward_dense on a strided (possibly overlapping) view of x: `strides` = element strides of
     (w, h, n); pixel (n, h, w) of the input the descriptor names starts n*s_n + h*s_h + w*s_w elements into x."""
-    _need_cuda(x, w, bias, y, ws, dev_status)
+    b = _binding()
+    if ws is None:
+        ws = _scratch(x)
     if y is None:
         y = _alloc_y(desc, x)
-    if ws is None:
-        ws = default_workspace(x.device)
-    ws_bytes = ws.nbytes
     s_w, s_h, s_n = (int(v) for v in strides)
-    f = lib().ssconv_forward_dense_strided
-    _check("ssconv_forward_dense_strided", f(ctypes.byref(desc), _ptr(x), s_w, s_h, s_n, _ptr(w), _ptr(bias), _ptr(y),
-                                             _ptr(ws), ws_bytes, _ptr(dev_status), _stream(stream)))
+    _check("ssconv_forward_dense_strided",
+           b.ssconv_forward_dense_strided(desc, x, s_w, s_h, s_n, w, bias, y, ws, ws, dev_status, stream))
     return y
 
 
@@ -535,13 +545,12 @@ def ssconv_forward_grouped(desc: Desc, groups: int, x: torch.Tensor, w_comp: tor
                            bias: Optional[torch.Tensor] = None, y: Optional[torch.Tensor] = None,
                            dev_status: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """2:4 masked grouped convolution (one launch, or one per group on channel slices)."""
-    _need_cuda(x, w_comp, meta, bias, y, dev_status)
+    b = _binding()
+    ws = _scratch(x)
     if y is None:
         y = _alloc_y(desc, x)
-    ws = default_workspace(x.device)
-    f = lib().ssconv_forward_grouped
-    _check("ssconv_forward_grouped", f(ctypes.byref(desc), groups, _ptr(x), _ptr(w_comp), _ptr(meta), _ptr(bias), _ptr(y),
-                                       _ptr(ws), ws.numel(), _ptr(dev_status), _stream(stream)))
+    _check("ssconv_forward_grouped",
+           b.ssconv_forward_grouped(desc, groups, x, w_comp, meta, bias, y, ws, ws, dev_status, stream))
     return y
 
 
@@ -549,24 +558,21 @@ def ssconv_forward_dense_grouped(desc: Desc, groups: int, x: torch.Tensor, w: to
                                  bias: Optional[torch.Tensor] = None, y: Optional[torch.Tensor] = None,
                                  dev_status: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Dense grouped convolution; w bf16 [C_out, KH, KW, C_in/groups]."""
-    _need_cuda(x, w, bias, y, dev_status)
+    b = _binding()
+    ws = _scratch(x)
     if y is None:
         y = _alloc_y(desc, x)
-    ws = default_workspace(x.device)
-    f = lib().ssconv_forward_dense_grouped
-    _check("ssconv_forward_dense_grouped", f(ctypes.byref(desc), groups, _ptr(x), _ptr(w), _ptr(bias), _ptr(y), _ptr(ws),
-                                             ws.numel(), _ptr(dev_status), _stream(stream)))
+    _check("ssconv_forward_dense_grouped", b.ssconv_forward_dense_grouped(desc, groups, x, w, bias, y, ws, ws, dev_status, stream))
     return y
 
 
 def ssconv_depthwise(desc: Desc, x: torch.Tensor, w: torch.Tensor, bias: Optional[torch.Tensor] = None,
                      y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Dense depthwise convolution; w bf16 tap-major [KH, KW, C]."""
-    _need_cuda(x, w, bias, y)
     if y is None:
+        _need_cuda(x)
         y = _alloc_y(desc, x)
-    f = lib().ssconv_depthwise
-    _check("ssconv_depthwise", f(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), _ptr(y), _stream(stream)))
+    _check("ssconv_depthwise", _binding().ssconv_depthwise(desc, x, w, bias, y, stream))
     return y
 
 
@@ -583,24 +589,22 @@ def ssconv_selftest_depthwise_give_up(desc: Desc, x: torch.Tensor, w: torch.Tens
 def ssconv_layernorm(x: torch.Tensor, gamma: torch.Tensor, beta: torch.Tensor, eps: float = 1e-6,
                      y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Layer normalisation over the last axis of x (bf16), gamma / beta fp32 [C]."""
-    _need_cuda(x, gamma, beta, y)
     c = x.shape[-1]
     if y is None:
+        _need_cuda(x)
         y = torch.empty_like(x)
-    f = lib().ssconv_layernorm
-    _check("ssconv_layernorm", f(_ptr(x), _ptr(gamma), _ptr(beta), float(eps), _ptr(y), x.numel() // c, c, _stream(stream)))
+    _check("ssconv_layernorm", _binding().ssconv_layernorm(x, gamma, beta, eps, y, x.numel() // c, c, stream))
     return y
 
 
 # ----------------------------------------------------------------------------- 8-bit (e4m3) operands
 def ssconv_quantize_e4m3(x: torch.Tensor, scale: float = 1.0, y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """uint8 e4m3 codes of x * scale (x bf16, an even number of elements), nearest even, saturating."""
-    _need_cuda(x, y)
+    _need_cuda(x)
     assert x.dtype == torch.bfloat16
     if y is None:
         y = torch.empty(x.shape, dtype=torch.uint8, device=x.device)
-    f = lib().ssconv_quantize_e4m3
-    _check("ssconv_quantize_e4m3", f(_ptr(x), _ptr(y), x.numel(), float(scale), _stream(stream)))
+    _check("ssconv_quantize_e4m3", _binding().ssconv_quantize_e4m3(x, y, x.numel(), scale, stream))
     return y
 
 
@@ -639,12 +643,10 @@ def ssconv_forward_fp8(desc: Desc, x: torch.Tensor, w_comp: torch.Tensor, meta: 
                        bias: Optional[torch.Tensor] = None, out_scale: float = 1.0, y: Optional[torch.Tensor] = None,
                        dev_status: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """2:4 masked convolution on e4m3 activations (uint8 NHWC) and compressed e4m3 weights; bf16 output."""
-    _need_cuda(x, w_comp, meta, bias, y, dev_status)
     if y is None:
+        _need_cuda(x)
         y = _alloc_y(desc, x)
-    f = lib().ssconv_forward_fp8
-    _check("ssconv_forward_fp8", f(ctypes.byref(desc), _ptr(x), _ptr(w_comp), _ptr(meta), _ptr(bias), float(out_scale),
-                                   _ptr(y), _ptr(dev_status), _stream(stream)))
+    _check("ssconv_forward_fp8", _binding().ssconv_forward_fp8(desc, x, w_comp, meta, bias, out_scale, y, dev_status, stream))
     return y
 
 
@@ -652,12 +654,10 @@ def ssconv_forward_dense_fp8(desc: Desc, x: torch.Tensor, w: torch.Tensor, bias:
                              out_scale: float = 1.0, y: Optional[torch.Tensor] = None,
                              dev_status: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Dense counterpart on e4m3 weights [C_out,KH,KW,C_in] (uint8)."""
-    _need_cuda(x, w, bias, y, dev_status)
     if y is None:
+        _need_cuda(x)
         y = _alloc_y(desc, x)
-    f = lib().ssconv_forward_dense_fp8
-    _check("ssconv_forward_dense_fp8", f(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(bias), float(out_scale), _ptr(y),
-                                         _ptr(dev_status), _stream(stream)))
+    _check("ssconv_forward_dense_fp8", _binding().ssconv_forward_dense_fp8(desc, x, w, bias, out_scale, y, dev_status, stream))
     return y
 
 
@@ -666,27 +666,24 @@ def ssconv_soft_mask(logits: torch.Tensor, noise: Optional[torch.Tensor], tau: f
                      z: Optional[torch.Tensor] = None, w_eff: Optional[torch.Tensor] = None):
     """(z fp32 [G,6] or None, w_eff bf16 shaped like w or None): relaxed choice (Eq. 3) and effective
     weights (Eq. 6 with the soft mask) of every group of four weights.  Output tensors may be passed in."""
-    _need_cuda(logits, noise, w, z, w_eff)
+    _need_cuda(logits, w)
     G = logits.shape[0]
     if z is None and want_z:
         z = torch.empty((G, 6), dtype=torch.float32, device=logits.device)
     if w_eff is None and want_w_eff:
         w_eff = torch.empty_like(w)
-    f = lib().ssconv_soft_mask
-    _check("ssconv_soft_mask", f(_ptr(logits), _ptr(noise), float(tau), _ptr(w), G, _ptr(z), _ptr(w_eff),
-                                 _stream(stream)))
+    _check("ssconv_soft_mask", _binding().ssconv_soft_mask(logits, noise, tau, w, G, z, w_eff, stream))
     return z, w_eff
 
 
 def ssconv_mask_grad(z: torch.Tensor, tau: float, w: torch.Tensor, g_w_eff: torch.Tensor,
                      g_logits: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """dL/dlogits fp32 [G,6] from dL/dw_eff (fp32, the shape of w)."""
-    _need_cuda(z, w, g_w_eff, g_logits)
+    _need_cuda(z)
     G = z.shape[0]
     if g_logits is None:
         g_logits = torch.empty((G, 6), dtype=torch.float32, device=z.device)
-    f = lib().ssconv_mask_grad
-    _check("ssconv_mask_grad", f(_ptr(z), float(tau), _ptr(w), _ptr(g_w_eff), G, _ptr(g_logits), _stream(stream)))
+    _check("ssconv_mask_grad", _binding().ssconv_mask_grad(z, tau, w, g_w_eff, G, g_logits, stream))
     return g_logits
 
 
@@ -701,16 +698,14 @@ def ssconv_wgrad(desc: Desc, x: torch.Tensor, dy: torch.Tensor, dw: Optional[tor
                  ws: Optional[torch.Tensor] = None, dev_status: Optional[torch.Tensor] = None,
                  stream=None) -> torch.Tensor:
     """Weight gradient fp32 [C_out,KH,KW,C_in] of the layer from its bf16 input x and output gradient dy."""
-    _need_cuda(x, dy, dw, ws, dev_status)
+    b = _binding()
+    _need_cuda(x)
     if dw is None:
         dw = torch.empty((desc.C_out, desc.KH, desc.KW, desc.C_in), dtype=torch.float32, device=x.device)
     if ws is None:
         need = ssconv_wgrad_ws_bytes(desc)
-        ws = torch.empty(need, dtype=torch.uint8, device=x.device) if need else None
-    ws_bytes = 0 if ws is None else ws.nbytes
-    f = lib().ssconv_wgrad
-    _check("ssconv_wgrad", f(ctypes.byref(desc), _ptr(x), _ptr(dy), _ptr(dw), _ptr(ws), ws_bytes, _ptr(dev_status),
-                             _stream(stream)))
+        ws = b.blob(need, x) if need else None
+    _check("ssconv_wgrad", b.ssconv_wgrad(desc, x, dy, dw, ws, ws, dev_status, stream))
     return dw
 
 
@@ -725,14 +720,13 @@ def ssconv_dgrad(desc: Desc, dy: torch.Tensor, w: torch.Tensor, dx: Optional[tor
                  ws: Optional[torch.Tensor] = None, dev_status: Optional[torch.Tensor] = None,
                  stream=None) -> torch.Tensor:
     """Input gradient bf16 [N,H,W,C_in] of the layer from its output gradient dy and bf16 weights, any stride."""
-    _need_cuda(dy, w, dx, ws, dev_status)
+    b = _binding()
+    _need_cuda(dy)
     if dx is None:
         dx = torch.empty((desc.N, desc.H, desc.W, desc.C_in), dtype=torch.bfloat16, device=dy.device)
     if ws is None:
-        ws = torch.empty((max(ssconv_dgrad_ws_bytes(desc), 16),), dtype=torch.uint8, device=dy.device)
-    f = lib().ssconv_dgrad
-    _check("ssconv_dgrad", f(ctypes.byref(desc), _ptr(dy), _ptr(w), _ptr(dx), _ptr(ws), ws.numel() * ws.element_size(),
-                             _ptr(dev_status), _stream(stream)))
+        ws = b.blob(max(ssconv_dgrad_ws_bytes(desc), 16), dy)
+    _check("ssconv_dgrad", b.ssconv_dgrad(desc, dy, w, dx, ws, ws, dev_status, stream))
     return dx
 
 
@@ -740,12 +734,11 @@ def ssconv_adamw(theta: torch.Tensor, g: torch.Tensor, m: torch.Tensor, v: torch
                  beta1: float = 0.9, beta2: float = 0.999, eps: float = 1e-8, weight_decay: float = 1e-4,
                  stream=None) -> torch.Tensor:
     """One AdamW update of fp32 parameters in place (theta, m, v are modified); step counts from 1."""
-    _need_cuda(theta, g, m, v)
+    _need_cuda(theta)
     assert theta.dtype == g.dtype == m.dtype == v.dtype == torch.float32
     assert theta.numel() == g.numel() == m.numel() == v.numel()
-    f = lib().ssconv_adamw
-    _check("ssconv_adamw", f(_ptr(theta), _ptr(g), _ptr(m), _ptr(v), theta.numel(), int(step), float(lr),
-                             float(beta1), float(beta2), float(eps), float(weight_decay), _stream(stream)))
+    _check("ssconv_adamw", _binding().ssconv_adamw(theta, g, m, v, theta.numel(), int(step), lr, beta1, beta2, eps,
+                                                   weight_decay, stream))
     return theta
 
 

@@ -1,14 +1,16 @@
-"""Compile the CUDA library (sm_100a only) into paper_2411_00288_b200/libssconv.so."""
+"""Compile the CUDA library (sm_100a only) into paper_2411_00288_b200/libssconv.so, and its CPython binding beside it."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libssconv.so")
+BINDING = os.path.join(_HERE, "_binding.so")
 SOURCES = ["api.cu", "mask.cu", "pool.cu", "depthwise.cu", "train.cu", "wgrad.cu", "forward.cu"]
 HEADERS = ["launch.cuh", "layout.cuh", "sm100_ptx.cuh"]
 
@@ -18,7 +20,29 @@ def _newest_source_mtime() -> float:
     return max(os.path.getmtime(f) for f in files)
 
 
+def build_binding(force: bool = False) -> str:
+    """_binding.so against the installed torch (csrc/binding.cpp); after the library, which it is linked with."""
+    sources = [os.path.join(CSRC, "binding.cpp"), os.path.join(ROOT, "include", "ssconv.h")]
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= max(os.path.getmtime(f) for f in sources):
+        return BINDING
+    import torch
+    t = os.path.dirname(torch.__file__)
+    includes = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(t, "include"),
+                os.path.join(t, "include", "torch", "csrc", "api", "include"),
+                os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
+    subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC"] + ["-I" + i for i in includes] +
+                   [sources[0], "-o", BINDING, "-L" + os.path.join(t, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu",
+                    "-lc10", "-lc10_cuda", "-L" + _HERE, "-l:libssconv.so", "-Wl,-rpath,$ORIGIN"], check=True)
+    return BINDING
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    _build_library(force, verbose)
+    build_binding(force)
+    return LIB
+
+
+def _build_library(force: bool, verbose: bool) -> str:
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source_mtime():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -1931,7 +1931,7 @@ static int ring_groups_for(uint32_t a_group_bytes, int BN, int stage_bufs) {
 }
 
 template <bool SPARSE>
-static double kblock_cycles(int BN, int stage_bufs, bool steady_ring = true) {
+static double model_kblock_cycles(int BN, int stage_bufs, bool steady_ring) {
   const double a_bytes = Cfg<SPARSE>::kAGroupBytes / 2.0;
   const double fill = (a_bytes + 128.0 * BN) / kFillBytesPerCycle;
   const double issue = SPARSE ? kIssueSparse : kIssueDense;
@@ -1946,6 +1946,21 @@ static double kblock_cycles(int BN, int stage_bufs, bool steady_ring = true) {
   // (a CTA of a split layer works through a handful of groups per tile and never reaches that
   // steady state: forced split plans measured fastest at the widths the other three terms choose)
   return (steady_ring && ring > t) ? ring : t;
+}
+// (a table: a call weighs some thirty of them against one another, with seven divisions each)
+template <bool SPARSE>
+struct KblockCycles {
+  double cycles[2][2][kBN / 16 + 1];  // [two or four staging buffers][steady ring][width / 16]
+  KblockCycles() {
+    for (int bufs = 0; bufs < 2; ++bufs)
+      for (int steady = 0; steady < 2; ++steady)
+        for (int w = 1; w <= kBN / 16; ++w) cycles[bufs][steady][w] = model_kblock_cycles<SPARSE>(16 * w, 2 + 2 * bufs, steady != 0);
+  }
+};
+template <bool SPARSE>
+static double kblock_cycles(int BN, int stage_bufs, bool steady_ring = true) {
+  static const KblockCycles<SPARSE> table;
+  return table.cycles[stage_bufs == 4 ? 1 : 0][steady_ring ? 1 : 0][BN / 16];
 }
 
 // Process-wide overrides of the planner (ssconv_tune): tile width (0 lets the model choose) and the
@@ -1997,6 +2012,10 @@ struct Plan {
   bool wide = false;  // one-CTA tiles with two sets of epilogue groups
   int cluster = 0;    // CTAs of a cluster that share each tile's K (ssconv_fwd_cluster_kernel); 0: none
 };
+// (32-bit divisions where the tiles allow it: a third of the time of 64-bit ones)
+static long long ceil_div(long long a, int b) {
+  return a <= 0x7FFFFFFFLL ? (long long)(((uint32_t)a + (uint32_t)(b - 1)) / (uint32_t)b) : (a + b - 1) / b;
+}
 template <bool SPARSE>
 static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force_split, int max_bn = kBN,
                        int stage_bufs = 2, bool allow_split = true, EpilogueCycles epilogue = kEpilogueHidden) {
@@ -2006,8 +2025,8 @@ static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force
   Plan best{max_bn, false};
   double best_cost = 0.0;
   for (int BN = max_bn; BN >= min_bn; BN -= 16) {
-    const long long tiles = ((Q + BN - 1) / BN) * geo.m_tiles;
-    const long long per_cta = (tiles + workers - 1) / workers;
+    const long long tiles = ceil_div(Q, BN) * geo.m_tiles;
+    const long long per_cta = ceil_div(tiles, workers);
     const int pieces = (BN / 2 + kPiece - 1) / kPiece;
     // (with at most three groups per tile the ring never reaches its steady state: such layers are paced
     // by their output stream, and measured fastest at the width the other terms choose)
@@ -2027,7 +2046,7 @@ static Plan plan_layer(long long Q, const Geometry& geo, int workers, bool force
     Plan best_split{kBN, true};
     double best_split_cost = 0.0;
     for (int BN = max_bn; BN >= min_bn; BN -= 16) {
-      const long long tiles = ((Q + BN - 1) / BN) * geo.m_tiles;
+      const long long tiles = ceil_div(Q, BN) * geo.m_tiles;
       const double units = (double)tiles * a_tiles;
       const double ctas = units < workers ? units : (double)workers;
       const int pieces = (BN / 2 + kPiece - 1) / kPiece;
@@ -2087,8 +2106,8 @@ static Plan plan_pair(long long Q, const Geometry& geo, int workers, bool forced
   for (int BN = max_bn; BN >= min_bn; BN -= 16) {
     const int groups = pair_ring_groups(Cfg<SPARSE>::kAGroupBytes, BN, geo.kblocks);
     if (groups < 2) continue;
-    const long long tiles = ((Q + BN - 1) / BN) * mp_tiles;
-    const long long per_pair = (tiles + pairs - 1) / pairs;
+    const long long tiles = ceil_div(Q, BN) * mp_tiles;
+    const long long per_pair = ceil_div(tiles, pairs);
     const int pieces = (BN / 2 + kPiece - 1) / kPiece;
     const double fill = (a_bytes + 64.0 * BN) / kFillBytesPerCyclePair;
     const double pipe = SPARSE ? 2.0 * (35.0 + 0.5 * BN) + 11.0 : 4.0 * (5.0 + 0.49 * BN);
@@ -2534,11 +2553,14 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
                                 CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
     // the last piece of a group may hold fewer positions: same view, shorter box
-    box[1] = (cuuint32_t)tail_cols;
-    r = g_encode_tiled(&tm_y_tail, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, y, dims, strides, box, estr,
-                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
+    tm_y_tail = tm_y;
+    if (tail_cols != kPiece) {
+      box[1] = (cuuint32_t)tail_cols;
+      r = g_encode_tiled(&tm_y_tail, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, y, dims, strides, box, estr,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+      if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
+    }
     // the residual tensor, when there is one, is read through the same two views
     tm_r = tm_y;
     tm_r_tail = tm_y_tail;
@@ -2549,11 +2571,14 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
-      box[1] = (cuuint32_t)tail_cols;
-      r = g_encode_tiled(&tm_r_tail, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, res, dims, strides, box, estr,
-                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-      if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
+      tm_r_tail = tm_r;
+      if (tail_cols != kPiece) {
+        box[1] = (cuuint32_t)tail_cols;
+        r = g_encode_tiled(&tm_r_tail, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, res, dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return SSCONV_ERR_CUDA;
+      }
     }
   }
 
