@@ -165,6 +165,10 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t sm
                ::"l"(map), "r"(smem_src), "r"(x), "r"(y), "r"(z), "r"(w)
                : "memory");
 }
+// Contiguous bytes (addresses and size multiples of 16) from shared memory.
+__device__ __forceinline__ void bulk_store(void* dst, uint32_t smem_src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(smem_src), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_group_read0() {
   asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");

@@ -15,14 +15,16 @@
 // forward kernel): N = 64 to 256 columns of dW per CTA, so the gradient tile is loaded once for up
 // to four taps.
 //
-// A CTA owns one work item: 128 output channels x T k-blocks x one range of positions, and walks
-// its positions 64 at a time through a 4-stage TMA ring (four producer threads, one MMA thread,
-// four epilogue warps, fp32 accumulator of 64 T columns in TMEM).  The accumulator has output
-// channels on TMEM lanes, so an epilogue thread holds one row of dW: it writes to a scratch slice
-// laid out [tile of 128 output channels][K][128], where the 32 lanes of a warp store 128 contiguous
-// bytes and a CTA's whole output is one contiguous block.  A second kernel
+// A CTA owns one work item: M tiles of 128 output channels x T k-blocks x one range of positions, and walks
+// its positions 64 at a time through a TMA ring (four producer threads, one MMA thread,
+// four epilogue warps, M fp32 accumulators of 64 T columns in TMEM).  With many positions and few k-blocks what paces it
+// is what its loads bring into shared memory: M tiles sharing the activation tiles take 128 M + 64 T rows of 128 bytes
+// per step where M items of one tile take 128 M + 64 T M (see wg_plan).  The accumulator has output
+// channels on TMEM lanes, so an epilogue thread holds one row of dW: it goes to a scratch slice
+// laid out [tile of 128 output channels][K][128] by way of the idle ring, where a k-block's 64 columns are one contiguous
+// block of 32 KB that one bulk copy takes out (4-byte stores per lane take 46 cycles each).  A second kernel
 // adds the slices of all position ranges in a fixed order (the result does not depend on timing)
-// and transposes 32 x 32 tiles through shared memory into dW [C_out][K].  All mbarrier waits are
+// and transposes tiles through shared memory into dW [C_out][K].  All mbarrier waits are
 // bounded (see sm100_ptx.cuh).
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -37,11 +39,22 @@ namespace ssconv {
 constexpr int kWgThreads = 288;        // warps 0, 6, 7, 8: TMA producers, warp 1: MMA, warps 2-5: epilogue
 constexpr int kWgPos = 64;             // positions per ring stage
 constexpr int kWgMaxT = 4;             // k-blocks per work item (N = 64 T <= 256)
-constexpr int kWgStages = 4;
+constexpr int kWgMaxM = 3;             // tiles of 128 output channels per work item
+constexpr int kWgMaxStages = 6;
 constexpr uint32_t kWgTileBytes = kWgPos * 128;                  // 64 positions x 64 channels bf16
-constexpr uint32_t kWgStageBytes = (2 + kWgMaxT) * kWgTileBytes;  // two gradient halves + T activation tiles
-constexpr uint32_t kWgTmemCols = 256;
-constexpr uint32_t kWgSmemBytes = 1024 + kWgStages * kWgStageBytes + 256;
+constexpr uint32_t kWgMaxSmemBytes = 232448;
+// ring stages of 2 M gradient tiles and T activation tiles
+__host__ __device__ constexpr uint32_t wg_stage_bytes(int M, int T) { return (uint32_t)(2 * M + T) * kWgTileBytes; }
+constexpr int wg_stages(int M, int T) {
+  const int n = (int)((kWgMaxSmemBytes - 1024 - 256) / wg_stage_bytes(M, T));
+  return n > kWgMaxStages ? kWgMaxStages : n;
+}
+constexpr uint32_t kWgOutBytes = kBlockK * kTileM * 4;   // a k-block of the result, staged in the ring
+static_assert(wg_stages(1, kWgMaxT) * wg_stage_bytes(1, kWgMaxT) >= kWgMaxT * kWgOutBytes &&
+                  wg_stages(kWgMaxM, 2) * wg_stage_bytes(kWgMaxM, 2) >= 2 * kWgMaxM * kWgOutBytes,
+              "the result fits in the ring");
+constexpr uint32_t wg_tmem_cols(int M, int T) { return 64 * M * T <= 128 ? 128 : 64 * M * T <= 256 ? 256 : 512; }
+static_assert(wg_stages(1, kWgMaxT) >= 4 && wg_stages(kWgMaxM, 2) >= 3 && 64 * kWgMaxM * 2 <= 512, "ring and TMEM");
 constexpr long long kWgWaitLimitCycles = 4000000000LL;
 
 struct WgParams {
@@ -50,6 +63,9 @@ struct WgParams {
   int taps, kblocks;       // k-blocks = channel chunks x taps, numbered chunk * taps + tap
   int T, items_b;          // k-blocks per item, items along K = ceil(kblocks / T)
   int m_tiles;
+  int M, items_m;          // channel tiles per item, items along C_out = ceil(m_tiles / M)
+  int stages;              // of the ring
+  uint32_t tmem_cols;
   int splits;              // position ranges
   int ksteps, ksteps_per_split;  // steps of 64 positions: in all, per range
   int dy_one_load;         // C_out % 64 == 0: both halves of a gradient tile come with one 3-D load
@@ -85,8 +101,8 @@ __device__ __forceinline__ WgItem wg_item(const WgParams& p) {
   int i = blockIdx.x;
   const int ib = i % p.items_b;
   i /= p.items_b;
-  it.m = i % p.m_tiles;
-  it.split = i / p.m_tiles;
+  it.m = (i % p.items_m) * p.M;
+  it.split = i / p.items_m;
   it.b0 = ib * p.T;
   it.nb = min(p.T, p.kblocks - it.b0);
   it.ks0 = it.split * p.ksteps_per_split;
@@ -99,11 +115,12 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
                     const WgParams p) {
   extern __shared__ uint8_t wg_smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(wg_smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kWgStages * kWgStageBytes);
-  uint64_t* bar_full = bars;                 // [kWgStages]
-  uint64_t* bar_empty = bars + kWgStages;    // [kWgStages]
-  uint64_t* bar_acc = bars + 2 * kWgStages;  // accumulator complete
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kWgStages + 1);
+  const uint32_t stage_bytes = wg_stage_bytes(p.M, p.T);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (uint32_t)p.stages * stage_bytes);
+  uint64_t* bar_full = bars;                    // [kWgMaxStages]
+  uint64_t* bar_empty = bars + kWgMaxStages;    // [kWgMaxStages]
+  uint64_t* bar_acc = bars + 2 * kWgMaxStages;  // accumulators complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kWgMaxStages + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5;
@@ -113,7 +130,7 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
 
   if (warp == 0) {
     if (lane == 0) {
-      for (int s = 0; s < kWgStages; ++s) {
+      for (int s = 0; s < kWgMaxStages; ++s) {
         mbar_init(&bar_full[s], producers);
         mbar_init(&bar_empty[s], 1u);
       }
@@ -127,7 +144,7 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
     }
     __syncwarp();
   } else if (warp == 1) {
-    tmem_alloc(tmem_slot, kWgTmemCols);
+    tmem_alloc(tmem_slot, p.tmem_cols);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -139,7 +156,7 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
   if (warp == 0 || warp >= 6) {
     // ------------------------------------------------------------------ TMA producers
     // A TMA instruction occupies its thread for a few hundred cycles, so the loads of a stage are
-    // spread over four threads: role 0 the gradient tile, roles 1-3 the activation tiles
+    // spread over four threads: role 0 the gradient tiles, roles 1-3 the activation tiles
     // (role 1 also the fourth one).
     const int role = (warp == 0) ? 0 : warp - 5;
     if (lane == 0 && role < (int)producers) {
@@ -148,16 +165,16 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
       for (int ks = item.ks0; ks < item.ks1; ++ks) {
         if (!mbar_wait_a(empty0 + 8u * s, ph ^ 1u, abort_flag, kWgWaitLimitCycles)) break;
         const uint32_t full = full0 + 8u * s;
-        const uint32_t dst = ring0 + s * kWgStageBytes;
+        const uint32_t dst = ring0 + s * stage_bytes;
         const int q0 = ks * kWgPos;
         if (role == 0) {
           // channels beyond C_out and positions beyond Q lie outside the tensor map: zeros
-          mbar_expect_tx_a(full, 2u * kWgTileBytes);
+          mbar_expect_tx_a(full, 2u * (uint32_t)p.M * kWgTileBytes);
           if (p.dy_one_load) {
             tma_load_3d_a(dst, &tm_dy, full, 0, q0, 2 * item.m);
           } else {
-            tma_load_2d_a(dst, &tm_dy, full, item.m * kTileM, q0);
-            tma_load_2d_a(dst + kWgTileBytes, &tm_dy, full, item.m * kTileM + 64, q0);
+            for (int h = 0; h < 2 * p.M; ++h)
+              tma_load_2d_a(dst + (uint32_t)h * kWgTileBytes, &tm_dy, full, item.m * kTileM + 64 * h, q0);
           }
         } else {
           const int rho = q0 / p.Wo;
@@ -174,11 +191,11 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
             const int tap = b - cc * p.taps;
             const int kh = tap / p.KW;
             const int kw = tap - kh * p.KW;
-            tma_load_im2col_4d_a(dst + (uint32_t)(2 + t) * kWgTileBytes, &tm_x, full, cc * kBlockK, base_w, base_h,
+            tma_load_im2col_4d_a(dst + (uint32_t)(2 * p.M + t) * kWgTileBytes, &tm_x, full, cc * kBlockK, base_w, base_h,
                                  n, (uint16_t)(kw * p.dil_w), (uint16_t)(kh * p.dil_h));
           }
         }
-        if (++s == kWgStages) {
+        if (++s == (uint32_t)p.stages) {
           s = 0;
           ph ^= 1u;
         }
@@ -193,16 +210,19 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
       bool ok = true;
       for (int ks = item.ks0; ks < item.ks1; ++ks) {
         if (!mbar_wait_a(full0 + 8u * s, ph, abort_flag, kWgWaitLimitCycles)) { ok = false; break; }
-        const uint32_t a_lo = wg_desc_lo(ring0 + s * kWgStageBytes);
-        const uint32_t b_lo = a_lo + ((2u * kWgTileBytes) >> 4);
+        const uint32_t a_lo = wg_desc_lo(ring0 + s * stage_bytes);
+        const uint32_t b_lo = a_lo + ((2u * (uint32_t)p.M * kWgTileBytes) >> 4);
         // 16 positions per MMA = two groups of 8 rows = 2048 B
+        for (int m = 0; m < p.M; ++m) {
+          const uint32_t am_lo = a_lo + (uint32_t)m * ((2u * kWgTileBytes) >> 4);
+          const uint32_t d_tmem = tmem_base + (uint32_t)(m * 64 * p.T);
 #pragma unroll
-        for (int i = 0; i < kWgPos / 16; ++i) {
-          tc_mma_dense_lo(tmem_base, a_lo + (uint32_t)i * 128u, b_lo + (uint32_t)i * 128u, idesc, accumulate);
-          accumulate = 1;
+          for (int i = 0; i < kWgPos / 16; ++i)
+            tc_mma_dense_lo(d_tmem, am_lo + (uint32_t)i * 128u, b_lo + (uint32_t)i * 128u, idesc, i == 0 ? accumulate : 1u);
         }
+        accumulate = 1;
         tc_commit_a(empty0 + 8u * s);
-        if (++s == kWgStages) {
+        if (++s == (uint32_t)p.stages) {
           s = 0;
           ph ^= 1u;
         }
@@ -217,27 +237,38 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
     if (got) {
       tc_fence_after();
       grid_dependency_wait();
+      const int m_here = min(p.M, p.m_tiles - item.m);
+      for (int mt = 0; mt < m_here * item.nb; ++mt) {
+        const int m = mt / item.nb, t = mt - m * item.nb;
+        // [column of the k-block][output channel] fp32, k-block after k-block
+        const uint32_t col0 = ring0 + (uint32_t)mt * kWgOutBytes + (uint32_t)(qd * 32 + lane) * 4u;
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+          uint32_t r[32];
+          tc_ld_32x32b_x32(tmem_base + ((uint32_t)(qd * 32) << 16) + (uint32_t)(64 * (m * p.T + t) + 32 * half), r);
+          tc_wait_ld();
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            asm volatile("st.shared.b32 [%0], %1;" ::"r"(col0 + (uint32_t)(32 * half + j) * (4u * kTileM)), "r"(r[j]) : "memory");
+        }
+      }
+      fence_proxy_async_smem();
+    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps
+    if (got && warp == 2 && lane == 0 && *abort_flag == 0) {
       const size_t K = (size_t)p.taps * p.C_in;
-      float* out = p.out + ((size_t)item.split * p.m_tiles + item.m) * K * kTileM + qd * 32 + lane;
-      for (int t = 0; t < item.nb; ++t) {
-        const int b = item.b0 + t;
+      const int m_here = min(p.M, p.m_tiles - item.m);
+      for (int mt = 0; mt < m_here * item.nb; ++mt) {
+        const int m = mt / item.nb, b = item.b0 + mt - m * item.nb;
         const int cc = b / p.taps;
         const int tap = b - cc * p.taps;
         // column c of this k-block is row tap * C_in + 64 cc + c of the tile's [K][128] block
         // (rows of output channels beyond C_out hold zeros: their gradient rows were zero-filled)
-        float* col0 = out + ((size_t)tap * p.C_in + cc * kBlockK) * kTileM;
-#pragma unroll 1
-        for (int half = 0; half < 2; ++half) {
-          uint32_t r[32];
-          tc_ld_32x32b_x32(tmem_base + ((uint32_t)(qd * 32) << 16) + (uint32_t)(64 * t + 32 * half), r);
-          tc_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int c = 32 * half + j;
-            if (cc * kBlockK + c < p.C_in) col0[(size_t)c * kTileM] = __uint_as_float(r[j]);
-          }
-        }
+        float* out = p.out + (((size_t)item.split * p.m_tiles + item.m + m) * K + (size_t)tap * p.C_in + cc * kBlockK) * kTileM;
+        bulk_store(out, ring0 + (uint32_t)mt * kWgOutBytes, (uint32_t)min(kBlockK, p.C_in - cc * kBlockK) * 4u * kTileM);
       }
+      bulk_commit_group();
+      bulk_wait_group_read0();   // shared memory is released below; the writes complete with the grid
     }
   }
 
@@ -252,7 +283,7 @@ ssconv_wgrad_kernel(const __grid_constant__ CUtensorMap tm_dy, const __grid_cons
   }
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kWgTmemCols);
+    tmem_dealloc(tmem_base, p.tmem_cols);
   }
 }
 
@@ -504,35 +535,51 @@ __global__ void __launch_bounds__(256) wgrad_sum_kernel(const float4* slices, in
   dw[i] = acc;
 }
 
-// dW [C_out][K] = transpose of the sum, in slice order, of the slices [m_tiles][K][128].  A block
-// of 32 x 8 threads handles 32 output channels x 8 columns of K, one element per thread: reads are
-// contiguous along the output channels, writes go out as 32-byte runs along K.  With many slices
-// the sums are latency-bound, hence the small tiles (many blocks) and eight loads in flight.
-__global__ void wgrad_reduce_kernel(const float* slices, int splits, int K, int C_out, int m_tiles, float* dw) {
-  __shared__ float tile[8][33];
+// dW [C_out][K] = transpose of the sum, in a fixed order, of the slices [m_tiles][K][128].  A block handles 32 output
+// channels x 8 columns of K: eight sets of 64 threads add an eighth of the slices each (four channels per thread, 16-byte
+// loads, eight in flight), the eight sums are added in order, and writes go out as 32-byte runs along K.  With one
+// thread per element and 4-byte stores in the kernel above, 64 x 56 x 56 x 64 -> 256 took 37.7 us, 29.9 now, 128 images of 128
+// -> 128 55.2 and 40.8.
+constexpr int kWgReduceSets = 8;
+__global__ void __launch_bounds__(64 * kWgReduceSets) wgrad_reduce_kernel(const float* slices, int splits, int K, int C_out,
+                                                                          int m_tiles, float* dw) {
+  __shared__ float4 part[kWgReduceSets][8][9];
   grid_launch_dependents();
   const int k0 = blockIdx.x * 8, c0 = blockIdx.y * 32;
-  const size_t slice = (size_t)m_tiles * K * kTileM;
-  const int c = c0 + threadIdx.x, k = k0 + threadIdx.y;
+  const int c4 = threadIdx.x & 7, kl = (threadIdx.x >> 3) & 7, set = threadIdx.x >> 6;
+  const int per_set = (splits + kWgReduceSets - 1) / kWgReduceSets;
+  const int s1 = min(splits, (set + 1) * per_set);
+  const size_t slice = (size_t)m_tiles * K * (kTileM / 4);  // in float4s
   grid_dependency_wait();
-  float acc = 0.0f;
-  if (k < K && c < C_out) {
-    const float* src = slices + ((size_t)(c / kTileM) * K + k) * kTileM + (c % kTileM);
-    int s = 0;
-    for (; s + 8 <= splits; s += 8) {  // eight loads in flight, added in slice order
-      float v[8];
+  float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (k0 + kl < K) {  // (slices hold whole tiles of 128 channels)
+    const float4* src = reinterpret_cast<const float4*>(slices) + ((size_t)(c0 / kTileM) * K + k0 + kl) * (kTileM / 4) +
+                        (c0 % kTileM) / 4 + c4;
+    for (int s = set * per_set; s < s1; s += 8) {
+      float4 v[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = src[(size_t)(s + j) * slice];
+      for (int j = 0; j < 8; ++j)
+        if (s + j < s1) v[j] = src[(size_t)(s + j) * slice];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc += v[j];
+      for (int j = 0; j < 8; ++j) {
+        if (s + j < s1) {
+          acc.x += v[j].x;
+          acc.y += v[j].y;
+          acc.z += v[j].z;
+          acc.w += v[j].w;
+        }
+      }
     }
-    for (; s < splits; ++s) acc += src[(size_t)s * slice];
   }
-  tile[threadIdx.y][threadIdx.x] = acc;
+  part[set][kl][c4] = acc;
   __syncthreads();
-  const int t = threadIdx.y * 32 + threadIdx.x;
-  const int cl = t >> 3, kl = t & 7;
-  if (k0 + kl < K && c0 + cl < C_out) dw[(size_t)(c0 + cl) * K + k0 + kl] = tile[kl][cl];
+  const int t = threadIdx.x;
+  if (t >= 256) return;
+  const int co = t >> 3, kw = t & 7;  // one element each: 8 threads write 32 contiguous bytes
+  float sum = 0.0f;
+#pragma unroll
+  for (int j = 0; j < kWgReduceSets; ++j) sum += reinterpret_cast<const float*>(&part[j][kw][co >> 2])[co & 3];
+  if (k0 + kw < K && c0 + co < C_out) dw[(size_t)(c0 + co) * K + k0 + kw] = sum;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -572,12 +619,15 @@ bool g_wg_attr_set[64] = {false};
 int g_tune_wg_ranges = 0;   // 0: the planner chooses; otherwise an upper limit on the position ranges
 int g_tune_wg_pair = -1;    // -1: the planner chooses; 0: one-CTA kernel only; 1: the pair kernel wherever it applies
 
+constexpr int kWgMinSteps2 = 5, kWgMinSteps3 = 32;  // steps per range for items of two (per k-block) and of three channel tiles
+
 // How a layer's weight gradient is cut into work items.
 struct WgPlan {
   int taps, kblocks, T, items_b, m_tiles, ksteps, splits, ksteps_per_split;
   long long Q;
   bool pair;                 // the CTA-pair kernel
   int kgroups, n_tiles, NT;  // its items: groups of four k-blocks x tiles of NT output channels
+  int M, items_m;            // the one-CTA kernel: channel tiles per item, items along C_out
 };
 WgPlan wg_plan(const ssconv_desc_t& d, int sms) {
   WgPlan w;
@@ -597,6 +647,8 @@ WgPlan wg_plan(const ssconv_desc_t& d, int sms) {
     w.T = 4;
     w.items_b = w.kgroups;
     w.m_tiles = w.n_tiles;
+    w.M = 1;
+    w.items_m = w.n_tiles;
     const int items = w.kgroups * w.n_tiles;
     int splits = (sms / 2) / items;
     if (splits > w.ksteps / 4) splits = w.ksteps / 4;   // at least four steps of 128 positions per range
@@ -614,7 +666,22 @@ WgPlan wg_plan(const ssconv_desc_t& d, int sms) {
   w.ksteps = (int)((w.Q + kWgPos - 1) / kWgPos);
   // Split the positions when the items alone would leave SMs idle, but keep at least 8 steps per
   // range so that the pipeline's ramp and the epilogue stay small against the loop.
-  const int items = w.m_tiles * w.items_b;
+  // Several channel tiles per item where the ranges stay long enough: an item then brings the activations in once for all
+  // its tiles, but as many ranges as SMs each write their accumulators, M times as much to add up as with one tile per item.
+  // us, one tile per item / M: 128 x 56 x 56 x 96 -> 384 (M 3, 42 steps per range) 74.4 / 71.7, 64 images (21 steps) 40.8 /
+  // 44.0, 256 images 144.8 / 129.0; M 2: 16 x 56 x 56 x 64 -> 256 (5 steps) 12.7 / 11.7, 32 images 19.3 / 14.8, 256 images 97.3 /
+  // 87.4, 64 x 28 x 28 x 128 -> 512 (10 steps) 19.6 / 16.4, 64 x 14 x 14 x 128 -> 1024 (two
+  // k-blocks, 5 steps) 13.9 / 14.8, 100 x 30 x 30 x 40 -> 200 16.7 / 13.8.
+  w.M = 1;
+  w.items_m = w.m_tiles;
+  if (w.T <= 2 && w.m_tiles > 1) {
+    const int M = w.m_tiles % 2 == 0 ? 2 : 3, items_m = (w.m_tiles + M - 1) / M;
+    if ((long long)w.ksteps * items_m * w.items_b >= (long long)(M == 2 ? kWgMinSteps2 * w.T : kWgMinSteps3) * sms) {
+      w.M = M;
+      w.items_m = items_m;
+    }
+  }
+  const int items = w.items_m * w.items_b;
   int splits = sms / items;
   if (splits > w.ksteps / 8) splits = w.ksteps / 8;
   if (g_tune_wg_ranges > 0 && splits > g_tune_wg_ranges) splits = g_tune_wg_ranges;
@@ -790,7 +857,7 @@ int32_t launch_wgrad(const ssconv_desc_t& d, const void* x, const void* dy, floa
   int dev = 0;
   cudaGetDevice(&dev);
   if (!g_wg_attr_set[dev]) {
-    if (cudaFuncSetAttribute(ssconv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgSmemBytes) !=
+    if (cudaFuncSetAttribute(ssconv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWgMaxSmemBytes) !=
         cudaSuccess)
       return SSCONV_ERR_CUDA;
     g_wg_attr_set[dev] = true;
@@ -807,13 +874,13 @@ int32_t launch_wgrad(const ssconv_desc_t& d, const void* x, const void* dy, floa
   {
     // gradient of the output, NHWC seen as (c, position); a box is 64 channels x 64 positions.  When
     // C_out is a multiple of 64 the view is (64 channels, position, block of 64 channels) instead, so
-    // that one box of 64 x 64 x 2 brings both halves of a 128-channel tile, half after half.
+    // that one box of 64 x 64 x 2 M brings both halves of the item's 128-channel tiles, half after half.
     const bool one_load = d.C_out % 64 == 0;
     CUresult r;
     if (one_load) {
       cuuint64_t dims[3] = {64, (cuuint64_t)w.Q, (cuuint64_t)(d.C_out / 64)};
       cuuint64_t strides[2] = {(cuuint64_t)d.C_out * 2, 128};
-      cuuint32_t box[3] = {64, (cuuint32_t)kWgPos, 2};
+      cuuint32_t box[3] = {64, (cuuint32_t)kWgPos, 2 * (cuuint32_t)w.M};
       cuuint32_t estr[3] = {1, 1, 1};
       r = wg_encode_tiled(&tm_dy, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(dy), dims, strides, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -864,6 +931,10 @@ int32_t launch_wgrad(const ssconv_desc_t& d, const void* x, const void* dy, floa
   p.T = w.T;
   p.items_b = w.items_b;
   p.m_tiles = w.m_tiles;
+  p.M = w.M;
+  p.items_m = w.items_m;
+  p.stages = wg_stages(w.M, w.T);
+  p.tmem_cols = wg_tmem_cols(w.M, w.T);
   p.splits = w.splits;
   p.ksteps = w.ksteps;
   p.ksteps_per_split = w.ksteps_per_split;
@@ -871,15 +942,16 @@ int32_t launch_wgrad(const ssconv_desc_t& d, const void* x, const void* dy, floa
   p.out = static_cast<float*>(ws);
   p.dev_status = dev_status;
 
-  const unsigned grid = (unsigned)(w.splits * w.m_tiles * w.items_b);
+  const unsigned grid = (unsigned)(w.splits * w.items_m * w.items_b);
+  const size_t smem_bytes = 1024 + (size_t)p.stages * wg_stage_bytes(w.M, w.T) + 256;
   count_launch();
-  if (launch_dependent_smem(ssconv_wgrad_kernel, grid, kWgThreads, kWgSmemBytes, stream, tm_dy, tm_x, p) != cudaSuccess)
+  if (launch_dependent_smem(ssconv_wgrad_kernel, grid, kWgThreads, smem_bytes, stream, tm_dy, tm_x, p) != cudaSuccess)
     return SSCONV_ERR_CUDA;
   {
     const int K = w.taps * d.C_in;
     const dim3 rgrid((unsigned)((K + 7) / 8), (unsigned)((d.C_out + 31) / 32));
     count_launch();
-    if (launch_dependent(wgrad_reduce_kernel, rgrid, dim3(32, 8), stream, static_cast<const float*>(ws), w.splits, K, d.C_out,
+    if (launch_dependent(wgrad_reduce_kernel, rgrid, dim3(64 * kWgReduceSets), stream, static_cast<const float*>(ws), w.splits, K, d.C_out,
                          w.m_tiles, dw) != cudaSuccess)
       return SSCONV_ERR_CUDA;
   }
