@@ -3,7 +3,22 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 namespace ssconv {
+
+// SMs of the current device (148 where it cannot be asked: grids are sized by it, nothing else).
+inline int device_sms() {
+  static std::atomic<int> known[64];
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  sms = known[dev].load(std::memory_order_relaxed);
+  if (sms == 0) {
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 148;
+    known[dev].store(sms, std::memory_order_relaxed);
+  }
+  return sms;
+}
 
 // Launch with programmatic stream serialisation, for kernels whose every thread calls grid_dependency_wait() before its
 // first access to global memory (by plain loads: read-only ones could be moved above the wait, or find a line that was

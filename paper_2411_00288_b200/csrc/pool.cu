@@ -705,6 +705,96 @@ __global__ void __launch_bounds__(256) layernorm_vec_kernel(const uint4* x, cons
   }
 }
 
+// The same for few pixels (a turn or a few per warp of the chip): the scale and shift are loaded with the first pixels, not
+// after their statistics, which is a latency less, and stay in registers for a warp's further pixels, whose loads are in
+// flight meanwhile.  us, the kernel above / this one: 3 x 56 x 56 x 96 2.7 / 2.2, 3 x 14 x 14 x 384 2.5 / 2.0, 16 x 14 x 14 x
+// 384 3.5 / 3.0 (one turn), 128 x 7 x 7 x 768 6.5 / 5.3 (3 turns); beyond the line 128 x 14 x 14 x 384 9.1 / 9.8 (5), 128 x 56 x
+// 56 x 96 29.8 / 35.4 (17): its 110 registers leave too few warps to keep memory busy.
+constexpr long long kLnFewTurns = 3;
+template <int V>
+__global__ void __launch_bounds__(128) layernorm_few_kernel(const uint4* x, const float* gamma, const float* beta, uint4* y,
+                                                            long long pixels, int C8, int G, float eps) {
+  grid_launch_dependents();
+  const int lane = threadIdx.x & 31;
+  const int sub = lane & (G - 1);
+  const int per_warp = 32 / G;
+  const long long step = (long long)gridDim.x * (blockDim.x >> 5) * per_warp;
+  long long pix = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp + lane / G;
+  grid_dependency_wait();
+  uint4 next[V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    next[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (pix < pixels && sub + k * G < C8) next[k] = x[pix * C8 + sub + k * G];
+  }
+  float gg[V][8], bb[V][8];
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const int idx = sub + k * G;
+    float4 g0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), g1 = g0, b0 = g0, b1 = g0;
+    if (idx < C8) {
+      g0 = reinterpret_cast<const float4*>(gamma)[2 * idx];
+      g1 = reinterpret_cast<const float4*>(gamma)[2 * idx + 1];
+      b0 = reinterpret_cast<const float4*>(beta)[2 * idx];
+      b1 = reinterpret_cast<const float4*>(beta)[2 * idx + 1];
+    }
+    gg[k][0] = g0.x; gg[k][1] = g0.y; gg[k][2] = g0.z; gg[k][3] = g0.w;
+    gg[k][4] = g1.x; gg[k][5] = g1.y; gg[k][6] = g1.z; gg[k][7] = g1.w;
+    bb[k][0] = b0.x; bb[k][1] = b0.y; bb[k][2] = b0.z; bb[k][3] = b0.w;
+    bb[k][4] = b1.x; bb[k][5] = b1.y; bb[k][6] = b1.z; bb[k][7] = b1.w;
+  }
+  // (a warp's lanes leave together: its first pixel decides)
+  for (long long first = pix - lane / G; first < pixels; first += step, pix += step) {
+    const bool live = pix < pixels;
+    float f[V][8];
+    float sum = 0.0f;
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      const uint32_t a[4] = {next[k].x, next[k].y, next[k].z, next[k].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        f[k][2 * j] = __uint_as_float(a[j] << 16);
+        f[k][2 * j + 1] = __uint_as_float(a[j] & 0xFFFF0000u);
+        sum += f[k][2 * j] + f[k][2 * j + 1];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      next[k] = make_uint4(0u, 0u, 0u, 0u);
+      if (pix + step < pixels && sub + k * G < C8) next[k] = x[(pix + step) * C8 + sub + k * G];
+    }
+    for (int o = G >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    const float inv_c = 1.0f / (float)(8 * C8);
+    const float mean = sum * inv_c;
+    float sq = 0.0f;
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      if (sub + k * G < C8) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float d = f[k][j] - mean;
+          sq += d * d;
+        }
+      }
+    }
+    for (int o = G >> 1; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    const float rstd = rsqrtf(sq * inv_c + eps);
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      const int idx = sub + k * G;
+      if (!live || idx >= C8) continue;
+      uint32_t o[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        __nv_bfloat162 p = __floats2bfloat162_rn((f[k][2 * j] - mean) * rstd * gg[k][2 * j] + bb[k][2 * j],
+                                                 (f[k][2 * j + 1] - mean) * rstd * gg[k][2 * j + 1] + bb[k][2 * j + 1]);
+        o[j] = *reinterpret_cast<uint32_t*>(&p);
+      }
+      y[pix * C8 + idx] = make_uint4(o[0], o[1], o[2], o[3]);
+    }
+  }
+}
+
 cudaError_t launch_layernorm(const void* x, const float* gamma, const float* beta, void* y, long long pixels, int C,
                              float eps, cudaStream_t st) {
   if (pixels == 0) return cudaSuccess;
@@ -724,16 +814,25 @@ cudaError_t launch_layernorm(const void* x, const float* gamma, const float* bet
     }
     const int V = (C8 + G - 1) / G;
     const long long warps = (pixels + (32 / G) - 1) / (32 / G);
-    const unsigned grid = (unsigned)((warps * 32 + T - 1) / T);
     const uint4* xp = static_cast<const uint4*>(x);
     uint4* yp = static_cast<uint4*>(y);
-    if (V == 1)
-      return launch_dependent(layernorm_vec_kernel<1>, grid, T, st, xp, gamma, beta, yp, pixels, C8, G, eps);
-    if (V == 2)
-      return launch_dependent(layernorm_vec_kernel<2>, grid, T, st, xp, gamma, beta, yp, pixels, C8, G, eps);
-    if (V == 3)
-      return launch_dependent(layernorm_vec_kernel<3>, grid, T, st, xp, gamma, beta, yp, pixels, C8, G, eps);
-    return launch_dependent(layernorm_vec_kernel<4>, grid, T, st, xp, gamma, beta, yp, pixels, C8, G, eps);
+    // blocks of four warps, as many as are resident at once, every warp with the same number of turns (or one fewer)
+    const long long most = 4ll * (V <= 2 ? 7 : V == 3 ? 5 : 4) * device_sms();
+    const long long turns = (warps + most - 1) / most;
+    if (turns <= kLnFewTurns) {
+      const unsigned few = (unsigned)(((warps + turns - 1) / turns + 3) / 4);
+      const auto kernel = V == 1   ? layernorm_few_kernel<1>
+                          : V == 2 ? layernorm_few_kernel<2>
+                          : V == 3 ? layernorm_few_kernel<3>
+                                   : layernorm_few_kernel<4>;
+      return launch_dependent(kernel, few, 128, st, xp, gamma, beta, yp, pixels, C8, G, eps);
+    }
+    const unsigned grid = (unsigned)((warps * 32 + T - 1) / T);
+    const auto kernel = V == 1   ? layernorm_vec_kernel<1>
+                        : V == 2 ? layernorm_vec_kernel<2>
+                        : V == 3 ? layernorm_vec_kernel<3>
+                                 : layernorm_vec_kernel<4>;
+    return launch_dependent(kernel, grid, T, st, xp, gamma, beta, yp, pixels, C8, G, eps);
   }
   layernorm_kernel<<<(unsigned)((pixels * 32 + T - 1) / T), T, 0, st>>>(static_cast<const __nv_bfloat16*>(x), gamma, beta,
                                                                         static_cast<__nv_bfloat16*>(y), pixels, C, eps);
