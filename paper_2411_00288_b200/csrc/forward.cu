@@ -43,7 +43,8 @@
 // ("stream-K").  A CTA writes a partly computed tile (fp32) to a scratch region of its own in
 // global memory; a second, small kernel (ssconv_split_finish_kernel) then sums the regions of
 // every split tile in a fixed order on all SMs and applies the same epilogue.  No CTA ever waits
-// for another, and the result does not depend on timing.
+// for another, and the result does not depend on timing.  Layers of very few tiles give each tile to a cluster of CTAs
+// instead, which add up its parts among themselves (ssconv_fwd_cluster_kernel).
 // All mbarrier waits are bounded; when one runs out the CTA raises a flag, every role leaves
 // its loop, TMEM is freed and SSCONV_ERR_TIMEOUT is stored to *dev_status.
 #include <cuda.h>
