@@ -91,7 +91,8 @@ int32_t ssconv_sizes(const ssconv_desc_t* desc, int64_t* G, size_t* w_comp_bytes
 /* How ssconv_forward (sparse != 0) or ssconv_forward_dense (sparse == 0) would run this layer on
  * the current device: positions per output tile (the N of the tensor-core instruction, a multiple
  * of 16 up to 240, chosen so that the tiles fill the SMs), whether the K range is split across
- * thread blocks (then a second, finishing kernel runs and ws is used), the number of thread
+ * thread blocks (over the grid: then a second, finishing kernel runs and ws is used; or, with very few
+ * tiles, over the blocks of a cluster per tile, in one kernel and without ws), the number of thread
  * blocks, the depth of the shared-memory ring in pairs of 64-column k-blocks, and whether the layer
  * runs on pairs of thread blocks that share tiles of 256 output channels (layers with more than 128
  * output channels and enough tiles; ctas is then twice the number of pairs).  A tuning aid with no
