@@ -343,10 +343,10 @@ cudaError_t launch_select(int mode, const void* scores, int64_t G, uint8_t* patt
   const int T = 256;
   count_launch();
   if (mode == SSCONV_MASK_LOGITS_F32)
-    return launch_dependent(select_logits_kernel, blocks_for(G, T), T, st, (const float2*)scores, G, pattern);
+    return launch_short(select_logits_kernel, blocks_for(G, T), T, st, (const float2*)scores, G, pattern);
   if (mode == SSCONV_MASK_MAGNITUDE_E4M3)
-    return launch_dependent(select_magnitude_e4m3_kernel, blocks_for(G, T), T, st, (const uint32_t*)scores, G, pattern);
-  return launch_dependent(select_magnitude_kernel, blocks_for(G, T), T, st, (const uint2*)scores, G, pattern);
+    return launch_short(select_magnitude_e4m3_kernel, blocks_for(G, T), T, st, (const uint32_t*)scores, G, pattern);
+  return launch_short(select_magnitude_kernel, blocks_for(G, T), T, st, (const uint2*)scores, G, pattern);
 }
 
 // All N-subsets of {0..M-1} in lexicographic order of the kept positions, as bitmasks.
@@ -402,7 +402,7 @@ cudaError_t launch_quantize_e4m3(const void* x, void* y, int64_t n, float scale,
   count_launch();
   const bool wide = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u) == 0;
   const int64_t pairs = n / 2, vectors = wide ? n / 16 : 0;
-  return launch_dependent(quantize_e4m3_kernel, blocks_for(vectors + (pairs - 8 * vectors), T), T, st, (const uint32_t*)x,
+  return launch_short(quantize_e4m3_kernel, blocks_for(vectors + (pairs - 8 * vectors), T), T, st, (const uint32_t*)x,
                           (uint16_t*)y, vectors, pairs, scale);
 }
 
@@ -437,7 +437,7 @@ cudaError_t launch_compress(const ssconv_desc_t& d, const void* w, const uint8_t
   Geometry geo = make_geometry(d);
   const int T = 256;
   count_launch();
-  return launch_dependent(compress_kernel, blocks_for((int64_t)geo.m_tiles * geo.stages * 512, T), T, st, d, geo, (const uint4*)w,
+  return launch_short(compress_kernel, blocks_for((int64_t)geo.m_tiles * geo.stages * 512, T), T, st, d, geo, (const uint4*)w,
                           pattern, (uint4*)w_comp, (uint32_t*)meta);
 }
 

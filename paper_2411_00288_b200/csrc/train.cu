@@ -3,7 +3,7 @@
 // M .* W (Eq. 6 with the soft mask) that the dense convolution then uses, and the gradient
 // from dL/dW_eff back to the choice weights.  One thread per group of four weights; both
 // kernels move 70-90 bytes per group and do a handful of flops: HBM-bound, or, on most layers, too short to be bound by
-// anything but their launches: the kernels of a step start while the one before them finishes (launch_dependent).
+// anything but their launches: the kernels of a step start while the one before them finishes (launch_short).
 #include <cuda_runtime.h>
 
 #include "launch.cuh"
@@ -146,7 +146,7 @@ cudaError_t launch_adamw(float* theta, const float* g, float* m, float* v, int64
   const int threads = 256;
   const int64_t work = (n >> 2) + (n & 3);
   count_launch();
-  return launch_dependent(adamw_kernel, (unsigned)((work + threads - 1) / threads), threads, st, theta, g, m, v, n, lr, beta1,
+  return launch_short(adamw_kernel, (unsigned)((work + threads - 1) / threads), threads, st, theta, g, m, v, n, lr, beta1,
                           beta2, eps, wd, c1, c2);
 }
 
@@ -360,7 +360,7 @@ cudaError_t launch_dgrad_fused_weights(const void* w, void* w_all, int C_out, in
   if (C_in == 0 || C_out == 0) return cudaSuccess;
   const dim3 grid((unsigned)((C_in + 31) / 32), (unsigned)((C_out + 31) / 32), (unsigned)(sh * sw * Jh * Jw));
   count_launch();
-  return launch_dependent(dgrad_fused_weights_kernel, grid, 256, st, (const uint16_t*)w, (uint16_t*)w_all, C_out, KH, KW, C_in,
+  return launch_short(dgrad_fused_weights_kernel, grid, 256, st, (const uint16_t*)w, (uint16_t*)w_all, C_out, KH, KW, C_in,
                           Jh, Jw, sh, sw);
 }
 
@@ -405,7 +405,7 @@ cudaError_t launch_dgrad_gather(const DgradClasses& cls, void* dx, int N, int H,
   const long long total = (long long)N * H * W * (C / 8);
   if (total == 0) return cudaSuccess;
   count_launch();
-  return launch_dependent(dgrad_gather_kernel, (unsigned)((total + 255) / 256), 256, st, cls, (uint4*)dx, total, H, W, C / 8,
+  return launch_short(dgrad_gather_kernel, (unsigned)((total + 255) / 256), 256, st, cls, (uint4*)dx, total, H, W, C / 8,
                           pitch / 8, sh, sw, ph, pw);
 }
 
@@ -414,7 +414,7 @@ cudaError_t launch_soft_mask(const float* logits, const float* noise, float tau,
   const int threads = 256;
   const int64_t blocks = (G + threads - 1) / threads;
   count_launch();
-  return launch_dependent(soft_mask_kernel, (unsigned)blocks, threads, st, logits, noise, 1.0f / tau, (const uint2*)w, G, z,
+  return launch_short(soft_mask_kernel, (unsigned)blocks, threads, st, logits, noise, 1.0f / tau, (const uint2*)w, G, z,
                           (uint2*)w_eff);
 }
 
@@ -423,7 +423,7 @@ cudaError_t launch_mask_grad(const float* z, float tau, const void* w, const flo
   const int threads = 256;
   const int64_t blocks = (G + threads - 1) / threads;
   count_launch();
-  return launch_dependent(mask_grad_kernel, (unsigned)blocks, threads, st, z, 1.0f / tau, (const uint2*)w,
+  return launch_short(mask_grad_kernel, (unsigned)blocks, threads, st, z, 1.0f / tau, (const uint2*)w,
                           (const float4*)g_w_eff, G, g_logits);
 }
 
