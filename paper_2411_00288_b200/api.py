@@ -1,14 +1,15 @@
 """Python binding of libssconv.so: the same entry points as include/ssconv.h.
 
 Only argument marshalling happens here; torch supplies device memory and the current
-stream.  The calls that a network makes per layer and step go through _binding.so (csrc/binding.cpp), which converts and
-checks their arguments in native code; the others through ctypes.  There is no CPU path: if the library is missing or a call fails, an exception
-is raised.
+stream.  The calls that a network makes per layer and step go through the native binding
+(csrc/binding.cpp), which converts and checks their arguments; the others through ctypes.
+There is no CPU path: if the library is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
 
 import ctypes
 import functools
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import Optional, Tuple
@@ -152,11 +153,19 @@ _native = None
 
 
 def _binding():
-    """The native binding (csrc/binding.cpp), loaded once; raise if it has not been built."""
+    """The native binding (csrc/binding.cpp), loaded once; raise if it has not been built for this torch and interpreter."""
     global _native
     if _native is None:
         lib()
-        from . import _binding as native
+        from .build import binding_path
+        path = binding_path()
+        if not os.path.exists(path):
+            raise FileNotFoundError(
+                f"{path} is missing: build it for torch {torch.__version__} with `python -m paper_2411_00288_b200.build` "
+                "(there is no fallback path)")
+        spec = importlib.util.spec_from_file_location(f"{__package__}._binding", path)
+        native = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(native)
         _native = native
     return _native
 

@@ -10,7 +10,6 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(_HERE)
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libssconv.so")
-BINDING = os.path.join(_HERE, "_binding.so")
 SOURCES = ["api.cu", "mask.cu", "pool.cu", "depthwise.cu", "train.cu", "wgrad.cu", "forward.cu"]
 HEADERS = ["launch.cuh", "layout.cuh", "sm100_ptx.cuh"]
 
@@ -20,20 +19,28 @@ def _newest_source_mtime() -> float:
     return max(os.path.getmtime(f) for f in files)
 
 
+def binding_path() -> str:
+    """The native binding's file.  It holds for one torch (whose C++ interface is no stable one) and one interpreter, so
+    both are part of its name: after a change of either another file is built and looked for."""
+    import torch
+    return os.path.join(_HERE, f"_binding.torch-{torch.__version__}{sysconfig.get_config_var('EXT_SUFFIX')}")
+
+
 def build_binding(force: bool = False) -> str:
-    """_binding.so against the installed torch (csrc/binding.cpp); after the library, which it is linked with."""
+    """The binding (csrc/binding.cpp) against the installed torch; after the library, which it is linked with."""
+    binding = binding_path()
     sources = [os.path.join(CSRC, "binding.cpp"), os.path.join(ROOT, "include", "ssconv.h")]
-    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= max(os.path.getmtime(f) for f in sources):
-        return BINDING
+    if not force and os.path.exists(binding) and os.path.getmtime(binding) >= max(os.path.getmtime(f) for f in sources):
+        return binding
     import torch
     t = os.path.dirname(torch.__file__)
     includes = [os.path.join(ROOT, "include"), sysconfig.get_paths()["include"], os.path.join(t, "include"),
                 os.path.join(t, "include", "torch", "csrc", "api", "include"),
                 os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")]
     subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC"] + ["-I" + i for i in includes] +
-                   [sources[0], "-o", BINDING, "-L" + os.path.join(t, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu",
+                   [sources[0], "-o", binding, "-L" + os.path.join(t, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu",
                     "-lc10", "-lc10_cuda", "-L" + _HERE, "-l:libssconv.so", "-Wl,-rpath,$ORIGIN"], check=True)
-    return BINDING
+    return binding
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -49,3 +49,12 @@ def test_the_librarys_status_comes_back(native):
     assert y.shape == (2, 4, 5, 40) and y.dtype == torch.bfloat16
     assert native.blob(7, torch.zeros(1)).shape == (7,)
     assert ctypes.sizeof(api.Desc) == 56
+
+
+def test_a_binding_built_for_another_torch_is_not_loaded(native, monkeypatch):
+    monkeypatch.setattr(api, "_native", None)
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    with pytest.raises(FileNotFoundError, match="python -m paper_2411_00288_b200.build"):
+        api._binding()
+    monkeypatch.undo()
+    assert api._binding() is not None
