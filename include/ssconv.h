@@ -358,7 +358,9 @@ int32_t ssconv_adamw(float* theta, const float* g, float* m, float* v, int64_t n
  * ws: scratch of at least ssconv_wgrad_ws_bytes, always needed: thread blocks store partial
  * gradients there (one slice per range of positions; layers with few weights and many positions
  * split the positions over thread blocks), and a second kernel adds the slices in a fixed order
- * and writes dw.  Needs no initialisation.  dev_status: as in ssconv_forward. */
+ * and writes dw.  Layers of one or two k-blocks and several tiles of 128 output channels may take up to three
+ * times the scratch of a tile per work item (one slice per SM, at most); they also run, more slowly, in what a
+ * tile per work item leaves: SMs / tiles slices of tiles x 128 x KH KW C_in floats.  Needs no initialisation.  dev_status: as in ssconv_forward. */
 int32_t ssconv_wgrad(const ssconv_desc_t* desc, const void* x, const void* dy, float* dw, void* ws,
                      size_t ws_bytes, int32_t* dev_status, void* stream);
 /* The gradient with respect to the layer's input in one call (Eq. 4 differentiated in x; the paper prints

@@ -629,7 +629,7 @@ struct WgPlan {
   int kgroups, n_tiles, NT;  // its items: groups of four k-blocks x tiles of NT output channels
   int M, items_m;            // the one-CTA kernel: channel tiles per item, items along C_out
 };
-WgPlan wg_plan(const ssconv_desc_t& d, int sms) {
+WgPlan wg_plan(const ssconv_desc_t& d, int sms, bool one_tile = false) {  // (one_tile: channel tiles one per item)
   WgPlan w;
   w.taps = d.KH * d.KW;
   w.kblocks = w.taps * ((d.C_in + kBlockK - 1) / kBlockK);
@@ -674,7 +674,7 @@ WgPlan wg_plan(const ssconv_desc_t& d, int sms) {
   // k-blocks, 5 steps) 13.9 / 14.8, 100 x 30 x 30 x 40 -> 200 16.7 / 13.8.
   w.M = 1;
   w.items_m = w.m_tiles;
-  if (w.T <= 2 && w.m_tiles > 1) {
+  if (w.T <= 2 && w.m_tiles > 1 && !one_tile) {
     const int M = w.m_tiles % 2 == 0 ? 2 : 3, items_m = (w.m_tiles + M - 1) / M;
     if ((long long)w.ksteps * items_m * w.items_b >= (long long)(M == 2 ? kWgMinSteps2 * w.T : kWgMinSteps3) * sms) {
       w.M = M;
@@ -689,6 +689,11 @@ WgPlan wg_plan(const ssconv_desc_t& d, int sms) {
   w.ksteps_per_split = (w.ksteps + splits - 1) / splits;
   w.splits = (w.ksteps + w.ksteps_per_split - 1) / w.ksteps_per_split;  // no empty range
   return w;
+}
+
+// Scratch of the one-CTA kernel: a slice per range.
+size_t wg_scratch_bytes(const ssconv_desc_t& d, const WgPlan& w) {
+  return (size_t)w.splits * w.m_tiles * kTileM * w.taps * d.C_in * sizeof(float);
 }
 
 int wg_sm_count(int* sms) {
@@ -727,7 +732,7 @@ int32_t wgrad_workspace_bytes(const ssconv_desc_t& d, size_t* bytes) {
   if (w.pair)
     *bytes = w.splits > 1 ? (size_t)w.splits * d.C_out * w.taps * d.C_in * sizeof(float) : 0;
   else
-    *bytes = (size_t)w.splits * w.m_tiles * kTileM * w.taps * d.C_in * sizeof(float);
+    *bytes = wg_scratch_bytes(d, w);
   return SSCONV_OK;
 }
 
@@ -862,13 +867,15 @@ int32_t launch_wgrad(const ssconv_desc_t& d, const void* x, const void* dy, floa
       return SSCONV_ERR_CUDA;
     g_wg_attr_set[dev] = true;
   }
-  const WgPlan w = wg_plan(d, sms);
+  WgPlan w = wg_plan(d, sms);
+  // Items of several channel tiles leave up to that many times the ranges; a caller whose scratch holds the slices of items
+  // of one tile gets those.
+  if (!w.pair && w.M > 1 && ws_bytes < wg_scratch_bytes(d, w)) w = wg_plan(d, sms, true);
   if (w.Q > 0x7FFFFF00LL) return SSCONV_ERR_UNSUPPORTED_SHAPE;
   const int Ho = wg_out_extent(d.H, d.KH, d.stride_h, d.pad_h, d.dil_h);
   const int Wo = wg_out_extent(d.W, d.KW, d.stride_w, d.pad_w, d.dil_w);
   if (w.pair) return launch_wgrad_pair(d, w, Ho, Wo, x, dy, dw, ws, ws_bytes, dev_status, stream);
-  const size_t slice_bytes = (size_t)w.m_tiles * kTileM * w.taps * d.C_in * sizeof(float);
-  if (ws == nullptr || ws_bytes < (size_t)w.splits * slice_bytes) return SSCONV_ERR_WORKSPACE;
+  if (ws == nullptr || ws_bytes < wg_scratch_bytes(d, w)) return SSCONV_ERR_WORKSPACE;
 
   CUtensorMap tm_dy, tm_x;
   {

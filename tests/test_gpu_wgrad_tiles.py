@@ -33,3 +33,26 @@ def test_wgrad_items_of_several_channel_tiles(case):
     assert int(status.item()) == 0
     assert rel <= 1e-4, f"{name}: {rel:.3e}"      # fp32 sums of exact products, as for every weight gradient
     assert torch.equal(dw, again)
+
+
+@pytest.mark.parametrize("case", CASES[:3], ids=[c[0] for c in CASES[:3]])
+def test_wgrad_in_the_scratch_of_items_of_one_channel_tile(case):
+    name, n, h, w, ci, co = case
+    n *= 2                                                      # (enough positions for items of several tiles)
+    g = torch.Generator(device=DEV).manual_seed(7150 + CASES.index(case))
+    desc = api.make_desc(n, h, w, ci, co, 1, 1, bias=False)
+    x = torch.randn((n, h, w, ci), generator=g, device=DEV).to(torch.bfloat16)
+    dy = torch.randn((n, h, w, co), generator=g, device=DEV).to(torch.bfloat16)
+    tiles, steps = -(-co // 128), -(-n * h * w // 64)
+    ranges = torch.cuda.get_device_properties(0).multi_processor_count // tiles
+    ranges = -(-steps // -(-steps // ranges))                   # (none of them empty)
+    small = ranges * tiles * 128 * ci * 4
+    need = api.ssconv_wgrad_ws_bytes(desc)
+    assert small < need
+    ws = torch.empty(need, dtype=torch.uint8, device=DEV)
+    ref = dy.reshape(-1, co).double().T @ x.reshape(-1, ci).double()
+    for size in (small, need - 16, need):
+        dw = api.ssconv_wgrad(desc, x, dy, ws=ws[:size])
+        assert float((dw.reshape(co, ci).double() - ref).norm() / ref.norm()) <= 1e-4, size
+    with pytest.raises(api.SsconvError):
+        api.ssconv_wgrad(desc, x, dy, ws=ws[:small - 16])
