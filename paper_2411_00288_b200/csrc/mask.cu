@@ -15,12 +15,14 @@ namespace ssconv {
 // ---------------------------------------------------------------------------------------
 
 // Eq. 1 without the one-hot: first maximum of the six scores of each group.
+template <bool EARLY>
 __global__ void select_logits_kernel(const float2* scores, int64_t G, uint8_t* pattern) {
-  grid_launch_dependents();
+  short_begin<EARLY>();
   int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  grid_dependency_wait();
+  short_wait<EARLY>();
   if (g >= G) return;
-  float2 a = scores[3 * g], b = scores[3 * g + 1], c = scores[3 * g + 2];
+  float2 a = short_load<EARLY>(scores + 3 * g), b = short_load<EARLY>(scores + 3 * g + 1),
+         c = short_load<EARLY>(scores + 3 * g + 2);
   float v[6] = {a.x, a.y, b.x, b.y, c.x, c.y};
   int best = 0;
   float bv = v[0];
@@ -61,22 +63,24 @@ __device__ __forceinline__ uint32_t magnitude_pattern(uint32_t lo, uint32_t hi) 
   return magnitude_pattern4(a);
 }
 
+template <bool EARLY>
 __global__ void select_magnitude_kernel(const uint2* w, int64_t G, uint8_t* pattern) {
-  grid_launch_dependents();
+  short_begin<EARLY>();
   int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  grid_dependency_wait();
+  short_wait<EARLY>();
   if (g >= G) return;
-  uint2 v = w[g];
+  uint2 v = short_load<EARLY>(w + g);
   pattern[g] = (uint8_t)magnitude_pattern(v.x, v.y);
 }
 
 // The same for e4m3 weights: a group is four bytes, a magnitude the 7 bits below the sign bit.
+template <bool EARLY>
 __global__ void select_magnitude_e4m3_kernel(const uint32_t* w, int64_t G, uint8_t* pattern) {
-  grid_launch_dependents();
+  short_begin<EARLY>();
   int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  grid_dependency_wait();
+  short_wait<EARLY>();
   if (g >= G) return;
-  const uint32_t v = w[g];
+  const uint32_t v = short_load<EARLY>(w + g);
   const uint32_t a[4] = {v & 0x7Fu, (v >> 8) & 0x7Fu, (v >> 16) & 0x7Fu, (v >> 24) & 0x7Fu};
   pattern[g] = (uint8_t)magnitude_pattern4(a);
 }
@@ -91,13 +95,15 @@ __device__ __forceinline__ uint32_t e4m3_pair(uint32_t v, float scale) {
   asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(out) : "f"(hi), "f"(lo));
   return out;
 }
+template <bool EARLY>
 __global__ void __launch_bounds__(256) quantize_e4m3_kernel(const uint32_t* x, uint16_t* y, int64_t vectors,
                                                             int64_t pairs, float scale) {
-  grid_launch_dependents();
+  short_begin<EARLY>();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  grid_dependency_wait();
+  short_wait<EARLY>();
   if (i < vectors) {
-    const uint4 a = reinterpret_cast<const uint4*>(x)[2 * i], b = reinterpret_cast<const uint4*>(x)[2 * i + 1];
+    const uint4* v = reinterpret_cast<const uint4*>(x) + 2 * i;
+    const uint4 a = short_load<EARLY>(v), b = short_load<EARLY>(v + 1);
     uint4 o;
     o.x = e4m3_pair(a.x, scale) | (e4m3_pair(a.y, scale) << 16);
     o.y = e4m3_pair(a.z, scale) | (e4m3_pair(a.w, scale) << 16);
@@ -258,11 +264,12 @@ __global__ void decompress_e4m3_kernel(ssconv_desc_t d, Geometry geo, const uint
 // patterns and writes 2 x 16 bytes of values; the eight threads of a row and stage write 128 bytes.  Values and
 // metadata in one launch: a layer's weights are small (0.1 to 2 MB), so a launch more costs as much as the work
 // (52 layers of a ResNet-50: 154 + 120 us for the two kernels with one thread per group, 180 us for this one).
+template <bool EARLY>
 __global__ void __launch_bounds__(256) compress_kernel(ssconv_desc_t d, Geometry geo, const uint4* w, const uint8_t* pattern,
                                                        uint4* w_comp, uint32_t* meta) {
-  grid_launch_dependents();
+  short_begin<EARLY>();
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  grid_dependency_wait();
+  short_wait<EARLY>();
   if (t >= (int64_t)geo.m_tiles * geo.stages * 512) return;
   const int half = (int)(t & 1), j = (int)(t >> 1) & 3, row = ((int)(t >> 3) & 7) + 16 * ((int)(t >> 6) & 7);
   const int64_t tile = t >> 9;  // (channel tile, stage)
@@ -271,22 +278,36 @@ __global__ void __launch_bounds__(256) compress_kernel(ssconv_desc_t d, Geometry
   const int tap = b % geo.taps;
   const int col = (j & 1) * 32 + 16 * half;  // dense column within the k-block
   const int c = (b / geo.taps) * kBlockK + col;
+  // both rows' loads first: plain ones may not pass the stores
+  const bool in = b < geo.kblocks && c < d.C_in, all = c + 8 < d.C_in;  // (input channels come in multiples of eight)
+  uint4 lo[2], hi[2];
+  uint32_t pat[2][4];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int co = mt * kTileM + row + 8 * h;
+    lo[h] = hi[h] = make_uint4(0u, 0u, 0u, 0u);
+    if (in && co < d.C_out) {
+      const int64_t g = ((int64_t)co * geo.taps + tap) * (d.C_in / 4) + c / 4;
+      lo[h] = short_load<EARLY>(w + g / 2);
+      if (all) hi[h] = short_load<EARLY>(w + g / 2 + 1);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i < 2 || all) pat[h][i] = short_load<EARLY>(pattern + g + i);
+    }
+  }
   uint32_t word = 0;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int co = mt * kTileM + row + 8 * h;
     uint32_t out[4] = {0u, 0u, 0u, 0u};
     uint32_t codes = 0x4444u;
-    if (co < d.C_out && b < geo.kblocks && c < d.C_in) {
-      const int64_t g = ((int64_t)co * geo.taps + tap) * (d.C_in / 4) + c / 4;
-      const bool all = c + 8 < d.C_in;  // (input channels come in multiples of eight)
-      const uint4 lo = w[g / 2];
-      const uint4 hi = all ? w[g / 2 + 1] : make_uint4(0u, 0u, 0u, 0u);
-      const uint2 v[4] = {make_uint2(lo.x, lo.y), make_uint2(lo.z, lo.w), make_uint2(hi.x, hi.y), make_uint2(hi.z, hi.w)};
+    if (in && co < d.C_out) {
+      const uint2 v[4] = {make_uint2(lo[h].x, lo[h].y), make_uint2(lo[h].z, lo[h].w), make_uint2(hi[h].x, hi[h].y),
+                          make_uint2(hi[h].z, hi[h].w)};
       codes = 0;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const uint32_t code = (i < 2 || all) ? pattern_code(pattern[g + i]) : 0x4u;
+        const uint32_t code = (i < 2 || all) ? pattern_code(pat[h][i]) : 0x4u;
         codes |= code << (4 * i);
         // bytes 2 p, 2 p + 1 of the group for each kept position p
         const uint32_t p0 = code & 3u, p1 = code >> 2;
@@ -343,10 +364,13 @@ cudaError_t launch_select(int mode, const void* scores, int64_t G, uint8_t* patt
   const int T = 256;
   count_launch();
   if (mode == SSCONV_MASK_LOGITS_F32)
-    return launch_short(select_logits_kernel, blocks_for(G, T), T, st, (const float2*)scores, G, pattern);
+    return launch_short(select_logits_kernel<true>, select_logits_kernel<false>, kEarlyBlocksLogits, blocks_for(G, T), T, st,
+                        (const float2*)scores, G, pattern);
   if (mode == SSCONV_MASK_MAGNITUDE_E4M3)
-    return launch_short(select_magnitude_e4m3_kernel, blocks_for(G, T), T, st, (const uint32_t*)scores, G, pattern);
-  return launch_short(select_magnitude_kernel, blocks_for(G, T), T, st, (const uint2*)scores, G, pattern);
+    return launch_short(select_magnitude_e4m3_kernel<true>, select_magnitude_e4m3_kernel<false>, kEarlyBlocks, blocks_for(G, T),
+                        T, st, (const uint32_t*)scores, G, pattern);
+  return launch_short(select_magnitude_kernel<true>, select_magnitude_kernel<false>, kEarlyBlocks, blocks_for(G, T), T, st,
+                      (const uint2*)scores, G, pattern);
 }
 
 // All N-subsets of {0..M-1} in lexicographic order of the kept positions, as bitmasks.
@@ -402,8 +426,8 @@ cudaError_t launch_quantize_e4m3(const void* x, void* y, int64_t n, float scale,
   count_launch();
   const bool wide = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u) == 0;
   const int64_t pairs = n / 2, vectors = wide ? n / 16 : 0;
-  return launch_short(quantize_e4m3_kernel, blocks_for(vectors + (pairs - 8 * vectors), T), T, st, (const uint32_t*)x,
-                          (uint16_t*)y, vectors, pairs, scale);
+  return launch_short(quantize_e4m3_kernel<true>, quantize_e4m3_kernel<false>, kEarlyBlocks,
+                      blocks_for(vectors + (pairs - 8 * vectors), T), T, st, (const uint32_t*)x, (uint16_t*)y, vectors, pairs, scale);
 }
 
 cudaError_t launch_compress_e4m3(const ssconv_desc_t& d, const void* w, const uint8_t* pattern, void* w_comp, void* meta,
@@ -437,8 +461,9 @@ cudaError_t launch_compress(const ssconv_desc_t& d, const void* w, const uint8_t
   Geometry geo = make_geometry(d);
   const int T = 256;
   count_launch();
-  return launch_short(compress_kernel, blocks_for((int64_t)geo.m_tiles * geo.stages * 512, T), T, st, d, geo, (const uint4*)w,
-                          pattern, (uint4*)w_comp, (uint32_t*)meta);
+  return launch_short(compress_kernel<true>, compress_kernel<false>, kEarlyBlocks,
+                      blocks_for((int64_t)geo.m_tiles * geo.stages * 512, T), T, st, d, geo, (const uint4*)w, pattern,
+                      (uint4*)w_comp, (uint32_t*)meta);
 }
 
 cudaError_t launch_decompress(const ssconv_desc_t& d, const void* w_comp, const void* meta, void* w_out,

@@ -22,9 +22,10 @@ __device__ __forceinline__ void block_from_choice(const float (&z)[6], float (&b
   b[3] = z[2] + z[4] + z[5];
 }
 
+template <bool EARLY>
 __device__ __forceinline__ void load6(const float* p, int64_t g, float (&v)[6]) {
   const float2* q = reinterpret_cast<const float2*>(p) + 3 * g;
-  const float2 a = q[0], b = q[1], c = q[2];
+  const float2 a = short_load<EARLY>(q), b = short_load<EARLY>(q + 1), c = short_load<EARLY>(q + 2);
   v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y; v[4] = c.x; v[5] = c.y;
 }
 __device__ __forceinline__ void store6(float* p, int64_t g, const float (&v)[6]) {
@@ -42,17 +43,18 @@ __device__ __forceinline__ uint32_t f32_pair_to_bf16(float lo, float hi) {
 
 // Eq. 3 in fp32: z = softmax((logits + noise) / tau), evaluated with the maximum subtracted
 // (which cancels in the quotient); then b = D z and W_eff = b .* W rounded once to bf16.
+template <bool EARLY>
 __global__ void soft_mask_kernel(const float* logits, const float* noise, float inv_tau, const uint2* w, int64_t G,
                                  float* z_out, uint2* w_eff) {
-  grid_launch_dependents();
+  short_begin<EARLY>();
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  grid_dependency_wait();
+  short_wait<EARLY>();
   if (g >= G) return;
   float s[6];
-  load6(logits, g, s);
+  load6<EARLY>(logits, g, s);
   if (noise != nullptr) {
     float n[6];
-    load6(noise, g, n);
+    load6<EARLY>(noise, g, n);
 #pragma unroll
     for (int i = 0; i < 6; ++i) s[i] += n[i];
   }
@@ -72,7 +74,7 @@ __global__ void soft_mask_kernel(const float* logits, const float* noise, float 
   if (w_eff != nullptr) {
     float b[4];
     block_from_choice(z, b);
-    const uint2 v = w[g];
+    const uint2 v = short_load<EARLY>(w + g);
     uint2 o;
     o.x = f32_pair_to_bf16(b[0] * bf16_bits_to_f32(v.x & 0xFFFFu), b[1] * bf16_bits_to_f32(v.x >> 16));
     o.y = f32_pair_to_bf16(b[2] * bf16_bits_to_f32(v.y & 0xFFFFu), b[3] * bf16_bits_to_f32(v.y >> 16));
@@ -82,16 +84,17 @@ __global__ void soft_mask_kernel(const float* logits, const float* noise, float 
 
 // Chain rule from G = dL/dW_eff to the choice weights: dL/db_j = G_j W_j, dL/dz_i = the sum of
 // dL/db over the two positions pattern i keeps, dL/dlogit_i = z_i (dL/dz_i - sum_k z_k dL/dz_k) / tau.
+template <bool EARLY>
 __global__ void mask_grad_kernel(const float* z_in, float inv_tau, const uint2* w, const float4* g_w_eff, int64_t G,
                                  float* g_logits) {
-  grid_launch_dependents();
+  short_begin<EARLY>();
   const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  grid_dependency_wait();
+  short_wait<EARLY>();
   if (g >= G) return;
   float z[6];
-  load6(z_in, g, z);
-  const uint2 v = w[g];
-  const float4 up = g_w_eff[g];
+  load6<EARLY>(z_in, g, z);
+  const uint2 v = short_load<EARLY>(w + g);
+  const float4 up = short_load<EARLY>(g_w_eff + g);
   const float gb0 = up.x * bf16_bits_to_f32(v.x & 0xFFFFu), gb1 = up.y * bf16_bits_to_f32(v.x >> 16);
   const float gb2 = up.z * bf16_bits_to_f32(v.y & 0xFFFFu), gb3 = up.w * bf16_bits_to_f32(v.y >> 16);
   const float gz[6] = {gb0 + gb1, gb0 + gb2, gb0 + gb3, gb1 + gb2, gb1 + gb3, gb2 + gb3};
@@ -113,13 +116,15 @@ __device__ __forceinline__ void adamw_one(float& t, float g, float& m, float& v,
   v = beta2 * v + (1.0f - beta2) * g * g;
   t = t - lr * (m * c1 / (sqrtf(v * c2) + eps) + wd * t);
 }
-// Four elements per thread (16-byte accesses); the last n % 4 elements are handled one by one.
+// Four elements per thread (16-byte accesses); the last n % 4 elements are handled one by one.  (Plain loads in both
+// forms: with read-only ones the arithmetic was contracted in another way, and its last bits differed.)
+template <bool EARLY>
 __global__ void adamw_kernel(float* theta, const float* g, float* m, float* v, int64_t n, float lr, float beta1, float beta2,
                              float eps, float wd, float c1, float c2) {
-  grid_launch_dependents();
+  short_begin<EARLY>();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t n4 = n >> 2;
-  grid_dependency_wait();
+  short_wait<EARLY>();
   if (i < n4) {
     float4 t = reinterpret_cast<float4*>(theta)[i];
     const float4 gi = reinterpret_cast<const float4*>(g)[i];
@@ -146,8 +151,8 @@ cudaError_t launch_adamw(float* theta, const float* g, float* m, float* v, int64
   const int threads = 256;
   const int64_t work = (n >> 2) + (n & 3);
   count_launch();
-  return launch_short(adamw_kernel, (unsigned)((work + threads - 1) / threads), threads, st, theta, g, m, v, n, lr, beta1,
-                          beta2, eps, wd, c1, c2);
+  return launch_short(adamw_kernel<true>, adamw_kernel<false>, kEarlyBlocks, (unsigned)((work + threads - 1) / threads),
+                      threads, st, theta, g, m, v, n, lr, beta1, beta2, eps, wd, c1, c2);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -324,12 +329,13 @@ __global__ void __launch_bounds__(256) dgrad_class_weights_kernel(const uint16_t
 //   w_all[k C_in + ci][u_h][u_w][co] = w[co][a + (Jh - 1 - u_h) s_h][b + (Jw - 1 - u_w) s_w][ci]  (0 past KH, KW).
 // One launch instead of s_h s_w small ones; the zero taps cost multiply-adds (16 tap-classes for the 9
 // taps of a 3x3 stride-2 layer, against 36 for the zero-spread form).
+template <bool EARLY>
 __global__ void __launch_bounds__(256) dgrad_fused_weights_kernel(const uint16_t* w, uint16_t* w_all,
                                                                   int C_out, int KH, int KW, int C_in, int Jh, int Jw,
                                                                   int sh, int sw) {
   // A block transposes one 32 (ci) x 32 (co) tile of one (class, tap): reads run along ci, writes along co.
   __shared__ uint16_t tile[32][33];
-  grid_launch_dependents();
+  short_begin<EARLY>();
   int z = blockIdx.z;
   const int uw = z % Jw;
   z /= Jw;
@@ -340,11 +346,11 @@ __global__ void __launch_bounds__(256) dgrad_fused_weights_kernel(const uint16_t
   const bool tap = kh < KH && kw < KW;
   const int ci0 = blockIdx.x * 32, co0 = blockIdx.y * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
-  grid_dependency_wait();
+  short_wait<EARLY>();
 #pragma unroll
   for (int r = ty; r < 32; r += 8) {
     const int co = co0 + r, ci = ci0 + tx;
-    tile[r][tx] = (tap && co < C_out && ci < C_in) ? w[(((int64_t)co * KH + kh) * KW + kw) * C_in + ci] : (uint16_t)0;
+    tile[r][tx] = (tap && co < C_out && ci < C_in) ? short_load<EARLY>(w + (((int64_t)co * KH + kh) * KW + kw) * C_in + ci) : (uint16_t)0;
   }
   __syncthreads();
 #pragma unroll
@@ -360,8 +366,8 @@ cudaError_t launch_dgrad_fused_weights(const void* w, void* w_all, int C_out, in
   if (C_in == 0 || C_out == 0) return cudaSuccess;
   const dim3 grid((unsigned)((C_in + 31) / 32), (unsigned)((C_out + 31) / 32), (unsigned)(sh * sw * Jh * Jw));
   count_launch();
-  return launch_short(dgrad_fused_weights_kernel, grid, 256, st, (const uint16_t*)w, (uint16_t*)w_all, C_out, KH, KW, C_in,
-                          Jh, Jw, sh, sw);
+  return launch_short(dgrad_fused_weights_kernel<true>, dgrad_fused_weights_kernel<false>, kEarlyBlocks, grid, 256, st,
+                      (const uint16_t*)w, (uint16_t*)w_all, C_out, KH, KW, C_in, Jh, Jw, sh, sw);
 }
 
 cudaError_t launch_dgrad_class_weights(const void* w, void* w_c, int C_out, int KH, int KW, int C_in, int a, int b,
@@ -378,11 +384,12 @@ cudaError_t launch_dgrad_class_weights(const void* w, void* w_c, int C_out, int 
 // padded position; zero for a class without taps and beyond a class tensor's extent (no filter placement
 // reaches those pixels).  `pitch8` = 16-byte units between pixels of a class tensor (C_in / 8, or the
 // channels of all classes when they share one tensor).  One thread per 16 bytes of dx.
+template <bool EARLY>
 __global__ void __launch_bounds__(256) dgrad_gather_kernel(DgradClasses cls, uint4* dx, long long total, int H,
                                                            int W, int C8, int pitch8, int sh, int sw, int ph, int pw) {
-  grid_launch_dependents();
+  short_begin<EARLY>();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  grid_dependency_wait();
+  short_wait<EARLY>();
   if (i >= total) return;
   const int c = (int)(i % C8);
   long long r = i / C8;
@@ -396,7 +403,7 @@ __global__ void __launch_bounds__(256) dgrad_gather_kernel(DgradClasses cls, uin
   uint4 v = make_uint4(0u, 0u, 0u, 0u);
   const uint4* t = static_cast<const uint4*>(cls.t[k]);
   if (t != nullptr && ih < cls.rows[k] && iw < cls.cols[k])
-    v = t[((n * cls.rows[k] + ih) * cls.cols[k] + iw) * pitch8 + c];
+    v = short_load<EARLY>(t + ((n * cls.rows[k] + ih) * cls.cols[k] + iw) * pitch8 + c);
   dx[i] = v;
 }
 
@@ -405,8 +412,8 @@ cudaError_t launch_dgrad_gather(const DgradClasses& cls, void* dx, int N, int H,
   const long long total = (long long)N * H * W * (C / 8);
   if (total == 0) return cudaSuccess;
   count_launch();
-  return launch_short(dgrad_gather_kernel, (unsigned)((total + 255) / 256), 256, st, cls, (uint4*)dx, total, H, W, C / 8,
-                          pitch / 8, sh, sw, ph, pw);
+  return launch_short(dgrad_gather_kernel<true>, dgrad_gather_kernel<false>, kEarlyBlocks, (unsigned)((total + 255) / 256), 256,
+                      st, cls, (uint4*)dx, total, H, W, C / 8, pitch / 8, sh, sw, ph, pw);
 }
 
 cudaError_t launch_soft_mask(const float* logits, const float* noise, float tau, const void* w, int64_t G, float* z,
@@ -414,8 +421,8 @@ cudaError_t launch_soft_mask(const float* logits, const float* noise, float tau,
   const int threads = 256;
   const int64_t blocks = (G + threads - 1) / threads;
   count_launch();
-  return launch_short(soft_mask_kernel, (unsigned)blocks, threads, st, logits, noise, 1.0f / tau, (const uint2*)w, G, z,
-                          (uint2*)w_eff);
+  return launch_short(soft_mask_kernel<true>, soft_mask_kernel<false>, kEarlyBlocks, (unsigned)blocks, threads, st, logits, noise,
+                      1.0f / tau, (const uint2*)w, G, z, (uint2*)w_eff);
 }
 
 cudaError_t launch_mask_grad(const float* z, float tau, const void* w, const float* g_w_eff, int64_t G,
@@ -423,8 +430,8 @@ cudaError_t launch_mask_grad(const float* z, float tau, const void* w, const flo
   const int threads = 256;
   const int64_t blocks = (G + threads - 1) / threads;
   count_launch();
-  return launch_short(mask_grad_kernel, (unsigned)blocks, threads, st, z, 1.0f / tau, (const uint2*)w,
-                          (const float4*)g_w_eff, G, g_logits);
+  return launch_short(mask_grad_kernel<true>, mask_grad_kernel<false>, kEarlyBlocks, (unsigned)blocks, threads, st, z, 1.0f / tau,
+                      (const uint2*)w, (const float4*)g_w_eff, G, g_logits);
 }
 
 }  // namespace ssconv
