@@ -8,6 +8,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 
 #include "launch.cuh"
@@ -705,12 +706,15 @@ __global__ void __launch_bounds__(256) layernorm_vec_kernel(const uint4* x, cons
   }
 }
 
-// The same for few pixels (a turn or a few per warp of the chip): the scale and shift are loaded with the first pixels, not
-// after their statistics, which is a latency less, and stay in registers for a warp's further pixels, whose loads are in
-// flight meanwhile.  us, the kernel above / this one: 3 x 56 x 56 x 96 2.7 / 2.2, 3 x 14 x 14 x 384 2.5 / 2.0, 16 x 14 x 14 x
-// 384 3.5 / 3.0 (one turn), 128 x 7 x 7 x 768 6.5 / 5.3 (3 turns); beyond the line 128 x 14 x 14 x 384 9.1 / 9.8 (5), 128 x 56 x
-// 56 x 96 29.8 / 35.4 (17): its 110 registers leave too few warps to keep memory busy.
-constexpr long long kLnFewTurns = 3;
+// The same for few pixels (a turn or a few per warp of the chip) of two to four pieces per lane: the scale and shift are
+// loaded with the first pixels, not after their statistics, which is a latency less, and stay in registers (86, 120 and 148 by
+// the pieces: five, four and three blocks per SM) for a warp's further pixels, whose loads are in flight meanwhile.  us, the
+// kernel above / this one, between launches of itself: 384 channels (three pieces), half a turn 4.0 / 3.1, one 4.2 / 3.2,
+// two 4.4 / 4.2, three 6.6 / 5.2, and beyond the line five 9.1 / 9.8; 1024 channels (four), half a turn 4.0 / 3.2, two 5.5 /
+// 4.3, three 7.2 / 5.4.  Before two pointwise layers, all three: 512 channels (two pieces), half a turn 12.8 / 12.5, one 15.6 /
+// 14.6, two 18.3 / 18.1, and beyond the line 2.1 turns 19.1 / 19.7; one piece (64, 128, 256 channels) within 4 % either way,
+// half a turn 13.1 / 12.7, 12.6 / 12.9, 12.0 / 11.1, a third 11.6 / 11.8, 11.6 / 11.7, 10.2 / 10.6: not worth a form.
+constexpr long long ln_few_turns(int V) { return V == 1 ? 0 : V == 2 ? 2 : 3; }
 template <int V>
 __global__ void __launch_bounds__(128) layernorm_few_kernel(const uint4* x, const float* gamma, const float* beta, uint4* y,
                                                             long long pixels, int C8, int G, float eps) {
@@ -795,6 +799,21 @@ __global__ void __launch_bounds__(128) layernorm_few_kernel(const uint4* x, cons
   }
 }
 
+// Blocks of layernorm_few_kernel<V> that an SM holds (asked once per device and form: seven, five and four were assumed, and
+// a grid of three turns ran in more waves; 1024 channels at 2.4 turns 5.35 us in the kernel above, 6.26 then, 5.41 now).
+using LnFewKernel = void (*)(const uint4*, const float*, const float*, uint4*, long long, int, int, float);
+static int layernorm_few_blocks(LnFewKernel kernel, int V) {
+  static std::atomic<int> known[64][5];
+  int dev = 0, blocks = 0;
+  const bool keep = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64;
+  if (keep) blocks = known[dev][V].load(std::memory_order_relaxed);
+  if (blocks == 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, 128, 0) != cudaSuccess || blocks <= 0) blocks = 1;
+    if (keep) known[dev][V].store(blocks, std::memory_order_relaxed);
+  }
+  return blocks;
+}
+
 cudaError_t launch_layernorm(const void* x, const float* gamma, const float* beta, void* y, long long pixels, int C,
                              float eps, cudaStream_t st) {
   if (pixels == 0) return cudaSuccess;
@@ -816,16 +835,15 @@ cudaError_t launch_layernorm(const void* x, const float* gamma, const float* bet
     const long long warps = (pixels + (32 / G) - 1) / (32 / G);
     const uint4* xp = static_cast<const uint4*>(x);
     uint4* yp = static_cast<uint4*>(y);
-    // blocks of four warps, as many as are resident at once, every warp with the same number of turns (or one fewer)
-    const long long most = 4ll * (V <= 2 ? 7 : V == 3 ? 5 : 4) * device_sms();
-    const long long turns = (warps + most - 1) / most;
-    if (turns <= kLnFewTurns) {
-      const unsigned few = (unsigned)(((warps + turns - 1) / turns + 3) / 4);
-      const auto kernel = V == 1   ? layernorm_few_kernel<1>
-                          : V == 2 ? layernorm_few_kernel<2>
-                          : V == 3 ? layernorm_few_kernel<3>
-                                   : layernorm_few_kernel<4>;
-      return launch_dependent(kernel, few, 128, st, xp, gamma, beta, yp, pixels, C8, G, eps);
+    // blocks of four warps, at most as many as are resident at once, every warp with the same number of turns (or one fewer)
+    if (V > 1) {
+      const auto few_kernel = V == 2 ? layernorm_few_kernel<2> : V == 3 ? layernorm_few_kernel<3> : layernorm_few_kernel<4>;
+      const long long most = 4ll * layernorm_few_blocks(few_kernel, V) * device_sms();
+      const long long turns = (warps + most - 1) / most;
+      if (turns <= ln_few_turns(V)) {
+        const unsigned few = (unsigned)(((warps + turns - 1) / turns + 3) / 4);
+        return launch_dependent(few_kernel, few, 128, st, xp, gamma, beta, yp, pixels, C8, G, eps);
+      }
     }
     const unsigned grid = (unsigned)((warps * 32 + T - 1) / T);
     const auto kernel = V == 1   ? layernorm_vec_kernel<1>
