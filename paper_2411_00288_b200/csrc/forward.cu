@@ -2732,9 +2732,31 @@ int32_t launch_forward_dense(const ssconv_desc_t& d, const void* x, const void* 
   return launch_forward_impl<false>(d, x, w, nullptr, bias, residual, y, ws, ws_bytes, dev_status, stream, kMaxWorkers,
                                     false, x_strides, 1.0f, 0, 1, gradient_weights);
 }
-// Whether launch_forward_dense takes the weights of the layer whose input gradient `d` computes as they are (the 8-channel
-// mode cuts its k-blocks across taps).
-bool takes_gradient_weights(const ssconv_desc_t& d) { return !small_channel_mode(d, false); }
+// Whether launch_forward_dense takes the weights of the layer whose input gradient `d` computes as they are.  Not in the
+// 8-channel mode, which cuts its k-blocks across taps.  And not where their rows, C_out bf16 values each, start between two
+// 32-byte sectors and a CTA has many k-blocks of them to bring in: each then takes some 0.1 us longer than from rearranged
+// weights with aligned rows (d.C_in % 16 == 0), less where those are unaligned too, more with at most 40 rows, where a k-block
+// of rearranged ones is that many rows and of these 64.  Rearranging takes 3 us, once.  us, rearranged first / as they are
+// (images x height x channels of the layer -> its output channels, filter; k-blocks per CTA):
+//   aligned        32 x 54 x 72 -> 256, 3 (108)  48.1 / 55.2    16 x 28 x 72 -> 512, 3 (72)  21.9 / 26.2    8 x 54 x 72 -> 256, 3 (36)
+//                  19.2 / 18.9
+//   unaligned      8 x 54 x 72 -> 280, 5 (83)  68.2 / 72.1      15 x 35 x 56 -> 200, 5 (52)  51.2 / 43.4
+//   at most 40     25 x 20 x 24 -> 480, 3 (72)  20.4 / 23.6     5 x 37 x 40 -> 1872, 1 (30)  12.3 / 14.9    64 x 28 x 40 -> 64, 3 (18)
+//                  20.9 / 18.5                                  13 x 39 x 40 -> 1512, 3 (121, unaligned)  80.2 / 92.8
+//   several channel tiles  32 x 28 x 200 -> 256, 3  38.2 / 35.8, 67 x 43 x 456 -> 224, 3  218 / 220
+//   rows of whole sectors  32 x 56 x 96 -> 384, 3 (162)  77.3 / 76.6, 54 x 63 x 48 -> 104, 5 (350)  229 / 207
+bool takes_gradient_weights(const ssconv_desc_t& d) {
+  if (small_channel_mode(d, false)) return false;
+  if (d.C_out % 16 == 0 || d.C_out > kTileM) return true;
+  int32_t bn = 0, split = 0, ctas = 0;
+  if (plan_query(d, false, &bn, &split, &ctas, nullptr, nullptr) != SSCONV_OK || bn <= 0 || ctas <= 0) return true;
+  const Geometry geo = layer_geometry(d, false);
+  const long long Q = (long long)d.N * out_extent(d.H, d.KH, d.stride_h, d.pad_h, d.dil_h) *
+                      out_extent(d.W, d.KW, d.stride_w, d.pad_w, d.dil_w);
+  const long long tiles = (Q + bn - 1) / bn;
+  const long long per_cta = split ? tiles * geo.kblocks / ctas : (tiles + ctas - 1) / ctas * geo.kblocks;
+  return per_cta <= (d.C_in % 16 == 0 ? 40 : 64) / (d.C_out <= 40 ? 2 : 1);
+}
 
 // Groups of a grouped convolution in one launch: what the model says of all groups' tiles dealt out together
 // against one launch per group (each of which may split K or use pairs, and starts and drains by itself).  A group's last

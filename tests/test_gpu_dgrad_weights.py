@@ -19,6 +19,8 @@ DGRAD = [
     ("pairs",           32, 28, 28, 256, 192, 3, 1, 1, 1),
     ("few_tiles",       1, 7,  7,  128, 512, 3, 1, 1, 1),
     ("spread",          2, 14, 14, 64,  72,  3, 2, 1, 2),
+    ("unaligned_long",  16, 28, 28, 72, 512, 3, 1, 1, 1),     # (rows between sectors, a long K: rearranged first)
+    ("unaligned_short", 5, 37, 37, 40,  512, 1, 1, 0, 1),
 ]
 
 
@@ -31,7 +33,11 @@ def test_dgrad_reads_the_layers_own_weights(case):
     wt = (torch.randn((co, k, k, ci), generator=g) / (k * k * co) ** 0.5).to(torch.bfloat16).to(DEV)
     dy = torch.randn((n, ho, wo, co), generator=g).to(torch.bfloat16).to(DEV)
     status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    launches = api.ssconv_launch_count()
     dx = api.ssconv_dgrad(desc, dy, wt, dev_status=status)
+    launches = api.ssconv_launch_count() - launches
+    if name.startswith("unaligned"):
+        assert launches == (2 if name == "unaligned_long" else 1)
     # every output pixel's gradient at the pixels that it was computed from, one matrix product per tap
     ref = torch.zeros((n, h + 2 * p, w + 2 * p, ci), dtype=torch.float64, device=DEV)
     for a in range(k):
