@@ -1202,7 +1202,9 @@ __global__ void __launch_bounds__(kFinishThreads) ssconv_split_finish_kernel(con
 // summed over the CTAs in rank order by 128 threads that read the peers' rings directly, and finished like a split tile.
 // Against the split over the whole grid there is no second launch (3 us of the caller's time, 2 us on the GPU) and no
 // scratch in global memory; against whole tiles the K loop is 2 to 8 times shorter.  Nothing waits for a CTA outside the
-// cluster, whose CTAs the hardware starts together.  The residual is read by the finishing threads.
+// cluster, whose CTAs the hardware starts together, nor do two clusters of different grids wait for each other's tensor
+// memory: this kernel's registers (118 x 384 threads), those of the pair kernel (102 and more x 384 or 448) and of the weight
+// gradient's (143 x 256) leave an SM room for one such CTA at a time.  The residual is read by the finishing threads.
 // Shared memory: ring, three 2-KB staging buffers (one per 128 threads), barriers.
 constexpr int kClusterThreads = kThreads;                          // 384: three sets of 128 finishing threads
 constexpr uint32_t kClusterStageBytes = 3u * 2048u;
@@ -2153,16 +2155,21 @@ constexpr double kPairAdvantage = 1.05;  // the pair kernel only if the model pr
 //                          3 x 7 x 3072 -> 768, 1   6.9 / 7.4 -> 6.2 / 7.4
 //     beyond the line      8 x 7 x 512 -> 264, 3 (9 groups per CTA)  7.8 / 8.1 -> 7.6 / 9.1,  1 x 28 x 512 -> 128, 1 (4 groups in
 //                          all)  3.9 / 4.6 -> 4.4 / 4.9
+//   dense layers of 10 to 15 groups and few tiles, 4 CTAs -> 8 (split over the grid)   7 x 12 x 160 -> 80, 3 (2)  6.4 -> 5.7 (6.1)
+//                          3 x 6 x 392 -> 72, 2  6.5 -> 5.8 (6.1)    16 x 2 x 1256 -> 176, 1  6.3 -> 5.8 (6.1)    12 tiles: 3 x 11 x
+//                          1376 -> 144, 1  6.1 -> 6.6 (6.4);  8 groups: 17 x 6 x 992 -> 40, 1  5.7 -> 6.0
 //   2 CTAs                 8 x 14 x 256 -> 256, 3  7.7 / 9.0 -> 7.4 / 9.1,  27 x 7 x 512 -> 512, 3  11.6 / 13.5 -> 11.2 / 14.0,
 //                          27 x 7 x 2048 -> 512, 1  7.6 / 10.2 -> 8.0 / 9.4: not worth a rule
 // (groups = pairs of k-blocks).  Of the widths, 48 where it covers the positions with fewer columns.
 constexpr int kClusterMinGroups = 8, kCluster8MinGroups = 16, kCluster8MaxGroups = 72, kCluster4MaxGroups = 24;
+constexpr int kCluster8MinGroupsDense = 10;
 // Clusters that the chip holds at once: its SMs come in groups that are no multiple of the cluster, so that a few stay out.
 static int max_clusters(int workers, int size) { return workers / size - (size == 8 ? 4 : size == 4 ? 3 : 2); }
 static int cluster_ring_groups(uint32_t a_group_bytes, int BN) {
   const int n = (int)((kMaxSmemBytes - 1024 - kBarrierBytes - kClusterStageBytes) / group_bytes(a_group_bytes, BN));
   return n > kMaxGroups ? kMaxGroups : n;
 }
+template <bool SPARSE>
 static Plan plan_cluster(long long Q, const Geometry& geo, int workers) {
   Plan none{0, false};
   // (an override of the width or of the pairs asks for the kernels that it is about)
@@ -2174,7 +2181,9 @@ static Plan plan_cluster(long long Q, const Geometry& geo, int workers) {
     if (g_tune_bn != 0) c.BN = g_tune_bn;
     return geo.stages < c.cluster || ((Q + c.BN - 1) / c.BN) * geo.m_tiles > max_clusters(workers, c.cluster) ? none : c;
   }
-  if (geo.stages >= kCluster8MinGroups && geo.stages <= kCluster8MaxGroups && tiles64 <= max_clusters(workers, 8)) {
+  const bool deep = geo.stages >= kCluster8MinGroups && tiles64 <= max_clusters(workers, 8);
+  const bool few = !SPARSE && geo.stages >= kCluster8MinGroupsDense && 2 * tiles64 <= max_clusters(workers, 8);
+  if ((deep || few) && geo.stages <= kCluster8MaxGroups) {
     c.cluster = 8;
     return c;
   }
@@ -2254,7 +2263,7 @@ template <bool SPARSE>
 static Plan choose_plan(const ssconv_desc_t& d, long long Q, const Geometry& geo, int workers, bool force_split,
                         bool allow_split = true, bool allow_wide = true, bool allow_pair = true, bool allow_cluster = true) {
   if (allow_cluster && !force_split && !small_channel_mode(d, SPARSE)) {
-    const Plan c = plan_cluster(Q, geo, workers);
+    const Plan c = plan_cluster<SPARSE>(Q, geo, workers);
     if (c.cluster != 0) return c;
   }
   const Plan plan = plan_layer<SPARSE>(Q, geo, workers, force_split, kBN, 2, allow_split);
@@ -2388,7 +2397,7 @@ static int32_t launch_forward_impl(const ssconv_desc_t& d, const void* x, const 
   // (a grouped layer's own launches per group keep the split over the grid)
   const bool allow_cluster = !FP8 && !force_split && !small_c && groups == 1 && y_pitch == 0;
   Plan plan{0, false};
-  if (allow_cluster) plan = plan_cluster(Q, geo, workers);
+  if (allow_cluster) plan = plan_cluster<SPARSE>(Q, geo, workers);
   if (plan.cluster == 0)
     plan = groups > 1 ? choose_plan<SPARSE>(d, Q, geo, workers, false, false, false, false, false)
            : (residual != nullptr || (FP8 && !SPARSE))

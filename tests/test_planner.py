@@ -58,6 +58,21 @@ def test_never_more_blocks_than_sms_and_scaling_with_the_sm_count():
         assert 1 <= p["ctas"] <= sms
 
 
+@pytest.mark.parametrize("layer, sparse, per_tile", [
+    ((3, 6, 392, 72, 2), False, 8),     # dense, 14 groups of k-blocks, 3 tiles: eight blocks share a tile's K,
+    ((3, 6, 392, 72, 2), True, 4),      # four in the 2:4 form, half of whose bytes a group brings in,
+    ((3, 11, 1376, 144, 1), False, 4),  # with 12 tiles,
+    ((17, 6, 992, 40, 1), False, 4),    # and with 8 groups
+], ids=["dense_few_tiles", "sparse", "dense_more_tiles", "dense_8_groups"])
+def test_blocks_that_share_the_k_of_a_tile(layer, sparse, per_tile):
+    n, h, c_in, c_out, k = layer
+    desc = api.make_desc(n, h, h, c_in, c_out, k, k, pad=k // 2)
+    p = api.ssconv_plan_for_sms(desc, sparse, SMS)
+    extent = h + 2 * (k // 2) - k + 1
+    tiles = -(-n * extent ** 2 // p["tile_positions"]) * -(-c_out // 128)
+    assert p["split"] and p["ctas"] == per_tile * tiles, p
+
+
 def test_window_extent_is_the_output_extent_formula():
     for cfg in (1, 2, 3, 4, 5):
         for s in synth.config_layers(cfg):
