@@ -14,6 +14,23 @@ from tests import parity
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
+
+@pytest.fixture
+def no_small_maps():
+    """Small maps on the tensor-core kernel, as larger ones are."""
+    api.ssconv_tune(api.TUNE_DEPTHWISE_SMALL, 0)
+    yield
+    api.ssconv_tune(api.TUNE_DEPTHWISE_SMALL, -1)
+
+
+@pytest.fixture(params=[0, -1], ids=["tensor_cores", "small_maps"])
+def either_kernel(request):
+    """Small maps on the tensor-core kernel, whose bands meet pixels outside an output's window, and on their own."""
+    api.ssconv_tune(api.TUNE_DEPTHWISE_SMALL, request.param)
+    yield
+    api.ssconv_tune(api.TUNE_DEPTHWISE_SMALL, -1)
+
+
 CASES = [  # N, H, W, C, pad, relu
     (1, 7, 7, 32, 0, False),      # one output
     (1, 1, 1, 32, 3, True),       # one pixel
@@ -57,16 +74,12 @@ def test_depthwise7_on_the_fp32_kernels(case):
 
 
 @pytest.mark.parametrize("case", CASES, ids=["x".join(map(str, c[:4])) + f"_p{c[4]}" for c in CASES])
-def test_depthwise7_without_the_kernel_for_small_maps(case):
+def test_depthwise7_without_the_kernel_for_small_maps(case, no_small_maps):
     # (most of the maps above are small: the tensor-core kernel at the edges of its own tiles)
-    api.ssconv_tune(api.TUNE_DEPTHWISE_SMALL, 0)
-    try:
-        _check_case(case)
-    finally:
-        api.ssconv_tune(api.TUNE_DEPTHWISE_SMALL, -1)
+    _check_case(case)
 
 
-@pytest.mark.parametrize("case", [
+SMALL_CASES = [
     (1, 4, 8, 32, 3, False),      # one tile exactly
     (2, 5, 9, 64, 3, True),       # one row and one column more
     (1, 10, 14, 32, 0, False),    # no padding: the tile's pixels are the map
@@ -74,16 +87,17 @@ def test_depthwise7_without_the_kernel_for_small_maps(case):
     (2, 1, 1, 960, 6, True),      # many channels, windows mostly outside
     (37, 14, 14, 160, 3, False),  # 1480 blocks: the most
     (38, 14, 14, 160, 3, False),  # (one image more: the tensor-core kernel)
-], ids=lambda c: "x".join(map(str, c[:4])) + f"_p{c[4]}")
+]
+
+
+@pytest.mark.parametrize("case", SMALL_CASES, ids=lambda c: "x".join(map(str, c[:4])) + f"_p{c[4]}")
 def test_depthwise7_on_small_maps(case):
-    if case not in CASES:
-        CASES.append(case)        # (its index seeds the inputs)
     _check_case(case)
 
 
 def _check_case(case):
     N, H, W, C, pad, relu = case
-    g = torch.Generator().manual_seed(synth.SEED_BASE + 7100 + CASES.index(case))
+    g = torch.Generator().manual_seed(synth.SEED_BASE + 7100 + (CASES + SMALL_CASES).index(case))
     x = torch.randn((N, H, W, C), generator=g).to(torch.bfloat16)
     w = (torch.randn((7, 7, C), generator=g) / 7).to(torch.bfloat16)
     bias = torch.randn((C,), generator=g) * 0.1
@@ -105,7 +119,7 @@ def _check_case(case):
 
 @pytest.mark.parametrize("polls", [0, 1, 3, 40])
 @pytest.mark.parametrize("case", [(17, 9, 8, 2560, 3, False), (24, 28, 28, 64, 3, True), (9, 27, 30, 160, 3, False)])
-def test_depthwise7_computes_everything_again_when_waits_run_out(case, polls):
+def test_depthwise7_computes_everything_again_when_waits_run_out(case, polls, no_small_maps):
     # (0: all waits give up; more: some warps of a block may give up and others not)
     N, H, W, C, pad, relu = case
     g = torch.Generator(device=DEV).manual_seed(synth.SEED_BASE + 7990)
@@ -124,7 +138,7 @@ def test_depthwise7_computes_everything_again_when_waits_run_out(case, polls):
         assert not torch.equal(y, ref)                                             # (computed another way: some roundings differ)
 
 
-def test_depthwise7_non_finite_pixels_reach_their_own_windows_only():
+def test_depthwise7_non_finite_pixels_reach_their_own_windows_only(either_kernel):
     N, H, W, C = 2, 20, 19, 64
     g = torch.Generator().manual_seed(synth.SEED_BASE + 7200)
     x = torch.randn((N, H, W, C), generator=g).to(torch.bfloat16)
@@ -176,7 +190,7 @@ def test_depthwise7_sums_are_as_exact_as_fp32_ones(data):
 
 @pytest.mark.parametrize("relu", [False, True], ids=["none", "relu"])
 @pytest.mark.parametrize("with_bias", [False, True], ids=["no_bias", "bias"])
-def test_depthwise7_non_finite_outputs_are_those_of_the_fp32_kernel(relu, with_bias):
+def test_depthwise7_non_finite_outputs_are_those_of_the_fp32_kernel(relu, with_bias, either_kernel):
     N, H, W, C = 3, 22, 25, 64
     g = torch.Generator(device=DEV).manual_seed(synth.SEED_BASE + 7250)
     x = torch.randn((N, H, W, C), generator=g, device=DEV).to(torch.bfloat16)

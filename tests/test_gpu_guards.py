@@ -3,8 +3,8 @@
 Guard bands: outputs and scratch buffers are carved out of larger allocations whose slack on both
 sides holds a sentinel pattern; after the calls the slack must be untouched.  Covered: the output of
 the one-block kernel (TMA stores, ragged channels and positions), of the K-split path (finishing
-kernel), of the pair kernel (tests/test_gpu_pair.py), the forward workspace and the weight gradient's
-scratch and output.
+kernel), of the cluster kernel, of the pair kernel (tests/test_gpu_pair.py), the forward workspace and the
+scratch and output of both weight-gradient kernels.
 
 Bounded wait: every mbarrier wait in the library gives up after a cycle limit, raises a flag and lets
 the kernel return with SSCONV_ERR_TIMEOUT in the caller's status word.  No product kernel is broken to
@@ -68,22 +68,82 @@ def test_forward_touches_neither_the_slack_around_y_nor_around_ws(case, sparse):
         assert bool((ws != 0x5A).any()), "the split path parks partial tiles in ws"
 
 
-def test_weight_gradient_touches_neither_the_slack_around_dw_nor_around_its_scratch():
-    spec = synth.LayerSpec("guard_wgrad", 4, 14, 14, 72, 136, 3, 3, 1, 1, 1, config=11, index=60)
-    inp = synth.make_inputs(spec, x_only=True)
-    tr = synth.make_train_inputs(spec)
-    desc = api.desc_from_spec(spec)
-    n_dw = spec.C_out * spec.K * 4
+@pytest.mark.parametrize("case", [
+    ("pairs", 4, 14, 14, 72, 136, 3, 1),                  # 3 x 3: thread-block pairs
+    ("one_tile", 7, 19, 23, 72, 72, 1, 0),                # pointwise: the one-block kernel, whose results leave by bulk copies,
+    ("ragged_two_tiles", 48, 33, 35, 40, 200, 1, 0),      # with items of two channel tiles
+    ("ragged_three_tiles", 100, 57, 56, 72, 328, 1, 0),   # and of three
+], ids=lambda c: c[0])
+def test_weight_gradient_touches_neither_the_slack_around_dw_nor_around_its_scratch(case):
+    name, n, h, w, ci, co, k, p = case
+    g = torch.Generator(device=DEV).manual_seed(synth.SEED_BASE + 60 + len(name))
+    desc = api.make_desc(n, h, w, ci, co, k, k, pad=p, bias=False)
+    x = torch.randn((n, h, w, ci), generator=g, device=DEV).to(torch.bfloat16)
+    dy = torch.randn((n, h, w, co), generator=g, device=DEV).to(torch.bfloat16)
+    n_dw = co * k * k * ci * 4
     dwbuf, dwmid = _banded(n_dw)
-    dw = dwmid.view(torch.float32).view(spec.C_out, spec.KH, spec.KW, spec.C_in)
+    dw = dwmid.view(torch.float32).view(co, k, k, ci)
     need = api.ssconv_wgrad_ws_bytes(desc)
+    if name.startswith("ragged"):   # items of all channel tiles: more ranges of positions than items of one would leave
+        tiles = -(-co // 128)
+        assert need // (tiles * 128 * ci * 4) > torch.cuda.get_device_properties(0).multi_processor_count // tiles
     wsbuf, ws = _banded(max(need, 256))
     status = torch.zeros(1, dtype=torch.int32, device=DEV)
-    api.ssconv_wgrad(desc, inp.x.to(DEV), tr.dy.to(DEV), dw=dw, ws=ws, dev_status=status)
+    api.ssconv_wgrad(desc, x, dy, dw=dw, ws=ws, dev_status=status)
     torch.cuda.synchronize()
     assert int(status.item()) == 0
     assert _bands_intact(dwbuf, n_dw) and _bands_intact(wsbuf, max(need, 256))
-    assert bool(torch.isfinite(dw).all())
+    xp = torch.nn.functional.pad(x, (0, 0, p, p, p, p)).double()
+    for a in range(k):
+        for b in range(k):
+            ref = dy.reshape(-1, co).double().T @ xp[:, a:a + h, b:b + w].reshape(-1, ci)
+            assert float((dw[:, a, b].double() - ref).norm() / ref.norm()) <= 1e-4
+
+
+def _cluster_layer(name, index, n, c_out):
+    """What a call of a layer needs whose tiles' K the blocks of clusters share: x, descriptor, packed weights, bias."""
+    spec = synth.LayerSpec(name, n, 7, 7, 512, c_out, 3, 3, 1, 1, 1, relu=True, w_std="fan_in", mask_source="magnitude",
+                           config=14, index=index)
+    inp = synth.make_inputs(spec)
+    desc = api.desc_from_spec(spec)
+    plan = api.ssconv_plan(desc, True)
+    tiles = -(-spec.P // plan["tile_positions"]) * -(-c_out // 128)
+    assert plan["split"] and plan["ctas"] == 8 * tiles, plan
+    return inp.x.to(DEV), desc, api.ssconv_compress(desc, inp.w.to(DEV), parity.gpu_pattern(inp, DEV)), inp.bias.to(DEV)
+
+
+def test_clusters_stay_inside_y_and_add_a_residual_in_place():
+    x, desc, packed, bias = _cluster_layer("cluster_guard", 10, 3, 264)        # 147 positions, 8 channels in the last tile
+    shape = (3, 7, 7, 264)
+    n_out = 3 * 49 * 264 * 2
+    ybuf, ymid = _banded(n_out)
+    y = ymid.view(torch.bfloat16).view(shape)
+    status = torch.zeros(1, dtype=torch.int32, device=DEV)
+    res = torch.randn(shape, generator=torch.Generator().manual_seed(3)).to(torch.bfloat16).to(DEV)
+    api.ssconv_forward(desc, x, *packed, bias, y=y, dev_status=status)
+    torch.cuda.synchronize()
+    assert _bands_intact(ybuf, n_out)
+    apart = api.ssconv_forward(desc, x, *packed, bias, residual=res, dev_status=status)
+    y.copy_(res)
+    api.ssconv_forward(desc, x, *packed, bias, y=y, residual=y, dev_status=status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    assert torch.equal(y, apart) and _bands_intact(ybuf, n_out)
+
+
+def test_clusters_on_two_streams_do_not_disturb_each_other():
+    # (an SM holds one of their blocks at a time: no two clusters can wait for each other's share of tensor memory)
+    ctx = [_cluster_layer("cluster_a", 11, 1, 512), _cluster_layer("cluster_b", 12, 4, 256)]
+    streams = [torch.cuda.Stream(device=DEV) for _ in ctx]
+    alone = [api.ssconv_forward(desc, x, *packed, bias) for x, desc, packed, bias in ctx]
+    torch.cuda.synchronize()
+    outs = [[torch.empty_like(a) for _ in range(12)] for a in alone]
+    for it in range(12):
+        for (x, desc, packed, bias), o, stream in zip(ctx, outs, streams):
+            api.ssconv_forward(desc, x, *packed, bias, y=o[it], stream=stream)
+    torch.cuda.synchronize()
+    for a, o in zip(alone, outs):
+        assert all(torch.equal(y, a) for y in o)
 
 
 def test_bounded_wait_runs_out_returns_a_status_and_leaves_the_context_usable():
@@ -102,13 +162,16 @@ def test_bounded_wait_runs_out_returns_a_status_and_leaves_the_context_usable():
         api.ssconv_selftest_wait_timeout(10, status)       # limit below the accepted range
 
 
-def test_calls_on_two_streams_with_their_own_scratch_do_not_disturb_each_other():
+def test_calls_on_two_streams_with_their_own_scratch_do_not_disturb_each_other(request):
     """The library keeps no hidden device state between calls (the one entry point that does says so in the
     header): two layers launched again and again on two streams that overlap on the GPU, each with its own
     scratch and status word, give bit for bit what they give alone.  A K-split layer (scratch + finishing
-    kernel) on one stream, a layer for the thread-block-pair kernel on the other."""
+    kernel; clusters, which would take so few tiles, are off) on one stream, a layer for the thread-block-pair kernel on
+    the other."""
+    request.addfinalizer(lambda: api.ssconv_tune(api.TUNE_CLUSTER, -1))
+    api.ssconv_tune(api.TUNE_CLUSTER, 0)
     specs = [synth.LayerSpec("deep_k_split", 2, 7, 7, 512, 128, 3, 3, 1, 1, 1, config=14, index=0),
-             synth.LayerSpec("pair_3x3", 8, 14, 14, 256, 256, 3, 3, 1, 1, 1, config=14, index=1)]
+             synth.LayerSpec("pair_3x3", 128, 14, 14, 256, 256, 3, 3, 1, 1, 1, config=14, index=1)]
     ctx = []
     for spec in specs:
         inp = synth.make_inputs(spec)
@@ -128,8 +191,12 @@ def test_calls_on_two_streams_with_their_own_scratch_do_not_disturb_each_other()
     alone = []
     for c in ctx:
         y = torch.empty((c["desc"].N, *api.ssconv_out_shape(c["desc"]), c["desc"].C_out), dtype=torch.bfloat16, device=DEV)
+        c["ws"].fill_(0x5A)
+        torch.cuda.synchronize()
         run(c, y)
         torch.cuda.synchronize()
+        assert api.ssconv_plan(c["desc"])["pair"] == (c is ctx[1])
+        assert bool((c["ws"] != 0x5A).any()) == (c is ctx[0])      # (only the split layer writes its scratch)
         alone.append(y.clone())
     outs = [[torch.empty_like(a) for _ in range(12)] for a in alone]
     for it in range(12):

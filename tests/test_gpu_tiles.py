@@ -34,20 +34,32 @@ def test_tile_width_sweep(hw, sparse):
     assert rel <= parity.REL_FRO_TOL and mx <= parity.MAX_ABS_TOL, f"{spec.name} {plan}: rel={rel:.3e} max={mx:.3e}"
 
 
-def test_split_plan_deep_k_few_tiles():
-    """512 -> 256 channels on 7x7 maps: few tiles, deep K: the K range is split and a second kernel finishes."""
+def test_split_plan_deep_k_few_tiles(request):
+    """512 -> 256 channels on 7x7 maps: few tiles, deep K: the K range is split over the grid and a second kernel finishes
+    (with clusters off: they would take a layer of so few tiles)."""
     spec = synth.LayerSpec("split_7x7", 8, 7, 7, 512, 256, 3, 3, 1, 1, 1, relu=True, w_std="fan_in",
                            mask_source="magnitude", config=8, index=20)
     desc = api.desc_from_spec(spec)
+    request.addfinalizer(lambda: api.ssconv_tune(api.TUNE_CLUSTER, -1))
+    api.ssconv_tune(api.TUNE_CLUSTER, 0)
+    inp = synth.make_inputs(spec)
+    x, w, bias = inp.x.to(DEV), inp.w.to(DEV), inp.bias.to(DEV)
+    packed = api.ssconv_compress(desc, w, parity.gpu_pattern(inp, DEV))
     for sparse in (True, False):
         plan = api.ssconv_plan(desc, sparse)
         assert plan["split"], plan
-        c0 = api.ssconv_launch_count()
         rel, mx = parity.check_layer(spec, DEV, sparse=sparse)
         assert rel <= parity.REL_FRO_TOL and mx <= parity.MAX_ABS_TOL, f"split {sparse}: rel={rel:.3e} max={mx:.3e}"
         rel, mx = parity.check_layer(spec, DEV, sparse=sparse, residual=True)  # the finishing kernel adds it
         assert rel <= parity.REL_FRO_TOL and mx <= parity.MAX_ABS_TOL, f"split+res {sparse}: rel={rel:.3e} max={mx:.3e}"
-        assert api.ssconv_launch_count() - c0 >= 2  # main + finishing kernel (+ select/compress when sparse)
+        ws = torch.full((api.ssconv_sizes(desc).ws_bytes_sparse,), 0x5A, dtype=torch.uint8, device=DEV)
+        c0 = api.ssconv_launch_count()
+        if sparse:
+            api.ssconv_forward(desc, x, *packed, bias, ws=ws)
+        else:
+            api.ssconv_forward_dense(desc, x, w, bias, ws=ws)
+        assert api.ssconv_launch_count() - c0 == 2       # main and finishing kernel
+        assert bool((ws != 0x5A).any())                  # partial tiles
 
 
 def test_zz_sweep_covered_several_widths():
