@@ -367,8 +367,9 @@ int32_t ssconv_wgrad(const ssconv_desc_t* desc, const void* x, const void* dy, f
  * no gradient):  dx[n,h,w,ci] = sum over (kh,kw,co) of dy[n,ho,wo,co] * w[co,kh,kw,ci]  for the outputs
  * (ho,wo) whose tap (kh,kw) read pixel (h,w).  dy: bf16 [N,H_out,W_out,C_out], w: bf16 [C_out,KH,KW,C_in],
  * dx: bf16 [N,H,W,C_in] (every element is written), all device, 16-byte aligned; one rounding to bf16.
- * With unit stride it is one convolution of dy with the reversed, channel-exchanged filter (as
- * ssconv_dgrad_prepare + ssconv_forward_dense).  With a stride s > 1 the input pixels are split into the
+ * With unit stride it is one convolution of dy with the reversed, channel-exchanged filter (what
+ * ssconv_dgrad_prepare + ssconv_forward_dense compute; the layer's own weights are read in that order, or written
+ * to scratch in it first where that is faster).  With a stride s > 1 the input pixels are split into the
  * s_h x s_w residue classes of their padded position: a pixel with (h + pad) mod s = a only met the taps
  * kh = a, a + s, ..., so each class is a unit-stride convolution of dy with its own few taps (all classes
  * together carry the layer's KH x KW taps, where ssconv_dgrad_spread makes every input pixel meet all of
@@ -376,8 +377,8 @@ int32_t ssconv_wgrad(const ssconv_desc_t* desc, const void* x, const void* dy, f
  * by a gather kernel.  Strided layers with a dilation other than 1 or a stride above 4 take the plain route
  * instead (dy spread out with zeros as by ssconv_dgrad_spread, into scratch, then one convolution).
  * The flags of desc are ignored (no bias, no activation).
- * ws: device scratch of ssconv_dgrad_ws_bytes(desc) bytes (reversed weights; per class its weights and
- * tensor, or the spread gradient), too small -> SSCONV_ERR_WORKSPACE.  SSCONV_ERR_UNSUPPORTED_SHAPE: padding
+ * ws: device scratch of ssconv_dgrad_ws_bytes(desc) bytes (room for the reversed weights; per class its weights
+ * and tensor, or the spread gradient; the convolution's own), too small -> SSCONV_ERR_WORKSPACE.  SSCONV_ERR_UNSUPPORTED_SHAPE: padding
  * beyond the filter's reach, C_out % 8 != 0. */
 int32_t ssconv_dgrad_ws_bytes(const ssconv_desc_t* desc, size_t* bytes);
 int32_t ssconv_dgrad(const ssconv_desc_t* desc, const void* dy, const void* w_bf16, void* dx, void* ws, size_t ws_bytes,

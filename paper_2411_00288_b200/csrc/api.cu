@@ -785,7 +785,8 @@ struct DgradPlan {
 size_t round256(size_t v) { return (v + 255) & ~size_t(255); }
 
 // Shape rules and workspace layout: per class its weights [C_in, Ja, Jb, C_out] and its tensor
-// [N, Ho + Ja - 1, Wo + Jb - 1, C_in]; with unit stride only the reversed weights.
+// [N, Ho + Ja - 1, Wo + Jb - 1, C_in]; with unit stride, and for the spread form, room for the reversed weights, which are
+// only written where the convolution does not read the layer's own (takes_gradient_weights): the size does not depend on it.
 int32_t dgrad_plan(const ssconv_desc_t& d, DgradPlan* p) {
   if (d.C_out % 8 != 0) return SSCONV_ERR_UNSUPPORTED_SHAPE;  // dy's channels are the convolutions' input channels
   if (d.dil_h * (d.KH - 1) < d.pad_h || d.dil_w * (d.KW - 1) < d.pad_w) return SSCONV_ERR_UNSUPPORTED_SHAPE;

@@ -533,9 +533,8 @@ depthwise7_mma_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_con
 // neighbouring outputs of one pair of channels from shared memory with fp32 multiply-adds, a filter row at a time (each row a
 // chain of its own, added to the sum: rms error in the units above .109 / .469 / .448).  Bound by that one latency and 196
 // multiply-adds per thread while the blocks are resident at once; every pixel is loaded 4.4 times, so larger maps are not
-// for it.us between other
-// launches, tensor-core kernel / this one: 3 x 56 x 56 x 96 9.3 / 5.8, 3 x 28 x 28 x 192 8.8 / 4.5, 3 x 14 x 14 x 384 8.8 / 3.2,
-// 3 x 7 x 7 x 768 8.1 / 2.6; with 64 threads of eight outputs each 5.6, 4.5, 3.4, 3.3.
+// for it.  us between other launches, tensor-core kernel / this one: 3 x 56 x 56 x 96 9.3 / 5.8, 3 x 28 x 28 x 192 8.8 / 4.5,
+// 3 x 14 x 14 x 384 8.8 / 3.2, 3 x 7 x 7 x 768 8.1 / 2.6; with 64 threads of eight outputs each 5.6, 4.5, 3.4, 3.3.
 constexpr int kDwSmallH = 4, kDwSmallW = 8, kDwSmallRun = 4;
 constexpr int kDwSmallThreads = 16 * kDwSmallH * (kDwSmallW / kDwSmallRun);
 constexpr int kDwSmallRows = kDwSmallH + kDw7K - 1, kDwSmallCols = kDwSmallW + kDw7K - 1;
@@ -683,10 +682,10 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Blocks of depthwise7_small_kernel for a map, and the most that it is used for.  us, tensor-core kernel /
+// Blocks of depthwise7_small_kernel for a map, and the most per SM that it is used for.  us on 148 SMs, tensor-core kernel /
 // small: 1152 blocks 12 x 14 x 14 x 384 9.7 / 6.9, 1536 blocks 32 x 7 x 7 x 768 8.5 / 8.3, 1764 blocks 6 x 56 x 56 x 96 10.0 /
 // 10.1, 2304 blocks 24 x 14 x 14 x 384 10.5 / 11.7.
-constexpr long long kDwSmallMaxBlocks = 10 * 148;
+constexpr int kDwSmallMaxBlocksPerSm = 10;
 static long long depthwise7_small_blocks(int N, int C, int Ho, int Wo) {
   return (long long)N * ((Ho + kDwSmallH - 1) / kDwSmallH) * ((Wo + kDwSmallW - 1) / kDwSmallW) * (C / kDw7Channels);
 }
@@ -797,7 +796,7 @@ bool launch_depthwise7(const void* x, const void* w, const float* bias, void* y,
                        int KH, int KW, int stride, int pad, int dil, uint32_t flags, int32_t polls, cudaStream_t st,
                        cudaError_t* result) {
   if (polls < 0 && KH == kDw7K && KW == kDw7K && stride == 1 && dil == 1 && C % kDw7Channels == 0 && g_tune_mma != 0 &&
-      g_tune_small != 0 && depthwise7_small_blocks(N, C, Ho, Wo) <= kDwSmallMaxBlocks) {
+      g_tune_small != 0 && depthwise7_small_blocks(N, C, Ho, Wo) <= kDwSmallMaxBlocksPerSm * device_sms()) {
     Dw7Params p{};
     p.x = static_cast<const uint32_t*>(x);
     p.w = static_cast<const uint32_t*>(w);

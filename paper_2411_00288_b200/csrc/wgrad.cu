@@ -619,7 +619,7 @@ bool g_wg_attr_set[64] = {false};
 int g_tune_wg_ranges = 0;   // 0: the planner chooses; otherwise an upper limit on the position ranges
 int g_tune_wg_pair = -1;    // -1: the planner chooses; 0: one-CTA kernel only; 1: the pair kernel wherever it applies
 
-constexpr int kWgMinSteps2 = 5, kWgMinSteps3 = 32;  // steps per range for items of two (per k-block) and of three channel tiles
+constexpr int kWgMinSteps2 = 5, kWgMinSteps3 = 32;  // steps per SM for items of two (per k-block) and of three channel tiles
 
 // How a layer's weight gradient is cut into work items.
 struct WgPlan {
@@ -664,14 +664,18 @@ WgPlan wg_plan(const ssconv_desc_t& d, int sms, bool one_tile = false) {  // (on
   w.items_b = (w.kblocks + w.T - 1) / w.T;
   w.m_tiles = (d.C_out + kTileM - 1) / kTileM;
   w.ksteps = (int)((w.Q + kWgPos - 1) / kWgPos);
-  // Split the positions when the items alone would leave SMs idle, but keep at least 8 steps per
-  // range so that the pipeline's ramp and the epilogue stay small against the loop.
-  // Several channel tiles per item where the ranges stay long enough: an item then brings the activations in once for all
-  // its tiles, but as many ranges as SMs each write their accumulators, M times as much to add up as with one tile per item.
-  // us, one tile per item / M: 128 x 56 x 56 x 96 -> 384 (M 3, 42 steps per range) 74.4 / 71.7, 64 images (21 steps) 40.8 /
-  // 44.0, 256 images 144.8 / 129.0; M 2: 16 x 56 x 56 x 64 -> 256 (5 steps) 12.7 / 11.7, 32 images 19.3 / 14.8, 256 images 97.3 /
-  // 87.4, 64 x 28 x 28 x 128 -> 512 (10 steps) 19.6 / 16.4, 64 x 14 x 14 x 128 -> 1024 (two
-  // k-blocks, 5 steps) 13.9 / 14.8, 100 x 30 x 30 x 40 -> 200 16.7 / 13.8.
+  // Several channel tiles per item where there are positions enough: an item then brings the activations in once for all
+  // its tiles, but each range writes M times the accumulators of an item of one tile, to be added up.  The line is drawn at
+  // steps x items / SMs, the steps per range if there were as many ranges as SMs; at its lower end the limit of eight steps per
+  // range (below) leaves fewer.  us, one tile per item / M tiles (steps per SM; ranges):
+  //   M 2   16 x 56 x 56 x 64 -> 256 (5; 98) 12.7 / 11.7, 32 images (11; 143) 19.3 / 14.8, 256 images (85; 148) 97.3 / 87.4, 64 x 28
+  //         x 28 x 128 -> 512 (11; 72) 19.6 / 16.4, 100 x 30 x 30 x 40 -> 200 (10; 141) 16.7 / 13.8; beyond the line, two k-blocks 64
+  //         x 14 x 14 x 128 -> 1024 (5; 22) 13.9 / 14.8
+  //   M 3   three tiles 128 x 56 x 56 x 96 -> 384 (42; 146) 74.4 / 71.7, 104 images -> 328 (34; 146) 69.6 / 60.1, 256 images (85)
+  //         144.8 / 129.0; five 60 images -> 640 (40; 74) 69.6 / 55.7, 64 images of 64 channels (42; 73) 66.3 / 53.4; seven 48 images ->
+  //         896 (48; 49) 72.1 / 58.4 (the places for an eighth and a ninth tile multiply zeros); beyond the line 64 images of 96 -> 384
+  //         (21) 40.8 / 44.0
+  // (the figures of three and more tiles but the first and the last compare the kernel before and after items of M tiles).
   w.M = 1;
   w.items_m = w.m_tiles;
   if (w.T <= 2 && w.m_tiles > 1 && !one_tile) {
@@ -682,6 +686,8 @@ WgPlan wg_plan(const ssconv_desc_t& d, int sms, bool one_tile = false) {  // (on
     }
   }
   const int items = w.items_m * w.items_b;
+  // Split the positions when the items alone would leave SMs idle, but keep at least 8 steps per
+  // range so that the pipeline's ramp and the epilogue stay small against the loop.
   int splits = sms / items;
   if (splits > w.ksteps / 8) splits = w.ksteps / 8;
   if (g_tune_wg_ranges > 0 && splits > g_tune_wg_ranges) splits = g_tune_wg_ranges;
