@@ -45,7 +45,7 @@ MIN_REGIONS = 30       # timed regions of --steps steps each; the median is repo
 # DRAM bytes of one step of the stack at batch 256, from the ncu counters summarised in
 # profiles/bench_resnet50_stack_dram_traffic.md; valid for the kernels whose sources hash to `sources`
 # (anything else reports null: the counters would have to be taken again).
-STACK_TRAFFIC = {"batch": 256, "read": 4518895616, "write": 5835668736, "sources": "d52e97fb8f841f07"}
+STACK_TRAFFIC = {"batch": 256, "read": 4518220544, "write": 5834922240, "sources": "7499c9ad41a6cde0"}
 TRAFFIC_SOURCES = ("paper_2411_00288_b200/csrc/forward.cu", "paper_2411_00288_b200/csrc/pool.cu",
                    "paper_2411_00288_b200/csrc/sm100_ptx.cuh", "paper_2411_00288_b200/csrc/layout.cuh",
                    "paper_2411_00288_b200/stack.py")
